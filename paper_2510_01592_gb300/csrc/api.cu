@@ -302,7 +302,7 @@ uint64_t map_footprint(const vm_map_params& p, const vm_segment_params& sp) {
     uint64_t nb = 1;
     for (int a = 0; a < 3; ++a) nb *= (uint64_t)((p.dims[a] + kBrick - 1) / kBrick);
     const uint64_t cap = p.brick_capacity && p.brick_capacity < nb ? p.brick_capacity : nb;
-    const uint64_t pool = nb * 4 + cap * 4 + cap * kBrickVox * (3 * 8 + 4) + cap * (kBrickVox / 8) +
+    const uint64_t pool = nb * 4 + cap * 4 + cap * kBrickVox * (3 * 8 + 4) + cap * 2 * (kBrickVox / 8) +
                           scroll_tmp_words((uint32_t)cap) * 4 + 4096;
     const uint64_t bricks = (nb + 1) * 4 + nb * 4 + cap * 8 + 4096;
     const size_t nv = (size_t)cap * kBrickVox;
@@ -730,6 +730,7 @@ vm_status vm_create(const vm_map_params* params, void* cuda_stream, vm_map** out
     dry.take<uint32_t>((size_t)m->capacity * kBrickVox);
     dry.take<MapCounters>(1);
     dry.take<uint32_t>((size_t)m->capacity * (kBrickVox / 32));
+    dry.take<uint32_t>((size_t)m->capacity * (kBrickVox / 32));
     dry.take<uint32_t>(4);
     dry.take<uint32_t>(scroll_tmp_words(m->capacity));
     dry.take<float>(4);
@@ -744,6 +745,7 @@ vm_status vm_create(const vm_map_params* params, void* cuda_stream, vm_map** out
     m->S = c.take<unsigned long long>((size_t)m->capacity * 3 * kBrickVox);
     m->C = c.take<uint32_t>((size_t)m->capacity * kBrickVox);
     m->ctr = c.take<MapCounters>(1);
+    m->occ = c.take<uint32_t>((size_t)m->capacity * (kBrickVox / 32));
     m->mark = c.take<uint32_t>((size_t)m->capacity * (kBrickVox / 32));
     m->err = c.take<uint32_t>(4);
     m->scroll_tmp = c.take<uint32_t>(scroll_tmp_words(m->capacity));
@@ -794,6 +796,7 @@ vm_status vm_reset(vm_map* m) {
     VM_CUDA(cudaMemsetAsync(m->S, 0, (size_t)m->capacity * 3 * kBrickVox * sizeof(unsigned long long), m->stream));
     VM_CUDA(cudaMemsetAsync(m->C, 0, (size_t)m->capacity * kBrickVox * sizeof(uint32_t), m->stream));
     VM_CUDA(cudaMemsetAsync(m->ctr, 0, sizeof(MapCounters), m->stream));
+    VM_CUDA(cudaMemsetAsync(m->occ, 0, (size_t)m->capacity * (kBrickVox / 32) * sizeof(uint32_t), m->stream));
     VM_CUDA(cudaMemsetAsync(m->mark, 0, (size_t)m->capacity * (kBrickVox / 32) * sizeof(uint32_t), m->stream));
     m->segmented = false;
     return VM_OK;
@@ -830,7 +833,7 @@ vm_status vm_scroll(vm_map* m, const int32_t shift[3]) {
     const float po2[3] = {(float)((double)g2.ox + (double)g2.ax / 1048576.0),
                           (float)((double)g2.oy + (double)g2.ay / 1048576.0),
                           (float)((double)g2.oz + (double)g2.az / 1048576.0)};
-    VM_CUDA(launch_scroll(m->g, g2, shift, po2, m->brick_table, m->nb_total, m->slot_key, m->S, m->C, m->ctr,
+    VM_CUDA(launch_scroll(m->g, g2, shift, po2, m->brick_table, m->nb_total, m->slot_key, m->S, m->C, m->occ, m->ctr,
                           m->capacity, m->scroll_tmp, m->stream));
     m->g = g2;
     return VM_OK;
@@ -918,12 +921,13 @@ vm_status vm_integrate_ex(vm_map* m, const float* xyz, uint32_t n, const float p
     StageHook* hk = m->fit.timer.hook();
     if (flags & VM_INTEGRATE_CLEAR) {
         VM_STAGE_BEGIN(hk, kStClear, m->stream);
-        VM_CUDA(launch_clear(d, n, P, m->g, m->brick_table, m->S, m->C, m->mark, m->ctr, m->capacity, m->stream));
+        VM_CUDA(launch_clear(d, n, P, m->g, m->brick_table, m->S, m->C, m->occ, m->mark, m->ctr, m->capacity,
+                             m->stream));
         VM_STAGE_END(hk, kStClear, m->stream);
     }
     VM_TRY(ensure(m->deferred, (size_t)n * sizeof(uint32_t)));
     VM_STAGE_BEGIN(hk, kStIntegrate, m->stream);
-    VM_CUDA(launch_integrate(d, n, P, m->g, m->brick_table, m->slot_key, m->S, m->C,
+    VM_CUDA(launch_integrate(d, n, P, m->g, m->brick_table, m->slot_key, m->S, m->C, m->occ,
                              static_cast<uint32_t*>(m->deferred.p), m->ctr, m->capacity, m->stream));
     VM_STAGE_END(hk, kStIntegrate, m->stream);
     return VM_OK;

@@ -4,7 +4,8 @@
 // Storage: a direct-indexed brick table (one int32 per 8^3-voxel brick of the
 // grid) maps a brick to a slot of a pool allocated on first touch.  A slot
 // holds, per voxel, the exact fixed-point coordinate sums S (int64, 2^-20 m
-// units relative to the window's anchor) and the point count C.  Eq. 1's
+// units relative to the window's anchor) and the point count C, and one bit
+// (occ) that says whether C > 0.  Eq. 1's
 // running mean is the ratio S / C, independent of the order the points arrive
 // in, so concurrent updates need only integer atomics.
 //
@@ -70,9 +71,11 @@ __device__ __forceinline__ Keyed key_point(const float* __restrict__ xyz, uint32
 // runs of consecutive lanes, a spinning LiDAR's beams interleave); each
 // group's integer sums are reduced and its lowest lane issues the group's
 // atomics (64-bit sums sign-extended: a group's sum is negative when its
-// points lie a quantum below the window's anchor).
+// points lie a quantum below the window's anchor).  occ: one bit per voxel
+// slot, set where C > 0.
 __device__ __forceinline__ void accumulate_warp(uint32_t key, int32_t v0, int32_t v1, int32_t v2,
-                                                unsigned long long* __restrict__ S, uint32_t* __restrict__ C) {
+                                                unsigned long long* __restrict__ S, uint32_t* __restrict__ C,
+                                                uint32_t* __restrict__ occ) {
     if (!__any_sync(0xffffffffu, key != kNone)) return;  // nothing in this warp lands in the map
     const uint32_t grp = __match_any_sync(0xffffffffu, key);
     const int32_t s0 = __reduce_add_sync(grp, v0), s1 = __reduce_add_sync(grp, v1), s2 = __reduce_add_sync(grp, v2);
@@ -83,6 +86,9 @@ __device__ __forceinline__ void accumulate_warp(uint32_t key, int32_t v0, int32_
         atomicAdd(s + kBrickVox, (unsigned long long)(long long)s1);
         atomicAdd(s + 2 * kBrickVox, (unsigned long long)(long long)s2);
         atomicAdd(C + key, (uint32_t)__popc(grp));
+        // the occupancy bit: a plain read, and an atomic only on a voxel's first points
+        const uint32_t bit = 1u << (key & 31);
+        if (!(__ldcg(occ + (key >> 5)) & bit)) atomicOr(occ + (key >> 5), bit);
     }
 }
 
@@ -111,8 +117,8 @@ __device__ __forceinline__ void count_points(uint32_t n_ok, uint32_t n_bad, uint
 __global__ void __launch_bounds__(kThreads) k_accum(const float* __restrict__ xyz, uint32_t n, Pose P, Grid g,
                                                    int32_t* __restrict__ table, int32_t* __restrict__ slot_key,
                                                    unsigned long long* __restrict__ S, uint32_t* __restrict__ C,
-                                                   uint32_t* __restrict__ deferred, MapCounters* __restrict__ ctr,
-                                                   uint32_t capacity) {
+                                                   uint32_t* __restrict__ occ, uint32_t* __restrict__ deferred,
+                                                   MapCounters* __restrict__ ctr, uint32_t capacity) {
     pdl_gate();
     const int lane = threadIdx.x & 31;
     const uint32_t warp_global = (blockIdx.x * kThreads + threadIdx.x) >> 5;
@@ -155,7 +161,7 @@ __global__ void __launch_bounds__(kThreads) k_accum(const float* __restrict__ xy
                 ++n_bad;
             }
         }
-        accumulate_warp(key, v0, v1, v2, S, C);
+        accumulate_warp(key, v0, v1, v2, S, C, occ);
     }
     count_points(n_ok, n_bad, n_full, ctr);
 }
@@ -165,7 +171,7 @@ __global__ void __launch_bounds__(kThreads) k_accum(const float* __restrict__ xy
 __global__ void __launch_bounds__(kThreads) k_accum_deferred(const float* __restrict__ xyz, Pose P, Grid g,
                                                             const int32_t* __restrict__ table,
                                                             unsigned long long* __restrict__ S,
-                                                            uint32_t* __restrict__ C,
+                                                            uint32_t* __restrict__ C, uint32_t* __restrict__ occ,
                                                             const uint32_t* __restrict__ deferred,
                                                             MapCounters* __restrict__ ctr) {
     pdl_gate();
@@ -189,7 +195,7 @@ __global__ void __launch_bounds__(kThreads) k_accum_deferred(const float* __rest
                 ++n_full;
             }
         }
-        accumulate_warp(key, v0, v1, v2, S, C);
+        accumulate_warp(key, v0, v1, v2, S, C, occ);
     }
     count_points(n_ok, 0, n_full, ctr);
     __threadfence();
@@ -211,16 +217,30 @@ __global__ void __launch_bounds__(kThreads) k_accum_deferred(const float* __rest
 // checked that the sensor is inside the grid.  An occupied voxel on the walk
 // gets its bit in the mark bitmap (a plain read skips the atomic when the bit
 // is already set).
+//
+// The walk is bound by instruction issue (a camera frame at 0.01 m takes about
+// 80 M steps), so it runs in two parts.  The first carries no test for the end
+// of an axis or of the grid: while the smallest boundary parameter lies below
+// thr, no axis can have passed its end (the boundary behind the end voxel has
+// parameter >= 1) or left the grid (the grid's face has its own), as thr stays
+// below both by more than the parameters' rounding (a parameter is a sum of at
+// most dims terms near 1, each addition and the increment itself rounded by
+// 2^-24; the margin is four times that).  A lane steps until it leaves the
+// cell whose occupancy it holds -- a whole brick while the brick is not
+// allocated, else one word of its bitmap (8 x 4 voxels of one z layer) -- so a
+// warp looks cells up once per several steps instead of whenever one of its
+// lanes crosses a border.  Coordinates are mirrored on falling axes (u = 8 m + 7
+// - q), which makes every step + 1 and every cell border a zero of its low
+// bits.  The second part takes the last steps with the tests.
 __global__ void __launch_bounds__(kThreads) k_clear_mark(const float* __restrict__ xyz, uint32_t n, Pose P, Grid g,
                                                         const int32_t* __restrict__ table,
-                                                        const uint32_t* __restrict__ C, uint32_t* mark,
+                                                        const uint32_t* __restrict__ occ, uint32_t* mark,
                                                         MapCounters* __restrict__ ctr) {
     pdl_gate();
+    const float inf = __int_as_float(0x7f800000);
     const float s[3] = {__fmul_rn(__fsub_rn(P.r[3], g.ox), g.inv_res), __fmul_rn(__fsub_rn(P.r[7], g.oy), g.inv_res),
                         __fmul_rn(__fsub_rn(P.r[11], g.oz), g.inv_res)};
-    const int dims[3] = {g.nx, g.ny, g.nz};
-    const int w0 = g.wx, w1 = g.wy, w2 = g.wz;
-    const long long cap = (long long)g.nx + g.ny + g.nz + 3;  // a walk inside the grid is never longer
+    const float margin = (float)(max(g.nx, max(g.ny, g.nz)) + 16) * 2.384185791015625e-07f;  // 2^-22
     for (uint32_t i = blockIdx.x * kThreads + threadIdx.x; i < n; i += gridDim.x * kThreads) {
         const float x = xyz[3 * (size_t)i + 0], y = xyz[3 * (size_t)i + 1], z = xyz[3 * (size_t)i + 2];
         float e[3];
@@ -235,80 +255,111 @@ __global__ void __launch_bounds__(kThreads) k_clear_mark(const float* __restrict
         for (int a = 0; a < 3; ++a) fin &= isfinite(e[a]) && fabsf(e[a]) < 1073741824.0f;
         if (!fin) continue;
         // Per-axis state in scalars (an array indexed by the chosen axis would
-        // live in local memory).  Keys fit in int32: the sensor is inside the
-        // grid and |e| < 2^30.
-        int v0, v1, v2, e0i, e1i, e2i, st0, st1, st2;
-        float t0, t1, t2, dl0, dl1, dl2;
-        auto axis = [](float sa, float ea, int& va, int& vea, int& sta, float& ta, float& dla) {
-            va = (int)floorf(sa);
-            vea = (int)floorf(ea);
+        // live in local memory): u the mirrored window coordinate, end the
+        // point's, lim the first one outside the grid, flip the mirror (q = u
+        // or flip - u), t the next boundary's parameter (infinite when the walk
+        // does not move on this axis).  Keys fit in int32: the sensor is inside
+        // the grid and |e| < 2^30.
+        int u0, u1, u2, end0, end1, end2, lim0, lim1, lim2, flip0, flip1, flip2;
+        float t0, t1, t2, dl0, dl1, dl2, thr = 1.0f;
+        auto axis = [&](float sa, float ea, int w, int dim, int& u, int& end, int& lim, int& flip, float& t,
+                        float& dl) {
+            const int va = (int)floorf(sa), q = va - w, qe = (int)floorf(ea) - w;
             const float d = __fsub_rn(ea, sa);
+            t = dl = inf;
+            flip = 0;
+            u = q;
+            end = qe;
+            lim = dim;
             if (d > 0.0f) {
-                sta = 1;
-                ta = __fdiv_rn(__fsub_rn(__int2float_rn(va + 1), sa), d);
-                dla = __fdiv_rn(1.0f, d);
+                t = __fdiv_rn(__fsub_rn(__int2float_rn(va + 1), sa), d);
+                dl = __fdiv_rn(1.0f, d);
+                thr = fminf(thr, __fdividef(__int2float_rn(w + dim) - sa, d));
             } else if (d < 0.0f) {
-                sta = -1;
-                ta = __fdiv_rn(__fsub_rn(__int2float_rn(va), sa), d);
-                dla = __fdiv_rn(-1.0f, d);
-            } else {
-                sta = 0;
-                ta = __int_as_float(0x7f800000);
-                dla = __int_as_float(0x7f800000);
+                t = __fdiv_rn(__fsub_rn(__int2float_rn(va), sa), d);
+                dl = __fdiv_rn(-1.0f, d);
+                flip = dim | 7;
+                u = flip - q;
+                end = flip - qe;
+                lim = flip + 1;
+                thr = fminf(thr, __fdividef(__int2float_rn(w) - sa, d));
             }
+            if (q == qe) t = inf;
         };
-        axis(s[0], e[0], v0, e0i, st0, t0, dl0);
-        axis(s[1], e[1], v1, e1i, st1, t1, dl1);
-        axis(s[2], e[2], v2, e2i, st2, t2, dl2);
-        const long long l64 = llabs((long long)e0i - v0) + llabs((long long)e1i - v1) + llabs((long long)e2i - v2);
-        int left = (int)(l64 < cap ? l64 : cap);  // the walk leaves the grid first
-        uint32_t cur_brick = kNone;  // the brick of the last step and its slot: one table read per brick crossed
-        int32_t cur_slot = -1;
-        for (; left > 0; --left) {
-            const int q0 = v0 - w0, q1 = v1 - w1, q2 = v2 - w2;  // window coordinates
-            const bool gone = (q0 < 0 && st0 <= 0) || (q0 >= dims[0] && st0 >= 0) || (q1 < 0 && st1 <= 0) ||
-                              (q1 >= dims[1] && st1 >= 0) || (q2 < 0 && st2 <= 0) || (q2 >= dims[2] && st2 >= 0);
-            if (gone) break;
-            if (q0 >= 0 && q0 < dims[0] && q1 >= 0 && q1 < dims[1] && q2 >= 0 && q2 < dims[2]) {
-                const uint32_t brick =
-                    ((uint32_t)(q2 >> 3) * (uint32_t)g.nby + (uint32_t)(q1 >> 3)) * (uint32_t)g.nbx +
-                    (uint32_t)(q0 >> 3);
-                if (brick != cur_brick) {
-                    cur_brick = brick;
-                    cur_slot = table[brick];
-                }
-                if (cur_slot >= 0) {
-                    const uint32_t idx =
-                        (uint32_t)cur_slot * kBrickVox + (uint32_t)((((q2 & 7) << 3) | (q1 & 7)) << 3 | (q0 & 7));
-                    const uint32_t bit = 1u << (idx & 31);
-                    if (C[idx] && !(__ldcg(mark + (idx >> 5)) & bit)) atomicOr(mark + (idx >> 5), bit);
-                }
+        axis(s[0], e[0], g.wx, g.nx, u0, end0, lim0, flip0, t0, dl0);
+        axis(s[1], e[1], g.wy, g.ny, u1, end1, lim1, flip1, t1, dl1);
+        axis(s[2], e[2], g.wz, g.nz, u2, end2, lim2, flip2, t2, dl2);
+        thr -= margin;
+        uint32_t widx = 0, word = 0;  // the bitmap word of the cell, 0 where the brick is not allocated
+        // the cell of the walk's voxel: its word, and whether the brick is allocated
+        auto look = [&]() {
+            const int q0 = flip0 ? flip0 - u0 : u0, q1 = flip1 ? flip1 - u1 : u1, q2 = flip2 ? flip2 - u2 : u2;
+            const int32_t slot = table[((uint32_t)(q2 >> 3) * (uint32_t)g.nby + (uint32_t)(q1 >> 3)) *
+                                           (uint32_t)g.nbx + (uint32_t)(q0 >> 3)];
+            word = 0;
+            if (slot >= 0) {
+                widx = (uint32_t)slot * (kBrickVox / 32) + (uint32_t)(((q2 & 7) << 1) | ((q1 & 7) >> 2));
+                word = occ[widx];
             }
-            // the axis whose next boundary comes first, ties to x, then y, then z, among those not at the end
-            int best = -1;
-            float bt = 0.0f;
-            if (v0 != e0i) { best = 0; bt = t0; }
-            if (v1 != e1i && (best < 0 || t1 < bt)) { best = 1; bt = t1; }
-            if (v2 != e2i && (best < 0 || t2 < bt)) best = 2;
-            if (best == 0) {
-                v0 += st0;
-                t0 = __fadd_rn(t0, dl0);
-            } else if (best == 1) {
-                v1 += st1;
-                t1 = __fadd_rn(t1, dl1);
+            return slot >= 0;
+        };
+        const int mir = ((flip1 ? 3 : 0) << 3) | (flip0 ? 7 : 0);  // mirrors a voxel's place in its word
+        auto touch = [&]() {
+            const uint32_t bit = 1u << ((((u1 & 3) << 3) | (u0 & 7)) ^ mir);
+            if ((word & bit) && !(__ldcg(mark + widx) & bit)) atomicOr(mark + widx, bit);
+        };
+        float tm = fminf(t0, fminf(t1, t2));
+        while (tm < thr) {
+            const bool fine = look();
+            const int m1 = fine ? 3 : 7, m2 = fine ? 0 : 7;  // the cell: 8 x 4 x 1 or 8 x 8 x 8 voxels
+            bool inside;
+            do {
+                if (word) touch();
+                const bool p0 = t0 <= t1 && t0 <= t2, p1 = !p0 && t1 <= t2, p2 = !p0 && !p1;  // ties to x, y, z
+                inside = true;
+                if (p0) {
+                    ++u0;
+                    t0 = __fadd_rn(t0, dl0);
+                    inside = (u0 & 7) != 0;
+                }
+                if (p1) {
+                    ++u1;
+                    t1 = __fadd_rn(t1, dl1);
+                    inside = (u1 & m1) != 0;
+                }
+                if (p2) {
+                    ++u2;
+                    t2 = __fadd_rn(t2, dl2);
+                    inside = (u2 & m2) != 0;
+                }
+                tm = fminf(t0, fminf(t1, t2));
+            } while (inside && tm < thr);
+        }
+        if (u0 == end0) t0 = inf;
+        if (u1 == end1) t1 = inf;
+        if (u2 == end2) t2 = inf;
+        while (!(t0 == inf && t1 == inf && t2 == inf)) {
+            look();
+            if (word) touch();
+            if (t0 <= t1 && t0 <= t2) {
+                if (++u0 == lim0) break;
+                t0 = u0 == end0 ? inf : __fadd_rn(t0, dl0);
+            } else if (t1 <= t2) {
+                if (++u1 == lim1) break;
+                t1 = u1 == end1 ? inf : __fadd_rn(t1, dl1);
             } else {
-                v2 += st2;
-                t2 = __fadd_rn(t2, dl2);
+                if (++u2 == lim2) break;
+                t2 = u2 == end2 ? inf : __fadd_rn(t2, dl2);
             }
         }
     }
 }
 
-// Clears the marked voxels of the allocated slots (sums and count to zero)
-// and their marks; counts the cleared voxels.
+// Clears the marked voxels of the allocated slots (sums and count to zero,
+// their occupancy bits) and their marks; counts the cleared voxels.
 __global__ void __launch_bounds__(kThreads) k_clear_apply(unsigned long long* __restrict__ S, uint32_t* __restrict__ C,
-                                                         uint32_t* __restrict__ mark, MapCounters* __restrict__ ctr,
-                                                         uint32_t capacity) {
+                                                         uint32_t* __restrict__ occ, uint32_t* __restrict__ mark,
+                                                         MapCounters* __restrict__ ctr, uint32_t capacity) {
     pdl_gate();
     const uint32_t nb = min(ctr->n_bricks, capacity);
     const size_t words = (size_t)nb * (kBrickVox / 32);
@@ -317,6 +368,7 @@ __global__ void __launch_bounds__(kThreads) k_clear_apply(unsigned long long* __
         uint32_t m = mark[w];
         if (!m) continue;
         mark[w] = 0;
+        occ[w] &= ~m;
         const uint32_t slot = (uint32_t)(w / (kBrickVox / 32));
         while (m) {
             const int b = __ffs(m) - 1;
@@ -387,7 +439,7 @@ __global__ void __launch_bounds__(kThreads) k_scroll_move(const MapCounters* __r
                                                          const uint32_t* __restrict__ n_keep,
                                                          const uint32_t* __restrict__ hole, int32_t* slot_key,
                                                          int shift_key, long long dax, long long day, long long daz,
-                                                         unsigned long long* S, uint32_t* C) {
+                                                         unsigned long long* S, uint32_t* C, uint32_t* occ) {
     pdl_gate();
     const uint32_t nb = min(ctr->n_bricks, capacity), nk = *n_keep;
     const uint32_t below = nk < nb ? kpos[nk] : nk;  // kept slots below the kept count
@@ -406,6 +458,8 @@ __global__ void __launch_bounds__(kThreads) k_scroll_move(const MapCounters* __r
             sd[2 * kBrickVox + l] = (unsigned long long)((long long)ss[2 * kBrickVox + l] - cc * daz);
             cd[l] = c;
         }
+        if (threadIdx.x < kBrickVox / 32)
+            occ[(size_t)d * (kBrickVox / 32) + threadIdx.x] = occ[(size_t)s * (kBrickVox / 32) + threadIdx.x];
         if (threadIdx.x == 0) slot_key[d] = slot_key[s] - shift_key;
     }
 }
@@ -413,7 +467,7 @@ __global__ void __launch_bounds__(kThreads) k_scroll_move(const MapCounters* __r
 // Zeroes the slots from the kept count to the old count (their bricks moved
 // or were evicted) so they can be claimed again.
 __global__ void k_scroll_zero(const uint32_t* __restrict__ n_keep, const MapCounters* __restrict__ ctr,
-                              uint32_t capacity, unsigned long long* S, uint32_t* C) {
+                              uint32_t capacity, unsigned long long* S, uint32_t* C, uint32_t* occ) {
     pdl_gate();
     const size_t lo = (size_t)*n_keep * kBrickVox, hi = (size_t)min(ctr->n_bricks, capacity) * kBrickVox;
     for (size_t i = lo + (size_t)blockIdx.x * kThreads + threadIdx.x; i < hi; i += (size_t)gridDim.x * kThreads) {
@@ -422,6 +476,7 @@ __global__ void k_scroll_zero(const uint32_t* __restrict__ n_keep, const MapCoun
         S[slot * 3 * kBrickVox + kBrickVox + l] = 0;
         S[slot * 3 * kBrickVox + 2 * kBrickVox + l] = 0;
         C[i] = 0;
+        if (!(l & 31)) occ[i >> 5] = 0;
     }
 }
 
@@ -454,7 +509,8 @@ size_t scroll_tmp_words(uint32_t capacity) {
 
 cudaError_t launch_scroll(const Grid& g, const Grid& g2, const int32_t shift[3], const float po2[3],
                           int32_t* brick_table, uint32_t nb_total, int32_t* slot_key, unsigned long long* S,
-                          uint32_t* C, MapCounters* ctr, uint32_t capacity, uint32_t* tmp, cudaStream_t s) {
+                          uint32_t* C, uint32_t* occ, MapCounters* ctr, uint32_t capacity, uint32_t* tmp,
+                          cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -476,10 +532,10 @@ cudaError_t launch_scroll(const Grid& g, const Grid& g2, const int32_t shift[3],
     const unsigned gm = capacity < (uint32_t)sms * 8 ? capacity : (uint32_t)sms * 8;
     launch_k(k_scroll_count, dim3(gm), dim3(kThreads), 0, s, keep, capacity, C, ctr);
     launch_k(k_scroll_move, dim3(gm), dim3(kThreads), 0, s, ctr, capacity, keep, kpos, word, hole, slot_key, shift_key,
-             g2.ax - g.ax, g2.ay - g.ay, g2.az - g.az, S, C);
+             g2.ax - g.ax, g2.ay - g.ay, g2.az - g.az, S, C, occ);
     const size_t zw = ((size_t)capacity * kBrickVox + kThreads - 1) / kThreads;
     launch_k(k_scroll_zero, dim3((unsigned)(zw < (size_t)sms * 8 ? zw : (size_t)sms * 8)), dim3(kThreads), 0, s, word,
-             ctr, capacity, S, C);
+             ctr, capacity, S, C, occ);
     if ((e = cudaMemsetAsync(brick_table, 0xFF, (size_t)nb_total * sizeof(int32_t), s)) != cudaSuccess) return e;
     launch_k(k_scroll_table, dim3(gs), dim3(kThreads), 0, s, word, slot_key, brick_table, ctr,
              const_cast<float*>(g2.po), po2[0], po2[1], po2[2]);
@@ -488,8 +544,8 @@ cudaError_t launch_scroll(const Grid& g, const Grid& g2, const int32_t shift[3],
 }
 
 cudaError_t launch_clear(const float* xyz, uint32_t n, const Pose& pose, const Grid& g, const int32_t* brick_table,
-                         unsigned long long* S, uint32_t* C, uint32_t* mark, MapCounters* ctr, uint32_t capacity,
-                         cudaStream_t s) {
+                         unsigned long long* S, uint32_t* C, uint32_t* occ, uint32_t* mark, MapCounters* ctr,
+                         uint32_t capacity, cudaStream_t s) {
     // A sensor outside the grid casts no rays (host check, same arithmetic as the walk's start).
     const float sx = (pose.r[3] - g.ox) * g.inv_res, sy = (pose.r[7] - g.oy) * g.inv_res,
                 sz = (pose.r[11] - g.oz) * g.inv_res;
@@ -502,28 +558,28 @@ cudaError_t launch_clear(const float* xyz, uint32_t n, const Pose& pose, const G
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint32_t want = (n + kThreads - 1) / kThreads;
     const uint32_t grid = want < (uint32_t)(sms * 8) ? want : (uint32_t)(sms * 8);
-    launch_k(k_clear_mark, dim3(grid), dim3(kThreads), 0, s, xyz, n, pose, g, brick_table, C, mark, ctr);
+    launch_k(k_clear_mark, dim3(grid), dim3(kThreads), 0, s, xyz, n, pose, g, brick_table, occ, mark, ctr);
     const size_t words = (size_t)capacity * (kBrickVox / 32);
     const size_t wgrid = (words + kThreads - 1) / kThreads;
     launch_k(k_clear_apply, dim3((unsigned)(wgrid < (size_t)sms * 8 ? wgrid : (size_t)sms * 8)), dim3(kThreads), 0, s,
-             S, C, mark, ctr, capacity);
+             S, C, occ, mark, ctr, capacity);
     count_launch(2);
     return cudaGetLastError();
 }
 
 cudaError_t launch_integrate(const float* xyz, uint32_t n, const Pose& pose, const Grid& g, int32_t* brick_table,
-                             int32_t* slot_key, unsigned long long* S, uint32_t* C, uint32_t* deferred,
-                             MapCounters* ctr, uint32_t capacity, cudaStream_t s) {
+                             int32_t* slot_key, unsigned long long* S, uint32_t* C, uint32_t* occ,
+                             uint32_t* deferred, MapCounters* ctr, uint32_t capacity, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint32_t want = (n + kThreads - 1) / kThreads;
     const uint32_t grid = want < (uint32_t)(sms * 8) ? want : (uint32_t)(sms * 8);
-    launch_k(k_accum, dim3(grid), dim3(kThreads), 0, s, xyz, n, pose, g, brick_table, slot_key, S, C, deferred, ctr,
-             capacity);
+    launch_k(k_accum, dim3(grid), dim3(kThreads), 0, s, xyz, n, pose, g, brick_table, slot_key, S, C, occ, deferred,
+             ctr, capacity);
     launch_k(k_accum_deferred, dim3(grid < (uint32_t)sms ? grid : (uint32_t)sms), dim3(kThreads), 0, s, xyz, pose, g,
-             brick_table, S, C, deferred, ctr);
+             brick_table, S, C, occ, deferred, ctr);
     count_launch(2);
     return cudaGetLastError();
 }

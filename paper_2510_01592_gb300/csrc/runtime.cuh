@@ -136,6 +136,7 @@ struct vm_map {
     uint32_t* C = nullptr;
     vmx::MapCounters* ctr = nullptr;
     uint32_t* err = nullptr;  // segmentation error word
+    uint32_t* occ = nullptr;  // occupancy bitmap, one bit per voxel slot (set where C > 0)
     uint32_t* mark = nullptr; // ray-cast clearing marks, one bit per voxel slot
     uint32_t* scroll_tmp = nullptr;  // window-scroll scratch (flags, positions, holes, scan state)
     float* po_dev = nullptr;         // position origin of the window, read by the segmentation

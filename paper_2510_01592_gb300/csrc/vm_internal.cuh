@@ -324,19 +324,21 @@ cudaError_t stable_sort_pairs_u32(uint32_t* keys, uint32_t* vals, uint32_t* keys
 size_t scroll_tmp_words(uint32_t capacity);
 cudaError_t launch_scroll(const Grid& g, const Grid& g2, const int32_t shift[3], const float po2[3],
                           int32_t* brick_table, uint32_t nb_total, int32_t* slot_key, unsigned long long* S,
-                          uint32_t* C, MapCounters* ctr, uint32_t capacity, uint32_t* tmp, cudaStream_t s);
-// deferred: room for n point indices (the frame's points whose brick another
+                          uint32_t* C, uint32_t* occ, MapCounters* ctr, uint32_t capacity, uint32_t* tmp,
+                          cudaStream_t s);
+// occ: the occupancy bitmap, capacity * 16 words (bit l of a slot: its voxel l
+// has points).  deferred: room for n point indices (the frame's points whose brick another
 // thread was claiming); the map counters' deferred words are zero between calls.
 cudaError_t launch_integrate(const float* xyz, uint32_t n, const Pose& pose, const Grid& g, int32_t* brick_table,
-                             int32_t* slot_key, unsigned long long* S, uint32_t* C, uint32_t* deferred,
-                             MapCounters* ctr, uint32_t capacity, cudaStream_t s);
+                             int32_t* slot_key, unsigned long long* S, uint32_t* C, uint32_t* occ,
+                             uint32_t* deferred, MapCounters* ctr, uint32_t capacity, cudaStream_t s);
 // Voxel information clearing (Sec. III.B, Eq. 2): marks every occupied voxel
 // that a point's ray from the sensor passes through before the point's own
 // voxel (mark: one bit per voxel slot, capacity * 16 words, zero between
 // calls), then clears the marked voxels and the marks.
 cudaError_t launch_clear(const float* xyz, uint32_t n, const Pose& pose, const Grid& g,
-                         const int32_t* brick_table, unsigned long long* S, uint32_t* C, uint32_t* mark,
-                         MapCounters* ctr, uint32_t capacity, cudaStream_t s);
+                         const int32_t* brick_table, unsigned long long* S, uint32_t* C, uint32_t* occ,
+                         uint32_t* mark, MapCounters* ctr, uint32_t capacity, cudaStream_t s);
 
 // ---------------------------------------------------------------- segment.cu
 struct SegBuffers {
