@@ -244,36 +244,50 @@ static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* 
 
 
 
-// Scan state for every scan of a segmentation (at most max(nv, bricks) + 1
-// elements); the radix sort has its own region (histograms and their scan).
+// Scan state for the brick ordering and every scan of a segmentation (at most
+// nv + 1 elements).
 static size_t vox_tmp_words(size_t nv, uint32_t nb_total) {
-    return scan_tmp_words((nv > (size_t)nb_total ? nv : (size_t)nb_total) + 1);
+    const size_t a = scan_tmp_words(nv + 1), b = order_tmp_words(nb_total);
+    return a > b ? a : b;
 }
 
-// The rank-dense voxel arrays of nv slots, carved in order.
+// The per-voxel arrays for at most nv occupied voxels, carved in order.
 static void vox_layout(Carver& c, SegBuffers& b, size_t nv, size_t tmp_words) {
-    b.M = c.take<int32_t>(3 * nv);
-    b.nrm = c.take<float>(3 * nv);
-    b.status = c.take<uint8_t>(nv);
-    b.nbr = c.take<uint8_t>(nv);
-    b.rec = c.take<float4>(2 * nv);
-    b.list_idx = c.take<uint32_t>(nv);
+    b.near = c.take<int32_t>(nv / kBrickVox * 27);
+    b.rows = c.take<uint4>(nv / kBrickVox * 100);
+    b.vox = c.take<uint32_t>(nv);
+    b.M = c.take<int4>(nv);
+    b.pos = c.take<float4>(nv);
+    b.nrm = c.take<float4>(nv);
     b.list_A = c.take<float>(6 * nv);
+    b.nbr = c.take<uint8_t>(nv);
+    b.lc = c.take<uint16_t>(nv);
+    b.lsize = c.take<uint32_t>(nv);
+    b.lroot = c.take<uint32_t>(nv);
     b.parent = c.take<uint32_t>(nv);
-    b.count = c.take<uint32_t>(nv);
-    b.cid = c.take<uint32_t>(nv + 1);
-    b.vert_flag = c.take<uint32_t>(nv + 1);
-    b.keys = c.take<uint32_t>(nv);
-    b.vals = c.take<uint32_t>(nv);
-    b.keys_alt = c.take<uint32_t>(nv);
-    b.vals_alt = c.take<uint32_t>(nv);
+    b.csize = c.take<uint32_t>(nv);
+    b.croot = c.take<uint32_t>(nv);
+    b.total = c.take<uint32_t>(nv);
+    b.ccl = c.take<uint32_t>(nv);
+    b.place = c.take<uint32_t>(nv);
+    b.pairs = c.take<unsigned long long>(nv);
     b.cl_size = c.take<uint32_t>(nv + 1);
     b.cl_off = c.take<uint32_t>(nv + 1);
     b.cl_label = c.take<uint32_t>(nv + 1);
     b.pts = c.take<float>(3 * nv);
     b.pt_vid = c.take<uint32_t>(nv);
     b.scan_tmp = c.take<uint32_t>(tmp_words);
-    b.sort_tmp = c.take<uint32_t>(sort_tmp_words(nv));
+}
+
+// The brick-level segmentation arrays of a map, carved in order.
+static void brick_layout(Carver& c, SegBuffers& b, size_t nb_total, size_t capacity) {
+    b.rank_table = c.take<int32_t>(nb_total);
+    b.sorted_slot = c.take<int32_t>(capacity);
+    b.sorted_key = c.take<int32_t>(capacity);
+    b.brec = c.take<BrickRec>(capacity + 1);
+    b.ncomp = c.take<uint32_t>(capacity + 1);
+    b.cbase = c.take<uint32_t>(capacity + 1);
+    b.ctr = c.take<SegCounters>(1);
 }
 
 vm_status alloc_vox(vm_map* m, uint32_t n_bricks) {
@@ -291,7 +305,6 @@ vm_status alloc_vox(vm_map* m, uint32_t n_bricks) {
     Carver c{static_cast<char*>(m->vox_mem.p)};
     vox_layout(c, m->seg, nv, tmp_words);
     VM_CUDA(cudaMemsetAsync(m->seg.scan_tmp, 0, tmp_words * sizeof(uint32_t), m->stream));  // scan states
-    VM_CUDA(cudaMemsetAsync(m->seg.sort_tmp, 0, sort_tmp_words(nv) * sizeof(uint32_t), m->stream));
     m->seg.nv = nv;
     m->seg.kcap = nv;
     m->seg_nv = nv;
@@ -304,10 +317,12 @@ uint64_t map_footprint(const vm_map_params& p, const vm_segment_params& sp) {
     const uint64_t cap = p.brick_capacity && p.brick_capacity < nb ? p.brick_capacity : nb;
     const uint64_t pool = nb * 4 + cap * 4 + cap * kBrickVox * (3 * 8 + 4) + cap * 2 * (kBrickVox / 8) +
                           scroll_tmp_words((uint32_t)cap) * 4 + 4096;
-    const uint64_t bricks = (nb + 1) * 4 + nb * 4 + cap * 8 + 4096;
     const size_t nv = (size_t)cap * kBrickVox;
-    Carver dry{nullptr};
     SegBuffers tmp{};
+    Carver bd{nullptr};
+    brick_layout(bd, tmp, nb, cap);
+    const uint64_t bricks = (uint64_t)bd.off + 4096;
+    Carver dry{nullptr};
     vox_layout(dry, tmp, nv, vox_tmp_words(nv, (uint32_t)nb));
     const uint32_t mc = sp.min_cluster > 16 ? sp.min_cluster : 16;
     const uint64_t kcap = nv / mc > 256 ? nv / mc : 256;
@@ -417,7 +432,7 @@ cudaError_t enqueue_front(vm_map* m, const vm_segment_params& p, StageHook* hk, 
     SegBuffers& b = m->seg;
     cudaError_t e;
     VM_STAGE_BEGIN(hk, kStOrder, s);
-    if ((e = seg_order_bricks(m->brick_table, m->nb_total, b, sms, s, m->err, also_zero)) != cudaSuccess) return e;
+    if ((e = seg_order_bricks(m->brick_table, m->nb_total, m->occ, b, s, m->err, also_zero)) != cudaSuccess) return e;
     VM_STAGE_END(hk, kStOrder, s);
     return seg_run(m->g, m->S, m->C, p, b, m->kcap, m->err, sms, s, hk);
 }
@@ -629,6 +644,7 @@ vm_status finish_segment(vm_map* m, const vm_segment_params& p, vm_planes* out) 
 vm_status read_result(vm_map* m, vm_planes* out) {
     const SegCounters* hdr = static_cast<const SegCounters*>(m->out_host);
     m->last = *hdr;
+
     m->segmented = true;
     const uint32_t K = hdr->n_planes, n_hull = hdr->n_hull;
     const size_t b_planes = (size_t)K * sizeof(vm_plane);
@@ -753,22 +769,14 @@ vm_status vm_create(const vm_map_params* params, void* cuda_stream, vm_map** out
     g.po = m->po_dev;
     // brick-level segmentation arrays
     Carver bd{nullptr};
-    bd.take<uint32_t>((size_t)m->nb_total + 1);
-    bd.take<int32_t>(m->nb_total);
-    bd.take<int32_t>(m->capacity);
-    bd.take<int32_t>(m->capacity);
-    bd.take<SegCounters>(1);
+    brick_layout(bd, m->seg, m->nb_total, m->capacity);
     st = ensure(m->brick_mem, bd.off + 256);
     if (st != VM_OK) {
         vm_destroy(m);
         return st;
     }
     Carver bc{static_cast<char*>(m->brick_mem.p)};
-    m->seg.flags = bc.take<uint32_t>((size_t)m->nb_total + 1);
-    m->seg.rank_table = bc.take<int32_t>(m->nb_total);
-    m->seg.sorted_slot = bc.take<int32_t>(m->capacity);
-    m->seg.sorted_key = bc.take<int32_t>(m->capacity);
-    m->seg.ctr = bc.take<SegCounters>(1);
+    brick_layout(bc, m->seg, m->nb_total, m->capacity);
     e = cudaMallocHost(reinterpret_cast<void**>(&m->hctr), sizeof(SegCounters));
     if (e != cudaSuccess) {
         vm_destroy(m);
@@ -1115,7 +1123,7 @@ vm_status vm_export_voxels(vm_map* m, uint32_t* vid, int64_t* sums, uint32_t* co
     }
     cudaStream_t s = m->stream;
     if (!m->vox_mem.p) VM_TRY(alloc_vox(m, 1));  // scan scratch
-    VM_CUDA(seg_order_bricks(m->brick_table, m->nb_total, m->seg, device_sms(), s));
+    VM_CUDA(seg_order_bricks(m->brick_table, m->nb_total, m->occ, m->seg, s));
     VM_CUDA(cudaMemcpyAsync(m->hctr, m->seg.ctr, sizeof(SegCounters), cudaMemcpyDeviceToHost, s));
     VM_CUDA(cudaStreamSynchronize(s));
     const uint32_t nb = m->hctr->n_sorted;
@@ -1158,40 +1166,46 @@ vm_status vm_export_labels(vm_map* m, uint32_t* vid, float* normal, uint8_t* sta
     *n = 0;
     if (!m->segmented) return VM_OK;
     cudaStream_t s = m->stream;
-    const uint32_t nb = m->last.n_sorted;
-    const size_t nv = (size_t)nb * kBrickVox;
+    const uint32_t nb = m->last.n_sorted, nc = m->last.n_comp;
+    const size_t nv = m->last.n_occ;
     std::vector<int32_t> key(nb);
-    std::vector<uint8_t> st(nv), nb8(nv);
-    std::vector<float> nrm(3 * nv);
-    std::vector<uint32_t> par(nv);
-    if (nb) {
-        VM_CUDA(cudaMemcpyAsync(key.data(), m->seg.sorted_key, nb * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        VM_CUDA(cudaMemcpyAsync(st.data(), m->seg.status, nv, cudaMemcpyDeviceToHost, s));
-        VM_CUDA(cudaMemcpyAsync(nb8.data(), m->seg.nbr, nv, cudaMemcpyDeviceToHost, s));
-        VM_CUDA(cudaMemcpyAsync(par.data(), m->seg.parent, nv * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        for (int a = 0; a < 3; ++a)
-            VM_CUDA(cudaMemcpyAsync(nrm.data() + a * nv, m->seg.nrm + a * m->seg.nv, nv * sizeof(float),
-                                    cudaMemcpyDeviceToHost, s));
+    std::vector<uint8_t> nb8(nv);
+    std::vector<uint16_t> lc(nv);
+    std::vector<float4> pos(nv), nrm(nv);
+    std::vector<uint32_t> vox(nv), cbase(nb), root(nc), croot(nc);
+    if (nv) {
+        const SegBuffers& b = m->seg;
+        VM_CUDA(cudaMemcpyAsync(key.data(), b.sorted_key, nb * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        VM_CUDA(cudaMemcpyAsync(cbase.data(), b.cbase, nb * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        VM_CUDA(cudaMemcpyAsync(vox.data(), b.vox, nv * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        VM_CUDA(cudaMemcpyAsync(pos.data(), b.pos, nv * sizeof(float4), cudaMemcpyDeviceToHost, s));
+        VM_CUDA(cudaMemcpyAsync(nrm.data(), b.nrm, nv * sizeof(float4), cudaMemcpyDeviceToHost, s));
+        VM_CUDA(cudaMemcpyAsync(nb8.data(), b.nbr, nv, cudaMemcpyDeviceToHost, s));
+        VM_CUDA(cudaMemcpyAsync(lc.data(), b.lc, nv * sizeof(uint16_t), cudaMemcpyDeviceToHost, s));
+        if (nc) {
+            VM_CUDA(cudaMemcpyAsync(root.data(), b.parent, nc * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+            VM_CUDA(cudaMemcpyAsync(croot.data(), b.croot, nc * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        }
     }
     VM_CUDA(cudaStreamSynchronize(s));
-    uint32_t k = 0;
-    for (size_t i = 0; i < nv; ++i) {
-        if (!st[i]) continue;
-        if (k < cap) {
-            const uint32_t v = (uint32_t)key[i / kBrickVox] * kBrickVox + (uint32_t)(i % kBrickVox);
-            if (vid) vid[k] = v;
-            if (normal)
-                for (int a = 0; a < 3; ++a) normal[3 * (size_t)k + a] = nrm[a * nv + i];
-            if (status) status[k] = st[i];
-            if (nbr) nbr[k] = nb8[i];
-            if (label) {
-                const uint32_t p = par[i];
-                label[k] = (p == kNone) ? kNone : (uint32_t)key[p / kBrickVox] * kBrickVox + p % kBrickVox;
-            }
+    const size_t k = nv < cap ? nv : cap;
+    for (size_t i = 0; i < k; ++i) {
+        const uint32_t r = vox[i] / kBrickVox;
+        if (vid) vid[i] = (uint32_t)key[r] * kBrickVox + vox[i] % kBrickVox;
+        if (normal) {
+            normal[3 * i] = nrm[i].x;
+            normal[3 * i + 1] = nrm[i].y;
+            normal[3 * i + 2] = nrm[i].z;
         }
-        ++k;
+        if (status) {
+            uint32_t st;
+            memcpy(&st, &pos[i].w, sizeof(st));
+            status[i] = (uint8_t)st;
+        }
+        if (nbr) nbr[i] = nb8[i];
+        if (label) label[i] = lc[i] == kNoComp ? kNone : croot[root[cbase[r] + lc[i]]];
     }
-    *n = k;
+    *n = (uint32_t)nv;
     return VM_OK;
 }
 

@@ -1,7 +1,6 @@
-// scan.cu -- device-wide exclusive prefix sum and a stable LSD radix sort of
-// (uint32 key, uint32 value) pairs.  These order the bricks and voxels by id,
-// number the kept clusters and lay the cluster members out contiguously in
-// voxel-id order (Sec. III.C: points sharing a label are grouped as clusters).
+// scan.cu -- device-wide exclusive prefix sum, and the ordering of the
+// allocated bricks and their occupied voxels by id that every per-voxel array
+// of a segmentation follows (Sec. III.C).
 #include "vm_internal.cuh"
 
 namespace vmx {
@@ -154,98 +153,170 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_lookback(const uint32_t* 
     }
 }
 
-// The allocated bricks in key order in one pass (a stream compaction with the
-// look-back scan above): tile t of the brick table flags its allocated
-// entries (slot >= 0), ranks them within the tile, looks back for the count
-// of allocated bricks before the tile, then writes every entry's rank (or -1)
-// and, per allocated brick, its slot and key at its rank.  The last tile
-// writes the count.  Block 0 also clears the words clear[1 .. n_clear) (a
-// counter block whose word 0 is the count) and zero0 / zero1 (may be null).
+// Looks back, a warp over 32 earlier tiles at a time, for the sum of the tiles
+// before `tile` in one array of status words, and publishes the inclusive sum.
+// Every earlier tile belongs to a CTA that has started; the wait is capped.
+__device__ __forceinline__ uint32_t warp_look_back(unsigned long long* status, uint32_t tile, uint32_t epoch,
+                                                   uint32_t agg, uint32_t* err) {
+    const int lane = threadIdx.x & 31;
+    uint32_t prefix = 0;
+    for (int64_t top = (int64_t)tile - 1; top >= 0; top -= 32) {
+        const int64_t p = top - lane;
+        unsigned long long w = 0;
+        bool ready = p < 0;
+        for (int it = 0; it < kLookbackCap; ++it) {
+            if (!ready) {
+                w = *(volatile unsigned long long*)(status + p);
+                ready = (uint32_t)(w >> 34) == (epoch & kEpochMask) && ((w >> 32) & 3ull);
+            }
+            // the nearest inclusive sum ends the walk: only the tiles up to it have to be there
+            const uint32_t inc = __ballot_sync(0xffffffffu, ready && p >= 0 && ((w >> 32) & 3ull) == kFlagInc);
+            const uint32_t need = inc ? (inc & (0u - inc)) * 2u - 1u : 0xffffffffu;
+            if ((__ballot_sync(0xffffffffu, ready) & need) == need) break;
+        }
+        const uint32_t inc = __ballot_sync(0xffffffffu, ready && p >= 0 && ((w >> 32) & 3ull) == kFlagInc);
+        const uint32_t need = inc ? (inc & (0u - inc)) * 2u - 1u : 0xffffffffu;
+        const bool in = (need >> lane) & 1u;
+        if (__any_sync(0xffffffffu, in && !ready)) {  // a predecessor never published: report, count it as 0
+            if (err && lane == 0) atomicOr(err, kErrTimeout);
+        }
+        prefix += __reduce_add_sync(0xffffffffu, in && ready && p >= 0 ? (uint32_t)(w & 0xffffffffull) : 0u);
+        if (inc) break;
+    }
+    if (lane == 0) atomicExch(status + tile, lb_word(epoch, kFlagInc, prefix + agg));
+    return prefix;
+}
+
+// The allocated bricks in key order and their occupied voxels' places, in one
+// pass (a stream compaction with the look-back scan above, over two sums at
+// once): tile t of the brick table lists its allocated entries (slot >= 0) and
+// their occupied voxels (from the pool's occupancy bitmap), looks back for the
+// bricks and the voxels before the tile, then writes every entry's rank (or
+// -1) and, per allocated brick, its slot, key and record at its rank.  The
+// last tile writes the two counts to clear[0] and clear[1].  Block 0 also
+// clears the words clear[2 .. n_clear) (a counter block that opens with the
+// two counts) and zero0 / zero1 (may be null).  Allocated bricks cluster (a
+// floor fills a whole z layer of the table), so tiles are small and a thread
+// takes a brick, its whole bitmap in four loads.
+constexpr int kOrdItems = 4;
+constexpr int kOrdTile = kScanThreads * kOrdItems;
+__device__ __forceinline__ void load_bits(const uint32_t* __restrict__ occ, int32_t slot, uint4 (&m)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) m[q] = reinterpret_cast<const uint4*>(occ + (size_t)slot * 16)[q];
+}
 __global__ void __launch_bounds__(kScanThreads) k_order_bricks(const int32_t* __restrict__ table, uint32_t nb,
+                                                               const uint32_t* __restrict__ occ,
                                                                int32_t* __restrict__ rank_table,
                                                                int32_t* __restrict__ sorted_slot,
                                                                int32_t* __restrict__ sorted_key,
+                                                               BrickRec* __restrict__ brec,
                                                                uint32_t* __restrict__ clear, int n_clear,
                                                                uint32_t* __restrict__ zero0,
                                                                uint32_t* __restrict__ zero1,
                                                                uint32_t* __restrict__ state, uint32_t* err) {
     pdl_gate();
-    __shared__ int32_t buf[kScanTile];
+    __shared__ int32_t buf[kOrdTile];    // the tile's table entries, then its allocated slots
+    __shared__ uint16_t lkey[kOrdTile];  // the allocated entries' places in the tile
+    __shared__ uint32_t lvox[kOrdTile];  // their occupied voxels, then the voxels before them
     __shared__ uint32_t ws[kScanThreads / 32];
-    __shared__ uint32_t tot, s_tile, s_prefix;
+    __shared__ uint32_t tot, s_tile, s_prefix[2];
+    const uint32_t nt_used = (nb + kOrdTile - 1) / kOrdTile;
     unsigned long long* status = reinterpret_cast<unsigned long long*>(state + 4);
     if (blockIdx.x == 0) {
-        for (int i = 1 + threadIdx.x; i < n_clear; i += kScanThreads) clear[i] = 0u;
+        for (int i = 2 + threadIdx.x; i < n_clear; i += kScanThreads) clear[i] = 0u;
         if (threadIdx.x == 0) {
             if (zero0) *zero0 = 0u;
             if (zero1) *zero1 = 0u;
         }
     }
-    const uint32_t nt_used = (nb + kScanTile - 1) / kScanTile;
     const uint32_t epoch = *(volatile uint32_t*)(state + 2);
     if (threadIdx.x == 0) s_tile = atomicAdd(state, 1u);
     __syncthreads();
     const uint32_t tile = s_tile;
     if (tile < nt_used) {
-        const uint32_t base = tile * kScanTile;
+        const uint32_t base = tile * kOrdTile;
 #pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
+        for (int i = 0; i < kOrdItems; ++i) {
             const uint32_t j = base + i * kScanThreads + threadIdx.x;
             buf[i * kScanThreads + threadIdx.x] = j < nb ? table[j] : -1;
         }
         __syncthreads();
-        int32_t v[kScanItems];
+        int32_t v[kOrdItems];
         uint32_t sum = 0;
 #pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
-            v[i] = buf[threadIdx.x * kScanItems + i];
+        for (int i = 0; i < kOrdItems; ++i) {
+            v[i] = buf[threadIdx.x * kOrdItems + i];
             sum += v[i] >= 0;
+            if (v[i] < 0 && base + threadIdx.x * kOrdItems + i < nb)
+                rank_table[base + threadIdx.x * kOrdItems + i] = -1;
         }
-        const uint32_t ex_local = block_excl_scan(sum, ws, &tot);
-        if (threadIdx.x == 0) {
-            const uint32_t agg = tot;
-            uint32_t prefix = 0;
-            if (tile == 0) {
-                atomicExch(status, lb_word(epoch, kFlagInc, agg));
-            } else {
-                atomicExch(status + tile, lb_word(epoch, kFlagAgg, agg));
-                for (int64_t p = (int64_t)tile - 1; p >= 0; --p) {
-                    unsigned long long w = 0;
-                    int it = 0;
-                    for (; it < kLookbackCap; ++it) {
-                        w = *(volatile unsigned long long*)(status + p);
-                        if ((uint32_t)(w >> 34) == (epoch & kEpochMask) && ((w >> 32) & 3ull)) break;
-                    }
-                    if (it == kLookbackCap) {  // the predecessor never published: report, count it as 0
-                        if (err) atomicOr(err, kErrTimeout);
-                        break;
-                    }
-                    prefix += (uint32_t)(w & 0xffffffffull);
-                    if (((w >> 32) & 3ull) == kFlagInc) break;
-                }
-                atomicExch(status + tile, lb_word(epoch, kFlagInc, prefix + agg));
+        uint32_t at = block_excl_scan(sum, ws, &tot);  // its barriers also end the reads of buf
+#pragma unroll
+        for (int i = 0; i < kOrdItems; ++i)
+            if (v[i] >= 0) {
+                buf[at] = v[i];
+                lkey[at++] = (uint16_t)(threadIdx.x * kOrdItems + i);
             }
-            s_prefix = prefix;
-            if (tile == nt_used - 1) clear[0] = prefix + agg;
+        __syncthreads();
+        const uint32_t nbr = tot;
+        for (uint32_t b = threadIdx.x; b < nbr; b += kScanThreads) {
+            uint4 m[4];
+            load_bits(occ, buf[b], m);
+            uint32_t c = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) c += __popc(m[q].x) + __popc(m[q].y) + __popc(m[q].z) + __popc(m[q].w);
+            lvox[b] = c;
         }
         __syncthreads();
-        uint32_t rank = ex_local + s_prefix;
+        uint32_t n[kOrdItems], nsum = 0;
 #pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
-            const uint32_t j = base + threadIdx.x * kScanItems + i;
-            if (j < nb) {
-                if (v[i] >= 0) {
-                    sorted_slot[rank] = v[i];
-                    sorted_key[rank] = (int32_t)j;
-                    rank_table[j] = (int32_t)rank;
-                    ++rank;
-                } else {
-                    rank_table[j] = -1;
-                }
+        for (int i = 0; i < kOrdItems; ++i) {
+            const uint32_t b = threadIdx.x * kOrdItems + i;
+            n[i] = b < nbr ? lvox[b] : 0u;
+            nsum += n[i];
+        }
+        uint32_t ex = block_excl_scan(nsum, ws, &tot);
+#pragma unroll
+        for (int i = 0; i < kOrdItems; ++i) {
+            const uint32_t b = threadIdx.x * kOrdItems + i;
+            if (b < nbr) lvox[b] = ex;
+            ex += n[i];
+        }
+        if (threadIdx.x < 64) {  // warp 0: bricks, warp 1: voxels (its status words lie behind the first's)
+            const int which = threadIdx.x >> 5;
+            const uint32_t agg = which ? tot : nbr;
+            unsigned long long* st = status + (which ? nt_used : 0);
+            if ((threadIdx.x & 31) == 0) atomicExch(st + tile, lb_word(epoch, tile ? kFlagAgg : kFlagInc, agg));
+            const uint32_t prefix = tile ? warp_look_back(st, tile, epoch, agg, err) : 0u;
+            if ((threadIdx.x & 31) == 0) {
+                s_prefix[which] = prefix;
+                if (tile == nt_used - 1) clear[which] = prefix + agg;
             }
+        }
+        __syncthreads();
+        const uint32_t rank0 = s_prefix[0], vox0 = s_prefix[1];
+        for (uint32_t b = threadIdx.x; b < nbr; b += kScanThreads) {
+            const int32_t slot = buf[b];
+            const uint32_t rank = rank0 + b, key = base + lkey[b];
+            uint4 m[4];
+            load_bits(occ, slot, m);
+            BrickRec* r = brec + rank;
+            uint32_t run = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                reinterpret_cast<uint4*>(r->mask)[q] = m[q];
+                const uint32_t p0 = run, p1 = p0 + __popc(m[q].x), p2 = p1 + __popc(m[q].y), p3 = p2 + __popc(m[q].z);
+                run = p3 + __popc(m[q].w);
+                reinterpret_cast<uint2*>(r->pre)[q] = make_uint2(p0 | (p1 << 16), p2 | (p3 << 16));
+            }
+            *reinterpret_cast<uint4*>(&r->base) = make_uint4(vox0 + lvox[b], run, key, (uint32_t)slot);
+            sorted_slot[rank] = slot;
+            sorted_key[rank] = (int32_t)key;
+            rank_table[key] = (int32_t)rank;
         }
     } else if (tile == 0 && threadIdx.x == 0) {  // an empty table
         clear[0] = 0u;
+        clear[1] = 0u;
     }
     if (threadIdx.x == 0) {
         __threadfence();
@@ -254,96 +325,6 @@ __global__ void __launch_bounds__(kScanThreads) k_order_bricks(const int32_t* __
             state[1] = 0;
             state[2] = epoch + 1;
             __threadfence();
-        }
-    }
-}
-
-// ------------------------------------------------------------------ radix sort
-constexpr int kSortThreads = 256;
-constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortIters = 8;                               // 32-item rounds per warp
-constexpr int kSortTile = kSortThreads * kSortIters;        // 2048
-
-// Pass `pass` of the sort runs only when some key reaches its digit: with a
-// device bound kb on the keys (every key < kb), pass p > 0 runs iff
-// kb > 2^(8p).  Tiles past the device count do nothing; the histograms are
-// laid out digit-major over the used tiles only, and *cnt receives their
-// count (the scan's length).
-__device__ __forceinline__ bool rs_pass_active(const uint32_t* kb, int pass) {
-    return pass == 0 || !kb || (unsigned long long)*kb > (1ull << (8 * pass));
-}
-
-__global__ void k_rs_hist(const uint32_t* __restrict__ keys, size_t n_cap, const uint32_t* __restrict__ n_dev, int pass,
-                          const uint32_t* __restrict__ kb, uint32_t* __restrict__ ghist, uint32_t* __restrict__ cnt) {
-    pdl_gate();
-    __shared__ uint32_t h[256];
-    const bool active = rs_pass_active(kb, pass);
-    const size_t n = active ? dev_count(n_cap, n_dev) : 0;
-    const size_t ntu = (n + kSortTile - 1) / kSortTile;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *cnt = (uint32_t)(256 * ntu);
-    if (blockIdx.x >= ntu) return;
-    const int shift = 8 * pass;
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const size_t base = (size_t)blockIdx.x * kSortTile;
-    for (int i = 0; i < kSortIters; ++i) {
-        size_t j = base + (size_t)i * kSortThreads + threadIdx.x;
-        if (j < n) atomicAdd(&h[(keys[j] >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    ghist[(size_t)threadIdx.x * ntu + blockIdx.x] = h[threadIdx.x];
-}
-
-// Stable scatter: warp w owns items [w*256, w*256+256) of the tile, in order.
-__global__ void k_rs_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                             uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, size_t n_cap,
-                             const uint32_t* __restrict__ n_dev, int pass, const uint32_t* __restrict__ kb,
-                             const uint32_t* __restrict__ goff) {
-    pdl_gate();
-    __shared__ uint32_t wc[kSortWarps][256];
-    if (!rs_pass_active(kb, pass)) return;
-    const size_t n = dev_count(n_cap, n_dev);
-    if ((size_t)blockIdx.x * kSortTile >= n) return;
-    const size_t nt = (n + kSortTile - 1) / kSortTile;  // used tiles: the histogram stride
-    const int shift = 8 * pass;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int d = threadIdx.x; d < kSortWarps * 256; d += kSortThreads) (&wc[0][0])[d] = 0;
-    __syncthreads();
-    const size_t base = (size_t)blockIdx.x * kSortTile + (size_t)w * (32 * kSortIters);
-    const uint32_t lt = (1u << lane) - 1u;
-    uint32_t rank[kSortIters], dig[kSortIters];
-#pragma unroll
-    for (int i = 0; i < kSortIters; ++i) {
-        size_t j = base + (size_t)i * 32 + lane;
-        uint32_t d = (j < n) ? ((kin[j] >> shift) & 255u) : 256u;
-        dig[i] = d;
-        uint32_t m = __match_any_sync(0xffffffffu, d);
-        uint32_t r = __popc(m & lt);
-        uint32_t b = (d < 256u) ? wc[w][d] : 0u;
-        __syncwarp();
-        if (d < 256u && r == 0) wc[w][d] = b + __popc(m);
-        __syncwarp();
-        rank[i] = b + r;
-    }
-    __syncthreads();
-    {   // exclusive offsets of each warp per digit
-        const int d = threadIdx.x;  // kSortThreads == 256 digits
-        uint32_t run = 0;
-        for (int q = 0; q < kSortWarps; ++q) {
-            uint32_t t = wc[q][d];
-            wc[q][d] = run;
-            run += t;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kSortIters; ++i) {
-        size_t j = base + (size_t)i * 32 + lane;
-        if (j < n) {
-            uint32_t d = dig[i];
-            uint32_t pos = goff[(size_t)d * nt + blockIdx.x] + wc[w][d] + rank[i];
-            kout[pos] = kin[j];
-            vout[pos] = vin[j];
         }
     }
 }
@@ -396,76 +377,10 @@ __global__ void __launch_bounds__(kSmallThreads) k_scan_small(const uint32_t* in
     }
 }
 
-// Two arrays of the same length scanned by one CTA (as k_scan_small, both at once).
-__global__ void __launch_bounds__(kSmallThreads) k_scan2_small(const uint32_t* in0, uint32_t* out0, uint32_t* total0,
-                                                               const uint32_t* in1, uint32_t* out1, uint32_t* total1,
-                                                               size_t n_cap, const uint32_t* __restrict__ n_dev) {
-    pdl_gate();
-    __shared__ uint32_t ws[2][kSmallThreads / 32];
-    __shared__ uint32_t round_total[2];
-    const size_t n = dev_count(n_cap, n_dev);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t carry0 = 0, carry1 = 0;
-    for (size_t base = 0; base < n; base += (size_t)kSmallThreads * kSmallItems) {
-        const size_t j0 = base + (size_t)threadIdx.x * kSmallItems;
-        uint32_t v0[kSmallItems], v1[kSmallItems], sum0 = 0, sum1 = 0;
-#pragma unroll
-        for (int i = 0; i < kSmallItems; ++i) {
-            v0[i] = (j0 + i < n) ? in0[j0 + i] : 0u;
-            v1[i] = (j0 + i < n) ? in1[j0 + i] : 0u;
-            sum0 += v0[i];
-            sum1 += v1[i];
-        }
-        const uint32_t inc0 = warp_incl_scan(sum0), inc1 = warp_incl_scan(sum1);
-        if (lane == 31) {
-            ws[0][w] = inc0;
-            ws[1][w] = inc1;
-        }
-        __syncthreads();
-        if (w < 2) {
-            const uint32_t t = ws[w][lane];
-            const uint32_t ti = warp_incl_scan(t);
-            ws[w][lane] = ti - t;
-            if (lane == 31) round_total[w] = ti;
-        }
-        __syncthreads();
-        uint32_t ex0 = carry0 + ws[0][w] + (inc0 - sum0), ex1 = carry1 + ws[1][w] + (inc1 - sum1);
-#pragma unroll
-        for (int i = 0; i < kSmallItems; ++i) {
-            if (j0 + i < n) {
-                out0[j0 + i] = ex0;
-                out1[j0 + i] = ex1;
-            }
-            ex0 += v0[i];
-            ex1 += v1[i];
-        }
-        carry0 += round_total[0];
-        carry1 += round_total[1];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        if (total0) *total0 = carry0;
-        if (total1) *total1 = carry1;
-    }
-}
-
 }  // namespace
 
+static_assert((size_t)kOrdTile == kOrderTileElems, "order_tmp_words assumes the ordering's tile size");
 static_assert((size_t)kScanTile == kScanTileElems, "scan_tmp_words assumes the scan's tile size");
-
-cudaError_t exclusive_scan2_dev(const uint32_t* in0, uint32_t* out0, uint32_t* total0, const uint32_t* in1,
-                                uint32_t* out1, uint32_t* total1, const uint32_t* n_dev, size_t n_cap, uint32_t* tmp,
-                                cudaStream_t s, uint32_t* err) {
-    if (n_cap > 0 && n_cap <= kSmallMax) {
-        launch_k(k_scan2_small, dim3(1), dim3(kSmallThreads), 0, s, in0, out0, total0, in1, out1, total1, n_cap,
-                 n_dev);
-        count_launch(1);
-        return cudaGetLastError();
-    }
-    cudaError_t e = exclusive_scan_dev(in0, out0, total0, n_dev, n_cap, tmp, s, err);
-    if (e != cudaSuccess) return e;
-    return exclusive_scan_dev(in1, out1, total1, n_dev, n_cap, tmp, s, err);
-}
 
 cudaError_t exclusive_scan_dev(const uint32_t* in, uint32_t* out, uint32_t* total, const uint32_t* n_dev, size_t n_cap,
                                uint32_t* tmp, cudaStream_t s, uint32_t* err, bool end) {
@@ -488,58 +403,15 @@ cudaError_t exclusive_scan_dev(const uint32_t* in, uint32_t* out, uint32_t* tota
     return cudaGetLastError();
 }
 
-cudaError_t order_bricks_dev(const int32_t* table, uint32_t nb, int32_t* rank_table, int32_t* sorted_slot,
-                             int32_t* sorted_key, uint32_t* clear, int n_clear, uint32_t* zero0, uint32_t* zero1,
-                             uint32_t* tmp, cudaStream_t s, uint32_t* err) {
+cudaError_t order_bricks_dev(const int32_t* table, uint32_t nb, const uint32_t* occ, int32_t* rank_table,
+                             int32_t* sorted_slot, int32_t* sorted_key, BrickRec* brec, uint32_t* clear, int n_clear,
+                             uint32_t* zero0, uint32_t* zero1, uint32_t* tmp, cudaStream_t s, uint32_t* err) {
     if (reinterpret_cast<uintptr_t>(tmp) & 7) return cudaErrorInvalidValue;  // 64-bit status words
-    const size_t nt = ((size_t)nb + kScanTile - 1) / kScanTile;
-    launch_k(k_order_bricks, dim3((unsigned)(nt ? nt : 1)), dim3(kScanThreads), 0, s, table, nb, rank_table,
-             sorted_slot, sorted_key, clear, n_clear, zero0, zero1, tmp, err);
+    const size_t nt = ((size_t)nb + kOrdTile - 1) / kOrdTile;
+    launch_k(k_order_bricks, dim3((unsigned)(nt ? nt : 1)), dim3(kScanThreads), 0, s, table, nb, occ, rank_table,
+             sorted_slot, sorted_key, brec, clear, n_clear, zero0, zero1, tmp, err);
     count_launch(1);
     return cudaGetLastError();
-}
-
-cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, uint32_t* total, size_t n, uint32_t* tmp,
-                               cudaStream_t s, uint32_t* err) {
-    return exclusive_scan_dev(in, out, total, nullptr, n, tmp, s, err);
-}
-
-size_t sort_tmp_words(size_t n) {
-    const size_t nt = (n + kSortTile - 1) / kSortTile;
-    return 256 * nt + 64 + scan_tmp_words(256 * nt);
-}
-
-cudaError_t stable_sort_pairs_dev(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
-                                  const uint32_t* n_dev, size_t n_cap, int bits, uint32_t* tmp, cudaStream_t s,
-                                  uint32_t* err, const uint32_t* key_bound) {
-    if (n_cap == 0 || bits <= 0) return cudaSuccess;
-    const size_t nt = (n_cap + kSortTile - 1) / kSortTile;
-    uint32_t* ghist = tmp;
-    uint32_t* cnt = tmp + 256 * nt;          // the histogram scan's length (device)
-    uint32_t* stmp = tmp + 256 * nt + 64;    // its look-back state
-    uint32_t *ki = keys, *vi = vals, *ko = keys_alt, *vo = vals_alt;
-    const int passes = (bits + 7) / 8;
-    for (int p = 0; p < passes; ++p) {
-        launch_k(k_rs_hist, dim3((unsigned)nt), dim3(kSortThreads), 0, s, ki, n_cap, n_dev, p, key_bound, ghist, cnt);
-        cudaError_t e = exclusive_scan_dev(ghist, ghist, nullptr, cnt, 256 * nt, stmp, s, err);
-        if (e != cudaSuccess) return e;
-        launch_k(k_rs_scatter, dim3((unsigned)nt), dim3(kSortThreads), 0, s, ki, vi, ko, vo, n_cap, n_dev, p, key_bound,
-                 ghist);
-        count_launch(2);
-        uint32_t* t;
-        t = ki; ki = ko; ko = t;
-        t = vi; vi = vo; vo = t;
-    }
-    if (!key_bound && ki != keys) {  // odd number of passes: copy back (n_cap elements; the tail is scratch)
-        cudaMemcpyAsync(keys, ki, n_cap * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(vals, vi, n_cap * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t stable_sort_pairs_u32(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, size_t n,
-                                  int bits, uint32_t* tmp, cudaStream_t s, uint32_t* err) {
-    return stable_sort_pairs_dev(keys, vals, keys_alt, vals_alt, nullptr, n, bits, tmp, s, err, nullptr);
 }
 
 }  // namespace vmx

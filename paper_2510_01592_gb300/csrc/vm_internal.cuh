@@ -122,9 +122,13 @@ struct SegCounters {
     uint32_t n_bricks;   // bricks allocated in the pool (copied at the end)
     uint32_t map_err;    // map error bits (copied at the end)
     uint32_t fit_err;    // fit error bits (copied at the end)
-    uint32_t n_list;     // occupied voxels listed for the eigen-solve
+    uint32_t n_vox;      // occupied voxels of the bricks that fit the scratch
     uint32_t n_planes;   // output plane records (k, or more with several extraction rounds)
     uint32_t k_need;     // kept clusters before clamping to the scratch (sizes a re-run)
+    uint32_t n_comp;     // in-brick components
+    uint32_t n_pairs;    // joined component pairs listed
+    uint32_t n_apart;    // of those, in different trees when they were looked at
+    uint32_t join_done;  // CTAs of the join that have finished
     uint32_t pad[2];
 };
 
@@ -262,56 +266,46 @@ vm_status ensure(DevBuf& b, size_t bytes);
     } while (0)
 
 // ---------------------------------------------------------------- scan.cu
-// Exclusive prefix sum of n uint32 values: out[i] = sum(in[0..i-1]); *total
-// (device) receives the sum.  in and out may alias.  tmp must hold
-// scan_tmp_words(n) words and be zeroed once when it is allocated (it keeps
-// the single-pass scan's look-back state, which every launch leaves ready
-// for the next).  err (device, may be null): kErrTimeout when a bounded
-// look-back wait ran out.
+// Exclusive prefix sum of uint32 values, out[i] = sum(in[0..i-1]); *total
+// (device, may be null) receives the sum.  in and out may alias.  The element
+// count is read on the device from n_dev (clamped to the host bound n_cap,
+// which sizes the grid): usable inside a CUDA graph.  tmp must hold
+// scan_tmp_words(n_cap) words and be zeroed once when it is allocated (it
+// keeps the single-pass scan's look-back state, which every launch leaves
+// ready for the next).  err (device, may be null): kErrTimeout when a bounded
+// look-back wait ran out.  end: also write the sum at out[n] (n the device
+// count clamped to n_cap; out then holds n_cap + 1 words), the closing offset
+// of an offsets array.
 // Elements per tile of the single-pass scan; its look-back state is a
 // ticket, a done count, an epoch, a pad word and one 64-bit word per tile.
 constexpr size_t kScanTileElems = 2048;
 constexpr size_t scan_tmp_words(size_t n) { return 4 + 2 * ((n + kScanTileElems - 1) / kScanTileElems) + 2; }
-cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, uint32_t* total, size_t n, uint32_t* tmp,
-                               cudaStream_t s, uint32_t* err);
-// Stable sort of (key, value) pairs by key, key < 2^bits (bits <= 32), LSD
-// 8-bit digits.  keys/vals are sorted in place using the alt buffers; tmp
-// (sort_tmp_words) zeroed once when allocated.
-// Variants whose element count is read on the device from n_dev (clamped to
-// the host bound n_cap, which sizes the grids): usable inside a CUDA graph.
-// end: also write the sum at out[n] (n the device count clamped to n_cap; out
-// then holds n_cap + 1 words), the closing offset of an offsets array.
 cudaError_t exclusive_scan_dev(const uint32_t* in, uint32_t* out, uint32_t* total, const uint32_t* n_dev, size_t n_cap,
                                uint32_t* tmp, cudaStream_t s, uint32_t* err, bool end = false);
-// Two arrays of the same length scanned as exclusive_scan_dev does (one
-// launch when n_cap is small).
-cudaError_t exclusive_scan2_dev(const uint32_t* in0, uint32_t* out0, uint32_t* total0, const uint32_t* in1,
-                                uint32_t* out1, uint32_t* total1, const uint32_t* n_dev, size_t n_cap, uint32_t* tmp,
-                                cudaStream_t s, uint32_t* err);
-// key_bound (device, may be null): every key is below *key_bound; passes whose
-// digit no key reaches are skipped on the device, and the result then lies in
-// (keys, vals) after an even number of executed passes and in the alt buffers
-// after an odd number (sort_result_alt tells which, on the device).  Without
-// a bound the result is always in (keys, vals).
-cudaError_t stable_sort_pairs_dev(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
-                                  const uint32_t* n_dev, size_t n_cap, int bits, uint32_t* tmp, cudaStream_t s,
-                                  uint32_t* err, const uint32_t* key_bound);
-__device__ __forceinline__ bool sort_result_alt(uint32_t key_bound, int bits) {
-    int executed = 1;
-    for (int p = 1; p < (bits + 7) / 8; ++p) executed += (unsigned long long)key_bound > (1ull << (8 * p));
-    return executed & 1;
-}
-size_t sort_tmp_words(size_t n);
+
+// One allocated brick, by rank: its occupied voxels as a bitmap (bit x of byte
+// 8 z + y: voxel (x, y, z) of the brick), the occupied voxels before each
+// bitmap word, the place of its first occupied voxel in the per-voxel arrays,
+// their count, the brick key and the pool slot.  One 128-byte line.
+struct alignas(128) BrickRec {
+    uint32_t mask[16];
+    uint16_t pre[16];
+    uint32_t base, n, key, slot;
+    uint32_t pad[4];
+};
+static_assert(sizeof(BrickRec) == 128, "one line a brick");
 // The allocated bricks of a brick table of nb entries in key order, in one
 // kernel: rank_table[j] = the rank of brick key j (-1: unallocated),
-// sorted_slot / sorted_key by rank; the count lands in clear[0] and the words
-// clear[1 .. n_clear) and zero0 / zero1 (may be null) are cleared.  tmp: the
-// look-back state of a scan of nb elements (scan_tmp_words(nb)), zeroed once.
-cudaError_t order_bricks_dev(const int32_t* table, uint32_t nb, int32_t* rank_table, int32_t* sorted_slot,
-                             int32_t* sorted_key, uint32_t* clear, int n_clear, uint32_t* zero0, uint32_t* zero1,
-                             uint32_t* tmp, cudaStream_t s, uint32_t* err);
-cudaError_t stable_sort_pairs_u32(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, size_t n,
-                                  int bits, uint32_t* tmp, cudaStream_t s, uint32_t* err);
+// sorted_slot / sorted_key / brec by rank (the occupied voxels from the pool's
+// bitmap occ); the brick and voxel counts land in clear[0] and clear[1] and
+// the words clear[2 .. n_clear) and zero0 / zero1 (may be null) are cleared.
+// tmp: order_tmp_words(nb) words of look-back state, zeroed once.
+// Two status words a tile.
+constexpr size_t kOrderTileElems = 1024;
+constexpr size_t order_tmp_words(size_t nb) { return 4 + 4 * ((nb + kOrderTileElems - 1) / kOrderTileElems) + 2; }
+cudaError_t order_bricks_dev(const int32_t* table, uint32_t nb, const uint32_t* occ, int32_t* rank_table,
+                             int32_t* sorted_slot, int32_t* sorted_key, BrickRec* brec, uint32_t* clear, int n_clear,
+                             uint32_t* zero0, uint32_t* zero1, uint32_t* tmp, cudaStream_t s, uint32_t* err);
 
 // ---------------------------------------------------------------- integrate.cu
 // Robot-centric window (Sec. III.B): moves the window of g by shift whole
@@ -341,29 +335,38 @@ cudaError_t launch_clear(const float* xyz, uint32_t n, const Pose& pose, const G
                          uint32_t* mark, MapCounters* ctr, uint32_t capacity, cudaStream_t s);
 
 // ---------------------------------------------------------------- segment.cu
+// Per-voxel arrays hold the occupied voxels only, in voxel-id order (bricks by
+// rank, voxels by index inside the brick): entry i of brick r is brec[r].base +
+// its place among the brick's occupied voxels.  Components are numbered in the
+// order of their smallest voxel: a brick's are cbase[r] .. cbase[r] + ncomp[r].
 struct SegBuffers {
     // brick order
-    uint32_t* flags;        // [nb_total + 1] scan scratch
     int32_t* rank_table;    // [nb_total]   brick key -> rank or -1
     int32_t* sorted_slot;   // [cap]        rank -> pool slot
     int32_t* sorted_key;    // [cap]        rank -> brick key
-    // rank-dense voxel arrays, index = rank * 512 + local
-    int32_t* M;             // [3][nv]  exact integer means (2^-20 m), INT32_MIN when empty
-    float* nrm;             // [3][nv]
-    uint8_t* status;        // [nv]     0 free, 1 occupied, 2 steppable
+    BrickRec* brec;         // [cap + 1]
+    uint32_t* ncomp;        // [cap + 1]    in-brick components
+    uint32_t* cbase;        // [cap + 1]    their first number
+    int32_t* near;          // [nv / 512][27]  rank of each brick around (-1: none)
+    uint4* rows;            // [nv / 512][100] halo rows (halo_row), row 10 (z + 1) + y + 1
+    // occupied voxels
+    uint32_t* vox;          // [nv]     rank * 512 + voxel index inside the brick
+    int4* M;                // [nv]     exact integer means (2^-20 m); w unused
+    float4* pos;            // [nv]     mean position, status bits (1 occupied, 2 steppable)
+    float4* nrm;            // [nv]     normal; w unused
+    float* list_A;          // [6][nv]  window covariances (FP32, rounded from exact integers)
     uint8_t* nbr;           // [nv]     occupied neighbours N
-    float4* rec;            // [2][nv]  packed (mu, status bits) and (normal, 0) per voxel
-    uint32_t* list_idx;     // [nv]     occupied voxels (rank-dense index), in no particular order
-    float* list_A;          // [6][nv]  their window covariances (FP32, rounded from exact integers)
-    uint32_t* parent;       // [nv]     union-find parent, kNone when not a vertex
-    uint32_t* count;        // [nv]     component sizes at roots
-    uint32_t* cid;          // [nv + 1] kept-root flags -> cluster index (scan)
-    uint32_t* vert_flag;    // [nv + 1] kept-vertex flags -> compact position (scan)
-    // compact kept vertices
-    uint32_t* keys;         // [nv] cluster index
-    uint32_t* vals;         // [nv] rank-dense voxel index
-    uint32_t* keys_alt;
-    uint32_t* vals_alt;
+    uint16_t* lc;           // [nv]     in-brick component, kNoComp when not a vertex
+    uint32_t* lsize;        // [nv]     vertices of component j of a brick, at its base + j; then pairs still apart
+    uint32_t* lroot;        // [nv]     its smallest voxel's id, likewise
+    // components
+    uint32_t* parent;       // [nv]     union-find parent, then the root
+    uint32_t* csize;        // [nv]     vertices of the in-brick component
+    uint32_t* croot;        // [nv]     its smallest voxel's id
+    uint32_t* total;        // [nv]     vertices of the whole component, at its root
+    uint32_t* ccl;          // [nv]     cluster number, kNone when not kept
+    uint32_t* place;        // [nv]     where the in-brick component's points start in the cluster lists
+    unsigned long long* pairs;  // [nv] joined components (lower << 32 | higher)
     // clusters
     uint32_t* cl_size;      // [kcap + 1]
     uint32_t* cl_off;       // [kcap + 1]
@@ -371,16 +374,16 @@ struct SegBuffers {
     float* pts;             // [nv][3]  cluster points in cluster order
     uint32_t* pt_vid;       // [nv]
     uint32_t* scan_tmp;     // look-back state of the segmentation's scans
-    uint32_t* sort_tmp;     // the radix sort's histograms and their scan state
     SegCounters* ctr;       // device
     size_t nv, kcap;
 };
+constexpr uint16_t kNoComp = 0xFFFFu;
 
-// Orders the allocated bricks by key (rank table, sorted slots/keys); the
-// brick count lands in b.ctr->n_sorted.  Clears b.ctr first, and the device
-// words zero0 / zero1 (either may be null).
-cudaError_t seg_order_bricks(const int32_t* brick_table, uint32_t nb_total, SegBuffers& b, int sms, cudaStream_t s,
-                             uint32_t* zero0 = nullptr, uint32_t* zero1 = nullptr);
+// Orders the allocated bricks by key (rank table, sorted slots/keys, brick
+// records); the brick and occupied-voxel counts land in b.ctr.  Clears b.ctr
+// first, and the device words zero0 / zero1 (either may be null).
+cudaError_t seg_order_bricks(const int32_t* brick_table, uint32_t nb_total, const uint32_t* occ, SegBuffers& b,
+                             cudaStream_t s, uint32_t* zero0 = nullptr, uint32_t* zero1 = nullptr);
 // Means, normals, classification, clustering, cluster numbering, the cluster
 // point lists in cluster order and their offsets, for the bricks ordered by
 // seg_order_bricks.  Every count is read on the device (clamped to the
