@@ -134,10 +134,10 @@ vm_status fit_prepare(FitContext& fc, size_t kcap, size_t npts, int H, int tile,
 void fit_release(FitContext& fc) {
     fc.timer.release();
     release(fc.mem);
-    release(fc.out);
     if (fc.host) cudaFreeHost(fc.host);
     fc.host = nullptr;
-    fc.host_bytes = 0;
+    fc.host_dev = nullptr;
+    fc.out_kcap = fc.out_hcap = 0;
     fc.kcap = fc.npts = fc.items = 0;
     fc.H = 0;
 }
@@ -178,46 +178,75 @@ vm_status check_single_round(const vm_segment_params* p) {
     return VM_OK;
 }
 
-// Runs the fit on k clusters and returns the packed result on the host.
+// The mapped result block of a calling thread's fits.
+static vm_status fit_out(FitContext& fc, uint32_t kcap, uint32_t hcap) {
+    if (fc.host && kcap <= fc.out_kcap && hcap <= fc.out_hcap) return VM_OK;
+    kcap = kcap > fc.out_kcap ? kcap + kcap / 4 + 16 : fc.out_kcap;
+    hcap = hcap > fc.out_hcap ? hcap : fc.out_hcap;
+    if (fc.host) cudaFreeHost(fc.host);
+    fc.host = nullptr;
+    fc.host_dev = nullptr;
+    fc.out_kcap = fc.out_hcap = 0;
+    const size_t bytes = out_xyz_off(kcap, hcap) + (size_t)hcap * 12 + 256;
+    count_alloc();
+    VM_CUDA(cudaHostAlloc(&fc.host, bytes, cudaHostAllocMapped));
+    void* d = nullptr;
+    VM_CUDA(cudaHostGetDevicePointer(&d, fc.host, 0));
+    fc.host_dev = static_cast<char*>(d);
+    fc.out_kcap = kcap;
+    fc.out_hcap = hcap;
+    return VM_OK;
+}
+
+// Runs the fit on k clusters and returns the packed result on the host.  The
+// kernels write the result into mapped host memory and check the batch's point
+// count against the scratch themselves, so a call waits for the device once;
+// a batch that does not fit (or the first of a thread) grows the scratch and
+// runs again.
 static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* off, const uint32_t* labels,
-                              uint32_t k, uint32_t npts, const vm_segment_params& p, const FitTuning& tune,
-                              cudaStream_t s, vm_planes* out) {
+                              uint32_t k, const vm_segment_params& p, const FitTuning& tune, cudaStream_t s,
+                              vm_planes* out) {
     memset(out, 0, sizeof(*out));
     if (k == 0) return VM_OK;
-    VM_TRY(fit_prepare(fc, k, npts, (int)p.n_hyp, tune.tile, s));
-    FitBuffers& fb = fc.fb;
-    VM_CUDA(cudaMemsetAsync(fb.err, 0, sizeof(uint32_t), s));
-    StageHook* hk = fc.timer.hook();
-    VM_CUDA(fit_set_count(fb.kdev, k, s));
-    VM_CUDA(launch_fit(pts, off, labels, fb.kdev, k, p, fb, tune, device_sms(), s, hk));
-    uint32_t hdr[2];
-    VM_CUDA(cudaMemcpyAsync(&hdr[0], fb.hull_cnt + k, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    VM_CUDA(cudaMemcpyAsync(&hdr[1], fb.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    VM_CUDA(cudaStreamSynchronize(s));
-    const uint32_t n_hull = hdr[0];
-    const size_t b_planes = (size_t)k * sizeof(vm_plane);
-    const size_t b_xy = (size_t)n_hull * 2 * sizeof(int32_t);
-    const size_t b_xyz = (size_t)n_hull * 3 * sizeof(float);
-    const size_t o_xy = (b_planes + 255) & ~(size_t)255;
-    const size_t o_xyz = (o_xy + b_xy + 255) & ~(size_t)255;
-    const size_t total = o_xyz + b_xyz + 256;
-    VM_TRY(ensure(fc.out, total));
-    char* d = static_cast<char*>(fc.out.p);
-    VM_STAGE_BEGIN(hk, kStPack, s);
-    VM_CUDA(launch_pack(fb, off, labels, fb.kdev, k, reinterpret_cast<vm_plane*>(d),
-                        reinterpret_cast<int32_t*>(d + o_xy), reinterpret_cast<float*>(d + o_xyz), n_hull, s));
-    if (fc.host_bytes < total) {
-        if (fc.host) cudaFreeHost(fc.host);
-        fc.host = nullptr;
-        fc.host_bytes = 0;
-        VM_CUDA(cudaMallocHost(&fc.host, total + total / 4));
-        fc.host_bytes = total + total / 4;
+    size_t npts = fc.npts;
+    if (!fc.mem.p || k > fc.kcap || (int)p.n_hyp > fc.H) {  // the scratch grows in any case: learn the point count
+        uint32_t n = 0;
+        VM_CUDA(cudaMemcpyAsync(&n, off + k, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        VM_CUDA(cudaStreamSynchronize(s));
+        npts = n;
     }
-    VM_CUDA(cudaMemcpyAsync(fc.host, d, total, cudaMemcpyDeviceToHost, s));
-    VM_STAGE_END(hk, kStPack, s);
-    VM_CUDA(cudaStreamSynchronize(s));
-    fc.timer.fold();
-    out->planes = static_cast<vm_plane*>(malloc(b_planes ? b_planes : 1));
+    uint32_t hull = k * 48u + 4096u;
+    StageHook* hk = fc.timer.hook();
+    FitHeader h;
+    for (int attempt = 0;; ++attempt) {
+        VM_TRY(fit_prepare(fc, k, npts, (int)p.n_hyp, tune.tile, s));
+        VM_TRY(fit_out(fc, k, hull));
+        FitBuffers& fb = fc.fb;
+        char* d = fc.host_dev;
+        VM_CUDA(fit_open(off, k, (uint32_t)(fc.npts < 0xFFFFFFFFull ? fc.npts : 0xFFFFFFFFull), fb, s));
+        VM_CUDA(launch_fit(pts, off, labels, fb.kdev, k, p, fb, tune, device_sms(), s, hk));
+        VM_STAGE_BEGIN(hk, kStPack, s);
+        VM_CUDA(launch_pack(fb, off, labels, fb.kdev, k, reinterpret_cast<vm_plane*>(d + out_planes_off()),
+                            reinterpret_cast<int32_t*>(d + out_xy_off(fc.out_kcap)),
+                            reinterpret_cast<float*>(d + out_xyz_off(fc.out_kcap, fc.out_hcap)), fc.out_hcap, s));
+        VM_CUDA(fit_close(fb, reinterpret_cast<FitHeader*>(d), s));
+        VM_STAGE_END(hk, kStPack, s);
+        VM_CUDA(cudaStreamSynchronize(s));
+        fc.timer.fold();
+        h = *static_cast<const FitHeader*>(fc.host);
+        const bool scratch = (h.err & kErrScratch) != 0;
+        if (!scratch && h.n_hull <= fc.out_hcap) break;
+        if (attempt == 3) {
+            set_error("fit scratch could not be sized for this batch");
+            return VM_ERR_OUT_OF_MEMORY;
+        }
+        if (scratch) npts = h.n_points;
+        else hull = h.n_hull + h.n_hull / 4;
+    }
+    const size_t b_planes = (size_t)k * sizeof(vm_plane);
+    const size_t b_xy = (size_t)h.n_hull * 2 * sizeof(int32_t);
+    const size_t b_xyz = (size_t)h.n_hull * 3 * sizeof(float);
+    out->planes = static_cast<vm_plane*>(malloc(b_planes));
     out->hull_xy = static_cast<int32_t*>(malloc(b_xy ? b_xy : 1));
     out->hull_xyz = static_cast<float*>(malloc(b_xyz ? b_xyz : 1));
     if (!out->planes || !out->hull_xy || !out->hull_xyz) {
@@ -225,24 +254,22 @@ static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* 
         set_error("host allocation of the result failed");
         return VM_ERR_OUT_OF_MEMORY;
     }
-    const char* h = static_cast<const char*>(fc.host);
-    memcpy(out->planes, h, b_planes);
-    memcpy(out->hull_xy, h + o_xy, b_xy);
-    memcpy(out->hull_xyz, h + o_xyz, b_xyz);
+    const char* hb = static_cast<const char*>(fc.host);
+    memcpy(out->planes, hb + out_planes_off(), b_planes);
+    memcpy(out->hull_xy, hb + out_xy_off(fc.out_kcap), b_xy);
+    memcpy(out->hull_xyz, hb + out_xyz_off(fc.out_kcap, fc.out_hcap), b_xyz);
     out->n_planes = k;
-    out->n_hull = n_hull;
-    if (hdr[1] & kErrTimeout) {
+    out->n_hull = h.n_hull;
+    if (h.err & kErrTimeout) {
         set_error("a bounded device loop reached its iteration cap during the plane fit");
         return VM_ERR_TIMEOUT;
     }
-    if (hdr[1] & kErrOverflow) {
+    if (h.err & kErrOverflow) {
         set_error("a cluster spans more than 2^28 hull quanta (4096 m) in its plane; its hull is not exact");
         return VM_ERR_EXTENT;
     }
     return VM_OK;
 }
-
-
 
 // Scan state for the brick ordering and every scan of a segmentation (at most
 // nv + 1 elements).
@@ -1105,8 +1132,7 @@ vm_status vm_get_stats(vm_map* m, vm_stats* out) {
     out->clustered_points = m->last.n_kept;
     out->voxels_cleared = c.cleared;
     out->voxels_evicted = c.evicted;
-    out->device_bytes = m->pool.bytes + m->stage.bytes + m->brick_mem.bytes + m->vox_mem.bytes + m->fit.mem.bytes +
-                        m->fit.out.bytes;
+    out->device_bytes = m->pool.bytes + m->stage.bytes + m->brick_mem.bytes + m->vox_mem.bytes + m->fit.mem.bytes;
     (void)0;
     if (c.err & kErrCapacity) {
         set_error("brick pool full");
@@ -1278,11 +1304,7 @@ vm_status vm_fit_planes(const float* xyz, const uint32_t* off, const uint32_t* l
     }
     memset(out, 0, sizeof(*out));
     if (k == 0) return VM_OK;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    uint32_t npts = 0;
-    VM_CUDA(cudaMemcpyAsync(&npts, off + k, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    VM_CUDA(cudaStreamSynchronize(s));
-    return fit_and_pack(tl_fit, xyz, off, labels, k, npts, *params, default_tuning(), s, out);
+    return fit_and_pack(tl_fit, xyz, off, labels, k, *params, default_tuning(), static_cast<cudaStream_t>(stream), out);
 }
 
 }  // extern "C"

@@ -1583,12 +1583,6 @@ void fit_init_attributes() {
     });
 }
 
-cudaError_t fit_set_count(uint32_t* kdev, uint32_t k, cudaStream_t s) {
-    launch_k(k_set_u32, dim3(1), dim3(1), 0, s, kdev, k);
-    count_launch(1);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* labels, const uint32_t* kp,
                        uint32_t kcap, const vm_segment_params& p, FitBuffers& fb, const FitTuning& t, int sms,
                        cudaStream_t s, StageHook* hk, uint32_t round) {

@@ -15,14 +15,6 @@ using namespace vmx;
 
 namespace vmx {
 
-// Result block header of a plan (the first 256 bytes of its mapped block).
-struct FitHeader {
-    uint32_t k;          // clusters fitted (0 when the batch did not fit the scratch)
-    uint32_t n_points;   // off[k] as read on the device
-    uint32_t n_hull;     // hull vertices written (may exceed the block's capacity)
-    uint32_t err;        // kErr* bits
-};
-
 // Starts the fit's error word and rejects a batch whose point count exceeds
 // the scratch: every later kernel then sees zero clusters, and the host grows
 // the scratch and runs again.
@@ -36,6 +28,16 @@ __global__ void k_fit_guard(const uint32_t* __restrict__ off, uint32_t* __restri
     if (n > ncap) *kdev = 0;
 }
 
+// The same for a cluster count known on the host.
+__global__ void k_fit_open(const uint32_t* __restrict__ off, uint32_t k, uint32_t ncap, uint32_t* __restrict__ kdev,
+                           uint32_t* __restrict__ err, uint32_t* __restrict__ n_out) {
+    pdl_gate();
+    const uint32_t n = off[k];
+    *n_out = n;
+    *err = n > ncap ? kErrScratch : 0u;
+    *kdev = n > ncap ? 0u : k;
+}
+
 __global__ void k_fit_header(const uint32_t* __restrict__ kdev, const uint32_t* __restrict__ n_pts,
                              const uint32_t* __restrict__ hull_off, const uint32_t* __restrict__ err,
                              FitHeader* __restrict__ out) {
@@ -46,6 +48,18 @@ __global__ void k_fit_header(const uint32_t* __restrict__ kdev, const uint32_t* 
     h.n_hull = hull_off[h.k];
     h.err = *err;
     *out = h;
+}
+
+cudaError_t fit_open(const uint32_t* off, uint32_t k, uint32_t ncap, FitBuffers& fb, cudaStream_t s) {
+    launch_k(k_fit_open, dim3(1), dim3(1), 0, s, off, k, ncap, fb.kdev, fb.err, fb.tot + 2);
+    count_launch(1);
+    return cudaGetLastError();
+}
+
+cudaError_t fit_close(const FitBuffers& fb, FitHeader* out, cudaStream_t s) {
+    launch_k(k_fit_header, dim3(1), dim3(1), 0, s, fb.kdev, fb.tot + 2, fb.hull_cnt, fb.err, out);
+    count_launch(1);
+    return cudaGetLastError();
 }
 
 }  // namespace vmx
@@ -137,10 +151,9 @@ cudaError_t enqueue_fit(vm_fit_plan* f, const float* x, const uint32_t* off, con
                     reinterpret_cast<int32_t*>(d + out_xy_off(f->out_kcap)),
                     reinterpret_cast<float*>(d + out_xyz_off(f->out_kcap, f->out_hcap)), f->out_hcap, s);
     if (e != cudaSuccess) return e;
-    launch_k(k_fit_header, dim3(1), dim3(1), 0, s, fb.kdev, fb.tot + 2, fb.hull_cnt, fb.err,
-             reinterpret_cast<FitHeader*>(d));
+    if ((e = fit_close(fb, reinterpret_cast<FitHeader*>(d), s)) != cudaSuccess) return e;
     VM_STAGE_END(hk, kStPack, s);
-    count_launch(2);
+    count_launch(1);
     return cudaGetLastError();
 }
 

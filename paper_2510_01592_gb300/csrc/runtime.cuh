@@ -88,10 +88,24 @@ struct FitContext {
     FitBuffers fb{};
     size_t kcap = 0, npts = 0, items = 0;
     int H = 0;
-    DevBuf out;          // device staging of planes / hull arrays
-    void* host = nullptr;  // pinned host staging
-    size_t host_bytes = 0;
+    // result block of vm_fit_planes: mapped pinned host memory, laid out as a plan's
+    void* host = nullptr;
+    char* host_dev = nullptr;
+    uint32_t out_kcap = 0, out_hcap = 0;
 };
+
+// Result block header of a batched fit (the first 256 bytes of its block).
+struct FitHeader {
+    uint32_t k;          // clusters fitted (0 when the batch did not fit the scratch)
+    uint32_t n_points;   // off[k] as read on the device
+    uint32_t n_hull;     // hull vertices written (may exceed the block's capacity)
+    uint32_t err;        // kErr* bits
+};
+// Before a fit of k clusters: the device's cluster count (0 when off[k] exceeds
+// ncap points, with kErrScratch) and a clear error word.  After it and its
+// pack: the header.
+cudaError_t fit_open(const uint32_t* off, uint32_t k, uint32_t ncap, FitBuffers& fb, cudaStream_t s);
+cudaError_t fit_close(const FitBuffers& fb, FitHeader* out, cudaStream_t s);
 
 void release(DevBuf& b);
 size_t fit_bytes(size_t kcap, size_t npts, size_t chunks, int H);

@@ -435,7 +435,6 @@ size_t fit_hull_smem();
 // captured in a CUDA graph.  Per-cluster records land in fb.cl, hull vertices
 // in fb.hull at each cluster's point offset and their offsets in fb.hull_cnt.
 void fit_init_attributes();
-cudaError_t fit_set_count(uint32_t* kdev, uint32_t k, cudaStream_t s);
 // round: the extraction round (Philox counter word 2; 0 for the paper's
 // single plane per cluster).
 cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* labels, const uint32_t* kp,

@@ -82,7 +82,7 @@ class Server:
         if not on_dev:
             xyz = np.ascontiguousarray(np.asarray(xyz, dtype=np.float32))
         n = int(xyz.shape[0])
-        pz = (C.c_float * 12)(*[float(v) for v in np.asarray(pose, dtype=np.float32).reshape(12)])
+        pz = vm._pose(pose)
         t = C.c_uint64()
         vm._check(vm.load().vm_server_submit(self._h, int(sid), vm._ptr(xyz), n, pz, 1 if on_dev else 0,
                                              float(t_arrival), C.byref(t)))

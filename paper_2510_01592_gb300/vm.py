@@ -189,23 +189,33 @@ def segment_params(n_th=3, theta_step_deg=15.0, d_th=0.05, theta_ccl_deg=15.0, m
                              np.float32(eps), seed, classify, planes_per_cluster)
 
 
-def _planes_to_numpy(out: vm_planes):
-    n = out.n_planes
-    dt = np.dtype([("normal", np.float32, 3), ("offset", np.float32), ("inlier_count", np.uint32),
+_PLANE = np.dtype([("normal", np.float32, 3), ("offset", np.float32), ("inlier_count", np.uint32),
                    ("label", np.uint32), ("ransac_normal", np.float32, 3), ("ransac_offset", np.float32),
                    ("basis_u", np.float32, 3), ("basis_v", np.float32, 3), ("hull_origin", np.float32, 3),
                    ("hull_offset", np.uint32), ("hull_count", np.uint32), ("n_points", np.uint32),
                    ("best_h", np.int32), ("flags", np.uint32)])
-    assert dt.itemsize == C.sizeof(vm_plane)
-    if n:
-        raw = C.string_at(out.planes, n * C.sizeof(vm_plane))
-        planes = np.frombuffer(raw, dtype=dt).copy()
-    else:
-        planes = np.zeros(0, dtype=dt)
+assert _PLANE.itemsize == C.sizeof(vm_plane)
+_Pose = C.c_float * 12
+
+
+def _copy(ptr, n, dtype):
+    """n records at ptr as an array of its own."""
+    return np.frombuffer(bytearray(C.string_at(ptr, n * dtype.itemsize)) if n else bytearray(), dtype)
+
+
+_I32, _F32 = np.dtype(np.int32), np.dtype(np.float32)
+
+
+def _planes_to_numpy(out: vm_planes):
     nh = out.n_hull
-    hull_xy = np.ctypeslib.as_array(out.hull_xy, shape=(nh, 2)).copy() if nh else np.zeros((0, 2), np.int32)
-    hull_xyz = np.ctypeslib.as_array(out.hull_xyz, shape=(nh, 3)).copy() if nh else np.zeros((0, 3), np.float32)
-    return {"planes": planes, "hull_xy": hull_xy, "hull_xyz": hull_xyz}
+    return {"planes": _copy(out.planes, out.n_planes, _PLANE),
+            "hull_xy": _copy(out.hull_xy, 2 * nh, _I32).reshape(nh, 2),
+            "hull_xyz": _copy(out.hull_xyz, 3 * nh, _F32).reshape(nh, 3)}
+
+
+def _pose(pose):
+    """12 floats as the library takes them."""
+    return _Pose.from_buffer_copy(np.ascontiguousarray(pose, np.float32).reshape(12))
 
 
 def _ptr(x):
@@ -270,7 +280,7 @@ class VoxelMap:
     def integrate(self, xyz, pose, clear=False):
         """xyz: float32 [n, 3] torch tensor (CUDA or CPU) or numpy array; pose: 12 floats, sensor->map.
         clear: first clear the voxels the points' rays pass through (Eq. 2)."""
-        pose = np.ascontiguousarray(pose, np.float32).reshape(12)
+        pose = _pose(pose)
         on_dev = 1 if (hasattr(xyz, "is_cuda") and xyz.is_cuda) else 0
         if hasattr(xyz, "is_contiguous"):
             assert xyz.dtype.is_floating_point and xyz.element_size() == 4 and xyz.is_contiguous()
@@ -279,8 +289,7 @@ class VoxelMap:
             xyz = np.ascontiguousarray(xyz, np.float32)
             n = xyz.size // 3
         order_after_torch(xyz, self._stream)
-        _check(load().vm_integrate_ex(self._h, _ptr(xyz), n, pose.ctypes.data_as(C.POINTER(C.c_float)), on_dev,
-                                      VM_INTEGRATE_CLEAR if clear else 0))
+        _check(load().vm_integrate_ex(self._h, _ptr(xyz), n, pose, on_dev, VM_INTEGRATE_CLEAR if clear else 0))
 
     def segment(self, params: vm_segment_params | None = None):
         params = params or segment_params()
