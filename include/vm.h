@@ -229,7 +229,8 @@ vm_status vm_fit_planes(const float* xyz, const uint32_t* off, const uint32_t* l
 typedef struct vm_fit_plan vm_fit_plan; /* opaque, library-owned */
 
 typedef struct {
-    uint32_t tile;           /* points per work item, a multiple of 256 in 256..16384       */
+    uint32_t tile;           /* points per work item, a multiple of 256 in 256..16384 (the default
+                                schedule takes a smaller one for a fit too small to fill the GPU) */
     uint32_t hyp_per_thread; /* hypotheses each thread holds in registers: 1, 2, 4 or 8    */
     uint32_t ctas_per_sm;    /* persistent scoring CTAs per SM, 1..16                      */
     uint32_t schedule;       /* 0: a 256-thread CTA per work item; 1: a warp per work item  */

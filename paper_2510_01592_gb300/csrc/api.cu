@@ -84,6 +84,7 @@ static void fit_layout(Carver& c, FitBuffers& fb, size_t kcap, size_t npts, size
     fb.inlier = c.take<uint8_t>(npts + 1);
     fb.part = c.take<float>((chunks + 1) * 10);
     fb.cen = c.take<float>(kcap * 6);
+    fb.poly = c.take<FitPoly>(kcap);
     fb.surv = c.take<int2>(npts + 1);
     fb.hull = c.take<int2>(npts + 1);
     fb.hull_cnt = c.take<uint32_t>(kcap + 1);

@@ -12,17 +12,19 @@
 //  k_select  stage c: max count, lowest hypothesis index on ties; in-plane
 //            basis and hull origin.
 //  k_extract inliers of the selected plane, centroid partial sums and the
-//            extreme inliers along 16 integer directions (exact integer keys).
+//            extreme inliers along 16 integer directions (exact integer keys);
+//            the CTA that completes a cluster forms its centroid and polygon.
 //  k_filter  covariance partial sums; points strictly inside the 16-gon of
 //            extreme points cannot be hull vertices and are dropped (the GPU
 //            filtering step of the cited convex-hull method), the rest are
 //            appended.
 //  k_refit   per cluster: TLS refit from the partial sums (double-float sums,
 //            adjugate power iteration).
-//  k_hull    per cluster: a second, 128-direction filter, then a bitonic sort
-//            of the remaining quantised points in shared memory and Andrew's
-//            monotone chain with exact int64 orientation tests; gift wrapping
-//            over global memory when too many remain for shared memory.
+//  k_hull    per cluster: a second, 128-direction filter, then a sort of the
+//            remaining quantised points in shared memory and Andrew's monotone
+//            chain with exact int64 orientation tests (few points: a rank sort
+//            and a test per point); gift wrapping over global memory when too
+//            many remain for shared memory.
 #include <climits>
 #include <mutex>
 #include <string>
@@ -244,10 +246,12 @@ template <int R>
 __global__ void __launch_bounds__(kT) k_score(const float* __restrict__ pts, const uint32_t* __restrict__ off,
                                               const uint32_t* __restrict__ item_off,
                                               const uint32_t* __restrict__ item_cl, const uint32_t* __restrict__ kp,
-                                              int H, int T, const float4* __restrict__ hyp,
-                                              uint32_t* __restrict__ counts, uint32_t* __restrict__ queue, float eps) {
+                                              int H, const uint32_t* __restrict__ tile,
+                                              const float4* __restrict__ hyp, uint32_t* __restrict__ counts,
+                                              uint32_t* __restrict__ queue, float eps) {
     pdl_wait();
     const uint32_t k = *kp;
+    const int T = (int)*tile;
     extern __shared__ float4 sp[];                // T staged points
     uint32_t* red = reinterpret_cast<uint32_t*>(sp + T);  // [P][G*R]
     __shared__ uint32_t s_item;
@@ -315,7 +319,6 @@ __device__ __forceinline__ int2 quantise(const FitCluster& f, float px, float py
 // (-1,2) (-1,1) (-2,1) (-1,0) (-2,-1) (-1,-1) (-1,-2) (0,-1) (1,-2) (1,-1) (2,-1);
 // direction d + 8 is direction d negated.  With |X|, |Y| < 2^28 every value
 // fits in int32.
-constexpr int kFiltDirs = 16;
 __device__ __forceinline__ int32_t dir_value(int dir, int2 p) {
     const int a = (dir == 0 || dir == 2 || dir == 3 || dir == 14 || dir == 13) ? 1
                 : (dir == 1 || dir == 15) ? 2
@@ -453,12 +456,14 @@ __device__ __forceinline__ df2 df_shfl_xor(df2 x, int o) {
 }
 
 // Sums NV double-float values over a CTA in a fixed order: a shuffle tree in
-// each warp, then the warps' results in warp order.  The total is valid in
-// thread 0.  sh: NV * (kT / 32) entries of shared memory.
+// each warp, then the warps' results in warp order, a thread per value.  The
+// totals end in tot (shared, valid after the call's last barrier); sh: NV * (kT
+// / 32) entries of shared memory.  Rolled loops: this code runs once a cluster,
+// and fetching it unrolled (10 KB) took longer than running it.
 template <int NV>
-__device__ __forceinline__ void block_df_sum(df2 (&v)[NV], df2* sh) {
+__device__ __forceinline__ void block_df_sum(df2 (&v)[NV], df2* sh, df2* tot) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
+#pragma unroll 1
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
         for (int e = 0; e < NV; ++e) v[e] = df_add(v[e], df_shfl_xor(v[e], o));
@@ -466,24 +471,85 @@ __device__ __forceinline__ void block_df_sum(df2 (&v)[NV], df2* sh) {
 #pragma unroll
         for (int e = 0; e < NV; ++e) sh[e * (kT / 32) + w] = v[e];
     __syncthreads();
-    if (threadIdx.x == 0)
+    if (threadIdx.x < NV) {
+        const df2* s = sh + threadIdx.x * (kT / 32);
+        df2 t = s[0];
+#pragma unroll 1
+        for (int q = 1; q < kT / 32; ++q) t = df_add(t, s[q]);
+        tot[threadIdx.x] = t;
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ long long cross3(int2 o, int2 a, int2 b) {
+    return (long long)(a.x - o.x) * (long long)(b.y - o.y) - (long long)(a.y - o.y) * (long long)(b.x - o.x);
+}
+
+// Forms cluster c's polygon, by one warp: a lane per direction.  A cluster with
+// inliers has an extreme in every direction, one without in none.  f: the
+// cluster's plane; its extremes are read from L2 (other CTAs wrote them).
+__device__ __forceinline__ void poly_warp(const FitCluster& f, const float* __restrict__ pts, uint32_t base,
+                                          FitPoly* __restrict__ out) {
+    const int lane = threadIdx.x & 31, d = lane & 15;
+    const unsigned long long key = __ldcg(&f.ext[d]);
+    int2 xy = make_int2(0, 0);
+    if (key) {
+        const float* p = pts + 3 * ((size_t)base + (uint32_t)(key & 0xffffffffu));
+        xy = quantise(f, p[0], p[1], p[2]);
+    }
+    const int px = __shfl_sync(0xffffffffu, xy.x, d ? d - 1 : 0), py = __shfl_sync(0xffffffffu, xy.y, d ? d - 1 : 0);
+    const uint32_t keep = __ballot_sync(0xffffffffu, key && lane < 16 && (d == 0 || xy.x != px || xy.y != py));
+    int m = __popc(keep);
+    // vertex i: the i-th kept direction's extreme
+    uint32_t rest = keep;
+    for (int i = 0; i < lane && i < kFiltDirs; ++i) rest &= rest - 1;
+    const int src = rest ? __ffs(rest) - 1 : 0;
+    const int ax = __shfl_sync(0xffffffffu, xy.x, src), ay = __shfl_sync(0xffffffffu, xy.y, src);
+    const int lx = __shfl_sync(0xffffffffu, ax, m ? m - 1 : 0), ly = __shfl_sync(0xffffffffu, ay, m ? m - 1 : 0);
+    const int fx = __shfl_sync(0xffffffffu, ax, 0), fy = __shfl_sync(0xffffffffu, ay, 0);
+    if (m > 1 && lx == fx && ly == fy) --m;
+    const int nx0 = __shfl_sync(0xffffffffu, ax, lane + 1 < m ? lane + 1 : 0);
+    const int ny0 = __shfl_sync(0xffffffffu, ay, lane + 1 < m ? lane + 1 : 0);
+    long long area2 = lane < m ? (long long)ax * ny0 - (long long)ay * nx0 : 0ll;
 #pragma unroll
-        for (int e = 0; e < NV; ++e) {
-            df2 t = sh[e * (kT / 32)];
-            for (int q = 1; q < kT / 32; ++q) t = df_add(t, sh[e * (kT / 32) + q]);
-            v[e] = t;
+    for (int o = 16; o > 0; o >>= 1) area2 += __shfl_xor_sync(0xffffffffu, area2, o);
+    if (m < 3 || area2 <= 0) m = 0;
+    // |X|, |Y| of every inlier: at most the extremes along +-x (directions 0, 8), +-y (4, 12)
+    int mx = key && !(d & 3) ? abs((int)((uint32_t)(key >> 32) ^ 0x80000000u)) : 0;
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    const float sM = (float)mx + 1.0f;
+    if (lane < kFiltDirs) {
+        float4 e = make_float4(0.0f, 0.0f, 2.0f, 0.0f);
+        if (lane < m) {
+            const long long ex = (long long)nx0 - ax, ey = (long long)ny0 - ay;
+            const long long cc = (long long)((unsigned long long)ex * (unsigned long long)(long long)ay -
+                                             (unsigned long long)ey * (unsigned long long)(long long)ax);
+            const float exf = (float)ex, eyf = (float)ey, cf = (float)cc;
+            const float sum = fabsf(exf) + fabsf(eyf);
+            const float E = 2.0f * (0.5f * sum + 4.76837158203125e-7f * (sum * sM + fabsf(cf)) + 1.0f);
+            e = make_float4(__fdiv_rn(exf, E), -__fdiv_rn(eyf, E), -__fdiv_rn(cf, E), 0.0f);
+            out->pt[lane] = make_int2(ax, ay);
+            if (lane == m - 1) out->pt[m] = make_int2(fx, fy);
         }
+        out->edge[lane] = e;
+    }
+    if (lane == 0) out->m = m;
 }
 
 // Inlier count and centroid of cluster c by a whole CTA: the per-chunk
 // partial sums (read from L2: other CTAs wrote them) added in double-float in
 // a fixed order (thread-strided, then block_df_sum), so the result does not
-// depend on scheduling.  The centroid is kept as (hi, lo) per axis.
-__device__ __forceinline__ void centroid_cta(uint32_t c, const uint32_t* __restrict__ off,
-                                             const uint32_t* __restrict__ item_off, int T,
-                                             const float* __restrict__ part, FitCluster* __restrict__ cl,
-                                             float* __restrict__ cen, df2* sh, uint32_t* shn) {
-    const uint32_t cpt = (uint32_t)T / kChunk;
+// depend on scheduling.  The centroid is kept as (hi, lo) per axis.  The last
+// warp forms the filter polygon meanwhile.
+struct CentroidShared {
+    df2 sh[3 * (kT / 32)], tot[3];
+    uint32_t n[kT / 32];
+};
+__device__ __forceinline__ void centroid_cta(uint32_t c, const float* __restrict__ pts,
+                                             const uint32_t* __restrict__ off, const uint32_t* __restrict__ item_off,
+                                             uint32_t cpt, const float* __restrict__ part,
+                                             FitCluster* __restrict__ cl, float* __restrict__ cen,
+                                             FitPoly* __restrict__ poly, CentroidShared& sm) {
     df2 v[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
     uint32_t n = 0;
     const uint32_t base = item_off[c] * cpt, nch = (off[c + 1] - off[c] + kChunk - 1) / kChunk;
@@ -495,24 +561,22 @@ __device__ __forceinline__ void centroid_cta(uint32_t c, const uint32_t* __restr
         v[1] = df_add(v[1], df2{__ldcg(pp + 2), 0.0f});
         v[2] = df_add(v[2], df2{__ldcg(pp + 3), 0.0f});
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
-    if ((threadIdx.x & 31) == 0) shn[threadIdx.x >> 5] = n;
-    block_df_sum<3>(v, sh);
-    if (threadIdx.x == 0) {
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0) sm.n[threadIdx.x >> 5] = n;
+    block_df_sum<3>(v, sm.sh, sm.tot);
+    FitCluster& f = cl[c];
+    if (threadIdx.x >= kT - 32) poly_warp(f, pts, off[c], poly + c);
+    if (threadIdx.x < 3) {
         n = 0;
-        for (int q = 0; q < kT / 32; ++q) n += shn[q];
-        FitCluster& f = cl[c];
-        f.inliers = n;
-        df2 cx{f.o[0], 0.0f}, cy{f.o[1], 0.0f}, cz{f.o[2], 0.0f};
-        if (n) {
-            cx = df_add(cx, df_div_count(v[0], n));
-            cy = df_add(cy, df_div_count(v[1], n));
-            cz = df_add(cz, df_div_count(v[2], n));
-        }
-        float* ce = cen + 6 * (size_t)c;
-        ce[0] = cx.hi; ce[1] = cx.lo; ce[2] = cy.hi; ce[3] = cy.lo; ce[4] = cz.hi; ce[5] = cz.lo;
-        f.c[0] = cx.hi; f.c[1] = cy.hi; f.c[2] = cz.hi;
+#pragma unroll
+        for (int q = 0; q < kT / 32; ++q) n += sm.n[q];
+        df2 x{f.o[threadIdx.x], 0.0f};
+        if (n) x = df_add(x, df_div_count(sm.tot[threadIdx.x], n));
+        float* ce = cen + 6 * (size_t)c + 2 * threadIdx.x;
+        ce[0] = x.hi;
+        ce[1] = x.lo;
+        f.c[threadIdx.x] = x.hi;
+        if (threadIdx.x == 0) f.inliers = n;
     }
     __syncthreads();  // shared partials reused next
 }
@@ -520,37 +584,41 @@ __device__ __forceinline__ void centroid_cta(uint32_t c, const uint32_t* __restr
 // After an extraction item of cluster c: the CTA that completes the cluster's
 // last item computes its centroid (out of line: the item loop keeps its
 // registers).
-__device__ __noinline__ void extract_tail(uint32_t c, const uint32_t* __restrict__ off,
-                                          const uint32_t* __restrict__ item_off, int T,
+__device__ __noinline__ void extract_tail(uint32_t c, const float* __restrict__ pts, const uint32_t* __restrict__ off,
+                                          const uint32_t* __restrict__ item_off, uint32_t cpt,
                                           const float* __restrict__ part, FitCluster* __restrict__ cl,
-                                          float* __restrict__ cen, uint32_t* __restrict__ done) {
-    __shared__ df2 sh[3 * (kT / 32)];
-    __shared__ uint32_t shn[kT / 32], s_last;
+                                          float* __restrict__ cen, FitPoly* __restrict__ poly,
+                                          uint32_t* __restrict__ done) {
+    __shared__ CentroidShared sm;
+    __shared__ uint32_t s_last;
     if (cta_last_item(done + 3 * (size_t)c + 1, item_off[c + 1] - item_off[c], &s_last))
-        centroid_cta(c, off, item_off, T, part, cl, cen, sh, shn);
+        centroid_cta(c, pts, off, item_off, cpt, part, cl, cen, poly, sm);
 }
 
 // Inliers, centroid partials (relative to the origin) and the extreme inliers
-// along the 16 filter directions (reduced per warp, then atomicMax).
+// along the 16 filter directions (reduced per CTA, then one atomicMax each: the
+// items of a large cluster meet on its 16 words).
 // kTail: the CTA that completes a cluster's last item computes its centroid
 // (done: the per-cluster completion counters).
 template <bool kTail>
 __global__ void __launch_bounds__(kT) k_extract(const float* __restrict__ pts, const uint32_t* __restrict__ off,
                                                 const uint32_t* __restrict__ item_off,
                                                 const uint32_t* __restrict__ item_cl, const uint32_t* __restrict__ kp,
-                                                int T, FitCluster* __restrict__ cl, uint8_t* __restrict__ inlier,
-                                                float* __restrict__ part, float eps, uint32_t* __restrict__ err,
-                                                uint32_t* __restrict__ done, float* __restrict__ cen) {
+                                                const uint32_t* __restrict__ tile, FitCluster* __restrict__ cl,
+                                                uint8_t* __restrict__ inlier, float* __restrict__ part, float eps,
+                                                uint32_t* __restrict__ err, uint32_t* __restrict__ done,
+                                                float* __restrict__ cen, FitPoly* __restrict__ poly) {
     pdl_gate();
-    const uint32_t k = *kp;
+    const uint32_t k = *kp, T = *tile;
     __shared__ float wp[kMaxChunksPerItem * (kT / 32) * 4];
+    __shared__ unsigned long long wext[kT / 32][kFiltDirs];
     const uint32_t n_items = item_off[k];
-    const uint32_t cpt = (uint32_t)T / kChunk;  // chunks per work item
+    const uint32_t cpt = T / kChunk;  // chunks per work item
     for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
         const uint32_t c = find_cluster(item_cl, item_off, k, it);
         const FitCluster f = cl[c];
-        const uint32_t start = off[c] + (it - item_off[c]) * (uint32_t)T;
-        const uint32_t end = min(off[c + 1], start + (uint32_t)T);
+        const uint32_t start = off[c] + (it - item_off[c]) * T;
+        const uint32_t end = min(off[c + 1], start + T);
         // per thread and direction d < 8: the largest value and its point (the
         // last one, i.e. the largest index, among equal values: points come in
         // index order), and the smallest value and its point; direction d + 8
@@ -593,41 +661,48 @@ __global__ void __launch_bounds__(kT) k_extract(const float* __restrict__ pts, c
         }
         chunks_out<4>(wp, j, part + (size_t)it * cpt * 10, 0);  // slot 0 holds the count (at most 256: exact)
         if (big) atomicOr(err, kErrOverflow);
-        // the warp's largest key per direction: the extreme value, then the
-        // largest index among the lanes that hold it
-        const bool lane0 = (threadIdx.x & 31) == 0;
+        // the warp's largest key per direction (the extreme value, then the
+        // largest index among the lanes that hold it), then the CTA's
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
         for (int d = 0; d < kFiltDirs / 2; ++d) {
             const int wmax = __reduce_max_sync(0xffffffffu, vmax[d]);
             const int wimax = __reduce_max_sync(0xffffffffu, vmax[d] == wmax ? imax[d] : 0);
             const int wmin = __reduce_min_sync(0xffffffffu, vmin[d]);
             const int wimin = __reduce_max_sync(0xffffffffu, vmin[d] == wmin ? imin[d] : 0);
-            if (lane0 && wmax != INT_MIN) atomicMax(&cl[c].ext[d], ext_key(wmax, (uint32_t)wimax));
-            if (lane0 && wmin != INT_MAX) atomicMax(&cl[c].ext[d + 8], ext_key(-wmin, (uint32_t)wimin));
+            if (lane == d) wext[w][d] = wmax != INT_MIN ? ext_key(wmax, (uint32_t)wimax) : 0ull;
+            if (lane == d + 8) wext[w][d + 8] = wmin != INT_MAX ? ext_key(-wmin, (uint32_t)wimin) : 0ull;
         }
         __syncthreads();
-        if constexpr (kTail) extract_tail(c, off, item_off, T, part, cl, cen, done);
+        if (threadIdx.x < kFiltDirs) {
+            unsigned long long key = 0;
+#pragma unroll
+            for (int q = 0; q < kT / 32; ++q) key = wext[q][threadIdx.x] > key ? wext[q][threadIdx.x] : key;
+            if (key) atomicMax(&cl[c].ext[threadIdx.x], key);
+        }
+        __syncthreads();
+        if constexpr (kTail) extract_tail(c, pts, off, item_off, cpt, part, cl, cen, poly, done);
     }
 }
 
-__device__ __forceinline__ long long cross3(int2 o, int2 a, int2 b) {
-    return (long long)(a.x - o.x) * (long long)(b.y - o.y) - (long long)(a.y - o.y) * (long long)(b.x - o.x);
-}
-
+struct RefitShared {
+    df2 sh[6 * (kT / 32)], tot[6];
+};
 __device__ __forceinline__ void refit_cta(uint32_t c, const uint32_t* __restrict__ off,
-                                          const uint32_t* __restrict__ item_off, int T, const float* __restrict__ part,
-                                          const float* __restrict__ cen, FitCluster* __restrict__ cl, df2* sh);
+                                          const uint32_t* __restrict__ item_off, uint32_t cpt,
+                                          const float* __restrict__ part, const float* __restrict__ cen,
+                                          FitCluster* __restrict__ cl, RefitShared& sm);
 
 // After a filter item of cluster c: the CTA that completes the cluster's last
 // item refits its plane (out of line).
 __device__ __noinline__ void filter_tail(uint32_t c, const uint32_t* __restrict__ off,
-                                         const uint32_t* __restrict__ item_off, int T, const float* __restrict__ part,
-                                         const float* __restrict__ cen, FitCluster* __restrict__ cl,
-                                         uint32_t* __restrict__ done) {
-    __shared__ df2 sh[6 * (kT / 32)];
+                                         const uint32_t* __restrict__ item_off, uint32_t cpt,
+                                         const float* __restrict__ part, const float* __restrict__ cen,
+                                         FitCluster* __restrict__ cl, uint32_t* __restrict__ done) {
+    __shared__ RefitShared sm;
     __shared__ uint32_t s_last;
     if (cta_last_item(done + 3 * (size_t)c + 2, item_off[c + 1] - item_off[c], &s_last))
-        refit_cta(c, off, item_off, T, part, cen, cl, sh);
+        refit_cta(c, off, item_off, cpt, part, cen, cl, sm);
 }
 
 // Covariance partials about the centroid, and the 16-gon filter: inliers
@@ -647,89 +722,43 @@ __device__ __noinline__ void filter_tail(uint32_t c, const uint32_t* __restrict_
 // and the two fused multiply-adds add at most 2^-22 ((|ex| + |ey|) M + |c|).
 // So min over the edges F > 1 means strictly inside every edge (the point is
 // dropped) and F < -1 on some edge means outside it (a survivor); the few
-// points in between take the exact integer test.  The edges' coefficients are
-// read from shared memory once per kBatch chunks.
+// points in between take the exact integer test.  The polygon is formed once a
+// cluster, with its centroid (poly_warp; one thread an item did it in 1.4 us).
+// The edges' coefficients are read from shared memory once per kBatch chunks.
 template <bool kTail>
 __global__ void __launch_bounds__(kT) k_filter(const float* __restrict__ pts, const uint32_t* __restrict__ off,
                                                const uint32_t* __restrict__ item_off,
                                                const uint32_t* __restrict__ item_cl, const uint32_t* __restrict__ kp,
-                                               int T, FitCluster* __restrict__ cl, const uint8_t* __restrict__ inlier,
-                                               const float* __restrict__ cen, float* __restrict__ part,
+                                               const uint32_t* __restrict__ tile, FitCluster* __restrict__ cl,
+                                               const uint8_t* __restrict__ inlier, const float* __restrict__ cen,
+                                               const FitPoly* __restrict__ poly_of, float* __restrict__ part,
                                                int2* __restrict__ surv, uint32_t* __restrict__ done) {
     pdl_gate();
-    const uint32_t k = *kp;
+    const uint32_t k = *kp, T = *tile;
     constexpr int kSurvBuf = 128;
     constexpr int kBatch = 4;  // chunks a thread tests against the edges together
     __shared__ float wp[kMaxChunksPerItem * (kT / 32) * 6];
-    __shared__ int2 sxy[kFiltDirs];
     __shared__ int2 poly[kFiltDirs + 1];
-    __shared__ float4 edge[kFiltDirs];  // (ex / E, -ey / E, -c / E): F = x bf + y af + z
+    __shared__ float4 edge[kFiltDirs];
     __shared__ int npoly;
-    __shared__ float sM;
     __shared__ int2 sbuf[kT / 32][kSurvBuf];
     int2* sb = sbuf[threadIdx.x >> 5];
     const uint32_t n_items = item_off[k];
     const int lane = threadIdx.x & 31;
-    const uint32_t cpt = (uint32_t)T / kChunk;
+    const uint32_t cpt = T / kChunk;
     for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
         const uint32_t c = find_cluster(item_cl, item_off, k, it);
         const FitCluster f = cl[c];
         const uint32_t base = off[c];
-        const uint32_t start = base + (it - item_off[c]) * (uint32_t)T;
-        const uint32_t end = min(off[c + 1], start + (uint32_t)T);
+        const uint32_t start = base + (it - item_off[c]) * T;
+        const uint32_t end = min(off[c + 1], start + T);
         __syncthreads();
-        if (threadIdx.x < kFiltDirs) {  // the extreme points, one direction a thread
-            const int d = threadIdx.x;
-            const unsigned long long key = cl[c].ext[d];  // not f.ext[d]: an indexed copy would live on the stack
-            int2 xy = make_int2(INT_MIN, INT_MIN);  // none
-            if (key) {
-                const float* p = pts + 3 * ((size_t)base + (uint32_t)(key & 0xffffffffu));
-                xy = quantise(f, p[0], p[1], p[2]);
-            }
-            sxy[d] = xy;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            // polygon through the extreme points, counter-clockwise, duplicates removed
-            int m = 0;
-            for (int d = 0; d < kFiltDirs; ++d) {
-                const int2 xy = sxy[d];
-                if (xy.x == INT_MIN && xy.y == INT_MIN) continue;
-                if (m && poly[m - 1].x == xy.x && poly[m - 1].y == xy.y) continue;
-                poly[m++] = xy;
-            }
-            if (m > 1 && poly[m - 1].x == poly[0].x && poly[m - 1].y == poly[0].y) --m;
-            // a degenerate (zero-area) polygon filters nothing
-            long long area2 = 0;
-            for (int i = 0; i < m; ++i) {
-                const int2 a = poly[i], b = poly[(i + 1) % m];
-                area2 += (long long)a.x * b.y - (long long)a.y * b.x;
-            }
-            npoly = (m >= 3 && area2 > 0) ? m : 0;
-            // |X|, |Y| of every inlier: at most the extremes along +-x (directions 0, 8), +-y (4, 12)
-            int mx = 0;
-            for (int d = 0; d < kFiltDirs; d += 4)
-                if (f.ext[d]) mx = max(mx, abs((int)((uint32_t)(f.ext[d] >> 32) ^ 0x80000000u)));
-            sM = (float)mx + 1.0f;
-        }
+        const FitPoly* fp = poly_of + c;
+        if (threadIdx.x < kFiltDirs) edge[threadIdx.x] = fp->edge[threadIdx.x];
+        if (threadIdx.x >= 32 && threadIdx.x - 32 <= kFiltDirs) poly[threadIdx.x - 32] = fp->pt[threadIdx.x - 32];
+        if (threadIdx.x == 64) npoly = fp->m;
         __syncthreads();
         const int m = npoly;
-        if (threadIdx.x < kFiltDirs) {  // the edges' scaled lines, one edge a thread; padding never decides
-            const int i = threadIdx.x;
-            float4 e = make_float4(0.0f, 0.0f, 2.0f, 0.0f);
-            if (i < m) {
-                const int2 A = poly[i], B = poly[(i + 1) % m];
-                const long long ex = (long long)B.x - A.x, ey = (long long)B.y - A.y;
-                const long long cc = (long long)((unsigned long long)ex * (unsigned long long)(long long)A.y -
-                                                 (unsigned long long)ey * (unsigned long long)(long long)A.x);
-                const float exf = (float)ex, eyf = (float)ey, cf = (float)cc;
-                const float sum = fabsf(exf) + fabsf(eyf);
-                const float E = 2.0f * (0.5f * sum + 4.76837158203125e-7f * (sum * sM + fabsf(cf)) + 1.0f);
-                e = make_float4(__fdiv_rn(exf, E), -__fdiv_rn(eyf, E), -__fdiv_rn(cf, E), 0.0f);
-            }
-            edge[i] = e;
-        }
-        __syncthreads();
         const float cx = cen[6 * c], cy = cen[6 * c + 2], cz = cen[6 * c + 4];  // nearest floats of the centroid
         int cnt = 0;  // survivors in this warp's buffer (warp-uniform)
         auto flush = [&]() {
@@ -781,7 +810,7 @@ __global__ void __launch_bounds__(kT) k_filter(const float* __restrict__ pts, co
                         xy = make_int2(__float2int_rn(af[u]), __float2int_rn(bf[u]));
                         if (m && !(fmin[u] < -1.0f)) {  // within the error band of an edge: the exact test
                             for (int i = 0; i < m; ++i) {  // strictly inside every edge -> not a hull vertex
-                                if (cross3(poly[i], poly[(i + 1) % m], xy) <= 0) break;
+                                if (cross3(poly[i], poly[i + 1], xy) <= 0) break;
                                 if (i == m - 1) keep = false;
                             }
                         }
@@ -798,96 +827,118 @@ __global__ void __launch_bounds__(kT) k_filter(const float* __restrict__ pts, co
         }
         if (cnt) flush();
         chunks_out<6>(wp, j, part + (size_t)it * cpt * 10, 4);
-        if constexpr (kTail) filter_tail(c, off, item_off, T, part, cen, cl, done);
+        if constexpr (kTail) filter_tail(c, off, item_off, cpt, part, cen, cl, done);
     }
 }
 
 // Refit of cluster c by a whole CTA: total least squares on the inliers.  The
 // covariance A about the centroid is summed in double-float over the
 // per-chunk partials and scaled by its trace.  Its smallest eigenvector is the
-// dominant eigenvector of the adjugate adj(A) (eigenvalues lambda_j lambda_k);
+// dominant eigenvector of its adjugate adj(A) (eigenvalues lambda_j lambda_k);
 // the adjugate's cofactors, where the cancellation is, are formed in
 // double-float and rounded, then six steps of power iteration in FP32 from
 // the selected RANSAC normal converge by lambda_min / lambda_mid per step.
 // n_z >= 0, d = -n . centroid (double-float); lambda_mid < 10 lambda_min
 // (from the trace, the Rayleigh quotient in double-float and
 // x^T adj(A) x = lambda_1 lambda_2) flags the plane ill-conditioned.
+// The double-float steps run a lane per value (six entries, six cofactors,
+// three rows), so that their code is short: it runs once a cluster, and
+// written out for one thread its 13 KB took 3.5 us, most of it fetching.
+__device__ __forceinline__ df2 df_shfl(df2 x, int src) {
+    return {__shfl_sync(0xffffffffu, x.hi, src), __shfl_sync(0xffffffffu, x.lo, src)};
+}
+// Lane's pick of a small table packed in 4-bit fields.
+__device__ __forceinline__ int nib(uint32_t table, int i) { return (int)((table >> (4 * i)) & 15u); }
 __device__ __forceinline__ void refit_cta(uint32_t c, const uint32_t* __restrict__ off,
-                                          const uint32_t* __restrict__ item_off, int T, const float* __restrict__ part,
-                                          const float* __restrict__ cen, FitCluster* __restrict__ cl, df2* sh) {
-    const uint32_t cpt = (uint32_t)T / kChunk;
-    {
-        df2 A[6];
+                                          const uint32_t* __restrict__ item_off, uint32_t cpt,
+                                          const float* __restrict__ part, const float* __restrict__ cen,
+                                          FitCluster* __restrict__ cl, RefitShared& sm) {
+    df2 A[6];
 #pragma unroll
-        for (int e = 0; e < 6; ++e) A[e] = df2{0.0f, 0.0f};
-        const uint32_t base = item_off[c] * cpt, nch = (off[c + 1] - off[c] + kChunk - 1) / kChunk;
+    for (int e = 0; e < 6; ++e) A[e] = df2{0.0f, 0.0f};
+    const uint32_t base = item_off[c] * cpt, nch = (off[c + 1] - off[c] + kChunk - 1) / kChunk;
 #pragma unroll 2
-        for (uint32_t j = threadIdx.x; j < nch; j += kT)
+    for (uint32_t j = threadIdx.x; j < nch; j += kT) {
+        float v[6];
 #pragma unroll
-            for (int e = 0; e < 6; ++e) A[e] = df_add(A[e], df2{__ldcg(part + (size_t)(base + j) * 10 + 4 + e), 0.0f});
-        block_df_sum<6>(A, sh);
-        if (threadIdx.x == 0) {
-            FitCluster& f = cl[c];
-            uint32_t flags = 0;
-            float rn[3] = {0.0f, 0.0f, 0.0f}, rd = 0.0f;
-            const float tr = __fadd_rn(__fadd_rn(A[0].hi, A[1].hi), A[2].hi);
-            if (f.best_h >= 0 && f.inliers > 0 && tr > 0.0f) {
-                // A / tr: entries of magnitude at most 1 (the diagonal is non-negative)
-                const float itr = __fdiv_rn(1.0f, tr);
-                df2 S[6];
-    #pragma unroll
-                for (int e = 0; e < 6; ++e) S[e] = df_mulf(A[e], itr);
-                const df2 a = S[0], b = S[1], cc = S[2], d = S[3], e = S[4], g = S[5];
-                // symmetric adjugate (cofactors) of [[a d e] [d b g] [e g cc]]
-                const float m00 = df_sub(df_mul(b, cc), df_mul(g, g)).hi, m11 = df_sub(df_mul(a, cc), df_mul(e, e)).hi;
-                const float m22 = df_sub(df_mul(a, b), df_mul(d, d)).hi, m01 = df_sub(df_mul(e, g), df_mul(d, cc)).hi;
-                const float m02 = df_sub(df_mul(d, g), df_mul(e, b)).hi, m12 = df_sub(df_mul(d, e), df_mul(a, g)).hi;
-                float x = f.n[0], y = f.n[1], z = f.n[2];
-                bool ok = true;
-                for (int it = 0; it < 6; ++it) {
-                    const float nx = __fmaf_rn(m02, z, __fmaf_rn(m01, y, __fmul_rn(m00, x)));
-                    const float ny = __fmaf_rn(m12, z, __fmaf_rn(m11, y, __fmul_rn(m01, x)));
-                    const float nz = __fmaf_rn(m22, z, __fmaf_rn(m12, y, __fmul_rn(m02, x)));
-                    const float q = __fmaf_rn(nz, nz, __fmaf_rn(ny, ny, __fmul_rn(nx, nx)));
-                    if (!(q > 1e-30f) || !(q < 1e30f)) { ok = false; break; }  // rank <= 1: keep the RANSAC normal
-                    const float sc = rsqrtf(q);
-                    x = __fmul_rn(nx, sc); y = __fmul_rn(ny, sc); z = __fmul_rn(nz, sc);
-                }
-                if (!ok) {
-                    x = f.n[0]; y = f.n[1]; z = f.n[2];
-                    flags |= 1u;
-                }
-                // unit length to FP32 accuracy
-                const float inv = __fdiv_rn(1.0f, __fsqrt_rn(__fmaf_rn(z, z, __fmaf_rn(y, y, __fmul_rn(x, x)))));
-                x = __fmul_rn(x, inv); y = __fmul_rn(y, inv); z = __fmul_rn(z, inv);
-                if (z < 0.0f || (z == 0.0f && (y < 0.0f || (y == 0.0f && x < 0.0f)))) { x = -x; y = -y; z = -z; }
-                // eigenvalues (scaled by 1 / tr) for the conditioning flag
-                const df2 ax = df_add(df_add(df_mulf(a, x), df_mulf(d, y)), df_mulf(e, z));
-                const df2 ay = df_add(df_add(df_mulf(d, x), df_mulf(b, y)), df_mulf(g, z));
-                const df2 az = df_add(df_add(df_mulf(e, x), df_mulf(g, y)), df_mulf(cc, z));
-                const float lmin = df_add(df_add(df_mulf(ax, x), df_mulf(ay, y)), df_mulf(az, z)).hi;
-                const float p12 = x * (m00 * x + m01 * y + m02 * z) + y * (m01 * x + m11 * y + m12 * z) +
-                                  z * (m02 * x + m12 * y + m22 * z);
-                const float Sx = 1.0f - lmin;
-                const float disc = fmaxf(Sx * Sx - 4.0f * p12, 0.0f);
-                const float lmax = 0.5f * (Sx + sqrtf(disc));
-                const float lmid = lmax > 0.0f ? p12 / lmax : 0.0f;  // no cancellation
-                if (!(lmid >= 10.0f * lmin)) flags |= 1u;
-                rn[0] = x; rn[1] = y; rn[2] = z;
+        for (int e = 0; e < 6; ++e) v[e] = __ldcg(part + (size_t)(base + j) * 10 + 4 + e);
+#pragma unroll
+        for (int e = 0; e < 6; ++e) A[e] = df_add(A[e], df2{v[e], 0.0f});
+    }
+    block_df_sum<6>(A, sm.sh, sm.tot);
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x, e6 = lane < 6 ? lane : 0, r3 = lane % 4 < 3 ? lane % 4 : 0;
+        FitCluster& f = cl[c];
+        uint32_t flags = 0;
+        const float fx = f.n[0], fy = f.n[1], fz = f.n[2];
+        const float tr = __fadd_rn(__fadd_rn(sm.tot[0].hi, sm.tot[1].hi), sm.tot[2].hi);
+        const bool found = f.best_h >= 0 && f.inliers > 0;
+        float x = fx, y = fy, z = fz;
+        df2 S{0.0f, 0.0f};
+        if (found && tr > 0.0f) {
+            // A / tr: entries of magnitude at most 1 (the diagonal is non-negative); lane e holds entry e of
+            // [[0 3 4] [3 1 5] [4 5 2]]
+            S = df_mulf(sm.tot[e6], __fdiv_rn(1.0f, tr));
+            // symmetric adjugate, lane e: S[i0] S[i1] - S[i2] S[i3] of m00, m11, m22, m01, m02, m12
+            const df2 a0 = df_shfl(S, nib(0x334001u, e6)), a1 = df_shfl(S, nib(0x455122u, e6));
+            const df2 a2 = df_shfl(S, nib(0x043345u, e6)), a3 = df_shfl(S, nib(0x512345u, e6));
+            const float m = df_sub(df_mul(a0, a1), df_mul(a2, a3)).hi;
+            const float m00 = __shfl_sync(0xffffffffu, m, 0), m11 = __shfl_sync(0xffffffffu, m, 1);
+            const float m22 = __shfl_sync(0xffffffffu, m, 2), m01 = __shfl_sync(0xffffffffu, m, 3);
+            const float m02 = __shfl_sync(0xffffffffu, m, 4), m12 = __shfl_sync(0xffffffffu, m, 5);
+            bool ok = true;
+#pragma unroll 1
+            for (int it = 0; it < 6; ++it) {
+                const float nx = __fmaf_rn(m02, z, __fmaf_rn(m01, y, __fmul_rn(m00, x)));
+                const float ny = __fmaf_rn(m12, z, __fmaf_rn(m11, y, __fmul_rn(m01, x)));
+                const float nz = __fmaf_rn(m22, z, __fmaf_rn(m12, y, __fmul_rn(m02, x)));
+                const float q = __fmaf_rn(nz, nz, __fmaf_rn(ny, ny, __fmul_rn(nx, nx)));
+                if (!(q > 1e-30f) || !(q < 1e30f)) { ok = false; break; }  // rank <= 1: keep the RANSAC normal
+                const float sc = rsqrtf(q);
+                x = __fmul_rn(nx, sc); y = __fmul_rn(ny, sc); z = __fmul_rn(nz, sc);
+            }
+            if (!ok) {
+                x = fx; y = fy; z = fz;
+                flags |= 1u;
+            }
+            // unit length to FP32 accuracy
+            const float inv = __fdiv_rn(1.0f, __fsqrt_rn(__fmaf_rn(z, z, __fmaf_rn(y, y, __fmul_rn(x, x)))));
+            x = __fmul_rn(x, inv); y = __fmul_rn(y, inv); z = __fmul_rn(z, inv);
+            if (z < 0.0f || (z == 0.0f && (y < 0.0f || (y == 0.0f && x < 0.0f)))) { x = -x; y = -y; z = -z; }
+            // eigenvalues (scaled by 1 / tr) for the conditioning flag: lanes 0 .. 2 hold the rows of A x, lanes 4
+            // .. 6 the centroid; each times its component, summed in lanes 0 and 4
+            const df2 s0 = df_shfl(S, nib(0x430u, r3)), s1 = df_shfl(S, nib(0x513u, r3)), s2 = df_shfl(S, nib(0x254u, r3));
+            df2 row = df_add(df_add(df_mulf(s0, x), df_mulf(s1, y)), df_mulf(s2, z));
+            if (lane & 4) row = df2{cen[6 * (size_t)c + 2 * r3], cen[6 * (size_t)c + 2 * r3 + 1]};
+            row = df_mulf(row, r3 == 0 ? x : (r3 == 1 ? y : z));
+            const df2 t1 = df_shfl(row, (lane & 4) + 1), t2 = df_shfl(row, (lane & 4) + 2);
+            const float dot = df_add(df_add(row, t1), t2).hi;
+            const float lmin = __shfl_sync(0xffffffffu, dot, 0), cd = __shfl_sync(0xffffffffu, dot, 4);
+            const float p12 = x * (m00 * x + m01 * y + m02 * z) + y * (m01 * x + m11 * y + m12 * z) +
+                              z * (m02 * x + m12 * y + m22 * z);
+            const float Sx = 1.0f - lmin;
+            const float disc = fmaxf(Sx * Sx - 4.0f * p12, 0.0f);
+            const float lmax = 0.5f * (Sx + sqrtf(disc));
+            const float lmid = lmax > 0.0f ? p12 / lmax : 0.0f;  // no cancellation
+            if (!(lmid >= 10.0f * lmin)) flags |= 1u;
+            if (lane == 0) {
+                f.refit_n[0] = x; f.refit_n[1] = y; f.refit_n[2] = z;
+                f.refit_d = -cd;
+                f.flags = flags;
+            }
+        } else if (lane == 0) {
+            float rd = 0.0f;
+            x = y = z = 0.0f;
+            if (found) {  // zero spread: no plane to fit; the RANSAC normal through the centroid
+                flags = 1u;
+                x = fx; y = fy; z = fz;
                 const float* ce = cen + 6 * (size_t)c;
-                const df2 dot = df_add(df_add(df_mulf(df2{ce[0], ce[1]}, x), df_mulf(df2{ce[2], ce[3]}, y)),
-                                       df_mulf(df2{ce[4], ce[5]}, z));
-                rd = -dot.hi;
-            } else if (f.best_h >= 0 && f.inliers > 0) {
-                flags |= 1u;  // zero spread: no plane to fit; the RANSAC normal through the centroid
-                rn[0] = f.n[0]; rn[1] = f.n[1]; rn[2] = f.n[2];
-                const float* ce = cen + 6 * (size_t)c;
-                rd = -df_add(df_add(df_mulf(df2{ce[0], ce[1]}, rn[0]), df_mulf(df2{ce[2], ce[3]}, rn[1])),
-                             df_mulf(df2{ce[4], ce[5]}, rn[2])).hi;
-        }
-        f.refit_n[0] = rn[0]; f.refit_n[1] = rn[1]; f.refit_n[2] = rn[2];
-        f.refit_d = rd;
-        f.flags = flags;
+                rd = -df_add(df_add(df_mulf(df2{ce[0], ce[1]}, x), df_mulf(df2{ce[2], ce[3]}, y)),
+                             df_mulf(df2{ce[4], ce[5]}, z)).hi;
+            }
+            f.refit_n[0] = x; f.refit_n[1] = y; f.refit_n[2] = z;
+            f.refit_d = rd;
+            f.flags = flags;
         }
     }
     __syncthreads();  // shared partials reused next
@@ -896,24 +947,25 @@ __device__ __forceinline__ void refit_cta(uint32_t c, const uint32_t* __restrict
 // The centroid and the refit of every cluster as kernels of their own (a CTA
 // per cluster), for fits too large for the per-cluster completion counters
 // to pay (launch_fit).
-__global__ void __launch_bounds__(kT) k_centroid(const uint32_t* __restrict__ off,
+__global__ void __launch_bounds__(kT) k_centroid(const float* __restrict__ pts, const uint32_t* __restrict__ off,
                                                  const uint32_t* __restrict__ item_off, const uint32_t* __restrict__ kp,
-                                                 int T, const float* __restrict__ part, FitCluster* __restrict__ cl,
-                                                 float* __restrict__ cen) {
+                                                 const uint32_t* __restrict__ tile, const float* __restrict__ part,
+                                                 FitCluster* __restrict__ cl, float* __restrict__ cen,
+                                                 FitPoly* __restrict__ poly) {
     pdl_gate();
-    const uint32_t k = *kp;
-    __shared__ df2 sh[3 * (kT / 32)];
-    __shared__ uint32_t shn[kT / 32];
-    for (uint32_t c = blockIdx.x; c < k; c += gridDim.x) centroid_cta(c, off, item_off, T, part, cl, cen, sh, shn);
+    const uint32_t k = *kp, cpt = *tile / kChunk;
+    __shared__ CentroidShared sm;
+    for (uint32_t c = blockIdx.x; c < k; c += gridDim.x) centroid_cta(c, pts, off, item_off, cpt, part, cl, cen, poly, sm);
 }
 
 __global__ void __launch_bounds__(kT) k_refit(const uint32_t* __restrict__ off, const uint32_t* __restrict__ item_off,
-                                              const uint32_t* __restrict__ kp, int T, const float* __restrict__ part,
-                                              const float* __restrict__ cen, FitCluster* __restrict__ cl) {
+                                              const uint32_t* __restrict__ kp, const uint32_t* __restrict__ tile,
+                                              const float* __restrict__ part, const float* __restrict__ cen,
+                                              FitCluster* __restrict__ cl) {
     pdl_gate();
-    const uint32_t k = *kp;
-    __shared__ df2 sh[6 * (kT / 32)];
-    for (uint32_t c = blockIdx.x; c < k; c += gridDim.x) refit_cta(c, off, item_off, T, part, cen, cl, sh);
+    const uint32_t k = *kp, cpt = *tile / kChunk;
+    __shared__ RefitShared sm;
+    for (uint32_t c = blockIdx.x; c < k; c += gridDim.x) refit_cta(c, off, item_off, cpt, part, cen, cl, sm);
 }
 
 __device__ __forceinline__ unsigned long long xy_key(int2 p) {
@@ -1037,16 +1089,18 @@ __global__ void __launch_bounds__(kT) k_hull(const uint32_t* __restrict__ off, c
                     if (v > bv[q]) { bv[q] = v; bi[q] = i; }
                 }
             }
+            // the warp's largest projection (its bits as an ordered integer), then the lowest index that has it
+            int at[kPer];
 #pragma unroll
             for (int q = 0; q < kPer; ++q) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const float ov = __shfl_xor_sync(0xffffffffu, bv[q], o);
-                    const int oi = __shfl_xor_sync(0xffffffffu, bi[q], o);
-                    if (ov > bv[q] || (ov == bv[q] && oi >= 0 && (bi[q] < 0 || oi < bi[q]))) { bv[q] = ov; bi[q] = oi; }
-                }
-                if (lane == 0) poly[kPer * w + q] = (bi[q] >= 0) ? sv[bi[q]] : make_int2(INT_MIN, INT_MIN);
+                const int b = __float_as_int(bv[q]), key = b ^ ((b >> 31) & 0x7fffffff);
+                const int top = __reduce_max_sync(0xffffffffu, key);
+                at[q] = __reduce_min_sync(0xffffffffu, key == top && bi[q] >= 0 ? bi[q] : INT_MAX);
             }
+            if (lane == 0)
+#pragma unroll
+                for (int q = 0; q < kPer; ++q)
+                    poly[kPer * w + q] = at[q] != INT_MAX ? sv[at[q]] : make_int2(INT_MIN, INT_MIN);
         }
         __syncthreads();
         // The polygon through the extremes, consecutive duplicates removed (and
@@ -1142,35 +1196,52 @@ __global__ void __launch_bounds__(kT) k_hull(const uint32_t* __restrict__ off, c
                 // (4') Andrew's chains by a test per candidate: in the sorted
                 // order, P_i is a vertex of the lower chain iff it is an end or
                 // cross(P_j, P_i, P_k) > 0 for every j < i < k -- the directions
-                // P_i - P_j lie in a half-plane (x >= 0, x = 0 only upwards) where
-                // cross orders them by angle, so it is enough that the most
-                // counter-clockwise of them turns left into the most clockwise of
-                // the P_k - P_i; the upper chain is the same over the reversed
-                // order.  Collinear points fail (cross = 0), as in the chains.
+                // P_i - P_j and P_k - P_i lie in a half-plane (x >= 0, x = 0 only
+                // upwards) where cross orders them by angle, so it is enough that
+                // the most counter-clockwise P_i - P_j turns left into the most
+                // clockwise P_k - P_i; of the upper chain iff the most clockwise
+                // P_i - P_j lies right of the most counter-clockwise P_k - P_i.
+                // Collinear points fail (cross = 0), as in the chains.  Few
+                // candidates share the threads, 4 or 2 to a candidate (48
+                // candidates took a thread each 4.3 us).
+                const int L = u <= kT / 4 ? 4 : (u <= kT / 2 ? 2 : 1), ci = (int)threadIdx.x / L;
+                const int sub = (int)threadIdx.x % L;
                 bool lo = false, hi = false;
-                if (i < u) {
-                    const int2 P = key_xy(uq[i]);
-                    if (i == 0 || i == u - 1) {
-                        lo = hi = true;
-                    } else {
-                        int2 D = make_int2(0, 0), E = make_int2(0, 0), D2 = make_int2(0, 0), E2 = make_int2(0, 0);
-                        for (int j = 0; j < i; ++j) {  // lower: P - P_j (most ccw); upper: P_j - P (most cw)
-                            const int2 Q = key_xy(uq[j]);
-                            const int2 d = make_int2(P.x - Q.x, P.y - Q.y), e2 = make_int2(Q.x - P.x, Q.y - P.y);
-                            if (j == 0 || cross3(make_int2(0, 0), D, d) > 0) D = d;
-                            if (j == 0 || cross3(make_int2(0, 0), e2, E2) > 0) E2 = e2;
-                        }
-                        for (int k2 = i + 1; k2 < u; ++k2) {  // lower: P_k - P (most cw); upper: P - P_k (most ccw)
-                            const int2 Q = key_xy(uq[k2]);
-                            const int2 e = make_int2(Q.x - P.x, Q.y - P.y), d2 = make_int2(P.x - Q.x, P.y - Q.y);
-                            if (k2 == i + 1 || cross3(make_int2(0, 0), e, E) > 0) E = e;
-                            if (k2 == i + 1 || cross3(make_int2(0, 0), D2, d2) > 0) D2 = d2;
-                        }
-                        lo = cross3(make_int2(0, 0), D, E) > 0;
-                        hi = cross3(make_int2(0, 0), D2, E2) > 0;
+                const auto turn = [](int2 a, int2 b) { return (long long)a.x * b.y - (long long)a.y * b.x; };
+                const int2 P = ci < u ? key_xy(uq[ci]) : make_int2(0, 0);
+                int2 dc[2], dw[2];  // most counter-clockwise and most clockwise, before and after; (0, 0): none yet
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    int2 C = make_int2(0, 0), W = make_int2(0, 0);
+                    const int q1 = ci < u ? (t ? u : ci) : 0;
+                    int q = (t ? ci + 1 : 0) + sub;
+                    if (q < q1) {
+                        const int2 Q = key_xy(uq[q]);
+                        C = W = t ? make_int2(Q.x - P.x, Q.y - P.y) : make_int2(P.x - Q.x, P.y - Q.y);
                     }
-                    lo &= i < u - 1;  // the lower chain's last point opens the upper chain
-                    hi &= i > 0;      // and the upper chain's last point is the first of the lower
+#pragma unroll 2
+                    for (q += L; q < q1; q += L) {
+                        const int2 Q = key_xy(uq[q]);
+                        const int2 d = t ? make_int2(Q.x - P.x, Q.y - P.y) : make_int2(P.x - Q.x, P.y - Q.y);
+                        if (turn(C, d) > 0) C = d;
+                        if (turn(d, W) > 0) W = d;
+                    }
+                    for (int o = 1; o < L; o <<= 1) {
+                        const int2 c2 = make_int2(__shfl_xor_sync(0xffffffffu, C.x, o), __shfl_xor_sync(0xffffffffu, C.y, o));
+                        const int2 w2 = make_int2(__shfl_xor_sync(0xffffffffu, W.x, o), __shfl_xor_sync(0xffffffffu, W.y, o));
+                        if (c2.x | c2.y) {
+                            if (!(C.x | C.y) || turn(C, c2) > 0) C = c2;
+                            if (!(W.x | W.y) || turn(w2, W) > 0) W = w2;
+                        }
+                    }
+                    dc[t] = C;
+                    dw[t] = W;
+                }
+                if (ci < u && sub == 0) {
+                    const bool end = ci == 0 || ci == u - 1;
+                    // the lower chain's last point opens the upper chain, whose last point is the lower's first
+                    lo = ci < u - 1 && (end || turn(dc[0], dw[1]) > 0);
+                    hi = ci > 0 && (end || turn(dc[1], dw[0]) > 0);
                 }
                 // lower vertices in increasing order, then upper vertices in decreasing order
                 const uint32_t bl = __ballot_sync(0xffffffffu, lo), bh = __ballot_sync(0xffffffffu, hi);
@@ -1186,8 +1257,8 @@ __global__ void __launch_bounds__(kT) k_hull(const uint32_t* __restrict__ off, c
                     plo += q < w ? (int)wsum[q] : 0;
                     phi += q > w ? (int)st_hi[q] : 0;
                 }
-                if (lo) out[plo] = key_xy(uq[i]);
-                if (hi) out[klo + phi] = key_xy(uq[i]);
+                if (lo) out[plo] = P;
+                if (hi) out[klo + phi] = P;
                 if (i == 0) hull_cnt[c] = (uint32_t)(klo + khi);
             }
         } else if (s2 <= kHullCap) {
@@ -1338,18 +1409,31 @@ __global__ void __launch_bounds__(kT) k_hull(const uint32_t* __restrict__ off, c
     }
 }
 
+// The tile of a fit: the tuning's, or, when the fit may choose (adapt_ctas),
+// the smallest multiple of a chunk that gives the points at most adapt_ctas
+// work items, so that a small fit's scoring, extraction and filter passes
+// spread over the GPU.  (240 thousand points of a walk map: 157 items of 2048
+// on 152 SMs scored in 21 us, 490 of 512 in 12 us; one 17,000-point cluster: 9
+// items in 14 us, 68 in 6 us.)  Results do not depend on the tile.
+__device__ __forceinline__ uint32_t choose_tile(uint32_t T, uint32_t n, uint32_t adapt_ctas) {
+    if (!adapt_ctas) return T;
+    const uint32_t want = (n / adapt_ctas + kChunk) / kChunk * kChunk;
+    return want < T ? want : T;
+}
+
 // Work items per cluster (scanned into the item offsets next) -- at least one,
 // so that an empty cluster's per-cluster steps still run -- the work queue's
 // heads and the per-cluster completion counters (done, may be null) cleared
-// for the fit that follows.
-__global__ void k_items(const uint32_t* __restrict__ off, const uint32_t* __restrict__ kp, int T,
-                        uint32_t* __restrict__ item_cnt, uint32_t* __restrict__ queue, uint32_t* __restrict__ done) {
+// for the fit that follows; queue[1] receives the tile.
+__global__ void k_items(const uint32_t* __restrict__ off, const uint32_t* __restrict__ kp, uint32_t tile,
+                        uint32_t adapt_ctas, uint32_t* __restrict__ item_cnt, uint32_t* __restrict__ queue,
+                        uint32_t* __restrict__ done) {
     pdl_gate();
-    const uint32_t k = *kp;
-    if (blockIdx.x == 0 && threadIdx.x < 4) queue[threadIdx.x] = 0;
+    const uint32_t k = *kp, T = choose_tile(tile, off[k], adapt_ctas);
+    if (blockIdx.x == 0 && threadIdx.x < 4) queue[threadIdx.x] = threadIdx.x == 1 ? T : 0u;
     for (uint32_t c = blockIdx.x * kT + threadIdx.x; c < k; c += gridDim.x * kT) {
         const uint32_t n = off[c + 1] - off[c];
-        item_cnt[c] = n ? (n + (uint32_t)T - 1) / (uint32_t)T : 1u;
+        item_cnt[c] = n ? (n + T - 1) / T : 1u;
         if (done) done[3 * (size_t)c] = done[3 * (size_t)c + 1] = done[3 * (size_t)c + 2] = 0u;
     }
 }
@@ -1360,22 +1444,22 @@ __global__ void k_items(const uint32_t* __restrict__ off, const uint32_t* __rest
 constexpr int kItemsScanT = 1024;
 constexpr uint32_t kItemsScanMax = 16384;
 __global__ void __launch_bounds__(kItemsScanT) k_items_scan(const uint32_t* __restrict__ off,
-                                                             const uint32_t* __restrict__ kp, int T,
-                                                             uint32_t* __restrict__ item_off,
+                                                             const uint32_t* __restrict__ kp, uint32_t tile,
+                                                             uint32_t adapt_ctas, uint32_t* __restrict__ item_off,
                                                              uint32_t* __restrict__ queue,
                                                              uint32_t* __restrict__ done) {
     pdl_gate();
     __shared__ uint32_t ws[kItemsScanT / 32];
-    const uint32_t k = *kp;
+    const uint32_t k = *kp, T = choose_tile(tile, off[k], adapt_ctas);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (threadIdx.x < 4) queue[threadIdx.x] = 0;
+    if (threadIdx.x < 4) queue[threadIdx.x] = threadIdx.x == 1 ? T : 0u;
     uint32_t carry = 0;
     for (uint32_t c0 = 0; c0 < k; c0 += kItemsScanT) {
         const uint32_t c = c0 + threadIdx.x;
         uint32_t v = 0;
         if (c < k) {
             const uint32_t n = off[c + 1] - off[c];
-            v = n ? (n + (uint32_t)T - 1) / (uint32_t)T : 1u;
+            v = n ? (n + T - 1) / T : 1u;
             if (done) done[3 * (size_t)c] = done[3 * (size_t)c + 1] = done[3 * (size_t)c + 2] = 0u;
         }
         uint32_t inc = v;
@@ -1423,11 +1507,13 @@ template <int R>
 __global__ void __launch_bounds__(kT) k_score_warp(const float* __restrict__ pts, const uint32_t* __restrict__ off,
                                                    const uint32_t* __restrict__ item_off,
                                                    const uint32_t* __restrict__ item_cl,
-                                                   const uint32_t* __restrict__ kp, int H, int T,
+                                                   const uint32_t* __restrict__ kp, int H,
+                                                   const uint32_t* __restrict__ tile,
                                                    const float4* __restrict__ hyp, uint32_t* __restrict__ counts,
                                                    uint32_t* __restrict__ queue, float eps) {
     pdl_wait();
     const uint32_t k = *kp;
+    const int T = (int)*tile;
     extern __shared__ float4 sp[];  // [kT / 32][T]
     const int lane = threadIdx.x & 31;
     float4* wp = sp + (size_t)(threadIdx.x >> 5) * T;
@@ -1488,7 +1574,8 @@ struct ScoreArgs {
     const uint32_t* item_off;
     const uint32_t* item_cl;  // item -> cluster table, or null for a binary search
     const uint32_t* kp;
-    int H, T;
+    int H, T;              // T: the largest tile, which sizes shared memory
+    const uint32_t* tile;  // the tile (device)
     const float4* hyp;
     uint32_t* counts;
     uint32_t* queue;
@@ -1501,7 +1588,7 @@ cudaError_t launch_score(const ScoreArgs& a, cudaStream_t s) {
     const int G = (a.H + R - 1) / R;
     const int P = kT / G;
     const size_t smem = (size_t)a.T * sizeof(float4) + (size_t)P * G * R * sizeof(uint32_t);
-    launch_full(k_score<R>, dim3(a.grid), dim3(kT), smem, s, a.pts, a.off, a.item_off, a.item_cl, a.kp, a.H, a.T,
+    launch_full(k_score<R>, dim3(a.grid), dim3(kT), smem, s, a.pts, a.off, a.item_off, a.item_cl, a.kp, a.H, a.tile,
                 a.hyp, a.counts, a.queue, a.eps);
     return cudaGetLastError();
 }
@@ -1510,7 +1597,7 @@ template <int R>
 cudaError_t launch_score_warp(const ScoreArgs& a, cudaStream_t s) {
     const size_t smem = (size_t)(kT / 32) * a.T * sizeof(float4);
     launch_full(k_score_warp<R>, dim3(a.grid), dim3(kT), smem, s, a.pts, a.off, a.item_off, a.item_cl, a.kp, a.H,
-                a.T, a.hyp, a.counts, a.queue, a.eps);
+                a.tile, a.hyp, a.counts, a.queue, a.eps);
     return cudaGetLastError();
 }
 
@@ -1518,7 +1605,7 @@ __global__ void k_set_u32(uint32_t* __restrict__ p, uint32_t v) { pdl_gate(); *p
 
 }  // namespace
 
-FitTuning default_tuning() { return FitTuning{2048, 4, 4, 0}; }
+FitTuning default_tuning() { return FitTuning{2048, 4, 4, 0, 1}; }
 
 // The scoring variant launch_fit picks for t and H: hypotheses per thread
 // and whether the warp schedule applies.
@@ -1592,12 +1679,15 @@ cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* la
     const int T = (t.tile + (int)kChunk - 1) / (int)kChunk * (int)kChunk;  // callers validate; never below a chunk
     cudaError_t e;
     VM_STAGE_BEGIN(hk, kStHyp, s);
+    const uint32_t adapt = t.adapt ? (uint32_t)(sms * t.ctas_per_sm) : 0u;
+    const uint32_t* tile = fb.queue + 1;
     if (kcap <= kItemsScanMax) {
-        launch_k(k_items_scan, dim3(1), dim3(kItemsScanT), 0, s, off, kp, T, fb.item_off, fb.queue, fb.done);
+        launch_k(k_items_scan, dim3(1), dim3(kItemsScanT), 0, s, off, kp, (uint32_t)T, adapt, fb.item_off, fb.queue,
+                 fb.done);
         count_launch(1);
     } else {
         const unsigned kgrid = (kcap + kT - 1) / kT < (uint32_t)sms * 8 ? (kcap + kT - 1) / kT : (uint32_t)sms * 8;
-        launch_k(k_items, dim3(kgrid), dim3(kT), 0, s, off, kp, T, fb.item_off, fb.queue, fb.done);
+        launch_k(k_items, dim3(kgrid), dim3(kT), 0, s, off, kp, (uint32_t)T, adapt, fb.item_off, fb.queue, fb.done);
         e = exclusive_scan_dev(fb.item_off, fb.item_off, fb.tot, kp, kcap, fb.scan_tmp, s, fb.err, true);
         if (e != cudaSuccess) return e;
         count_launch(1);
@@ -1623,7 +1713,7 @@ cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* la
     // Results are the same.
     uint32_t* done = fb.npts_cap <= kFusedFitPoints ? fb.done : nullptr;
     VM_STAGE_BEGIN(hk, kStScore, s);
-    const ScoreArgs sa{pts, off, fb.item_off, fb.item_cl, kp, H, T, fb.hyp, fb.counts, fb.queue, p.eps, grid};
+    const ScoreArgs sa{pts, off, fb.item_off, fb.item_cl, kp, H, T, tile, fb.hyp, fb.counts, fb.queue, p.eps, grid};
     if (warp) {
         switch (R) {
             case 1: e = launch_score_warp<1>(sa, s); break;
@@ -1651,18 +1741,19 @@ cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* la
     count_launch(1);
     const unsigned igrid = (unsigned)sms * 8;
     launch_full(done ? k_extract<true> : k_extract<false>, dim3(igrid), dim3(kT), 0, s, pts, off, fb.item_off,
-                fb.item_cl, kp, T, fb.cl, fb.inlier, fb.part, p.eps, fb.err, done, fb.cen);
+                fb.item_cl, kp, tile, fb.cl, fb.inlier, fb.part, p.eps, fb.err, done, fb.cen, fb.poly);
     if (!done) {
-        launch_k(k_centroid, dim3(cgrid), dim3(kT), 0, s, off, fb.item_off, kp, T, fb.part, fb.cl, fb.cen);
+        launch_k(k_centroid, dim3(cgrid), dim3(kT), 0, s, pts, off, fb.item_off, kp, tile, fb.part, fb.cl,
+                 fb.cen, fb.poly);
         count_launch(1);
     }
     launch_full(done ? k_filter<true> : k_filter<false>, dim3(igrid), dim3(kT), 0, s, pts, off, fb.item_off,
-                fb.item_cl, kp, T, fb.cl, fb.inlier, fb.cen, fb.part, fb.surv, done);
+                fb.item_cl, kp, tile, fb.cl, fb.inlier, fb.cen, fb.poly, fb.part, fb.surv, done);
     VM_STAGE_END(hk, kStExtract, s);
     count_launch(2);
     VM_STAGE_BEGIN(hk, kStHull, s);
     if (!done) {
-        launch_k(k_refit, dim3(cgrid), dim3(kT), 0, s, off, fb.item_off, kp, T, fb.part, fb.cen, fb.cl);
+        launch_k(k_refit, dim3(cgrid), dim3(kT), 0, s, off, fb.item_off, kp, tile, fb.part, fb.cen, fb.cl);
         count_launch(1);
     }
     launch_k(k_hull, dim3(cgrid), dim3(kT), fit_hull_smem(), s, off, kp, fb.cl, fb.surv, fb.hull, fb.hull_cnt, fb.err,
@@ -1800,7 +1891,7 @@ extern "C" vm_status vm_ransac_static(const float* xyz, const uint32_t* off, con
     fit_init_attributes();
     // the work queue starts at zero every call (k_items); counts are zeroed by k_hyp
     launch_k(k_set_u32, dim3(1), dim3(1), 0, s, kdev, k);
-    launch_k(k_items, dim3((k + kT - 1) / kT), dim3(kT), 0, s, off, kdev, t.tile, item_off, queue,
+    launch_k(k_items, dim3((k + kT - 1) / kT), dim3(kT), 0, s, off, kdev, (uint32_t)t.tile, 0u, item_off, queue,
              static_cast<uint32_t*>(nullptr));
     if ((e = exclusive_scan_dev(item_off, item_off, total, kdev, k, scan_tmp, s, nullptr, true)) != cudaSuccess)
         return cuda_status(e, "scan");
@@ -1817,7 +1908,7 @@ extern "C" vm_status vm_ransac_static(const float* xyz, const uint32_t* off, con
     bool warp;
     score_variant(tc, H, R, warp);
     const int grid = sms * t.ctas_per_sm;
-    const ScoreArgs sa{xyz, off, item_off, nullptr, kdev, H, t.tile, hyp, counts, queue, params->eps, grid};
+    const ScoreArgs sa{xyz, off, item_off, nullptr, kdev, H, t.tile, queue + 1, hyp, counts, queue, params->eps, grid};
     switch (R) {
         case 1: e = launch_score<1>(sa, s); break;
         case 2: e = launch_score<2>(sa, s); break;

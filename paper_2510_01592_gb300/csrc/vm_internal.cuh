@@ -150,6 +150,15 @@ struct FitCluster {
     unsigned long long ext[16]; // filter extremes: (biased value << 32) | point index
 };
 
+// The filter polygon of a cluster: the distinct extreme inliers along the 16
+// filter directions, counter-clockwise, and each edge's scaled line (k_filter).
+constexpr int kFiltDirs = 16;
+struct alignas(16) FitPoly {
+    float4 edge[kFiltDirs];  // (ex / E, -ey / E, -c / E): F = x bf + y af + z; padding never decides
+    int2 pt[kFiltDirs + 1];  // the vertices, the first one again after the last
+    int m;                   // vertices; 0: a degenerate (zero-area) polygon filters nothing
+};
+
 // One cluster's output record: the refit plane, the selected hypothesis, the
 // hull basis and origin; ho / hn: its first hull vertex and vertex count.
 __device__ __forceinline__ vm_plane make_plane(const FitCluster& f, uint32_t label, uint32_t n_points, uint32_t ho,
@@ -401,9 +410,10 @@ struct FitBuffers {
     FitCluster* cl;         // [kcap]
     uint32_t* item_off;     // [kcap + 1] work-item offsets (scan)
     uint32_t* item_cl;      // [items] the cluster of each work item
-    uint32_t* queue;        // [4] work-queue heads
+    uint32_t* queue;        // [4] work-queue head, the tile, -, the hull pass's count
     uint8_t* inlier;        // [npts]
     float* part;            // [items][10] per-item partial sums
+    FitPoly* poly;          // [kcap] filter polygons
     float* cen;             // [kcap][3][2] inlier centroids, double-float (hi, lo)
     int2* surv;             // [npts] hull candidates (per-cluster segments at cluster offsets)
     int2* hull;             // [npts] hull vertices (per-cluster segments at cluster offsets)
@@ -422,11 +432,13 @@ struct FitTuning {
     int hyp_per_thread;     // hypotheses held in registers per thread
     int ctas_per_sm;        // persistent CTAs per SM
     int schedule;           // 0: a CTA per work item; 1: a warp per work item
+    int adapt;              // 1: a small fit may take a smaller tile (the default schedule)
 };
 FitTuning default_tuning();
 // Resident scoring CTAs per SM for tuning t and H hypotheses (0 on error).
 int score_max_ctas_per_sm(const FitTuning& t, int H);
 size_t fit_hull_smem();
+
 
 // Runs RANSAC, selection, extraction, refit and hull for the clusters whose
 // points are pts[off[c]..off[c+1]) (device), labels (device, or nullptr for
