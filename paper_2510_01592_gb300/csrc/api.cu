@@ -84,6 +84,8 @@ static void fit_layout(Carver& c, FitBuffers& fb, size_t kcap, size_t npts, size
     fb.inlier = c.take<uint8_t>(npts + 1);
     fb.part = c.take<float>((chunks + 1) * 10);
     fb.cen = c.take<float>(kcap * 6);
+    fb.ref = c.take<float4>(kcap);
+    fb.lower = c.take<uint32_t>(kcap);
     fb.poly = c.take<FitPoly>(kcap);
     fb.surv = c.take<int2>(npts + 1);
     fb.hull = c.take<int2>(npts + 1);
@@ -120,7 +122,7 @@ vm_status fit_prepare(FitContext& fc, size_t kcap, size_t npts, int H, int tile,
     fit_layout(c, fb, k2, n2, c2, H2);
     VM_CUDA(cudaMemsetAsync(fb.scan_tmp, 0, scan_tmp_words(k2 + 1) * sizeof(uint32_t), s));  // scan state
     fb.kcap = k2;
-    fb.npts_cap = n2;
+    fb.npts_cap = fb.npts_expect = n2;
     fb.items_cap = c2;
     fb.H = H2;
     fc.fb = fb;
@@ -470,6 +472,8 @@ cudaError_t enqueue_segment(vm_map* m, const vm_segment_params& p, StageHook* hk
     const int sms = device_sms();
     SegBuffers& b = m->seg;
     FitBuffers& fb = m->fit.fb;
+    // the scratch has room for every slot of the bricks; about a fifth hold a clustered voxel
+    fb.npts_expect = m->last.n_kept ? (size_t)m->last.n_kept + m->last.n_kept / 4 : m->seg_nv / 4;
     cudaError_t e;
     if ((e = enqueue_front(m, p, hk, fb.err)) != cudaSuccess) return e;
     char* d = m->out_dev;

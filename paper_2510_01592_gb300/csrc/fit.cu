@@ -8,7 +8,8 @@
 //            work items from an atomic queue, stage the tile in shared memory
 //            and test every point against every hypothesis held in registers;
 //            integer counts are summed in shared memory and added to global
-//            memory with integer atomics (order-free, hence exact).
+//            memory with integer atomics (order-free, hence exact).  Large fits
+//            take k_score_slab, which bounds most tests instead of making them.
 //  k_select  stage c: max count, lowest hypothesis index on ties; in-plane
 //            basis and hull origin.
 //  k_extract inliers of the selected plane, centroid partial sums and the
@@ -37,7 +38,8 @@ namespace {
 constexpr int kT = 256;
 constexpr int kHullCap = 2048;   // hull candidates sorted in shared memory
 constexpr int kSurvCap = 12288;  // first-filter survivors staged in shared memory
-constexpr size_t kFusedFitPoints = size_t(4) << 20;  // fits of at most this many points: per-cluster tails fused
+constexpr size_t kFusedFitPoints = size_t(4) << 20;  // fits expected to have at most this many points: per-cluster
+                                                     // tails fused, every test of stage b made
 
 // ---------------------------------------------------------------- Philox
 __device__ __forceinline__ void philox4x64_10(const unsigned long long ctr[4], const unsigned long long key[2],
@@ -80,6 +82,21 @@ __device__ __forceinline__ void count_point(const float4 (&pl)[R], float4 p, flo
     }
 }
 
+// Two points at once: the two masks come off the count in one three-input add.
+template <int R>
+__device__ __forceinline__ void count_points2(const float4 (&pl)[R], float4 p, float4 q, float eps,
+                                              uint32_t (&acc)[R]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float a = plane_dist(pl[r].x, pl[r].y, pl[r].z, pl[r].w, p.x, p.y, p.z);
+        const float b = plane_dist(pl[r].x, pl[r].y, pl[r].z, pl[r].w, q.x, q.y, q.z);
+        uint32_t t, u;
+        asm("set.le.u32.f32 %0, %1, %2;" : "=r"(t) : "f"(a), "f"(eps));
+        asm("set.le.u32.f32 %0, %1, %2;" : "=r"(u) : "f"(b), "f"(eps));
+        acc[r] = acc[r] - t - u;
+    }
+}
+
 // The cluster of work item it: one load from the item -> cluster table k_hyp
 // writes (item_cl), else a binary search over the item offsets.
 __device__ __forceinline__ uint32_t find_cluster(const uint32_t* __restrict__ item_cl,
@@ -95,12 +112,13 @@ __device__ __forceinline__ uint32_t find_cluster(const uint32_t* __restrict__ it
 
 // ---------------------------------------------------------------- stage a
 // Also writes the item -> cluster table (item_cl, when not null): the thread
-// of hypothesis 0 of each cluster fills its cluster's items.
+// of hypothesis 0 of each cluster fills its cluster's items.  from_all: the
+// counts start at the cluster's size (k_score_slab takes the misses off).
 __global__ void k_hyp(const float* __restrict__ pts, const uint32_t* __restrict__ off,
                       const uint32_t* __restrict__ labels, const uint32_t* __restrict__ kp, int H,
                       unsigned long long seed, uint32_t round, float4* __restrict__ hyp, uint8_t* __restrict__ valid,
                       uint32_t* __restrict__ counts, const uint32_t* __restrict__ item_off,
-                      uint32_t* __restrict__ item_cl) {
+                      uint32_t* __restrict__ item_cl, uint32_t* __restrict__ lower, bool from_all) {
     pdl_gate();
     const uint32_t k = *kp;
     const size_t total = (size_t)k * H;
@@ -115,7 +133,7 @@ __global__ void k_hyp(const float* __restrict__ pts, const uint32_t* __restrict_
         philox4x64_10(ctr, key, r);
         const uint32_t i0 = (uint32_t)__umul64hi(r[0], n), i1 = (uint32_t)__umul64hi(r[1], n),
                        i2 = (uint32_t)__umul64hi(r[2], n);
-        counts[t] = 0;
+        if (from_all && h == 0) lower[c] = 0;
         uint8_t ok = (i0 != i1) && (i0 != i2) && (i1 != i2);
         float4 pl = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(0x7f800000));  // never an inlier
         if (ok) {
@@ -139,6 +157,7 @@ __global__ void k_hyp(const float* __restrict__ pts, const uint32_t* __restrict_
         }
         hyp[t] = pl;
         valid[t] = ok;
+        counts[t] = from_all && fabsf(pl.w) < __int_as_float(0x7f800000) ? n : 0u;  // no point is near any other plane
     }
 }
 
@@ -1567,6 +1586,336 @@ __global__ void __launch_bounds__(kT) k_score_warp(const float* __restrict__ pts
     }
 }
 
+// ---------------------------------------------------------------- stage b, large fits
+// The reference plane of each cluster for k_score_slab: the hypothesis with the
+// most inliers among kRefPts points spread over the cluster (any plane serves;
+// a good one decides more tiles at once).  w is infinite when no hypothesis is
+// valid.  One CTA a cluster, a thread per hypothesis.
+constexpr int kRefPts = 64;
+__global__ void __launch_bounds__(kT) k_score_ref(const float* __restrict__ pts, const uint32_t* __restrict__ off,
+                                                  const uint32_t* __restrict__ kp, int H,
+                                                  const float4* __restrict__ hyp, float4* __restrict__ ref, float eps) {
+    pdl_gate();
+    const uint32_t k = *kp;
+    __shared__ float4 sp[kRefPts];
+    __shared__ unsigned long long wbest[kT / 32];
+    for (uint32_t c = blockIdx.x; c < k; c += gridDim.x) {
+        const uint32_t base = off[c], n = off[c + 1] - base, m = n < (uint32_t)kRefPts ? n : (uint32_t)kRefPts;
+        __syncthreads();
+        if (threadIdx.x < m) {
+            const float* p = pts + 3 * ((size_t)base + (size_t)threadIdx.x * n / m);
+            sp[threadIdx.x] = make_float4(p[0], p[1], p[2], 0.0f);
+        }
+        __syncthreads();
+        unsigned long long best = 0;  // inliers + 1 << 32 | ~h
+        for (int h = threadIdx.x; h < H; h += kT) {
+            const float4 pl[1] = {hyp[(size_t)c * H + h]};
+            if (!(fabsf(pl[0].w) < __int_as_float(0x7f800000))) continue;
+            uint32_t in[1] = {1u};
+            for (uint32_t q = 0; q < m; ++q) count_point<1>(pl, sp[q], eps, in);
+            const unsigned long long key = ((unsigned long long)in[0] << 32) | (uint32_t)~(uint32_t)h;
+            best = key > best ? key : best;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long t = __shfl_xor_sync(0xffffffffu, best, o);
+            best = t > best ? t : best;
+        }
+        if ((threadIdx.x & 31) == 0) wbest[threadIdx.x >> 5] = best;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < kT / 32; ++w) best = wbest[w] > best ? wbest[w] : best;
+            ref[c] = best ? hyp[(size_t)c * H + (int)(~(uint32_t)(best & 0xffffffffu))]
+                          : make_float4(0.0f, 0.0f, 0.0f, __int_as_float(0x7f800000));
+        }
+    }
+}
+
+// A float's order as an integer's.
+__device__ __forceinline__ int ord(float x) {
+    const int b = __float_as_int(x);
+    return b ^ ((b >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float unord(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
+
+// The inliers of each cluster's reference plane: a lower bound of the best count.
+__global__ void __launch_bounds__(kT) k_score_lower(const float* __restrict__ pts, const uint32_t* __restrict__ off,
+                                                    const uint32_t* __restrict__ item_off,
+                                                    const uint32_t* __restrict__ item_cl,
+                                                    const uint32_t* __restrict__ kp, const uint32_t* __restrict__ tile,
+                                                    const float4* __restrict__ ref, uint32_t* __restrict__ lower,
+                                                    float eps) {
+    pdl_gate();
+    const uint32_t k = *kp, T = *tile, n_items = item_off[k];
+    for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
+        const uint32_t c = find_cluster(item_cl, item_off, k, it);
+        const uint32_t start = off[c] + (it - item_off[c]) * T, end = min(off[c + 1], start + T);
+        const float4 r0[1] = {ref[c]};
+        uint32_t in[1] = {0u};
+#pragma unroll 4
+        for (uint32_t q = start + threadIdx.x; q < end; q += kT)
+            count_point<1>(r0, make_float4(pts[3 * (size_t)q], pts[3 * (size_t)q + 1], pts[3 * (size_t)q + 2], 0.0f), eps, in);
+        in[0] = __reduce_add_sync(0xffffffffu, in[0]);
+        if ((threadIdx.x & 31) == 0 && in[0]) atomicAdd(lower + c, in[0]);
+    }
+}
+
+// Stage b for large fits: the best count, and every count that could be it, with
+// far fewer tests than k_score.
+// (1) A tile's points within eps / 2 of the cluster's reference plane (n0, d0),
+// the near points, are bounded by their range of residuals and a box aligned
+// with the plane and their longest direction.  For a hypothesis (n, d) the
+// residual of a near point is its reference residual plus (n - n0) . p + (d -
+// d0), which is linear, so the box bounds it; when the bound lies within eps
+// every near point is an inlier, and when it lies beyond eps none is: no test
+// is made.  The points off the plane (outliers) are tested against every
+// hypothesis, the near points against those the bound leaves open.  All tests
+// are count_point's, and the bound is widened by 2^-16 (|d| + |d0| + sum of the
+// largest |coordinates|), over 250 rounding units of every quantity that enters
+// it or the test (their sum stays below 150), so the counts are exact.
+// (2) counts start at the cluster's size and lose a tile's misses.  A
+// hypothesis whose count has fallen below the reference plane's inliers cannot
+// be selected any more and is dropped; its count stays below the best one.  The
+// tiles of a cluster are taken spread over the launch, so that a poor
+// hypothesis is dropped after a few of them.
+// On the batch of 2,000 clusters (48 M points, 5 % outliers, H = 256, tile 2048)
+// about a fifth of the tests remain (two fifths without (2)): 1.23 ms in place
+// of 2.86 ms, and 0.11 ms for the two passes before it.
+constexpr float kSlabErr = 1.52587890625e-05f;  // 2^-16
+template <int R>
+__global__ void __launch_bounds__(kT) k_score_slab(const float* __restrict__ pts, const uint32_t* __restrict__ off,
+                                                   const uint32_t* __restrict__ item_off,
+                                                   const uint32_t* __restrict__ item_cl,
+                                                   const uint32_t* __restrict__ kp, int H,
+                                                   const uint32_t* __restrict__ tile,
+                                                   const float4* __restrict__ hyp, const float4* __restrict__ ref,
+                                                   const uint32_t* __restrict__ lower, uint32_t* __restrict__ counts,
+                                                   uint32_t* __restrict__ queue, float eps) {
+    pdl_wait();
+    const uint32_t k = *kp;
+    const int T = (int)*tile;
+    extern __shared__ float4 sp[];                         // T points: the near ones from the front, the others from the back
+    uint32_t* hc = reinterpret_cast<uint32_t*>(sp + T);    // [H] inliers of the tile
+    uint16_t* open = reinterpret_cast<uint16_t*>(hc + H);  // [H] hypotheses the bound leaves open
+    uint16_t* alive = open + H;                            // [H] hypotheses still in the race
+    __shared__ uint32_t s_item, s_near, s_far, s_open, s_alive, s_step;
+    __shared__ int smin[kT / 32][4], smax[kT / 32][4];
+    __shared__ unsigned long long sfar[kT / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t n_items = item_off[k];
+    const float inf = __int_as_float(0x7f800000);
+    if (threadIdx.x == 0) {
+        uint32_t step = (uint32_t)(0.618034 * (double)n_items) | 1u;
+        for (;; ++step) {  // ends: n_items + 1 is coprime to n_items
+            uint32_t a = step, b = n_items;
+            while (b) {
+                const uint32_t t = a % b;
+                a = b;
+                b = t;
+            }
+            if (a == 1u || step > n_items) break;
+        }
+        s_step = step;
+    }
+    for (int guard = 0; guard < kLoopCap; ++guard) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_item = atomicAdd(queue, 1u);
+            s_near = s_far = s_open = s_alive = 0;
+        }
+        for (int h = threadIdx.x; h < H; h += kT) hc[h] = 0;
+        __syncthreads();
+        if (s_item >= n_items) break;
+        // a step coprime to the item count spreads each cluster's tiles over the launch
+        const uint32_t it = (uint32_t)((unsigned long long)s_item * s_step % n_items);
+        const uint32_t c = find_cluster(item_cl, item_off, k, it);
+        const uint32_t start = off[c] + (it - item_off[c]) * (uint32_t)T;
+        const int cnt = (int)(min(off[c + 1], start + (uint32_t)T) - start);
+        const float4 r0 = ref[c];
+        const float4* hy = hyp + (size_t)c * H;
+        // near and other points; the near ones' bounds: x, y, z and the residual
+        float lo[4] = {inf, inf, inf, inf}, hi[4] = {-inf, -inf, -inf, -inf};
+#pragma unroll 4
+        for (int q0 = 0; q0 < cnt; q0 += kT) {
+            const int q = q0 + threadIdx.x;
+            float v[4] = {0.0f, 0.0f, 0.0f, inf};
+            if (q < cnt) {
+                const float* p = pts + 3 * ((size_t)start + q);
+                v[0] = p[0]; v[1] = p[1]; v[2] = p[2];
+                v[3] = __fmaf_rn(r0.z, v[2], __fmaf_rn(r0.y, v[1], __fmaf_rn(r0.x, v[0], r0.w)));
+            }
+            const bool near = fabsf(v[3]) <= 0.5f * eps, far = q < cnt && !near;  // not a number: far
+            const uint32_t bn = __ballot_sync(0xffffffffu, near), bf = __ballot_sync(0xffffffffu, far);
+            uint32_t an = 0, af = 0;
+            if (lane == 0) {
+                if (bn) an = atomicAdd(&s_near, (uint32_t)__popc(bn));
+                if (bf) af = atomicAdd(&s_far, (uint32_t)__popc(bf));
+            }
+            an = __shfl_sync(0xffffffffu, an, 0) + __popc(bn & lt);
+            af = __shfl_sync(0xffffffffu, af, 0) + __popc(bf & lt);
+            if (near | far) sp[near ? (int)an : T - 1 - (int)af] = make_float4(v[0], v[1], v[2], 0.0f);
+            if (near)
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    lo[a] = fminf(lo[a], v[a]);
+                    hi[a] = fmaxf(hi[a], v[a]);
+                }
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int l = __reduce_min_sync(0xffffffffu, ord(lo[a])), g = __reduce_max_sync(0xffffffffu, ord(hi[a]));
+            if (lane == a) {
+                smin[w][a] = l;
+                smax[w][a] = g;
+            }
+        }
+        __syncthreads();
+        const int nn = (int)s_near, nf = (int)s_far;
+        float ctr[3], half[3], sumM = 0.0f, rlo = 0.0f, rhi = 0.0f;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            int l = smin[0][a], g = smax[0][a];
+#pragma unroll
+            for (int q = 1; q < kT / 32; ++q) {
+                l = min(l, smin[q][a]);
+                g = max(g, smax[q][a]);
+            }
+            const float fl = unord(l), fg = unord(g);
+            if (a < 3) {
+                ctr[a] = 0.5f * (fl + fg);
+                half[a] = 0.5f * (fg - fl);
+                sumM += fmaxf(fabsf(fl), fabsf(fg));
+            } else {
+                rlo = fl;
+                rhi = fg;
+            }
+        }
+        // the longest direction: towards the near point farthest from the box's centre
+        unsigned long long best = 0;
+        for (int q = threadIdx.x; q < nn; q += kT) {
+            const float4 p = sp[q];
+            const float dx = p.x - ctr[0], dy = p.y - ctr[1], dz = p.z - ctr[2];
+            const unsigned long long key =
+                ((unsigned long long)__float_as_uint(dx * dx + dy * dy + dz * dz) << 32) | (uint32_t)q;
+            best = key > best ? key : best;
+        }
+        const uint32_t top = __reduce_max_sync(0xffffffffu, (uint32_t)(best >> 32));
+        const uint32_t who = __reduce_max_sync(0xffffffffu, (uint32_t)(best >> 32) == top ? (uint32_t)best : 0u);
+        if (lane == 0) sfar[w] = ((unsigned long long)top << 32) | who;
+        __syncthreads();
+        best = sfar[0];
+#pragma unroll
+        for (int q = 1; q < kT / 32; ++q) best = sfar[q] > best ? sfar[q] : best;
+        float ax = 0.0f, ay = 0.0f, az = 0.0f;
+        if (nn) {
+            const float4 p = sp[(uint32_t)best];
+            ax = p.x - ctr[0];
+            ay = p.y - ctr[1];
+            az = p.z - ctr[2];
+        }
+        const float along = ax * r0.x + ay * r0.y + az * r0.z;
+        ax -= along * r0.x;
+        ay -= along * r0.y;
+        az -= along * r0.z;
+        const float len2 = ax * ax + ay * ay + az * az;
+        const bool framed = len2 > 1e-12f && len2 < 1e12f;  // else the axis-aligned box alone
+        const float il = framed ? rsqrtf(len2) : 0.0f;
+        ax *= il;
+        ay *= il;
+        az *= il;
+        const float bx = r0.y * az - r0.z * ay, by = r0.z * ax - r0.x * az, bz = r0.x * ay - r0.y * ax;
+        float ea = 0.0f, eb = 0.0f;
+        for (int q = threadIdx.x; q < nn; q += kT) {
+            const float4 p = sp[q];
+            const float dx = p.x - ctr[0], dy = p.y - ctr[1], dz = p.z - ctr[2];
+            ea = fmaxf(ea, fabsf(dx * ax + dy * ay + dz * az));
+            eb = fmaxf(eb, fabsf(dx * bx + dy * by + dz * bz));
+        }
+        const uint32_t ua = __reduce_max_sync(0xffffffffu, __float_as_uint(ea));
+        const uint32_t ub = __reduce_max_sync(0xffffffffu, __float_as_uint(eb));
+        __syncthreads();  // smin / smax read above
+        if (lane == 0) {
+            smax[w][0] = (int)ua;
+            smax[w][1] = (int)ub;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kT / 32; ++q) {
+            ea = fmaxf(ea, __int_as_float(smax[q][0]));
+            eb = fmaxf(eb, __int_as_float(smax[q][1]));
+        }
+        const float rc = r0.x * ctr[0] + r0.y * ctr[1] + r0.z * ctr[2] + r0.w;
+        const float er = fmaxf(fabsf(rhi - rc), fabsf(rlo - rc));
+        // each hypothesis: out of the race, or all near points, none of them, or open
+        const uint32_t least = lower[c];
+        for (int h0 = 0; h0 < H; h0 += kT) {
+            const int h = h0 + threadIdx.x;
+            bool is_alive = false, is_open = false;
+            if (h < H) {
+                const float4 pl = hy[h];
+                is_alive = fabsf(pl.w) < inf && __ldcg(counts + (size_t)c * H + h) >= least;
+                if (is_alive && nn) {
+                    const float dot = pl.x * r0.x + pl.y * r0.y + pl.z * r0.z, sg = dot < 0.0f ? -1.0f : 1.0f;
+                    const float gx = sg * pl.x - r0.x, gy = sg * pl.y - r0.y, gz = sg * pl.z - r0.z;
+                    const float mid = gx * ctr[0] + gy * ctr[1] + gz * ctr[2] + (sg * pl.w - r0.w);
+                    float spread = fabsf(gx) * half[0] + fabsf(gy) * half[1] + fabsf(gz) * half[2];
+                    if (framed)
+                        spread = fminf(spread, fabsf(gx * ax + gy * ay + gz * az) * ea +
+                                                   fabsf(gx * bx + gy * by + gz * bz) * eb +
+                                                   fabsf(gx * r0.x + gy * r0.y + gz * r0.z) * er);
+                    spread += kSlabErr * (fabsf(pl.w) + fabsf(r0.w) + sumM);
+                    const float s_lo = rlo + mid - spread, s_hi = rhi + mid + spread;
+                    if (s_lo >= -eps && s_hi <= eps) hc[h] = (uint32_t)nn;
+                    else is_open = !(s_lo > eps || s_hi < -eps);
+                }
+            }
+            const uint32_t bo = __ballot_sync(0xffffffffu, is_open), ba = __ballot_sync(0xffffffffu, is_alive);
+            uint32_t ao = 0, aa = 0;
+            if (lane == 0) {
+                if (bo) ao = atomicAdd(&s_open, (uint32_t)__popc(bo));
+                if (ba) aa = atomicAdd(&s_alive, (uint32_t)__popc(ba));
+            }
+            ao = __shfl_sync(0xffffffffu, ao, 0) + __popc(bo & lt);
+            aa = __shfl_sync(0xffffffffu, aa, 0) + __popc(ba & lt);
+            if (is_open) open[ao] = (uint16_t)h;
+            if (is_alive) alive[aa] = (uint16_t)h;
+        }
+        __syncthreads();
+        // the points off the plane against every live hypothesis, the near ones against the open ones
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+            const int nh = (int)(pass ? s_open : s_alive), np = pass ? nn : nf;
+            if (!nh || !np) continue;
+            const int G = (nh + R - 1) / R, P = kT / G;  // threads per point subset, point subsets
+            const int g = threadIdx.x / G, j = threadIdx.x % G;
+            if (g >= P) continue;
+            const float4* src = pass ? sp : sp + (T - nf);
+            float4 pl[R];
+            uint32_t acc[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int h = j * R + r;
+                pl[r] = h < nh ? hy[pass ? open[h] : alive[h]] : make_float4(0.0f, 0.0f, 0.0f, inf);
+                acc[r] = 0;
+            }
+            int q = g;
+            for (; q + P < np; q += 2 * P) count_points2<R>(pl, src[q], src[q + P], eps, acc);
+            if (q < np) count_point<R>(pl, src[q], eps, acc);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int h = j * R + r;
+                if (h < nh && acc[r]) atomicAdd(&hc[pass ? (int)open[h] : (int)alive[h]], acc[r]);
+            }
+        }
+        __syncthreads();
+        for (uint32_t a = threadIdx.x; a < s_alive; a += kT) {
+            const int h = alive[a];
+            if (hc[h] < (uint32_t)cnt) atomicSub(&counts[(size_t)c * H + h], (uint32_t)cnt - hc[h]);
+        }
+    }
+}
+
 // The scoring launch's arguments (stage b).
 struct ScoreArgs {
     const float* pts;
@@ -1590,6 +1939,20 @@ cudaError_t launch_score(const ScoreArgs& a, cudaStream_t s) {
     const size_t smem = (size_t)a.T * sizeof(float4) + (size_t)P * G * R * sizeof(uint32_t);
     launch_full(k_score<R>, dim3(a.grid), dim3(kT), smem, s, a.pts, a.off, a.item_off, a.item_cl, a.kp, a.H, a.tile,
                 a.hyp, a.counts, a.queue, a.eps);
+    return cudaGetLastError();
+}
+
+// Large fits: the reference planes and their inliers, then the slab scoring.
+template <int R>
+cudaError_t launch_score_slab(const ScoreArgs& a, float4* ref, uint32_t* lower, unsigned cgrid, unsigned igrid,
+                              cudaStream_t s) {
+    const size_t smem = (size_t)a.T * sizeof(float4) + (size_t)a.H * 8;
+    launch_k(k_score_ref, dim3(cgrid), dim3(kT), 0, s, a.pts, a.off, a.kp, a.H, a.hyp, ref, a.eps);
+    launch_full(k_score_lower, dim3(igrid), dim3(kT), 0, s, a.pts, a.off, a.item_off, a.item_cl, a.kp, a.tile, ref,
+                lower, a.eps);
+    launch_full(k_score_slab<R>, dim3(a.grid), dim3(kT), smem, s, a.pts, a.off, a.item_off, a.item_cl, a.kp, a.H,
+                a.tile, a.hyp, ref, lower, a.counts, a.queue, a.eps);
+    count_launch(2);
     return cudaGetLastError();
 }
 
@@ -1664,9 +2027,13 @@ void fit_init_attributes() {
         cudaFuncSetAttribute(k_score<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         cudaFuncSetAttribute(k_score<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         cudaFuncSetAttribute(k_score_warp<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(k_score_slab<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024);
         cudaFuncSetAttribute(k_score_warp<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(k_score_slab<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024);
         cudaFuncSetAttribute(k_score_warp<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(k_score_slab<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024);
         cudaFuncSetAttribute(k_score_warp<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(k_score_slab<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024);
     });
 }
 
@@ -1692,13 +2059,6 @@ cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* la
         if (e != cudaSuccess) return e;
         count_launch(1);
     }
-    const size_t kh = (size_t)kcap * H;
-    const unsigned hgrid = (unsigned)((kh + kT - 1) / kT < (size_t)sms * 16 ? (kh + kT - 1) / kT : (size_t)sms * 16);
-    launch_k(k_hyp, dim3(hgrid), dim3(kT), 0, s, pts, off, labels, kp, H, p.seed, round, fb.hyp, fb.hyp_valid,
-             fb.counts, fb.item_off, fb.item_cl);
-    VM_STAGE_END(hk, kStHyp, s);
-    count_launch(1);
-    const int grid = sms * t.ctas_per_sm;
     // The warp schedule needs ceil(H / R) <= 32 lanes with R <= 8 and its
     // per-warp tiles within the shared-memory limit; otherwise the CTA one
     // runs, with at most one subset row of kT threads.
@@ -1710,16 +2070,34 @@ cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* la
     // counters: that removes two dependent launches.  In large batches the
     // counters' fences wait, per work item, for the item's contended atomics,
     // which costs more than the launches; they take the separate kernels.
-    // Results are the same.
-    uint32_t* done = fb.npts_cap <= kFusedFitPoints ? fb.done : nullptr;
+    // Large fits also score by k_score_slab, which makes two passes more and
+    // far fewer tests (small ones are bound by their launches).  Results are
+    // the same.
+    uint32_t* done = fb.npts_expect <= kFusedFitPoints ? fb.done : nullptr;
+    const bool slab = !done && !warp && p.eps < 1e6f;
+    const size_t kh = (size_t)kcap * H;
+    const unsigned hgrid = (unsigned)((kh + kT - 1) / kT < (size_t)sms * 16 ? (kh + kT - 1) / kT : (size_t)sms * 16);
+    launch_k(k_hyp, dim3(hgrid), dim3(kT), 0, s, pts, off, labels, kp, H, p.seed, round, fb.hyp, fb.hyp_valid,
+             fb.counts, fb.item_off, fb.item_cl, fb.lower, slab);
+    VM_STAGE_END(hk, kStHyp, s);
+    count_launch(1);
+    const int grid = sms * t.ctas_per_sm;
     VM_STAGE_BEGIN(hk, kStScore, s);
     const ScoreArgs sa{pts, off, fb.item_off, fb.item_cl, kp, H, T, tile, fb.hyp, fb.counts, fb.queue, p.eps, grid};
+    const unsigned cgrid = kcap < (uint32_t)sms * 8 ? kcap : (uint32_t)sms * 8, igrid = (unsigned)sms * 8;
     if (warp) {
         switch (R) {
             case 1: e = launch_score_warp<1>(sa, s); break;
             case 2: e = launch_score_warp<2>(sa, s); break;
             case 4: e = launch_score_warp<4>(sa, s); break;
             default: e = launch_score_warp<8>(sa, s); break;
+        }
+    } else if (slab) {
+        switch (R) {
+            case 1: e = launch_score_slab<1>(sa, fb.ref, fb.lower, cgrid, igrid, s); break;
+            case 2: e = launch_score_slab<2>(sa, fb.ref, fb.lower, cgrid, igrid, s); break;
+            case 8: e = launch_score_slab<8>(sa, fb.ref, fb.lower, cgrid, igrid, s); break;
+            default: e = launch_score_slab<4>(sa, fb.ref, fb.lower, cgrid, igrid, s); break;
         }
     } else {
         switch (R) {
@@ -1735,11 +2113,9 @@ cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* la
     // stage c (k_select, a CTA per cluster), then the extraction; with the
     // completion counters the centroid runs in the extraction kernel and the
     // refit in the filter kernel, otherwise as kernels of their own
-    const unsigned cgrid = kcap < (uint32_t)sms * 8 ? kcap : (uint32_t)sms * 8;
     VM_STAGE_BEGIN(hk, kStExtract, s);
     launch_k(k_select, dim3(cgrid), dim3(kT), 0, s, pts, off, kp, H, fb.hyp, fb.hyp_valid, fb.counts, fb.cl);
     count_launch(1);
-    const unsigned igrid = (unsigned)sms * 8;
     launch_full(done ? k_extract<true> : k_extract<false>, dim3(igrid), dim3(kT), 0, s, pts, off, fb.item_off,
                 fb.item_cl, kp, tile, fb.cl, fb.inlier, fb.part, p.eps, fb.err, done, fb.cen, fb.poly);
     if (!done) {
@@ -1898,7 +2274,7 @@ extern "C" vm_status vm_ransac_static(const float* xyz, const uint32_t* off, con
     const size_t kh = (size_t)k * H;
     const unsigned hgrid = (unsigned)((kh + kT - 1) / kT < (size_t)sms * 16 ? (kh + kT - 1) / kT : (size_t)sms * 16);
     launch_k(k_hyp, dim3(hgrid), dim3(kT), 0, s, xyz, off, labels, kdev, H, params->seed, 0u, hyp, valid, counts,
-             item_off, static_cast<uint32_t*>(nullptr));
+             item_off, static_cast<uint32_t*>(nullptr), static_cast<uint32_t*>(nullptr), false);
     // The CTA-per-item schedule whatever the tuning asks for: with no
     // item -> cluster table here, the clusters of work items come from a
     // binary search, which only that schedule does.

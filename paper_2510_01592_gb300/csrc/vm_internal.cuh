@@ -413,6 +413,8 @@ struct FitBuffers {
     uint32_t* queue;        // [4] work-queue head, the tile, -, the hull pass's count
     uint8_t* inlier;        // [npts]
     float* part;            // [items][10] per-item partial sums
+    float4* ref;            // [kcap] reference planes of a large fit's scoring
+    uint32_t* lower;        // [kcap] their inliers
     FitPoly* poly;          // [kcap] filter polygons
     float* cen;             // [kcap][3][2] inlier centroids, double-float (hi, lo)
     int2* surv;             // [npts] hull candidates (per-cluster segments at cluster offsets)
@@ -424,6 +426,7 @@ struct FitBuffers {
     uint32_t* kdev;         // cluster count when the caller supplies it
     uint32_t* done;         // [kcap][3] per-cluster completion counters (scoring, extraction, filter)
     size_t kcap, npts_cap, items_cap;  // items_cap: 256-point partial-sum chunks
+    size_t npts_expect;     // points a fit is likely to have (picks kernels; results do not depend on it)
     int H;
 };
 
