@@ -396,7 +396,10 @@ __device__ __forceinline__ uint32_t back_cell(uint32_t at, uint32_t win, int k) 
 // edge lies between two trees: usually there is none from the start.  (Joining
 // each edge with a CAS loop contended for the few roots: single bricks took 30
 // us.  Testing on demand only the neighbours in other trees made fewer tests
-// but one long chain of them: 27 us for the walk map's 2,535 bricks.)  The
+// but one long chain of them.)  A brick whose vertices are one tree after the
+// first flattening needs neither edges between trees nor a numbering: 26 us for
+// the walk map's 2,535 bricks (27.6 without that exit), 110 for the 8 x 8 x 3 m
+// map's 16 thousand (119).  The instructions of the 13 tests bound it.  The
 // brick's components are numbered in the order of their smallest vertex, and
 // each one's size and smallest voxel id are kept at the brick's first entry
 // plus its number.
@@ -442,6 +445,7 @@ __global__ void __launch_bounds__(kLocalT, 14) k_ccl_local(SegCounters* __restri
             }
         }
         __syncthreads();
+        uint32_t nroot = 0, nhere = 0;
         for (uint32_t p = threadIdx.x; p < n; p += kLocalT) {
             const float4 a = A[p], an = B[p];
             const int l = sl[p], lx = l & 7, ly = (l >> 3) & 7, lz = l >> 6;
@@ -462,11 +466,33 @@ __global__ void __launch_bounds__(kLocalT, 14) k_ccl_local(SegCounters* __restri
                     }
                 }
             }
-            nvert += vert;
+            nroot += vert && par == p;
+            nhere += vert;
             lpar[p] = vert ? par : kNone;
             sedge[p] = vert ? (uint16_t)edges : 0;
         }
+        nvert += nhere;
+        nroot = __reduce_add_sync(0xffffffffu, nroot);
+        nhere = __reduce_add_sync(0xffffffffu, nhere);
+        if (lane == 0) wcnt[wid] = nroot << 16 | nhere;
         __syncthreads();
+        nroot = nhere = 0;
+#pragma unroll
+        for (int q = 0; q < kLocalT / 32; ++q) {
+            nroot += wcnt[q] >> 16;
+            nhere += wcnt[q] & 0xffffu;
+        }
+        if (nroot <= 1) {  // one tree (three bricks of four on the walk map): no labels to find
+            for (uint32_t p = threadIdx.x; p < n; p += kLocalT) {
+                lc[base + p] = lpar[p] == kNone ? kNoComp : (uint16_t)0;
+                if (lpar[p] == p) {
+                    lroot[base] = hd.z * kBrickVox + sl[p];
+                    lsize[base] = nhere;
+                }
+            }
+            if (threadIdx.x == 0) ncomp[r] = nroot;
+            continue;
+        }
         for (int round = 0; round < kBrickVox; ++round) {  // every round with an edge apart joins two trees or more
             for (int jump = 0; jump < 32; ++jump) {        // a tree over 512 voxels is flat after at most 9
                 bool more = false;
@@ -693,22 +719,37 @@ __global__ void __launch_bounds__(kT, 4)
 }
 
 // Joins the listed pairs.  While the components fit one SM's shared memory
-// (kSmemComps) the forest that the hooks of k_ccl_cross left is copied there (a
-// step of a walk takes 30 cycles; the chains, a hundred bricks long across a
-// floor, took 68 us to walk in global memory) and joined in rounds without any
-// loop over contended roots: each pair hooks the larger of its roots under the
-// smaller one (an atomic minimum; a hook that another one replaces is found
-// again), until no pair is apart.  Up to kJoinPairs pairs one CTA does this,
-// its pairs in registers.  With more, every CTA first walks its share of the
-// pairs in a copy of its own and lists those that are apart (a third of the
-// LiDAR map's 95 thousand), a thread per component stores its root, and the
-// last CTA to finish joins the list.  With more components, or pairs the list
-// had no room for, the grid joins pair by pair in global memory (which took 51
-// us for the walk map's 16 thousand pairs: the threads meet on the few large
-// roots).
-constexpr uint32_t kSmemComps = 56000;  // below 2^16: a pair packs into a word
-constexpr int kJoinIt = 16;
-constexpr uint32_t kJoinPairs = kOneT * kJoinIt;
+// (kSmemComps) the forest that the hooks of k_ccl_cross left is copied there and
+// joined in rounds: pointer jumping flattens the trees; each pair then reads its
+// two roots, and a pair that is apart hooks the larger under the smaller one (an
+// atomic minimum; a hook that another one replaces is found again), until no
+// pair is apart.  Only the roots that the first flattening leaves take part in
+// the later ones.  Pairs that fit beside the forest are joined by one CTA.  With
+// more, every CTA first walks its share of the pairs in a copy of its own, lists
+// those that are apart (a third of the LiDAR map's 95 thousand) and stores the
+// roots of its share of the components; the last CTA to finish joins the list.
+// With more components, or pairs the list had no room for, the grid joins pair
+// by pair in global memory (51 us for the walk map's 17 thousand pairs: the
+// threads meet on the few large roots).  One SM's instruction rate bounds the
+// rounds: what is touched in a round, not the steps of a chain, counts.  13.6 us
+// for the walk map (2.7 thousand components), 85 us for the 8 x 8 x 3 m one (29
+// thousand); reading each pair's chains in every round took 18 and 93 us.
+constexpr uint32_t kJoinWords = 57344;  // 224 KB: the forest, the roots, the pairs
+constexpr uint32_t kSmemComps = 36864;  // below 2^16: a pair packs into a word
+// Flattens the trees over the elements list[0 .. n) (null: 0 .. n).
+__device__ __forceinline__ void join_flatten(uint32_t* P, const uint16_t* list, uint32_t n) {
+    for (int round = 0; round < 64; ++round) {  // every round at least doubles the reach
+        bool more = false;
+        for (uint32_t i = threadIdx.x; i < n; i += kOneT) {
+            const uint32_t c = list ? list[i] : i, p = P[c], a = P[p];
+            if (a != p) {
+                P[c] = P[a];
+                more = true;
+            }
+        }
+        if (!__syncthreads_or(more)) break;
+    }
+}
 // The root of x in P, halving the path: a parent only moves to a smaller ancestor.
 __device__ __forceinline__ uint32_t join_root(uint32_t* P, uint32_t x, uint32_t K, uint32_t* err) {
     volatile uint32_t* V = P;
@@ -722,37 +763,13 @@ __device__ __forceinline__ uint32_t join_root(uint32_t* P, uint32_t x, uint32_t 
     atomicOr(err, kErrTimeout);
     return x;
 }
-// A round of the whole CTA over up to kJoinPairs pairs in registers (0: none or
-// together): first every pair's roots, then the hooks.  Apart, because a path
-// halved across a hook that another one then replaces would cut the tree: a
-// hook may only be replaced while nothing but its own pair has followed it.
-__device__ __forceinline__ bool join_round(uint32_t* P, uint32_t (&pr)[kJoinIt], uint32_t K, uint32_t* err) {
-#pragma unroll
-    for (int i = 0; i < kJoinIt; ++i) {
-        if (!pr[i]) continue;
-        const uint32_t a = join_root(P, pr[i] >> 16, K, err), b = join_root(P, pr[i] & 0xffffu, K, err);
-        pr[i] = a == b ? 0u : min(a, b) << 16 | max(a, b);  // the roots stand for the pair from here on
-    }
-    __syncthreads();
-    bool apart = false;
-#pragma unroll
-    for (int i = 0; i < kJoinIt; ++i)
-        if (pr[i]) {
-            atomicMin(&P[pr[i] & 0xffffu], pr[i] >> 16);
-            apart = true;
-        }
-    return __syncthreads_or(apart);
-}
-__device__ __forceinline__ uint32_t pack_pair(unsigned long long key) {
-    return (uint32_t)(key >> 32) << 16 | (uint32_t)key;
-}
 __global__ void __launch_bounds__(kOneT, 1) k_comp_join(SegCounters* __restrict__ ctr, uint32_t pair_cap,
-                                                     const unsigned long long* __restrict__ pairs, uint32_t* list,
-                                                     uint32_t* parent, const uint32_t* __restrict__ over,
-                                                     uint32_t* err) {
+                                                        const unsigned long long* __restrict__ pairs, uint32_t* list,
+                                                        uint32_t* parent, const uint32_t* __restrict__ over,
+                                                        uint32_t* err) {
     pdl_gate();
     extern __shared__ uint32_t P[];
-    __shared__ uint32_t s_last;
+    __shared__ uint32_t s_last, s_roots;
     const uint32_t K = ctr->n_comp, all = ctr->n_pairs, np = min(all, pair_cap);
     if (K > kSmemComps || all > pair_cap) {
         for (uint32_t q = blockIdx.x * kOneT + threadIdx.x; q < np; q += gridDim.x * kOneT) {
@@ -764,80 +781,95 @@ __global__ void __launch_bounds__(kOneT, 1) k_comp_join(SegCounters* __restrict_
                 if (over[c] != c) uf_union(parent, over[c], c, err);
         return;
     }
-    const bool one = np <= kJoinPairs;
+    uint16_t* roots = reinterpret_cast<uint16_t*>(P + K);  // the roots left by the first flattening
+    uint32_t* L = P + K + (K + 1) / 2;                     // pairs in shared memory (0: none, or together)
+    const uint32_t room = kJoinWords - K - (K + 1) / 2;
+    const bool one = np <= room;
     const uint32_t G = one ? 1u : min(gridDim.x, (np + kOneT - 1) / kOneT), g = blockIdx.x;
     if (g >= G) return;
     const int lane = threadIdx.x & 31;
-    uint32_t pr[kJoinIt];
+    const auto pack = [](unsigned long long key) { return (uint32_t)(key >> 32) << 16 | (uint32_t)key; };
+    if (threadIdx.x == 0) s_roots = 0;
+#pragma unroll 8
+    for (uint32_t c = threadIdx.x; c < K; c += kOneT) P[c] = __ldcg(parent + c);
     if (one)
-#pragma unroll
-        for (int i = 0; i < kJoinIt; ++i) {
-            const uint32_t q = threadIdx.x + i * kOneT;
-            pr[i] = q < np ? pack_pair(pairs[q]) : 0u;
-        }
-    constexpr int kIt = 8;
-    for (uint32_t c0 = threadIdx.x; c0 < K; c0 += kOneT * kIt) {
-        uint32_t v[kIt];
-#pragma unroll
-        for (int i = 0; i < kIt; ++i) v[i] = c0 + i * kOneT < K ? __ldcg(parent + c0 + i * kOneT) : 0u;
-#pragma unroll
-        for (int i = 0; i < kIt; ++i)
-            if (c0 + i * kOneT < K) P[c0 + i * kOneT] = v[i];
-    }
+#pragma unroll 8
+        for (uint32_t q = threadIdx.x; q < np; q += kOneT) L[q] = pack(__ldcg(pairs + q));
     __syncthreads();
+    uint32_t n = np;
     if (one) {
-        for (uint32_t round = 0; round <= K; ++round)  // a round with a pair apart joins two trees or more
-            if (!join_round(P, pr, K, err)) break;
-        for (uint32_t c = threadIdx.x; c < K; c += kOneT) parent[c] = join_root(P, c, K, err);
-        return;
-    }
-    for (uint32_t q0 = g * kOneT; q0 < np; q0 += G * kOneT) {
-        const uint32_t q = q0 + threadIdx.x;
-        uint32_t a = 0, b = 0;
-        if (q < np) {
-            const unsigned long long key = pairs[q];
-            a = join_root(P, (uint32_t)(key >> 32), K, err);
-            b = join_root(P, (uint32_t)key, K, err);
-        }
-        const uint32_t m = __ballot_sync(0xffffffffu, a != b);
-        uint32_t at = 0;
-        if (lane == 0 && m) at = atomicAdd(&ctr->n_apart, (uint32_t)__popc(m));
-        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
-        if (a != b) list[at] = min(a, b) << 16 | max(a, b);
-    }
-    // another CTA still copying the forest reads a parent or its root: either is an ancestor
-    for (uint32_t c = g * kOneT + threadIdx.x; c < K; c += G * kOneT) parent[c] = join_root(P, c, K, err);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&ctr->join_done, 1u) + 1u == G;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    const uint32_t n = *(volatile uint32_t*)&ctr->n_apart;
-    for (uint32_t round = 0; round <= K; ++round) {
-        bool more = false;
-        for (uint32_t q0 = 0; q0 < n; q0 += kJoinPairs) {
-            if (round == 0 || n > kJoinPairs)
-#pragma unroll
-                for (int i = 0; i < kJoinIt; ++i) {
-                    const uint32_t q = q0 + i * kOneT + threadIdx.x;
-                    pr[i] = q < n ? __ldcg(list + q) : 0u;
-                }
-            more |= join_round(P, pr, K, err);
-        }
-        if (!more) break;
-    }
-    for (uint32_t q0 = threadIdx.x; q0 < n; q0 += kJoinPairs) {
-#pragma unroll
-        for (int i = 0; i < kJoinIt; ++i) pr[i] = q0 + i * kOneT < n ? __ldcg(list + q0 + i * kOneT) : 0u;
-#pragma unroll
-        for (int i = 0; i < kJoinIt; ++i)
-            if (pr[i]) {
-                const uint32_t a = pr[i] >> 16, b = pr[i] & 0xffffu, r = join_root(P, a, K, err);
-                parent[a] = r;
-                parent[b] = r;
+        join_flatten(P, nullptr, K);
+    } else {
+        for (uint32_t q0 = g * kOneT; q0 < np; q0 += G * kOneT) {
+            const uint32_t q = q0 + threadIdx.x;
+            uint32_t a = 0, b = 0;
+            if (q < np) {
+                const uint32_t pr = pack(pairs[q]);
+                a = join_root(P, pr >> 16, K, err);
+                b = join_root(P, pr & 0xffffu, K, err);
             }
+            const uint32_t m = __ballot_sync(0xffffffffu, a != b);
+            uint32_t at = 0;
+            if (lane == 0 && m) at = atomicAdd(&ctr->n_apart, (uint32_t)__popc(m));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+            if (a != b) list[at] = min(a, b) << 16 | max(a, b);
+        }
+        // another CTA still copying the forest reads a parent or its root: either is an ancestor
+        for (uint32_t c = g * kOneT + threadIdx.x; c < K; c += G * kOneT) parent[c] = join_root(P, c, K, err);
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) s_last = atomicAdd(&ctr->join_done, 1u) + 1u == G;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        n = *(volatile uint32_t*)&ctr->n_apart;
+        if (n <= room)
+#pragma unroll 8
+            for (uint32_t q = threadIdx.x; q < n; q += kOneT) L[q] = __ldcg(list + q);
     }
+    for (uint32_t c0 = 0; c0 < K; c0 += kOneT) {
+        const uint32_t c = c0 + threadIdx.x;
+        const uint32_t m = __ballot_sync(0xffffffffu, c < K && P[c] == c);
+        uint32_t at = 0;
+        if (lane == 0 && m) at = atomicAdd(&s_roots, (uint32_t)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+        if (c < K && P[c] == c) roots[at] = (uint16_t)c;
+    }
+    __syncthreads();
+    const uint32_t nr = s_roots;
+    const bool here = n <= room;
+    for (uint32_t round = 0;; ++round) {
+        // the roots of every pair, then the hooks: apart, because a pair must not be taken for joined by a hook
+        // that another one then replaces
+        bool apart = false;
+#pragma unroll 4
+        for (uint32_t q = threadIdx.x; q < n; q += kOneT) {
+            const uint32_t pr = here ? L[q] : __ldcg(list + q);
+            if (!pr) continue;
+            const uint32_t a = P[pr >> 16], b = P[pr & 0xffffu], now = a == b ? 0u : min(a, b) << 16 | max(a, b);
+            if (here) L[q] = now;
+            else list[q] = now;
+            apart |= now != 0u;
+        }
+        if (!__syncthreads_or(apart)) break;
+        if (round > K) {  // every round with a pair apart joins two trees or more
+            if (threadIdx.x == 0) atomicOr(err, kErrTimeout);
+            break;
+        }
+#pragma unroll 4
+        for (uint32_t q = threadIdx.x; q < n; q += kOneT) {
+            const uint32_t pr = here ? L[q] : __ldcg(list + q);
+            // most pairs of a large tree name its root: a look first spares the meeting atomics
+            if (pr && *(volatile uint32_t*)&P[pr & 0xffffu] > pr >> 16) atomicMin(&P[pr & 0xffffu], pr >> 16);
+        }
+        __syncthreads();
+        join_flatten(P, roots, nr);
+    }
+    // a component's root of the first flattening, then that one's
+    if (one)
+        for (uint32_t c = threadIdx.x; c < K; c += kOneT) parent[c] = P[P[c]];
+    else
+        for (uint32_t i = threadIdx.x; i < nr; i += kOneT) parent[roots[i]] = P[roots[i]];
 }
 
 // Read-only walk to the root.  Used once linking is over: every thread writes
@@ -1146,7 +1178,7 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
                     SegBuffers& b, uint32_t kcap, uint32_t* err, int sms, cudaStream_t s, StageHook* hk) {
     static std::once_flag once;
     std::call_once(once, [] {
-        cudaFuncSetAttribute(k_comp_join, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemComps * 4));
+        cudaFuncSetAttribute(k_comp_join, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kJoinWords * 4));
         cudaFuncSetAttribute(k_cluster_place, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kPlaceWords * 4));
     });
     const uint32_t cap_b = (uint32_t)(b.nv / kBrickVox);
@@ -1177,7 +1209,7 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
     launch_k(k_ccl_cross, dim3(vgrid), dim3(kT), 0, s, b.ctr, b.brec, b.near, b.rows, b.vox, b.pos, b.nrm, b.lc,
              b.ncomp, b.cbase, b.lsize, b.lroot, b.csize, b.croot, b.total, b.parent, over, b.pairs, pair_cap,
              p.d_th2, p.cos_ccl, err);
-    launch_k(k_comp_join, dim3(sms), dim3(kOneT), kSmemComps * 4, s, b.ctr, pair_cap, b.pairs, b.lsize,
+    launch_k(k_comp_join, dim3(sms), dim3(kOneT), kJoinWords * 4, s, b.ctr, pair_cap, b.pairs, b.lsize,
              b.parent, over, err);
     VM_STAGE_END(hk, kStCcl, s);
     VM_STAGE_BEGIN(hk, kStClusters, s);
