@@ -814,7 +814,14 @@ vm_status vm_create(const vm_map_params* params, void* cuda_stream, vm_map** out
         vm_destroy(m);
         return cuda_status(e, "cudaMallocHost");
     }
-    st = vm_reset(m);
+    // the pool starts out zero; a reset then clears only the slots that were claimed
+    e = cudaMemsetAsync(m->S, 0, (size_t)m->capacity * 3 * kBrickVox * sizeof(unsigned long long), m->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->C, 0, (size_t)m->capacity * kBrickVox * sizeof(uint32_t), m->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->ctr, 0, sizeof(MapCounters), m->stream);
+    const size_t bits = (size_t)m->capacity * (kBrickVox / 32) * sizeof(uint32_t);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->occ, 0, bits, m->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->mark, 0, bits, m->stream);
+    st = e == cudaSuccess ? vm_reset(m) : cuda_status(e, "map initialisation");
     if (st == VM_OK) {
         const float po[4] = {g.ox, g.oy, g.oz, 0.0f};
         e = cudaMemsetAsync(m->scroll_tmp, 0, scroll_tmp_words(m->capacity) * sizeof(uint32_t), m->stream);
@@ -832,12 +839,7 @@ vm_status vm_create(const vm_map_params* params, void* cuda_stream, vm_map** out
 
 vm_status vm_reset(vm_map* m) {
     VM_TRY(check_map(m));
-    VM_CUDA(cudaMemsetAsync(m->brick_table, 0xFF, (size_t)m->nb_total * sizeof(int32_t), m->stream));
-    VM_CUDA(cudaMemsetAsync(m->S, 0, (size_t)m->capacity * 3 * kBrickVox * sizeof(unsigned long long), m->stream));
-    VM_CUDA(cudaMemsetAsync(m->C, 0, (size_t)m->capacity * kBrickVox * sizeof(uint32_t), m->stream));
-    VM_CUDA(cudaMemsetAsync(m->ctr, 0, sizeof(MapCounters), m->stream));
-    VM_CUDA(cudaMemsetAsync(m->occ, 0, (size_t)m->capacity * (kBrickVox / 32) * sizeof(uint32_t), m->stream));
-    VM_CUDA(cudaMemsetAsync(m->mark, 0, (size_t)m->capacity * (kBrickVox / 32) * sizeof(uint32_t), m->stream));
+    VM_CUDA(launch_reset(m->brick_table, m->nb_total, m->S, m->C, m->occ, m->mark, m->ctr, m->capacity, m->stream));
     m->segmented = false;
     return VM_OK;
 }

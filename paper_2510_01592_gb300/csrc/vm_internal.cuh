@@ -107,6 +107,7 @@ struct MapCounters {
     unsigned long long evicted;  // occupied voxels evicted by scrolling the window
     uint32_t n_deferred;         // points of the frame waiting for their brick's claim (k_accum_deferred)
     uint32_t deferred_done;      // CTAs of k_accum_deferred finished
+    uint32_t reset_done;         // CTAs of k_reset finished
 };
 
 // Counters produced by one segmentation, read back by the host.
@@ -339,6 +340,8 @@ cudaError_t launch_integrate(const float* xyz, uint32_t n, const Pose& pose, con
 // that a point's ray from the sensor passes through before the point's own
 // voxel (mark: one bit per voxel slot, capacity * 16 words, zero between
 // calls), then clears the marked voxels and the marks.
+cudaError_t launch_reset(int32_t* brick_table, uint32_t nb_total, unsigned long long* S, uint32_t* C, uint32_t* occ,
+                         uint32_t* mark, MapCounters* ctr, uint32_t capacity, cudaStream_t s);
 cudaError_t launch_clear(const float* xyz, uint32_t n, const Pose& pose, const Grid& g,
                          const int32_t* brick_table, unsigned long long* S, uint32_t* C, uint32_t* occ,
                          uint32_t* mark, MapCounters* ctr, uint32_t capacity, cudaStream_t s);
