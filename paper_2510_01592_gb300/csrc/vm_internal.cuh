@@ -311,7 +311,7 @@ static_assert(sizeof(BrickRec) == 128, "one line a brick");
 // the words clear[2 .. n_clear) and zero0 / zero1 (may be null) are cleared.
 // tmp: order_tmp_words(nb) words of look-back state, zeroed once.
 // Two status words a tile.
-constexpr size_t kOrderTileElems = 1024;
+constexpr size_t kOrderTileElems = 256;
 constexpr size_t order_tmp_words(size_t nb) { return 4 + 4 * ((nb + kOrderTileElems - 1) / kOrderTileElems) + 2; }
 cudaError_t order_bricks_dev(const int32_t* table, uint32_t nb, const uint32_t* occ, int32_t* rank_table,
                              int32_t* sorted_slot, int32_t* sorted_key, BrickRec* brec, uint32_t* clear, int n_clear,
