@@ -24,8 +24,8 @@ def test_order_and_sums(orc, bricks):
     from paper_2510_01592_gb300 import vm
     rng = np.random.default_rng(sum(bricks))
     dims = tuple(8 * b for b in bricks)
-    ext = np.array(dims) * 0.05
-    gm, om = vm.VoxelMap(dims, (0.0, 0.0, 0.0), 0.05), orc.OracleMap(dims, (0.0, 0.0, 0.0), 0.05)
+    ext = np.array(dims) * 0.005
+    gm, om = vm.VoxelMap(dims, (0.0, 0.0, 0.0), 0.005), orc.OracleMap(dims, (0.0, 0.0, 0.0), 0.005)
     sizes = list(range(1, 34)) * 3 + [64, 100, 1, 1, 1, 2, 2, 31, 32, 33] + [1] * 64
     for n_groups in (1, len(sizes)):
         p = _grouped(rng, ext, sizes[-n_groups:])
