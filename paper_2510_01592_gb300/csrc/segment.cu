@@ -386,7 +386,7 @@ __device__ __forceinline__ uint32_t back_cell(uint32_t at, uint32_t win, int k) 
     return k == 0 ? at - 1u : (k == 1 ? at : at + ((win >> 1) & 1u));
 }
 
-// The intra-brick half of Algorithm 1, one 64-thread CTA per brick.  Every
+// The intra-brick half of Algorithm 1, one 128-thread CTA per brick.  Every
 // vertex tests its 13 backward neighbours (independent tests, so their loads
 // and arithmetic overlap) and hooks under the smallest one it has an edge with,
 // without atomics; pointer jumping flattens the trees (a brick is 8 voxels
@@ -397,15 +397,17 @@ __device__ __forceinline__ uint32_t back_cell(uint32_t at, uint32_t win, int k) 
 // each edge with a CAS loop contended for the few roots: single bricks took 30
 // us.  Testing on demand only the neighbours in other trees made fewer tests
 // but one long chain of them.)  A brick whose vertices are one tree after the
-// first flattening needs neither edges between trees nor a numbering: 26 us for
-// the walk map's 2,535 bricks (27.6 without that exit), 110 for the 8 x 8 x 3 m
-// map's 16 thousand (119).  The instructions of the 13 tests bound it.  The
+// first flattening needs neither edges between trees nor a numbering.  Latency
+// bounds it (an instruction in a third of the issue slots), so 128 threads, one a
+// voxel in most bricks, take a brick, and the grid is left to the hardware's
+// scheduler: 20 us for the walk map's 2,535 bricks, 85 for the 8 x 8 x 3 m map's
+// 16 thousand; 64 threads and a grid of about one wave took 26 and 110.  The
 // brick's components are numbered in the order of their smallest vertex, and
 // each one's size and smallest voxel id are kept at the brick's first entry
 // plus its number.
-constexpr int kLocalT = 64;
+constexpr int kLocalT = 128;
 constexpr uint32_t kStage = 256;  // records staged in shared memory; a fuller brick's are read from the caches
-__global__ void __launch_bounds__(kLocalT, 14) k_ccl_local(SegCounters* __restrict__ ctr, uint32_t cap_b,
+__global__ void __launch_bounds__(kLocalT, 11) k_ccl_local(SegCounters* __restrict__ ctr, uint32_t cap_b,
                                                            const BrickRec* __restrict__ brec,
                                                            const uint32_t* __restrict__ vox,
                                                            const float4* __restrict__ pos,
@@ -429,12 +431,11 @@ __global__ void __launch_bounds__(kLocalT, 14) k_ccl_local(SegCounters* __restri
         const uint4 hd = *reinterpret_cast<const uint4*>(&br->base);  // base, n, key, slot
         const uint32_t base = hd.x, n = hd.y;
         __syncthreads();
-        {
+        if (threadIdx.x < 64) {
             const uint32_t m = br->mask[threadIdx.x >> 2], sh = (threadIdx.x & 3) * 8;
             rowt[threadIdx.x] = ((br->pre[threadIdx.x >> 2] + __popc(m & ((1u << sh) - 1u))) << 8) | ((m >> sh) & 0xffu);
         }
         const bool staged = n <= kStage;
-        const float4 *A = staged ? sA : pos + base, *B = staged ? sB : nrm + base;
 #pragma unroll 2
         for (uint32_t p = threadIdx.x; p < n; p += kLocalT) {
             sl[p] = (uint16_t)(vox[base + p] % kBrickVox);
@@ -446,31 +447,35 @@ __global__ void __launch_bounds__(kLocalT, 14) k_ccl_local(SegCounters* __restri
         }
         __syncthreads();
         uint32_t nroot = 0, nhere = 0;
-        for (uint32_t p = threadIdx.x; p < n; p += kLocalT) {
-            const float4 a = A[p], an = B[p];
-            const int l = sl[p], lx = l & 7, ly = (l >> 3) & 7, lz = l >> 6;
-            const bool vert = __float_as_int(a.w) >= want;
-            uint32_t par = p, edges = 0;
-#pragma unroll
-            for (int q = 0; q < 5; ++q) {
-                uint32_t at = 0;
-                const uint32_t win = back_row(rowt, q, lx, ly, lz, at);
-#pragma unroll
-                for (int k = 0; k < (q == 0 ? 1 : 3); ++k) {
-                    const bool on = (win >> k) & 1u;
-                    const uint32_t j = on ? back_cell(at, win, k) : p;
-                    const float4 c = A[j];
-                    if (on && __float_as_int(c.w) >= want && ccl_edge4(a, an, c, B[j], d_th2, cos_ccl)) {
-                        edges |= 1u << (3 * q + k);
-                        par = min(par, j);
+        const auto tests = [&](const float4* A, const float4* B) {  // apart for the two memories: plain shared loads
+            for (uint32_t p = threadIdx.x; p < n; p += kLocalT) {
+                const float4 a = A[p], an = B[p];
+                const int l = sl[p], lx = l & 7, ly = (l >> 3) & 7, lz = l >> 6;
+                const bool vert = __float_as_int(a.w) >= want;
+                uint32_t par = p, edges = 0;
+    #pragma unroll
+                for (int q = 0; q < 5; ++q) {
+                    uint32_t at = 0;
+                    const uint32_t win = back_row(rowt, q, lx, ly, lz, at);
+    #pragma unroll
+                    for (int k = 0; k < (q == 0 ? 1 : 3); ++k) {
+                        const bool on = (win >> k) & 1u;
+                        const uint32_t j = on ? back_cell(at, win, k) : p;
+                        const float4 c = A[j];
+                        if (on && __float_as_int(c.w) >= want && ccl_edge4(a, an, c, B[j], d_th2, cos_ccl)) {
+                            edges |= 1u << (3 * q + k);
+                            par = min(par, j);
+                        }
                     }
                 }
+                nroot += vert && par == p;
+                nhere += vert;
+                lpar[p] = vert ? par : kNone;
+                sedge[p] = vert ? (uint16_t)edges : 0;
             }
-            nroot += vert && par == p;
-            nhere += vert;
-            lpar[p] = vert ? par : kNone;
-            sedge[p] = vert ? (uint16_t)edges : 0;
-        }
+        };
+        if (staged) tests(sA, sB);
+        else tests(pos + base, nrm + base);
         nvert += nhere;
         nroot = __reduce_add_sync(0xffffffffu, nroot);
         nhere = __reduce_add_sync(0xffffffffu, nhere);
@@ -1187,7 +1192,9 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
     uint32_t* over = b.place;                                   // k_cluster_place writes it after the last join
     uint32_t* scratch = reinterpret_cast<uint32_t*>(b.pairs);   // free once the pairs are joined
     const auto clampg = [&](uint32_t want, uint32_t mx) { return want < mx ? (want ? want : 1u) : mx; };
-    const unsigned bgrid = clampg(cap_b, sms * 16), vgrid = clampg((uint32_t)((b.nv + kT - 1) / kT), sms * 8);
+    // Several waves of short CTAs: with about one, some SMs got a CTA more than others for the whole pass (the per-voxel
+    // passes of the 8 x 8 x 3 m map 248 us at 8 CTAs an SM, 219 at 24; at 64 a walk map's empty CTAs cost it 8 us).
+    const unsigned bgrid = clampg(cap_b, sms * 64), vgrid = clampg((uint32_t)((b.nv + kT - 1) / kT), sms * 24);
     VM_STAGE_BEGIN(hk, kStFinalize, s);
     launch_k(k_finalize, dim3(clampg((cap_b + kFinWarps - 1) / kFinWarps, sms * 8)), dim3(kT), 0, s, b.ctr, cap_b, g,
              b.brec, b.rank_table, S, C, b.M, b.vox, b.near, b.rows);
