@@ -37,7 +37,7 @@ namespace {
 
 constexpr int kT = 256;
 constexpr int kHullCap = 2048;   // hull candidates sorted in shared memory
-constexpr int kSurvCap = 12288;  // first-filter survivors staged in shared memory
+constexpr int kSurvCap = 10240;  // first-filter survivors staged in shared memory: two CTAs of k_hull fit an SM
 constexpr size_t kFusedFitPoints = size_t(4) << 20;  // fits expected to have at most this many points: per-cluster
                                                      // tails fused, every test of stage b made
 
@@ -618,15 +618,18 @@ __device__ __noinline__ void extract_tail(uint32_t c, const float* __restrict__ 
 // along the 16 filter directions (reduced per CTA, then one atomicMax each: the
 // items of a large cluster meet on its 16 words).
 // kTail: the CTA that completes a cluster's last item computes its centroid
-// (done: the per-cluster completion counters).
+// (done: the per-cluster completion counters).  Loads in flight bound it, so
+// registers are held to what lets a small fit's items, four an SM, all run at
+// once (a walk map 13.2 -> 11 us, 16 clusters 14.2 -> 10.9), and a large fit's
+// CTAs be five an SM (2,000 clusters 376 -> 349 us); the few spilled words cost
+// less.
 template <bool kTail>
-__global__ void __launch_bounds__(kT) k_extract(const float* __restrict__ pts, const uint32_t* __restrict__ off,
-                                                const uint32_t* __restrict__ item_off,
-                                                const uint32_t* __restrict__ item_cl, const uint32_t* __restrict__ kp,
-                                                const uint32_t* __restrict__ tile, FitCluster* __restrict__ cl,
-                                                uint8_t* __restrict__ inlier, float* __restrict__ part, float eps,
-                                                uint32_t* __restrict__ err, uint32_t* __restrict__ done,
-                                                float* __restrict__ cen, FitPoly* __restrict__ poly) {
+__global__ void __launch_bounds__(kT, kTail ? 4 : 5)
+k_extract(const float* __restrict__ pts, const uint32_t* __restrict__ off, const uint32_t* __restrict__ item_off,
+          const uint32_t* __restrict__ item_cl, const uint32_t* __restrict__ kp, const uint32_t* __restrict__ tile,
+          FitCluster* __restrict__ cl, uint8_t* __restrict__ inlier, float* __restrict__ part, float eps,
+          uint32_t* __restrict__ err, uint32_t* __restrict__ done, float* __restrict__ cen,
+          FitPoly* __restrict__ poly) {
     pdl_gate();
     const uint32_t k = *kp, T = *tile;
     __shared__ float wp[kMaxChunksPerItem * (kT / 32) * 4];
@@ -744,14 +747,15 @@ __device__ __noinline__ void filter_tail(uint32_t c, const uint32_t* __restrict_
 // points in between take the exact integer test.  The polygon is formed once a
 // cluster, with its centroid (poly_warp; one thread an item did it in 1.4 us).
 // The edges' coefficients are read from shared memory once per kBatch chunks.
+// Registers are held down as in k_extract, six CTAs an SM in a large fit (2,000
+// clusters 376 -> 292 us).
 template <bool kTail>
-__global__ void __launch_bounds__(kT) k_filter(const float* __restrict__ pts, const uint32_t* __restrict__ off,
-                                               const uint32_t* __restrict__ item_off,
-                                               const uint32_t* __restrict__ item_cl, const uint32_t* __restrict__ kp,
-                                               const uint32_t* __restrict__ tile, FitCluster* __restrict__ cl,
-                                               const uint8_t* __restrict__ inlier, const float* __restrict__ cen,
-                                               const FitPoly* __restrict__ poly_of, float* __restrict__ part,
-                                               int2* __restrict__ surv, uint32_t* __restrict__ done) {
+__global__ void __launch_bounds__(kT, kTail ? 4 : 6)
+k_filter(const float* __restrict__ pts, const uint32_t* __restrict__ off, const uint32_t* __restrict__ item_off,
+         const uint32_t* __restrict__ item_cl, const uint32_t* __restrict__ kp, const uint32_t* __restrict__ tile,
+         FitCluster* __restrict__ cl, const uint8_t* __restrict__ inlier, const float* __restrict__ cen,
+         const FitPoly* __restrict__ poly_of, float* __restrict__ part, int2* __restrict__ surv,
+         uint32_t* __restrict__ done) {
     pdl_gate();
     const uint32_t k = *kp, T = *tile;
     constexpr int kSurvBuf = 128;
@@ -1056,7 +1060,7 @@ __global__ void __launch_bounds__(kT) k_hull(const uint32_t* __restrict__ off, c
     unsigned long long* uq = sk + kHullCap;
     uint32_t* st_lo = reinterpret_cast<uint32_t*>(uq + kHullCap);
     uint32_t* st_hi = st_lo + kHullCap;
-    int2* ssv = reinterpret_cast<int2*>(st_hi + kHullCap);  // kSurvCap staged survivors
+    int2* ssv = reinterpret_cast<int2*>(uq);  // kSurvCap staged survivors, done with before the unique keys
     __shared__ uint32_t wsum[kT / 32];
     __shared__ int s_klo, s_khi, s_m, s_cnt;
     __shared__ int2 poly[kHullDirs + 1];   // the extreme point of each direction
@@ -1930,6 +1934,7 @@ struct ScoreArgs {
     uint32_t* queue;
     float eps;
     int grid;
+    bool early;  // launched while stage a runs (see launch_fit)
 };
 
 template <int R>
@@ -1937,7 +1942,7 @@ cudaError_t launch_score(const ScoreArgs& a, cudaStream_t s) {
     const int G = (a.H + R - 1) / R;
     const int P = kT / G;
     const size_t smem = (size_t)a.T * sizeof(float4) + (size_t)P * G * R * sizeof(uint32_t);
-    launch_full(k_score<R>, dim3(a.grid), dim3(kT), smem, s, a.pts, a.off, a.item_off, a.item_cl, a.kp, a.H, a.tile,
+    launch_as(a.early, k_score<R>, dim3(a.grid), dim3(kT), smem, s, a.pts, a.off, a.item_off, a.item_cl, a.kp, a.H, a.tile,
                 a.hyp, a.counts, a.queue, a.eps);
     return cudaGetLastError();
 }
@@ -2015,7 +2020,9 @@ int score_max_ctas_per_sm(const FitTuning& t, int H) {
 }
 
 size_t fit_hull_smem() {
-    return (size_t)kHullCap * (2 * sizeof(unsigned long long) + 2 * sizeof(uint32_t)) + (size_t)kSurvCap * sizeof(int2);
+    constexpr size_t chains = kHullCap * (sizeof(unsigned long long) + 2 * sizeof(uint32_t));
+    constexpr size_t staged = kSurvCap * sizeof(int2);
+    return kHullCap * sizeof(unsigned long long) + (chains > staged ? chains : staged);
 }
 
 void fit_init_attributes() {
@@ -2083,8 +2090,14 @@ cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* la
     count_launch(1);
     const int grid = sms * t.ctas_per_sm;
     VM_STAGE_BEGIN(hk, kStScore, s);
-    const ScoreArgs sa{pts, off, fb.item_off, fb.item_cl, kp, H, T, tile, fb.hyp, fb.counts, fb.queue, p.eps, grid};
-    const unsigned cgrid = kcap < (uint32_t)sms * 8 ? kcap : (uint32_t)sms * 8, igrid = (unsigned)sms * 8;
+    // Scoring launched while stage a runs lands unevenly beside stage a's CTAs (a walk map: 13.9 us for 12.1); where
+    // those take at most half of the SMs it does not, and a direct fit gains the 2 us of a launch.
+    const bool early = hgrid * 2 <= (unsigned)sms;
+    const ScoreArgs sa{pts, off, fb.item_off, fb.item_cl, kp, H, T, tile, fb.hyp, fb.counts, fb.queue, p.eps, grid, early};
+    const unsigned cgrid = kcap < (uint32_t)sms * 8 ? kcap : (uint32_t)sms * 8;
+    // A small fit has about four items an SM.  Of a large fit's many a CTA takes few, so that the last ones to finish
+    // leave little idle (2,000 clusters, extraction and filter: 776 us at 8 CTAs an SM, 740 at 64, 765 at 256).
+    const unsigned igrid = (unsigned)sms * (done ? 8 : 64);
     if (warp) {
         switch (R) {
             case 1: e = launch_score_warp<1>(sa, s); break;
@@ -2116,14 +2129,14 @@ cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* la
     VM_STAGE_BEGIN(hk, kStExtract, s);
     launch_k(k_select, dim3(cgrid), dim3(kT), 0, s, pts, off, kp, H, fb.hyp, fb.hyp_valid, fb.counts, fb.cl);
     count_launch(1);
-    launch_full(done ? k_extract<true> : k_extract<false>, dim3(igrid), dim3(kT), 0, s, pts, off, fb.item_off,
+    launch_as(done != nullptr, done ? k_extract<true> : k_extract<false>, dim3(igrid), dim3(kT), 0, s, pts, off, fb.item_off,
                 fb.item_cl, kp, tile, fb.cl, fb.inlier, fb.part, p.eps, fb.err, done, fb.cen, fb.poly);
     if (!done) {
         launch_k(k_centroid, dim3(cgrid), dim3(kT), 0, s, pts, off, fb.item_off, kp, tile, fb.part, fb.cl,
                  fb.cen, fb.poly);
         count_launch(1);
     }
-    launch_full(done ? k_filter<true> : k_filter<false>, dim3(igrid), dim3(kT), 0, s, pts, off, fb.item_off,
+    launch_as(done != nullptr, done ? k_filter<true> : k_filter<false>, dim3(igrid), dim3(kT), 0, s, pts, off, fb.item_off,
                 fb.item_cl, kp, tile, fb.cl, fb.inlier, fb.cen, fb.poly, fb.part, fb.surv, done);
     VM_STAGE_END(hk, kStExtract, s);
     count_launch(2);
@@ -2284,7 +2297,7 @@ extern "C" vm_status vm_ransac_static(const float* xyz, const uint32_t* off, con
     bool warp;
     score_variant(tc, H, R, warp);
     const int grid = sms * t.ctas_per_sm;
-    const ScoreArgs sa{xyz, off, item_off, nullptr, kdev, H, t.tile, queue + 1, hyp, counts, queue, params->eps, grid};
+    const ScoreArgs sa{xyz, off, item_off, nullptr, kdev, H, t.tile, queue + 1, hyp, counts, queue, params->eps, grid, false};
     switch (R) {
         case 1: e = launch_score<1>(sa, s); break;
         case 2: e = launch_score<2>(sa, s); break;
