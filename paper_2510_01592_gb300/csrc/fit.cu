@@ -1038,15 +1038,23 @@ __device__ __forceinline__ bool jarvis_better(int2 cur, int2 a, bool a_ok, int2 
 // it lies in the convex hull of the polygon's vertices and is not an extreme
 // point); the directions only decide how much it removes.
 constexpr int kHullDirs = 128;
+constexpr int kFewDirs = 32;
+constexpr int kFewSurv = 96;    // survivors that are not worth a pass
+constexpr int kFewCand = 128;   // candidates that are not worth a second one
 constexpr int kSmallHull = kT;  // candidates ranked and tested in parallel, one a thread
 
 // Per cluster hull of the first filter's survivors: (1) extreme survivors along
-// kHullDirs directions; (2) survivors strictly inside the polygon they span
+// kFewDirs or kHullDirs directions; (2) survivors strictly inside the polygon they span
 // are dropped (none of them can be a hull vertex), the rest gathered in shared
-// memory;
+// memory; when many are left, both once more with kHullDirs directions;
 // (3) bitonic sort by (X, Y), duplicates removed; (4) monotone chain, lower
 // and upper halves built concurrently by two threads.  If more than
 // kHullCap points remain, gift wrapping runs over the survivors instead.
+// Most clusters leave some 20 survivors, and these go straight to (3'): a pass
+// costs 4 us however few they are.  A first pass of 32 directions is cheap where
+// there are many survivors (1,500 cost 128 directions 10 us) and enough where
+// there are few; in between, 128 at once spare a second pass.  16 clusters: 8.4 ->
+// 7.5 us, 2,000 clusters 58 -> 43, the 5 x 5 x 5 m window 21.8 -> 14.5.
 // hull_ctr: a word that is zero at launch; the last CTA to finish turns
 // hull_cnt into the hulls' offsets (exclusive scan, the total at [k]) and
 // zeroes the word again.
@@ -1063,7 +1071,7 @@ __global__ void __launch_bounds__(kT) k_hull(const uint32_t* __restrict__ off, c
     int2* ssv = reinterpret_cast<int2*>(uq);  // kSurvCap staged survivors, done with before the unique keys
     __shared__ uint32_t wsum[kT / 32];
     __shared__ int s_klo, s_khi, s_m, s_cnt;
-    __shared__ int2 poly[kHullDirs + 1];   // the extreme point of each direction
+    __shared__ int2 poly[kHullDirs];       // the extreme point of each direction
     __shared__ int2 hpoly[kHullDirs + 1];  // the filter polygon
     __shared__ long long warea[kT / 32];
     __shared__ int2 sdir[kHullDirs];
@@ -1071,83 +1079,95 @@ __global__ void __launch_bounds__(kT) k_hull(const uint32_t* __restrict__ off, c
     __shared__ int jok[kT];
     __shared__ unsigned long long wmin[kT / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int j = threadIdx.x; j < kHullDirs; j += kT) {
-        const float t = (float)j * (2.0f / kHullDirs);
-        sdir[j] = make_int2(__float2int_rn(1024.0f * cospif(t)), __float2int_rn(1024.0f * sinpif(t)));
-    }
+    bool dirs = false;  // sdir is there
     for (uint32_t c = blockIdx.x; c < k; c += gridDim.x) {
         __syncthreads();
         const uint32_t base = off[c];
         const int s = (int)cl[c].n_surv;
         int2* out = hull + base;
-        if (threadIdx.x == 0) s_cnt = 0;
         // stage the survivors (when they fit) so the scans below read shared memory
         const int2* sv = surv + base;
         if (s <= kSurvCap) {
             for (int i = threadIdx.x; i < s; i += kT) ssv[i] = sv[i];
             sv = ssv;
-            __syncthreads();
         }
-        // (1) extreme points along kHullDirs directions, warp w taking 16 of
-        // them.  The projections are FP32: any closed polygon through input
-        // points serves the filter below (which is exact), so an extreme point
-        // only has to be an input point, not the exact maximiser.
-        {
-            constexpr int kPer = kHullDirs / (kT / 32);
-            float dxq[kPer], dyq[kPer], bv[kPer];
-            int bi[kPer];
-#pragma unroll
-            for (int q = 0; q < kPer; ++q) {
-                dxq[q] = (float)sdir[kPer * w + q].x;
-                dyq[q] = (float)sdir[kPer * w + q].y;
-                bv[q] = -INFINITY;
-                bi[q] = -1;
+        if (s > kFewSurv && !dirs) {
+            for (int j = threadIdx.x; j < kHullDirs; j += kT) {
+                const float t = (float)j * (2.0f / kHullDirs);
+                sdir[j] = make_int2(__float2int_rn(1024.0f * cospif(t)), __float2int_rn(1024.0f * sinpif(t)));
             }
-            for (int i = lane; i < s; i += 32) {
-                const int2 p = sv[i];
-                const float fx = (float)p.x, fy = (float)p.y;
-#pragma unroll
-                for (int q = 0; q < kPer; ++q) {
-                    const float v = fmaf(dxq[q], fx, dyq[q] * fy);
-                    if (v > bv[q]) { bv[q] = v; bi[q] = i; }
-                }
-            }
-            // the warp's largest projection (its bits as an ordered integer), then the lowest index that has it
-            int at[kPer];
-#pragma unroll
-            for (int q = 0; q < kPer; ++q) {
-                const int b = __float_as_int(bv[q]), key = b ^ ((b >> 31) & 0x7fffffff);
-                const int top = __reduce_max_sync(0xffffffffu, key);
-                at[q] = __reduce_min_sync(0xffffffffu, key == top && bi[q] >= 0 ? bi[q] : INT_MAX);
-            }
-            if (lane == 0)
-#pragma unroll
-                for (int q = 0; q < kPer; ++q)
-                    poly[kPer * w + q] = at[q] != INT_MAX ? sv[at[q]] : make_int2(INT_MIN, INT_MIN);
+            dirs = true;
         }
         __syncthreads();
-        // The polygon through the extremes, consecutive duplicates removed (and
-        // the last vertex when it repeats the first), in parallel: a direction's
-        // extreme is kept unless it repeats the previous direction's; a ballot
-        // places the kept ones.  Every direction has an extreme when s > 0.
-        {
-            const bool valid = s > 0 && threadIdx.x < kHullDirs;
+        // (1), (2): from `from`, n points, to `to`; the candidates so far are cand[0 .. s2)
+        const int2* cand = sv;
+        int s2 = s;
+        for (int pass = 0, D = s > 160 && s <= 512 ? kHullDirs : kFewDirs; pass < 2; ++pass, D = kHullDirs) {
+            const int2* from = cand;
+            int2* to = reinterpret_cast<int2*>(sk);
+            int n = s2;
+            if (pass == 0 ? s <= kFewSurv : s2 <= kFewCand) break;
+            if (pass && s2 > kHullCap) {  // from the survivors again: the first polygon dropped too few
+                from = sv;
+                n = s;
+            } else if (pass) {
+                to = reinterpret_cast<int2*>(uq);  // the staged survivors are done with
+            }
+            // (1) extreme points along D directions, four a warp at a time.  The
+            // projections are FP32: any closed polygon through input points
+            // serves the filter below (which is exact), so an extreme point only
+            // has to be an input point, not the exact maximiser.
+            for (int d0 = 4 * w; d0 < D; d0 += 4 * (kT / 32)) {
+                float dxq[4], dyq[4], bv[4];
+                int bi[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int2 dir = sdir[(d0 + q) * (kHullDirs / D)];
+                    dxq[q] = (float)dir.x;
+                    dyq[q] = (float)dir.y;
+                    bv[q] = -INFINITY;
+                    bi[q] = -1;
+                }
+#pragma unroll 2
+                for (int i = lane; i < n; i += 32) {
+                    const int2 p = from[i];
+                    const float fx = (float)p.x, fy = (float)p.y;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float v = fmaf(dxq[q], fx, dyq[q] * fy);
+                        if (v > bv[q]) { bv[q] = v; bi[q] = i; }
+                    }
+                }
+                // the warp's largest projection (its bits as an ordered integer), then the lowest index that has it
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int b = __float_as_int(bv[q]), key = b ^ ((b >> 31) & 0x7fffffff);
+                    const int top = __reduce_max_sync(0xffffffffu, key);
+                    const int at = __reduce_min_sync(0xffffffffu, key == top && bi[q] >= 0 ? bi[q] : INT_MAX);
+                    if (lane == q) poly[d0 + q] = at != INT_MAX ? from[at] : make_int2(INT_MIN, INT_MIN);
+                }
+            }
+            __syncthreads();
+            // The polygon through the extremes, consecutive duplicates removed (and
+            // the last vertex when it repeats the first), in parallel: a direction's
+            // extreme is kept unless it repeats the previous direction's; a ballot
+            // places the kept ones.  Every direction has an extreme: n > 0.
             int2 p = make_int2(0, 0);
             bool keep = false;
-            if (valid) {
+            if (threadIdx.x < D) {
                 p = poly[threadIdx.x];
                 const int2 q = poly[threadIdx.x ? threadIdx.x - 1 : 0];
                 keep = threadIdx.x == 0 || p.x != q.x || p.y != q.y;
             }
-            const uint32_t b = __ballot_sync(0xffffffffu, keep);
-            if (lane == 0) wsum[w] = __popc(b);
+            const uint32_t kb = __ballot_sync(0xffffffffu, keep);
+            if (lane == 0) wsum[w] = __popc(kb);
             __syncthreads();
-            uint32_t pos = __popc(b & ((1u << lane) - 1u)), m0 = 0;
+            uint32_t at = __popc(kb & ((1u << lane) - 1u)), m0 = 0;
             for (int q = 0; q < kT / 32; ++q) {
-                pos += q < w ? wsum[q] : 0u;
+                at += q < w ? wsum[q] : 0u;
                 m0 += wsum[q];
             }
-            if (keep) hpoly[pos] = p;
+            if (keep) hpoly[at] = p;
             __syncthreads();
             if (m0 > 1 && hpoly[m0 - 1].x == hpoly[0].x && hpoly[m0 - 1].y == hpoly[0].y) --m0;
             // twice the signed area: a degenerate (zero-area) polygon filters nothing
@@ -1164,47 +1184,57 @@ __global__ void __launch_bounds__(kT) k_hull(const uint32_t* __restrict__ off, c
                 long long area2 = 0;
                 for (int q = 0; q < kT / 32; ++q) area2 += warea[q];
                 s_m = (m0 >= 3 && area2 > 0) ? (int)m0 : 0;
+                hpoly[m0] = hpoly[0];
+                s_cnt = 0;
             }
-        }
-        __syncthreads();
-        const int m = s_m;
-        // (2) drop survivors strictly inside the polygon
-        for (int i0 = 0; i0 < s; i0 += kT) {
-            const int i = i0 + threadIdx.x;
-            bool keep = false;
-            int2 p = make_int2(0, 0);
-            if (i < s) {
-                p = sv[i];
-                keep = (m == 0);
-                for (int e = 0; e < m; ++e) {
-                    if (cross3(hpoly[e], hpoly[e + 1 < m ? e + 1 : 0], p) <= 0) { keep = true; break; }
+            __syncthreads();
+            const int m = s_m;
+            // (2) drop the points strictly inside the polygon
+            for (int i0 = 0; i0 < n; i0 += kT) {
+                const int i = i0 + threadIdx.x;
+                bool out_or_on = false;
+                int2 pt = make_int2(0, 0);
+                if (i < n) {
+                    pt = from[i];
+                    out_or_on = (m == 0);
+#pragma unroll 4
+                    for (int e = 0; e < m; ++e) out_or_on |= cross3(hpoly[e], hpoly[e + 1], pt) <= 0;
                 }
+                const uint32_t b = __ballot_sync(0xffffffffu, out_or_on);
+                int pos = 0;
+                if (lane == 0 && b) pos = atomicAdd(&s_cnt, __popc(b));
+                pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(b & ((1u << lane) - 1u));
+                if (out_or_on && pos < kHullCap) to[pos] = pt;
             }
-            const uint32_t b = __ballot_sync(0xffffffffu, keep);
-            int pos = 0;
-            if (lane == 0 && b) pos = atomicAdd(&s_cnt, __popc(b));
-            pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(b & ((1u << lane) - 1u));
-            if (keep && pos < kHullCap) sk[pos] = xy_key(p);
+            __syncthreads();
+            cand = to;
+            s2 = s_cnt;
         }
+        if (s2 <= kHullCap)
+            for (int i = threadIdx.x; i < s2; i += kT) sk[i] = xy_key(cand[i]);
         __syncthreads();
-        const int s2 = s_cnt;
         if (s2 <= kSmallHull) {
             // (3') at most kT candidates: rank sort with duplicates removed --
             // a candidate is kept if no earlier one has its key, and lands at
             // the number of kept keys below it
-            const int i = threadIdx.x;
+            // (few candidates share the threads, 4 or 2 to one)
+            const int i = threadIdx.x, Lr = s2 <= kT / 4 ? 4 : (s2 <= kT / 2 ? 2 : 1), cr = i / Lr, sr = i % Lr;
             unsigned long long key = 0;
-            bool first = false;
-            if (i < s2) {
-                key = sk[i];
-                first = true;
-                for (int j = 0; j < i; ++j) first &= sk[j] != key;
+            int twin = 0;
+            if (cr < s2) {
+                key = sk[cr];
+#pragma unroll 4
+                for (int j = sr; j < cr; j += Lr) twin |= sk[j] == key;
             }
-            st_lo[i] = first;  // kT flags
+            for (int o = 1; o < Lr; o <<= 1) twin |= __shfl_xor_sync(0xffffffffu, twin, o);
+            const bool uniq = cr < s2 && !twin, first = uniq && sr == 0;
+            if (sr == 0) st_lo[cr] = first;
             __syncthreads();
             int rank = 0;
-            if (first)
-                for (int j = 0; j < s2; ++j) rank += (st_lo[j] != 0u) & (sk[j] < key);
+            if (uniq)
+#pragma unroll 4
+                for (int j = sr; j < s2; j += Lr) rank += (st_lo[j] != 0u) & (sk[j] < key);
+            for (int o = 1; o < Lr; o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
             const uint32_t b = __ballot_sync(0xffffffffu, first);
             if (lane == 0) wsum[w] = __popc(b);
             __syncthreads();
