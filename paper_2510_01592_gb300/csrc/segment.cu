@@ -251,10 +251,13 @@ __device__ __forceinline__ float mean_pos(float o, int32_t m) {
 // cells of its 3x3x3 window are occupied and where their integer means lie;
 // the means are read straight from the caches (neighbours of a warp's voxels
 // share lines) and give the covariance of the window's mean positions (self
-// included) as the exact integer matrix N' sum(dd^T) - (sum d)(sum d)^T of
-// offsets d = M_j - M_i, rounded to FP32.  A free cell is read as the voxel
-// itself (d = 0 adds nothing), so a row's three loads carry no condition; rows
-// without an occupied cell are skipped.
+// included) as the exact integer matrix N' sum(MM^T) - (sum M)(sum M)^T,
+// rounded to FP32.  The matrix does not depend on the origin of the means, so
+// they are taken as they are, from the window's anchor: a map is at most 16 m
+// wide, 2^24 quanta, so the products' sums stay below 2^53 and N' times them
+// below 2^58.  A free cell's load is left out and adds zero.  Wide multiplies
+// and the loads' latency bound it: 12.4 us for the walk map's 0.28 M voxels, 66
+// for the 8 x 8 x 3 m map's 1.4 M (14 and 71 with offsets from the own mean).
 __global__ void __launch_bounds__(kT) k_moments(const SegCounters* __restrict__ ctr, const float* __restrict__ po,
                                                 const uint4* __restrict__ rows, const uint32_t* __restrict__ vox,
                                                 const int4* __restrict__ M, float4* __restrict__ pos,
@@ -274,21 +277,22 @@ __global__ void __launch_bounds__(kT) k_moments(const SegCounters* __restrict__ 
         int cnt = 0;
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
-            const uint4 row = rw[(q / 3) * 10 + q % 3];
             uint32_t win, idx[3];
-            row_window(row, lx, win, idx);
-            if (!win) continue;
+            row_window(rw[(q / 3) * 10 + q % 3], lx, win, idx);
+            cnt += __popc(win);
             int4 a[3];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) a[k] = M[(win >> k) & 1u ? idx[k] : i];
+            for (int k = 0; k < 3; ++k) {
+                a[k] = make_int4(0, 0, 0, 0);
+                if ((win >> k) & 1u) a[k] = M[idx[k]];
+            }
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const int32_t ex = a[k].x - m.x, ey = a[k].y - m.y, ez = a[k].z - m.z;
-                s1x += ex; s1y += ey; s1z += ez;
-                sxx += (long long)ex * ex; syy += (long long)ey * ey; szz += (long long)ez * ez;
-                sxy += (long long)ex * ey; sxz += (long long)ex * ez; syz += (long long)ey * ez;
+                const int32_t x = a[k].x, y = a[k].y, z = a[k].z;
+                s1x += x; s1y += y; s1z += z;
+                sxx += (long long)x * x; syy += (long long)y * y; szz += (long long)z * z;
+                sxy += (long long)x * y; sxz += (long long)x * z; syz += (long long)y * z;
             }
-            cnt += __popc(win);
         }
         const long long N = cnt;
         list_A[i] = __ll2float_rn(N * sxx - (long long)s1x * s1x);
