@@ -38,12 +38,12 @@ N_FRAMES = 300
 # stat its work scales with: {stage: (bytes per unit, stat)}.  Remove a
 # kernel's entry when the kernel changes.
 TRAFFIC_PER_UNIT = {
-    # 60-frame trajectory case (1,498 bricks; profiles/segment_kernels_60frames.md): the halo is staged
-    # per brick, so the traffic scales with the allocated bricks
-    "ccl_local": (14557952.0 / 1498, "bricks_allocated"),
-    "ccl_cross": ((15073792.0 + 1536.0) / 1498, "bricks_allocated"),
-    "moments": ((9291776.0 + 0.0) / 1498, "bricks_allocated"),
-    "eigen": ((4150016.0 + 77568.0) / 1498, "bricks_allocated"),
+    # 60-frame trajectory case (135,050 occupied voxels; profiles/segment_kernels_60frames.md): the
+    # arrays hold the occupied voxels only; the cross-brick stage is its three kernels together
+    "ccl_local": (5093632.0 / 135050, "occupied_voxels"),
+    "ccl_cross": ((14336.0 + 5942272.0 + 113408.0) / 135050, "occupied_voxels"),
+    "moments": (3901440.0 / 135050, "occupied_voxels"),
+    "eigen": (3390720.0 / 135050, "occupied_voxels"),
 }
 METRIC = "0.01 m integrate+segment: frames/s, p50/p99 ms, batched/served vs plain GPU"
 WORKLOAD = ("paper-scale trajectory: 4x4x2 m map at 0.01 m (sparse 8^3 bricks), 640x480 depth camera "
@@ -185,7 +185,9 @@ def batching_variant(dev, stream, alu_peak):
         "stages_ms": {kk: round(v[0], 4) for kk, v in st.items()},
         "ransac_score_roofline": {"bound": "alu", "achieved": round(ach, 3), "peak": round(alu_peak, 2),
                                   "unit": "T instr/s", "frac": round(ach / alu_peak, 4),
-                                  "point_tests_per_s": round(H * n / (score_ms / 1e3), 1)},
+                                  "point_tests_per_s": round(H * n / (score_ms / 1e3), 1),
+                                  "note": "priced as if every point were tested against every hypothesis; the "
+                                          "scoring decides most of these tests by a bound and makes about a fifth"},
     }
 
 
@@ -1166,26 +1168,28 @@ def kernel_table(stages, st, peaks, n_points_segment, frame_points=0, frame_voxe
     occupied voxel; eigen ~520 FP32 instructions per occupied voxel; CCL 24 B
     (mean, normal) + 4 B label x (1 + 1 pass) per vertex (steppable voxel):
     the in-brick pass is priced at 24 B + 4 B (its reads and its labels), the
-    cross-brick pass, which completes the labels, at the whole 32 B;
+    cross-brick stage (numbering, pairs, join), which completes the labels, at
+    the whole 32 B;
     RANSAC scoring 5 instructions per point-hypothesis test.  staged_bytes:
     what the kernel as written reads and writes for the same launch, where
-    it differs (per-slot staging of allocated bricks: slots = bricks x 512).
-    kernels: launches in the stage; only single-kernel stages are roofline
+    it differs (its own records per occupied voxel, halo rows per brick).
+    kernels: launches in the stage (the cross-brick stage's three count as
+    one, the method's unit); only single-kernel stages are roofline
     candidates."""
     hbm = peaks["hbm_gbs"] if peaks else 6800.0
     clk = (peaks or {}).get("sm_max_mhz", 2070.0) * 1e6
     alu_peak = SM_COUNT * FP32_LANES * clk / 1e12  # T instructions/s
     occ = st["occupied_voxels"]
     vert = st["steppable_voxels"]
-    slots = st["bricks_allocated"] * 512
+    bricks = st["bricks_allocated"]
     model = {  # name: (bound, algorithmic amount, staged bytes or None, kernels in the stage)
         "integrate": ("hbm", frame_points * (12 + 4) + frame_voxels * 28,
                       frame_points * (12 * 2 + 4) + frame_voxels * 28, 2),
-        "finalize": ("hbm", occ * (28 + 12 + 4), slots * (4 + 1 + 12) + occ * 24, 1),
-        "moments": ("hbm", occ * (12 + 1), slots * (12 + 16 + 8) + occ * (4 + 24 + 1), 1),
+        "finalize": ("hbm", occ * (28 + 12 + 4), occ * (28 + 16 + 4) + bricks * (128 + 108 + 1600), 1),
+        "moments": ("hbm", occ * (12 + 1), occ * (16 + 4 + 24 + 1 + 16 + 8) + bricks * 1600, 1),
         "eigen": ("alu", occ * 520, None, 1),
-        "ccl_local": ("hbm", vert * (24 + 4), None, 1),
-        "ccl_cross": ("hbm", vert * (24 + 4 * 2), None, 1),
+        "ccl_local": ("hbm", vert * (24 + 4), occ * (4 + 32 + 2) + bricks * 128, 1),
+        "ccl_cross": ("hbm", vert * (24 + 4 * 2), None, 1),  # numbering, pairs and join: one unit of work
         "ransac_score": ("alu", n_points_segment * n_hyp * 5, None, 1),
     }
     out = {}

@@ -21,7 +21,7 @@
 //            appended.
 //  k_refit   per cluster: TLS refit from the partial sums (double-float sums,
 //            adjugate power iteration).
-//  k_hull    per cluster: a second, 128-direction filter, then a sort of the
+//  k_hull    per cluster: a finer filter where many are left, then a sort of the
 //            remaining quantised points in shared memory and Andrew's monotone
 //            chain with exact int64 orientation tests (few points: a rank sort
 //            and a test per point); gift wrapping over global memory when too

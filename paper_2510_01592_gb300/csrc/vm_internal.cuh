@@ -25,7 +25,7 @@ namespace vmx {
 // griddepcontrol.launch_dependents lets the next kernel on the stream start
 // launching.  So each launch, and the rasterisation of its CTAs, overlaps the
 // kernel before it instead of following it: in a chain of small kernels (a
-// segmentation is ~40) that gap, not the work, is most of the time.  A kernel
+// segmentation is 20) that gap, not the work, is most of the time.  A kernel
 // touches no global memory before the gate, so ordering is that of plain
 // stream launches.  A long, issue-bound kernel that leaves room on its SMs
 // (the persistent RANSAC scoring) waits without the early trigger
@@ -60,9 +60,9 @@ cudaError_t launch_k(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, c
     return launch_as(true, kernel, grid, block, smem, s, std::forward<A>(args)...);
 }
 // A plain launch, for a kernel whose grid is sized to fill the GPU and whose
-// work is balanced by that placement (the persistent scoring, the chunked
-// extraction passes): launched early beside the kernel before it, its CTAs
-// would land unevenly on the SMs that kernel frees first.
+// work is balanced by that placement (the persistent scoring, a large fit's
+// chunked extraction passes): launched early beside the kernel before it, its
+// CTAs would land unevenly on the SMs that kernel frees first.
 template <typename... K, typename... A>
 cudaError_t launch_full(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
     return launch_as(false, kernel, grid, block, smem, s, std::forward<A>(args)...);
