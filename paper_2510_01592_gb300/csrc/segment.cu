@@ -735,18 +735,23 @@ __global__ void __launch_bounds__(kT, 4)
 // two roots, and a pair that is apart hooks the larger under the smaller one (an
 // atomic minimum; a hook that another one replaces is found again), until no
 // pair is apart.  Only the roots that the first flattening leaves take part in
-// the later ones.  Pairs that fit beside the forest are joined by one CTA.  With
-// more, every CTA first walks its share of the pairs in a copy of its own, lists
-// those that are apart (a third of the LiDAR map's 95 thousand) and stores the
-// roots of its share of the components; the last CTA to finish joins the list.
+// the later ones.  Few pairs are joined by one CTA.  With more, every CTA first
+// walks its share of the pairs in a copy of its own, lists those that are apart
+// (a third of the LiDAR map's 95 thousand) and stores the roots of its share of
+// the components; the last CTA to finish numbers the roots (9 of 29 thousand) and
+// joins the list over these numbers, so that forest and list fit beside each
+// other.
 // With more components, or pairs the list had no room for, the grid joins pair
 // by pair in global memory (51 us for the walk map's 17 thousand pairs: the
 // threads meet on the few large roots).  One SM's instruction rate bounds the
-// rounds: what is touched in a round, not the steps of a chain, counts.  13.6 us
-// for the walk map (2.7 thousand components), 85 us for the 8 x 8 x 3 m one (29
-// thousand); reading each pair's chains in every round took 18 and 93 us.
+// rounds: what is touched in a round, not the steps of a chain, counts.  So a few
+// thousand pairs are joined by one CTA, and more are thinned first: the walk
+// map's 17 thousand take 14.1 us alone and 12.7 thinned, the 5 x 5 x 5 m window's
+// 23 thousand 24.8 and 16.3.  The 8 x 8 x 3 m map's 95 thousand: 54 us (85 with
+// its list in global memory, 93 with each pair's chains read in every round).
 constexpr uint32_t kJoinWords = 57344;  // 224 KB: the forest, the roots, the pairs
 constexpr uint32_t kSmemComps = 36864;  // below 2^16: a pair packs into a word
+constexpr uint32_t kJoinAlone = 8192;   // pairs that one CTA joins by itself
 // Flattens the trees over the elements list[0 .. n) (null: 0 .. n).
 __device__ __forceinline__ void join_flatten(uint32_t* P, const uint16_t* list, uint32_t n) {
     for (int round = 0; round < 64; ++round) {  // every round at least doubles the reach
@@ -775,12 +780,12 @@ __device__ __forceinline__ uint32_t join_root(uint32_t* P, uint32_t x, uint32_t 
     return x;
 }
 __global__ void __launch_bounds__(kOneT, 1) k_comp_join(SegCounters* __restrict__ ctr, uint32_t pair_cap,
-                                                        const unsigned long long* __restrict__ pairs, uint32_t* list,
-                                                        uint32_t* parent, const uint32_t* __restrict__ over,
-                                                        uint32_t* err) {
+                                                        unsigned long long* pairs, uint32_t* list, uint32_t* parent,
+                                                        const uint32_t* __restrict__ over, uint32_t* err) {
     pdl_gate();
     extern __shared__ uint32_t P[];
-    __shared__ uint32_t s_last, s_roots;
+    __shared__ uint32_t ws[33];
+    __shared__ uint32_t s_last;
     const uint32_t K = ctr->n_comp, all = ctr->n_pairs, np = min(all, pair_cap);
     if (K > kSmemComps || all > pair_cap) {
         for (uint32_t q = blockIdx.x * kOneT + threadIdx.x; q < np; q += gridDim.x * kOneT) {
@@ -795,12 +800,11 @@ __global__ void __launch_bounds__(kOneT, 1) k_comp_join(SegCounters* __restrict_
     uint16_t* roots = reinterpret_cast<uint16_t*>(P + K);  // the roots left by the first flattening
     uint32_t* L = P + K + (K + 1) / 2;                     // pairs in shared memory (0: none, or together)
     const uint32_t room = kJoinWords - K - (K + 1) / 2;
-    const bool one = np <= room;
+    const bool one = np <= min(room, kJoinAlone);
     const uint32_t G = one ? 1u : min(gridDim.x, (np + kOneT - 1) / kOneT), g = blockIdx.x;
     if (g >= G) return;
     const int lane = threadIdx.x & 31;
     const auto pack = [](unsigned long long key) { return (uint32_t)(key >> 32) << 16 | (uint32_t)key; };
-    if (threadIdx.x == 0) s_roots = 0;
 #pragma unroll 8
     for (uint32_t c = threadIdx.x; c < K; c += kOneT) P[c] = __ldcg(parent + c);
     if (one)
@@ -834,33 +838,66 @@ __global__ void __launch_bounds__(kOneT, 1) k_comp_join(SegCounters* __restrict_
         if (!s_last) return;
         __threadfence();
         n = *(volatile uint32_t*)&ctr->n_apart;
-        if (n <= room)
-#pragma unroll 8
-            for (uint32_t q = threadIdx.x; q < n; q += kOneT) L[q] = __ldcg(list + q);
     }
-    for (uint32_t c0 = 0; c0 < K; c0 += kOneT) {
-        const uint32_t c = c0 + threadIdx.x;
-        const uint32_t m = __ballot_sync(0xffffffffu, c < K && P[c] == c);
-        uint32_t at = 0;
-        if (lane == 0 && m) at = atomicAdd(&s_roots, (uint32_t)__popc(m));
-        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
-        if (c < K && P[c] == c) roots[at] = (uint16_t)c;
+    // The roots, in order: a warp takes a run of components, counts its roots and lists them from there.
+    const uint32_t half = (K + 1) / 2;
+    uint16_t* rank = reinterpret_cast<uint16_t*>(P + kJoinWords - half);  // a root's number among the roots
+    uint32_t* comp = reinterpret_cast<uint32_t*>(pairs);                  // and back (the pairs are read)
+    const uint32_t run = (K + kOneT - 1) / kOneT * 32, c0 = (threadIdx.x >> 5) * run, c1 = min(K, c0 + run);
+    uint32_t nr, at = 0;
+    for (uint32_t c = c0 + lane; c - lane < c1; c += 32) at += __popc(__ballot_sync(0xffffffffu, c < c1 && P[c] == c));
+    at = cta_warps_excl(at, ws, &nr);
+    const bool rerank = !one && n + max(half, nr) <= kJoinWords;
+    for (uint32_t c = c0 + lane; c - lane < c1; c += 32) {
+        const bool root = c < c1 && P[c] == c;
+        const uint32_t m = __ballot_sync(0xffffffffu, root), i = at + __popc(m & ((1u << lane) - 1u));
+        if (root && rerank) {
+            rank[c] = (uint16_t)i;
+            comp[i] = c;
+        } else if (root) {
+            roots[i] = (uint16_t)c;
+        }
+        at += __popc(m);
     }
     __syncthreads();
-    const uint32_t nr = s_roots;
-    const bool here = n <= room;
+    uint32_t* F = P;              // the forest of the rounds
+    const uint16_t* flat = roots; // its members
+    bool here = n <= room;        // its pairs lie in L
+    if (rerank) {
+        // over the roots' numbers, which keep their order, the pairs fit beside the forest
+        L = P;
+#pragma unroll 8
+        for (uint32_t q = threadIdx.x; q < n; q += kOneT) {
+            const uint32_t pr = __ldcg(list + q);
+            L[q] = (uint32_t)rank[pr >> 16] << 16 | rank[pr & 0xffffu];
+        }
+        __syncthreads();
+        F = P + kJoinWords - nr;
+        flat = nullptr;
+        here = true;
+        for (uint32_t i = threadIdx.x; i < nr; i += kOneT) F[i] = i;
+        __syncthreads();
+    } else if (!one && here) {
+#pragma unroll 8
+        for (uint32_t q = threadIdx.x; q < n; q += kOneT) L[q] = __ldcg(list + q);
+        __syncthreads();
+    }
     for (uint32_t round = 0;; ++round) {
         // the roots of every pair, then the hooks: apart, because a pair must not be taken for joined by a hook
-        // that another one then replaces
+        // that another one then replaces.  The pairs of a list name roots that are apart.
         bool apart = false;
+        if (!one && round == 0) {
+            apart = threadIdx.x < n;
+        } else {
 #pragma unroll 4
-        for (uint32_t q = threadIdx.x; q < n; q += kOneT) {
-            const uint32_t pr = here ? L[q] : __ldcg(list + q);
-            if (!pr) continue;
-            const uint32_t a = P[pr >> 16], b = P[pr & 0xffffu], now = a == b ? 0u : min(a, b) << 16 | max(a, b);
-            if (here) L[q] = now;
-            else list[q] = now;
-            apart |= now != 0u;
+            for (uint32_t q = threadIdx.x; q < n; q += kOneT) {
+                const uint32_t pr = here ? L[q] : __ldcg(list + q);
+                if (!pr) continue;
+                const uint32_t a = F[pr >> 16], b = F[pr & 0xffffu], now = a == b ? 0u : min(a, b) << 16 | max(a, b);
+                if (here) L[q] = now;
+                else list[q] = now;
+                apart |= now != 0u;
+            }
         }
         if (!__syncthreads_or(apart)) break;
         if (round > K) {  // every round with a pair apart joins two trees or more
@@ -871,14 +908,16 @@ __global__ void __launch_bounds__(kOneT, 1) k_comp_join(SegCounters* __restrict_
         for (uint32_t q = threadIdx.x; q < n; q += kOneT) {
             const uint32_t pr = here ? L[q] : __ldcg(list + q);
             // most pairs of a large tree name its root: a look first spares the meeting atomics
-            if (pr && *(volatile uint32_t*)&P[pr & 0xffffu] > pr >> 16) atomicMin(&P[pr & 0xffffu], pr >> 16);
+            if (pr && *(volatile uint32_t*)&F[pr & 0xffffu] > pr >> 16) atomicMin(&F[pr & 0xffffu], pr >> 16);
         }
         __syncthreads();
-        join_flatten(P, roots, nr);
+        join_flatten(F, flat, nr);
     }
     // a component's root of the first flattening, then that one's
     if (one)
         for (uint32_t c = threadIdx.x; c < K; c += kOneT) parent[c] = P[P[c]];
+    else if (rerank)
+        for (uint32_t i = threadIdx.x; i < nr; i += kOneT) parent[comp[i]] = comp[F[i]];
     else
         for (uint32_t i = threadIdx.x; i < nr; i += kOneT) parent[roots[i]] = P[roots[i]];
 }
@@ -1199,8 +1238,10 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
     uint32_t* scratch = reinterpret_cast<uint32_t*>(b.pairs);   // free once the pairs are joined
     const auto clampg = [&](uint32_t want, uint32_t mx) { return want < mx ? (want ? want : 1u) : mx; };
     // Several waves of short CTAs: with about one, some SMs got a CTA more than others for the whole pass (the per-voxel
-    // passes of the 8 x 8 x 3 m map 248 us at 8 CTAs an SM, 219 at 24; at 64 a walk map's empty CTAs cost it 8 us).
-    const unsigned bgrid = clampg(cap_b, sms * 64), vgrid = clampg((uint32_t)((b.nv + kT - 1) / kT), sms * 24);
+    // passes of the 8 x 8 x 3 m map 248 us at 8 CTAs an SM, 219 at 24).  A CTA per two bricks covers their occupied
+    // voxels (about a fifth of the slots the scratch has room for); the empty CTAs of larger grids stand in the way of
+    // other streams (16 maps served at once: 1.14 ms a pass with a grid for every slot, 1.07 so).
+    const unsigned bgrid = clampg(cap_b, sms * 64), vgrid = clampg(cap_b / 2, sms * 24);
     VM_STAGE_BEGIN(hk, kStFinalize, s);
     launch_k(k_finalize, dim3(clampg((cap_b + kFinWarps - 1) / kFinWarps, sms * 8)), dim3(kT), 0, s, b.ctr, cap_b, g,
              b.brec, b.rank_table, S, C, b.M, b.vox, b.near, b.rows);
@@ -1222,16 +1263,19 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
     launch_k(k_ccl_cross, dim3(vgrid), dim3(kT), 0, s, b.ctr, b.brec, b.near, b.rows, b.vox, b.pos, b.nrm, b.lc,
              b.ncomp, b.cbase, b.lsize, b.lroot, b.csize, b.croot, b.total, b.parent, over, b.pairs, pair_cap,
              p.d_th2, p.cos_ccl, err);
-    launch_k(k_comp_join, dim3(sms), dim3(kOneT), kJoinWords * 4, s, b.ctr, pair_cap, b.pairs, b.lsize,
-             b.parent, over, err);
+    // a CTA per thousand pairs, of which a brick has about six: each needs a whole SM's shared memory, and other streams'
+    // kernels wait for it
+    launch_k(k_comp_join, dim3(clampg(cap_b / 128, sms)), dim3(kOneT), kJoinWords * 4, s, b.ctr, pair_cap, b.pairs,
+             b.lsize, b.parent, over, err);
     VM_STAGE_END(hk, kStCcl, s);
     VM_STAGE_BEGIN(hk, kStClusters, s);
-    launch_k(k_comp_size, dim3(clampg((uint32_t)((b.nv + kT - 1) / kT), sms * 2)), dim3(kT), 0, s, b.ctr, b.parent,
+    launch_k(k_comp_size, dim3(clampg(cap_b / 64, sms * 2)), dim3(kT), 0, s, b.ctr, b.parent,
              b.csize, b.total, err);
     const uint32_t min_cl = p.min_cluster ? p.min_cluster : 1u;
     launch_k(k_cluster_number, dim3(1), dim3(kOneT), 0, s, b.ctr, min_cl, kcap, b.total, b.croot, b.ccl, b.cl_size,
              b.cl_label, b.cl_off, scratch);
-    launch_k(k_cluster_place, dim3(clampg((uint32_t)sms, kPlaceCtas)), dim3(kOneT), kPlaceWords * 4, s, b.ctr,
+    // a CTA per thousand components, of which a brick has one or two, for the reason given at k_comp_join
+    launch_k(k_cluster_place, dim3(clampg(cap_b / 512 + 1, kPlaceCtas)), dim3(kOneT), kPlaceWords * 4, s, b.ctr,
              b.parent, b.csize, b.ccl, b.cl_off, b.place, scratch, (uint32_t)(2 * b.nv), err);
     launch_k(k_cluster_scatter, dim3(clampg((cap_b + kScatWarps - 1) / kScatWarps, sms * 8)), dim3(kScatWarps * 32), 0,
              s, b.ctr, cap_b, b.brec, b.ncomp, b.cbase, b.ccl, b.place, b.lc, b.vox, b.pos, b.pts, b.pt_vid);
