@@ -2175,7 +2175,10 @@ cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* la
         launch_k(k_refit, dim3(cgrid), dim3(kT), 0, s, off, fb.item_off, kp, tile, fb.part, fb.cen, fb.cl);
         count_launch(1);
     }
-    launch_k(k_hull, dim3(cgrid), dim3(kT), fit_hull_smem(), s, off, kp, fb.cl, fb.surv, fb.hull, fb.hull_cnt, fb.err,
+    // as many CTAs as run at once: a cluster takes about as long as another, and the last CTA's count of the finished ones
+    // is shorter (a walk map 231 us for 234 with a CTA for every cluster the scratch has room for)
+    const unsigned hull_grid = cgrid < (unsigned)sms * 2 ? cgrid : (unsigned)sms * 2;
+    launch_k(k_hull, dim3(hull_grid), dim3(kT), fit_hull_smem(), s, off, kp, fb.cl, fb.surv, fb.hull, fb.hull_cnt, fb.err,
              fb.queue + 3);
     VM_STAGE_END(hk, kStHull, s);
     count_launch(1);
