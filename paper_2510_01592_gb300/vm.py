@@ -200,7 +200,10 @@ _Pose = C.c_float * 12
 
 def _copy(ptr, n, dtype):
     """n records at ptr as an array of its own."""
-    return np.frombuffer(bytearray(C.string_at(ptr, n * dtype.itemsize)) if n else bytearray(), dtype)
+    size = n * dtype.itemsize
+    if size > 0x7FFFFFFF:  # string_at takes the size as a C int
+        return np.frombuffer((C.c_char * size).from_address(C.cast(ptr, C.c_void_p).value), dtype).copy()
+    return np.frombuffer(bytearray(C.string_at(ptr, size)) if n else bytearray(), dtype)
 
 
 _I32, _F32 = np.dtype(np.int32), np.dtype(np.float32)
