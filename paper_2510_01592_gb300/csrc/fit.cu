@@ -1706,7 +1706,15 @@ __global__ void __launch_bounds__(kT) k_score_lower(const float* __restrict__ pt
 // hypothesis, the near points against those the bound leaves open.  All tests
 // are count_point's, and the bound is widened by 2^-16 (|d| + |d0| + sum of the
 // largest |coordinates|), over 250 rounding units of every quantity that enters
-// it or the test (their sum stays below 150), so the counts are exact.
+// it or the test (their sum stays below 150), so the counts are exact.  The
+// in-plane axis is a difference, whose rounding leaves 2^-22 r / s of the normal
+// in it when the farthest point lies r from the box's centre but only s from it
+// in the plane: that costs 64 units more while the hypothesis leans from the
+// reference by less than 16 s / r (angle t), and nothing beyond: no near point is
+// farther than r from the centre, so one at an angle a from the farthest has a
+// residual lower by r (1 - cos a), and the box adds r (1 - cos t) (1 + cos a) for
+// it along the normal, together more than the r sin a sin t that it can lose, as
+// cos(t - a) + cos t < 2.
 // (2) counts start at the cluster's size and lose a tile's misses.  A
 // hypothesis whose count has fallen below the reference plane's inliers cannot
 // be selected any more and is dropped; its count stays below the best one.  The
@@ -1853,7 +1861,10 @@ __global__ void __launch_bounds__(kT) k_score_slab(const float* __restrict__ pts
         ay -= along * r0.y;
         az -= along * r0.z;
         const float len2 = ax * ax + ay * ay + az * az;
-        const bool framed = len2 > 1e-12f && len2 < 1e12f;  // else the axis-aligned box alone
+        // else the axis-aligned box alone: no direction, or a normal whose square left the range of normal floats
+        // (samples closer than 1e-9 m, or beyond 1e9 m, apart) and that is not a unit vector
+        const float n2 = r0.x * r0.x + r0.y * r0.y + r0.z * r0.z;
+        const bool framed = len2 > 1e-12f && len2 < 1e12f && fabsf(n2 - 1.0f) < 9.5367431640625e-07f;  // 2^-20
         const float il = framed ? rsqrtf(len2) : 0.0f;
         ax *= il;
         ay *= il;
