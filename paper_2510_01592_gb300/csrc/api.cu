@@ -72,11 +72,11 @@ void release(DevBuf& b) {
 
 
 // The fit scratch for kcap clusters, npts points, `chunks` 256-point partial
-// sums and H hypotheses, carved in order.
-static void fit_layout(Carver& c, FitBuffers& fb, size_t kcap, size_t npts, size_t chunks, int H) {
-    fb.hyp = c.take<float4>(kcap * H);
-    fb.hyp_valid = c.take<uint8_t>(kcap * H);
-    fb.counts = c.take<uint32_t>(kcap * H);
+// sums and `slots` hypotheses of all clusters together, carved in order.
+static void fit_layout(Carver& c, FitBuffers& fb, size_t kcap, size_t npts, size_t chunks, size_t slots) {
+    fb.hyp = c.take<float4>(slots);
+    fb.hyp_valid = c.take<uint8_t>(slots);
+    fb.counts = c.take<uint32_t>(slots);
     fb.cl = c.take<FitCluster>(kcap);
     fb.item_off = c.take<uint32_t>(kcap + 1);
     fb.item_cl = c.take<uint32_t>(chunks + 1);  // items never outnumber the chunk slots
@@ -97,10 +97,10 @@ static void fit_layout(Carver& c, FitBuffers& fb, size_t kcap, size_t npts, size
     fb.done = c.take<uint32_t>(kcap * 3);
 }
 
-size_t fit_bytes(size_t kcap, size_t npts, size_t chunks, int H) {
+static size_t fit_bytes(size_t kcap, size_t npts, size_t chunks, size_t slots) {
     Carver dry{nullptr};
     FitBuffers fb{};
-    fit_layout(dry, fb, kcap, npts, chunks, H);
+    fit_layout(dry, fb, kcap, npts, chunks, slots);
     return dry.off + 256;
 }
 
@@ -110,27 +110,41 @@ static size_t fit_chunks(size_t kcap, size_t npts, int tile) {
     return (npts / (size_t)tile + kcap + 1) * ((size_t)tile / 256);
 }
 
+// A limit that is too small grows with headroom and the others stay, so that a
+// caller whose batches alternate between shapes comes to rest.  Where the device
+// has no room for the largest of every limit together, the request's own remain.
 vm_status fit_prepare(FitContext& fc, size_t kcap, size_t npts, int H, int tile, cudaStream_t s) {
     const size_t chunks = fit_chunks(kcap, npts, tile);
-    if (fc.mem.p && kcap <= fc.kcap && npts <= fc.npts && chunks <= fc.items && H <= fc.H) return VM_OK;
-    const size_t k2 = kcap + kcap / 4 + 16, n2 = npts + npts / 4 + 1024;
-    const size_t c2 = fit_chunks(k2, n2, tile) > fc.items ? fit_chunks(k2, n2, tile) : fc.items;
-    const int H2 = H > fc.H ? H : fc.H;
-    VM_TRY(ensure(fc.mem, fit_bytes(k2, n2, c2, H2)));
+    if (fc.mem.p && kcap <= fc.kcap && npts <= fc.npts && chunks <= fc.items && kcap * H <= fc.slots) return VM_OK;
+    size_t k2 = 0, n2 = 0, c2 = 0, h2 = 0;
+    const auto limits = [&](bool keep) {
+        k2 = keep && kcap <= fc.kcap ? fc.kcap : kcap + kcap / 4 + 16;
+        n2 = keep && npts <= fc.npts ? fc.npts : npts + npts / 4 + 1024;
+        c2 = fit_chunks(k2, n2, tile);
+        h2 = (kcap + kcap / 4 + 16) * H;
+        if (keep && c2 < fc.items) c2 = fc.items;
+        if (keep && h2 < fc.slots) h2 = fc.slots;
+    };
+    limits(fc.mem.p != nullptr);
+    vm_status st = ensure(fc.mem, fit_bytes(k2, n2, c2, h2));
+    if (st == VM_ERR_OUT_OF_MEMORY) {
+        limits(false);
+        st = ensure(fc.mem, fit_bytes(k2, n2, c2, h2));
+    }
+    if (st != VM_OK) return st;
     Carver c{static_cast<char*>(fc.mem.p)};
     FitBuffers fb{};
-    fit_layout(c, fb, k2, n2, c2, H2);
+    fit_layout(c, fb, k2, n2, c2, h2);
     VM_CUDA(cudaMemsetAsync(fb.scan_tmp, 0, scan_tmp_words(k2 + 1) * sizeof(uint32_t), s));  // scan state
     fb.kcap = k2;
     fb.npts_cap = fb.npts_expect = n2;
     fb.items_cap = c2;
-    fb.H = H2;
     fc.fb = fb;
     fc.gen++;
     fc.kcap = k2;
     fc.npts = n2;
     fc.items = c2;
-    fc.H = H2;
+    fc.slots = h2;
     return VM_OK;
 }
 
@@ -141,8 +155,7 @@ void fit_release(FitContext& fc) {
     fc.host = nullptr;
     fc.host_dev = nullptr;
     fc.out_kcap = fc.out_hcap = 0;
-    fc.kcap = fc.npts = fc.items = 0;
-    fc.H = 0;
+    fc.kcap = fc.npts = fc.items = fc.slots = 0;
 }
 
 int device_sms() {
@@ -212,7 +225,7 @@ static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* 
     memset(out, 0, sizeof(*out));
     if (k == 0) return VM_OK;
     size_t npts = fc.npts;
-    if (!fc.mem.p || k > fc.kcap || (int)p.n_hyp > fc.H) {  // the scratch grows in any case: learn the point count
+    if (!fc.mem.p || k > fc.kcap || (size_t)k * p.n_hyp > fc.slots) {  // the scratch grows in any case: learn the point count
         uint32_t n = 0;
         VM_CUDA(cudaMemcpyAsync(&n, off + k, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         VM_CUDA(cudaStreamSynchronize(s));

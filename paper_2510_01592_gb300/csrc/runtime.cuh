@@ -86,8 +86,7 @@ struct FitContext {
     uint64_t gen = 0;      // bumps whenever the scratch moves
     DevBuf mem;
     FitBuffers fb{};
-    size_t kcap = 0, npts = 0, items = 0;
-    int H = 0;
+    size_t kcap = 0, npts = 0, items = 0, slots = 0;  // slots: hypotheses of all clusters
     // result block of vm_fit_planes: mapped pinned host memory, laid out as a plan's
     void* host = nullptr;
     char* host_dev = nullptr;
@@ -108,7 +107,6 @@ cudaError_t fit_open(const uint32_t* off, uint32_t k, uint32_t ncap, FitBuffers&
 cudaError_t fit_close(const FitBuffers& fb, FitHeader* out, cudaStream_t s);
 
 void release(DevBuf& b);
-size_t fit_bytes(size_t kcap, size_t npts, size_t chunks, int H);
 // Sizes fit scratch (zeroing its scan state on s when it is re-allocated).
 vm_status fit_prepare(FitContext& fc, size_t kcap, size_t npts, int H, int tile, cudaStream_t s);
 void fit_release(FitContext& fc);

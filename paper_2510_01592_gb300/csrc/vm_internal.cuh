@@ -430,7 +430,6 @@ struct FitBuffers {
     uint32_t* done;         // [kcap][3] per-cluster completion counters (scoring, extraction, filter)
     size_t kcap, npts_cap, items_cap;  // items_cap: 256-point partial-sum chunks
     size_t npts_expect;     // points a fit is likely to have (picks kernels; results do not depend on it)
-    int H;
 };
 
 struct FitTuning {

@@ -1,0 +1,58 @@
+"""GPU: a thread's direct fits (vm_fit_planes) share one scratch and one result
+block; calls of different shapes on one thread give the plan's outputs, and come
+to rest: no more launches or allocations a call than the shape takes alone."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _clusters(k, n, seed):
+    """k patches of n points, with outliers; offsets int32 [k + 1]."""
+    import torch
+    rng = np.random.default_rng(seed)
+    p = rng.uniform(-0.5, 0.5, (k, n, 3)) * np.array([1, 1, 0.004]) + rng.uniform(-4, 4, (k, 1, 3))
+    off = np.arange(0, k * n + 1, n, dtype=np.int32)
+    return torch.from_numpy(p.reshape(-1, 3).astype(np.float32)).cuda(), torch.from_numpy(off).cuda()
+
+
+def _cost(vm, call):
+    """Launches and allocations of a call."""
+    a = vm.launch_count(), vm.allocation_count()
+    call()
+    return vm.launch_count() - a[0], vm.allocation_count() - a[1]
+
+
+def _in_thread(work):
+    """Runs work in a thread of its own (the scratch is a thread's)."""
+    import threading
+    out = []
+
+    def body():
+        try:
+            out.append(work())
+        except BaseException as e:  # handed to the caller
+            out.append(e)
+
+    t = threading.Thread(target=body)
+    t.start()
+    t.join()
+    if isinstance(out[0], BaseException):
+        raise out[0]
+    return out[0]
+
+
+def test_alternating_shapes_come_to_rest():
+    from paper_2510_01592_gb300 import vm
+    prm, few, many, wide = vm.segment_params(seed=3), *(_clusters(16, 16000, 1), _clusters(2000, 50, 2)), _clusters(3, 64, 4)
+    wide_prm = vm.segment_params(n_hyp=1024, seed=3)
+    batches = [(few, prm), (many, prm), (wide, wide_prm)]
+
+    def work():
+        for (xyz, off), p in batches:
+            vm.fit_planes(xyz, off, p)
+        return [[_cost(vm, lambda: vm.fit_planes(xyz, off, p)) for (xyz, off), p in batches] for _ in range(3)]
+
+    alone = [_in_thread(lambda: (vm.fit_planes(*b, p), _cost(vm, lambda: vm.fit_planes(*b, p)))[1]) for b, p in batches]
+    assert all(a[1] == 0 for a in alone)
+    assert _in_thread(work) == [alone] * 3
