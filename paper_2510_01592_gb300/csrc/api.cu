@@ -218,7 +218,9 @@ static vm_status fit_out(FitContext& fc, uint32_t kcap, uint32_t hcap) {
 // kernels write the result into mapped host memory and check the batch's point
 // count against the scratch themselves, so a call waits for the device once;
 // a batch that does not fit (or the first of a thread) grows the scratch and
-// runs again.
+// runs again.  The result block starts with room for 48 hull vertices a cluster,
+// for large batches a million altogether; a batch with more is packed again into
+// a block of its size (its hulls are still in the scratch).
 static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* off, const uint32_t* labels,
                               uint32_t k, const vm_segment_params& p, const FitTuning& tune, cudaStream_t s,
                               vm_planes* out) {
@@ -231,33 +233,35 @@ static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* 
         VM_CUDA(cudaStreamSynchronize(s));
         npts = n;
     }
-    uint32_t hull = k * 48u + 4096u;
     StageHook* hk = fc.timer.hook();
     FitHeader h;
     for (int attempt = 0;; ++attempt) {
         VM_TRY(fit_prepare(fc, k, npts, (int)p.n_hyp, tune.tile, s));
-        VM_TRY(fit_out(fc, k, hull));
         FitBuffers& fb = fc.fb;
-        char* d = fc.host_dev;
         VM_CUDA(fit_open(off, k, (uint32_t)(fc.npts < 0xFFFFFFFFull ? fc.npts : 0xFFFFFFFFull), fb, s));
         VM_CUDA(launch_fit(pts, off, labels, fb.kdev, k, p, fb, tune, device_sms(), s, hk));
-        VM_STAGE_BEGIN(hk, kStPack, s);
-        VM_CUDA(launch_pack(fb, off, labels, fb.kdev, k, reinterpret_cast<vm_plane*>(d + out_planes_off()),
-                            reinterpret_cast<int32_t*>(d + out_xy_off(fc.out_kcap)),
-                            reinterpret_cast<float*>(d + out_xyz_off(fc.out_kcap, fc.out_hcap)), fc.out_hcap, s));
-        VM_CUDA(fit_close(fb, reinterpret_cast<FitHeader*>(d), s));
-        VM_STAGE_END(hk, kStPack, s);
-        VM_CUDA(cudaStreamSynchronize(s));
-        fc.timer.fold();
-        h = *static_cast<const FitHeader*>(fc.host);
-        const bool scratch = (h.err & kErrScratch) != 0;
-        if (!scratch && h.n_hull <= fc.out_hcap) break;
+        size_t hull = (size_t)k * 48 + 4096;
+        if (hull > (1u << 20)) hull = 1u << 20;
+        do {
+            VM_TRY(fit_out(fc, k, (uint32_t)(hull < 0xFFFFFFFFull ? hull : 0xFFFFFFFFull)));
+            char* d = fc.host_dev;
+            VM_STAGE_BEGIN(hk, kStPack, s);
+            VM_CUDA(launch_pack(fb, off, labels, fb.kdev, k, reinterpret_cast<vm_plane*>(d + out_planes_off()),
+                                reinterpret_cast<int32_t*>(d + out_xy_off(fc.out_kcap)),
+                                reinterpret_cast<float*>(d + out_xyz_off(fc.out_kcap, fc.out_hcap)), fc.out_hcap, s));
+            VM_CUDA(fit_close(fb, reinterpret_cast<FitHeader*>(d), s));
+            VM_STAGE_END(hk, kStPack, s);
+            VM_CUDA(cudaStreamSynchronize(s));
+            fc.timer.fold();
+            h = *static_cast<const FitHeader*>(fc.host);
+            hull = (size_t)h.n_hull + h.n_hull / 4;
+        } while (h.n_hull > fc.out_hcap);
+        if (!(h.err & kErrScratch)) break;
         if (attempt == 3) {
             set_error("fit scratch could not be sized for this batch");
             return VM_ERR_OUT_OF_MEMORY;
         }
-        if (scratch) npts = h.n_points;
-        else hull = h.n_hull + h.n_hull / 4;
+        npts = h.n_points;
     }
     const size_t b_planes = (size_t)k * sizeof(vm_plane);
     const size_t b_xy = (size_t)h.n_hull * 2 * sizeof(int32_t);

@@ -56,3 +56,41 @@ def test_alternating_shapes_come_to_rest():
     alone = [_in_thread(lambda: (vm.fit_planes(*b, p), _cost(vm, lambda: vm.fit_planes(*b, p)))[1]) for b, p in batches]
     assert all(a[1] == 0 for a in alone)
     assert _in_thread(work) == [alone] * 3
+
+
+def test_hulls_past_the_result_block_are_packed_again_only():
+    """The first call of a thread, with more hull vertices than its result block starts with (48 a cluster and 4096):
+    the fit runs once."""
+    import torch
+    from paper_2510_01592_gb300 import vm
+    k, n = 200, 20000
+    rng = np.random.default_rng(7)
+    r, a = np.sqrt(rng.random((k, n))), rng.random((k, n)) * 2 * np.pi
+    p = np.stack([r * np.cos(a), r * np.sin(a), rng.normal(0, 0.001, (k, n))], -1).reshape(-1, 3).astype(np.float32)
+    xyz = torch.from_numpy(p).cuda()
+    off = torch.arange(0, k * n + 1, n, dtype=torch.int32, device="cuda")
+    prm = vm.segment_params(n_hyp=32, seed=1)
+
+    def work():
+        first = _cost(vm, lambda: res.append(vm.fit_planes(xyz, off, prm)))
+        return first[0], _cost(vm, lambda: res.append(vm.fit_planes(xyz, off, prm)))
+
+    res = []
+    first, second = _in_thread(work)
+    assert len(res[0]["hull_xy"]) > 48 * k + 4096
+    assert second[1] == 0 and first <= second[0] + 2  # the pack and its header
+    want = vm.FitPlan(k, k * n, prm).run(xyz, off)
+    for key in ("planes", "hull_xy", "hull_xyz"):
+        assert res[0][key].tobytes() == res[1][key].tobytes() == want[key].tobytes(), key
+
+
+def test_many_small_clusters_with_over_a_million_hull_vertices():
+    from paper_2510_01592_gb300 import vm
+    k = 150_000
+    xyz, off = _clusters(k, 24, 5)
+    prm = vm.segment_params(n_hyp=8, seed=2)
+    got = _in_thread(lambda: vm.fit_planes(xyz, off, prm))
+    assert len(got["hull_xy"]) > 1 << 20
+    want = vm.FitPlan(k, k * 24, prm).run(xyz, off)
+    for key in ("planes", "hull_xy", "hull_xyz"):
+        assert got[key].tobytes() == want[key].tobytes(), key
