@@ -481,7 +481,7 @@ cudaError_t enqueue_front(vm_map* m, const vm_segment_params& p, StageHook* hk, 
     VM_STAGE_BEGIN(hk, kStOrder, s);
     if ((e = seg_order_bricks(m->brick_table, m->nb_total, m->occ, b, s, m->err, also_zero)) != cudaSuccess) return e;
     VM_STAGE_END(hk, kStOrder, s);
-    return seg_run(m->g, m->S, m->C, p, b, m->kcap, m->err, sms, s, hk);
+    return seg_run(m->g, m->S, m->C, p, b, m->kcap, m->many, m->err, sms, s, hk);
 }
 
 cudaError_t enqueue_segment(vm_map* m, const vm_segment_params& p, StageHook* hk) {
@@ -574,6 +574,7 @@ vm_status capture_segment(vm_map* m, const vm_segment_params& p) {
     uncount_launch(m->glaunches);  // counted when replayed, not when captured
     m->ggen = m->gen;
     m->gprm = p;
+    m->gmany = m->many;
     return VM_OK;
 }
 
@@ -596,7 +597,8 @@ vm_status launch_segment(vm_map* m, const vm_segment_params& p) {
     VM_TRY(plan_capacity(m, p, true));
     m->seg_rounds = p.planes_per_cluster > 1 ? p.planes_per_cluster : 1;
     StageHook* hk = m->fit.timer.hook();
-    if (m->use_graph && !hk && (!m->gexec || m->ggen != m->gen || memcmp(&m->gprm, &p, sizeof(p)) != 0)) {
+    if (m->use_graph && !hk && (!m->gexec || m->ggen != m->gen || m->gmany != m->many ||
+                                memcmp(&m->gprm, &p, sizeof(p)) != 0)) {
         if (capture_segment(m, p) != VM_OK) {  // e.g. a stream that cannot be captured: launch eagerly
             cudaGetLastError();
             m->use_graph = false;
@@ -637,6 +639,7 @@ static vm_status capture_front(vm_map* m, const vm_segment_params& p) {
     }
     m->fgen = m->gen;
     m->fprm = p;
+    m->fmany = m->many;
     return VM_OK;
 }
 
@@ -649,7 +652,8 @@ vm_status launch_front(vm_map* m, const vm_segment_params& p) {
         m->brick_hint = c.n_bricks < m->capacity ? c.n_bricks : m->capacity;
     }
     VM_TRY(plan_capacity(m, p, false));
-    if (m->use_graph && (!m->fexec || m->fgen != m->gen || memcmp(&m->fprm, &p, sizeof(p)) != 0)) {
+    if (m->use_graph && (!m->fexec || m->fgen != m->gen || m->fmany != m->many ||
+                         memcmp(&m->fprm, &p, sizeof(p)) != 0)) {
         if (capture_front(m, p) != VM_OK) {
             cudaGetLastError();
             m->use_graph = false;
@@ -673,6 +677,8 @@ bool take_hints(vm_map* m) {
     m->k_hint = hdr->k_need > hdr->k ? hdr->k_need : hdr->k;
     m->hull_hint = hdr->n_hull;
     m->rec_hint = hdr->n_planes;
+    // more than eight components a brick, until they are fewer than four: the graph is captured anew where it changes
+    m->many = hdr->n_comp > (uint64_t)hdr->n_sorted * (m->many ? 4 : 8);
     return (hdr->err & kErrScratch) || hdr->n_hull > m->out_hcap || hdr->n_planes > m->out_kcap;
 }
 

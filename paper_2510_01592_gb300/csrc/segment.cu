@@ -935,13 +935,22 @@ __device__ __forceinline__ uint32_t uf_root(const uint32_t* P, uint32_t x, uint3
     return x;
 }
 
+// Words of the scratch that k_cluster_number and k_cluster_place share, zero when
+// they start (k_comp_size): a flag a CTA of the placement, the tickets, and whose
+// turn a tile of the placement is; then a 64-bit word a CTA of the numbering.
+constexpr uint32_t kPlaceCtas = 128;  // CTAs of either at most
+constexpr uint32_t kPlaceTicket = kPlaceCtas, kPlaceTurn = kPlaceCtas + 1, kNumberTicket = kPlaceCtas + 2;
+constexpr uint32_t kNumberWords = kPlaceCtas + 4, kPlaceHead = kNumberWords + 2 * kPlaceCtas;
+
 // Every component's root, and the vertices of each whole component at its
 // root (lanes with equal roots add up first).
 __global__ void __launch_bounds__(kT) k_comp_size(const SegCounters* __restrict__ ctr, uint32_t* parent,
                                                   const uint32_t* __restrict__ csize, uint32_t* __restrict__ total,
-                                                  uint32_t* err) {
+                                                  uint32_t* __restrict__ scratch, uint32_t* err) {
     pdl_gate();
     const uint32_t K = ctr->n_comp;
+    if (blockIdx.x == 0)
+        for (uint32_t q = threadIdx.x; q < kPlaceHead; q += kT) scratch[q] = 0;
     for (uint32_t base = (blockIdx.x * kT + threadIdx.x) & ~31u; base < K; base += gridDim.x * kT) {
         const uint32_t c = base + (threadIdx.x & 31);
         uint32_t root = kNone, n = 0;
@@ -956,60 +965,92 @@ __global__ void __launch_bounds__(kT) k_comp_size(const SegCounters* __restrict_
     }
 }
 
-constexpr uint32_t kPlaceCtas = 128;  // CTAs of k_cluster_place
-
 // Kept components (at least min_cluster vertices) numbered in the order of
-// their roots (= label order) with their sizes and labels, and the cluster
-// offsets, in one CTA.  Clusters beyond the scratch flag a re-run, and the
-// count is clamped for the kernels after this one.
+// their roots (= label order) with their sizes, labels and offsets.  One CTA
+// takes up to kNumberRun components; more are cut into stretches, a CTA each,
+// which adds up its own, publishes the two sums and waits for the CTAs before it
+// (a ticket numbers them as they start, so each of those is running; the wait is
+// bounded).  Clusters beyond the scratch flag a re-run, and the count is clamped
+// for the kernels after this one.  next: the offsets again, which the placement
+// moves on where it goes tile by tile.  (A floor has a component or two a brick
+// and one CTA is done with its few thousand in 5 us; a 1 x 1 x 1 m map with every
+// second cell at 0.01 m occupied has hundreds a brick: 191 us in one CTA, 12 so.)
+constexpr uint32_t kNumberRun = kOneT * kRun;
 __global__ void __launch_bounds__(kOneT, 1) k_cluster_number(SegCounters* __restrict__ ctr, uint32_t min_cluster,
                                                           uint32_t kcap, const uint32_t* __restrict__ total,
                                                           const uint32_t* __restrict__ croot,
                                                           uint32_t* __restrict__ ccl, uint32_t* __restrict__ cl_size,
                                                           uint32_t* __restrict__ cl_label,
-                                                          uint32_t* __restrict__ cl_off,
-                                                          uint32_t* __restrict__ flags) {
+                                                          uint32_t* __restrict__ cl_off, uint32_t* scratch,
+                                                          uint32_t* err) {
     pdl_gate();
     __shared__ uint32_t ws[33];
+    __shared__ uint32_t s_ticket;
     const int lane = threadIdx.x & 31;
-    const uint32_t K = ctr->n_comp;
-    if (threadIdx.x <= kPlaceCtas) flags[threadIdx.x] = 0;  // k_cluster_place's, and its ticket
-    uint32_t k = 0;
-    for (uint32_t b0 = 0; b0 < K; b0 += kOneT * kRun) {
-        const uint32_t c0 = b0 + (threadIdx.x >> 5) * (32 * kRun) + lane;
-        uint32_t sz[kRun], kept[kRun], sum = 0;
+    const uint32_t w = threadIdx.x >> 5, K = ctr->n_comp;
+    const uint32_t stretch = max(kNumberRun, ((K + gridDim.x - 1) / gridDim.x + 1023u) & ~1023u);
+    const uint32_t G = max(1u, (K + stretch - 1) / stretch);
+    if (blockIdx.x >= G) return;
+    uint32_t g = 0, k = 0, off = 0;  // this CTA, the clusters and the vertices before it
+    uint32_t tot, tot2;
+    if (G > 1) {
+        volatile unsigned long long* words = reinterpret_cast<volatile unsigned long long*>(scratch + kNumberWords);
+        if (threadIdx.x == 0) s_ticket = atomicAdd(scratch + kNumberTicket, 1u);
+        __syncthreads();
+        g = s_ticket;
+        uint32_t mk = 0, mv = 0;
+        const uint32_t end = min(K, (g + 1) * stretch);
+#pragma unroll 8
+        for (uint32_t c = g * stretch + threadIdx.x; c < end; c += kOneT) {
+            const uint32_t n = total[c];  // 0 but at roots
+            mk += n >= min_cluster;
+            mv += n >= min_cluster ? n : 0u;
+        }
+        cta_warps_excl(__reduce_add_sync(0xffffffffu, mk), ws, &tot);
+        cta_warps_excl(__reduce_add_sync(0xffffffffu, mv), ws, &tot2);
+        // one word: the sums and that they are there
+        if (threadIdx.x == 0) words[g] = 1ull << 63 | (unsigned long long)tot << 32 | tot2;
+        unsigned long long before = 0;
+        if (threadIdx.x < g) {
+            int it = 0;
+            while (!((before = words[threadIdx.x]) >> 63) && it < kLoopCap) ++it;
+            if (it == kLoopCap) atomicOr(err, kErrTimeout);
+        }
+        cta_warps_excl(__reduce_add_sync(0xffffffffu, (uint32_t)(before >> 32) & 0x7fffffffu), ws, &k);
+        cta_warps_excl(__reduce_add_sync(0xffffffffu, (uint32_t)before), ws, &off);
+    }
+    uint32_t* next = scratch + kPlaceHead;
+    const uint32_t first = g * stretch, end = min(K, first + stretch);
+    for (uint32_t b0 = first; b0 < end; b0 += kNumberRun) {
+        const uint32_t c0 = b0 + w * (32 * kRun) + lane;
+        uint32_t sz[kRun], kept[kRun], inc[kRun], nk = 0, nv = 0;
 #pragma unroll
-        for (int i = 0; i < kRun; ++i) sz[i] = c0 + i * 32 < K ? total[c0 + i * 32] : 0u;  // 0 but at roots
+        for (int i = 0; i < kRun; ++i) sz[i] = c0 + i * 32 < end ? total[c0 + i * 32] : 0u;
 #pragma unroll
         for (int i = 0; i < kRun; ++i) {
             if (sz[i] < min_cluster) sz[i] = 0;
             kept[i] = __ballot_sync(0xffffffffu, sz[i] != 0);
-            sum += __popc(kept[i]);
+            nk += __popc(kept[i]);
+            inc[i] = nv + warp_incl(sz[i]);
+            nv = __shfl_sync(0xffffffffu, inc[i], 31);
         }
-        uint32_t tot;
-        uint32_t at = k + cta_warps_excl(sum, ws, &tot);
+        uint32_t at = k + cta_warps_excl(nk, ws, &tot);
+        const uint32_t av = off + cta_warps_excl(nv, ws, &tot2);
 #pragma unroll
         for (int i = 0; i < kRun; ++i) {
             const uint32_t c = c0 + i * 32, me = at + __popc(kept[i] & ((1u << lane) - 1u));
-            if (c < K) ccl[c] = sz[i] ? me : kNone;  // of roots; the others follow in k_cluster_place
+            if (c < end) ccl[c] = sz[i] ? me : kNone;  // of roots; the others follow in k_cluster_place
             if (sz[i]) {
                 cl_size[me] = sz[i];
                 cl_label[me] = croot[c];
+                cl_off[me] = next[me] = av + inc[i] - sz[i];
             }
             at += __popc(kept[i]);
         }
         k += tot;
+        off += tot2;
     }
-    __syncthreads();  // cl_size, by this CTA
-    uint32_t off = 0;
-    for (uint32_t b0 = 0; b0 < k; b0 += kOneT) {
-        const uint32_t c = b0 + threadIdx.x;
-        uint32_t tot;
-        const uint32_t at = off + cta_excl(c < k ? cl_size[c] : 0u, ws, &tot);
-        if (c < k) cl_off[c] = at;
-        off += tot;
-    }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && g == G - 1) {
         cl_off[k] = off;
         ctr->n_kept = off;
         ctr->tot = off;
@@ -1021,18 +1062,170 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_number(SegCounters* __rest
 
 // Where each in-brick component's points start in the cluster lists: its
 // cluster's offset plus the vertices of the cluster's components before it.
-// The components are cut into stretches, a CTA each, and a CTA's into 32, a
-// warp each: a warp adds up its components' vertices per cluster, the sums are
+// The components are cut into stretches, a CTA each, and a CTA's into at most 32,
+// a warp each: a warp adds up its components' vertices per cluster, the sums are
 // scanned over the CTA's warps, each CTA publishes its sums per cluster and
 // waits for the CTAs before it (a ticket numbers them as they start, so each
-// of those is running; the wait is bounded), and each warp walks its components again, 32 at a time, one scan
-// per cluster among them.  scratch: a flag per CTA and the ticket (zero at
-// launch), then the CTAs' sums.  Where the warps' counts do not fit shared memory or the sums
-// the scratch, one CTA takes everything, its counts in scratch.
-constexpr uint32_t kPlaceWords = 49152;  // 192 KB
+// of those is running; the wait is bounded), and each warp walks its components
+// again, 32 at a time, one scan per cluster among them.  scratch: kPlaceHead words,
+// then the CTAs' sums.  The counts of 32 warps fit shared memory up to kPlaceWords /
+// 32 clusters; with more, fewer warps count.  Where one warp's do not fit, or the
+// sums the scratch, the CTAs take tiles of kPlaceTile components instead
+// (place_tiles).  With all of it in one CTA from 1,536 clusters on, 4 x 4 x 1 m of
+// noise at 0.01 m took 1.75 ms for 12 thousand clusters (0.28 with one warp a CTA
+// counting) and 36.7 ms for 616 thousand (0.46 tile by tile) with the numbering and
+// the lists.
+constexpr uint32_t kPlaceWords = 24576;  // 96 KB: another stream's kernels fit the SM beside it
+constexpr uint32_t kPlaceTile = 8192;    // its keys and counts take them all
+constexpr uint32_t kTileBits = 13;
+static_assert(kPlaceTile == 1u << kTileBits && kPlaceTile * 3 <= kPlaceWords, "a tile's keys and counts fit");
+
+// The placement tile by tile, however many clusters there are.  A component that is
+// its whole cluster starts at the cluster's offset.  A tile's others are sorted by
+// (cluster, component) and a scan gives each one the vertices before it in its
+// cluster and tile.  A cluster that lies in one tile starts at its offset; of the
+// others the tiles, in turn, take the place so far (next) and move it on by their
+// own vertices.  A tile's turn comes when the one before it, which another CTA has
+// taken already, has had its own (the wait is bounded); only that step is serial.
+__device__ __noinline__ void place_tiles(uint32_t K, const uint32_t* __restrict__ parent,
+                                         const uint32_t* __restrict__ csize, uint32_t* ccl,
+                                         const uint32_t* __restrict__ cl_size, const uint32_t* __restrict__ cl_off,
+                                         uint32_t* __restrict__ place, uint32_t* scratch, uint32_t* sm, uint32_t* err) {
+    constexpr int kEach = kPlaceTile / kOneT;
+    __shared__ uint32_t ws[33];
+    __shared__ uint32_t s_tile, s_m;
+    unsigned long long* key = reinterpret_cast<unsigned long long*>(sm);  // cluster << kTileBits | component of the tile
+    uint32_t* cnt = sm + 2 * kPlaceTile;                                  // vertices, then places
+    uint32_t* next = scratch + kPlaceHead;
+    const uint32_t tid = threadIdx.x, tiles = (K + kPlaceTile - 1) / kPlaceTile;
+    const uint32_t lt = (1u << (tid & 31)) - 1u;
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) {
+            s_tile = atomicAdd(scratch + kPlaceTicket, 1u);
+            s_m = 0;
+        }
+        __syncthreads();
+        const uint32_t tile = s_tile, base = tile * kPlaceTile;
+        if (tile >= tiles) break;
+        uint32_t cl[kEach], n[kEach], all[kEach];
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+            const uint32_t c = base + i * kOneT + tid;
+            cl[i] = c < K ? parent[c] : kNone;
+            n[i] = c < K ? csize[c] : 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < kEach; ++i)  // a root's entry is read and rewritten with the same value
+            if (cl[i] != kNone) ccl[base + i * kOneT + tid] = cl[i] = __ldcg(ccl + cl[i]);
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) all[i] = cl[i] != kNone ? cl_size[cl[i]] : 0u;
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+            const uint32_t q = i * kOneT + tid;
+            const bool part = n[i] < all[i];
+            if (cl[i] != kNone && !part) place[base + q] = cl_off[cl[i]];
+            const uint32_t b = __ballot_sync(0xffffffffu, part);
+            uint32_t at = 0;
+            if (!(tid & 31) && b) at = atomicAdd(&s_m, (uint32_t)__popc(b));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & lt);
+            if (part) {
+                key[at] = (unsigned long long)cl[i] << kTileBits | q;
+                cnt[q] = n[i];
+            }
+        }
+        __syncthreads();
+        const uint32_t m = s_m;
+        uint32_t m2 = 1;
+        while (m2 < m) m2 <<= 1;
+        for (uint32_t q = m + tid; q < m2; q += kOneT) key[q] = ~0ull;
+        __syncthreads();
+        for (uint32_t size = 2; size <= m2; size <<= 1)
+            for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+                for (uint32_t p = tid; p < m2 / 2; p += kOneT) {
+                    const uint32_t i = 2 * p - (p & (stride - 1)), j = i + stride;
+                    const unsigned long long a = key[i], b = key[j];
+                    if ((a > b) == !(i & size)) {
+                        key[i] = b;
+                        key[j] = a;
+                    }
+                }
+                __syncthreads();
+            }
+        // a thread takes kEach places of the sorted order: the vertices before each in its cluster and tile
+        uint32_t rel[kEach], head[kEach], sum = 0, tot, lasts = 0;  // lasts: those that a later tile's follow
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+            const uint32_t q = tid * kEach + i;
+            n[i] = q < m ? cnt[key[q] & (kPlaceTile - 1)] : 0u;
+            sum += n[i];
+        }
+        uint32_t at = cta_excl(sum, ws, &tot);  // its barriers come after every read of the counts
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+            cnt[tid * kEach + i] = rel[i] = at;
+            at += n[i];
+        }
+        __syncthreads();
+        uint32_t whole = 0;  // the last ones of clusters that lie in this tile
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+            const uint32_t q = tid * kEach + i;
+            head[i] = 0;
+            if (q >= m) continue;
+            const unsigned long long c = key[q] >> kTileBits;
+            if (i && c == key[q - 1] >> kTileBits) {
+                head[i] = head[i - 1];
+            } else {  // the first place of the cluster
+                uint32_t lo = 0, hi = q;
+                while (lo < hi) {
+                    const uint32_t mid = (lo + hi) >> 1;
+                    if (key[mid] >> kTileBits < c) lo = mid + 1;
+                    else hi = mid;
+                }
+                head[i] = lo;
+            }
+            rel[i] -= cnt[head[i]];
+            if (q + 1 == m || key[q + 1] >> kTileBits != c) {
+                if (rel[i] + n[i] == cl_size[c]) whole |= 1u << i;
+                else lasts |= 1u << i;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kEach; ++i)
+            if ((whole >> i) & 1u) cnt[head[i]] = cl_off[key[tid * kEach + i] >> kTileBits];
+        if (tid == 0 && tile) {
+            volatile uint32_t* turn = scratch + kPlaceTurn;
+            int it = 0;
+            while (*turn != tile && it < kLoopCap) ++it;
+            if (it == kLoopCap) atomicOr(err, kErrTimeout);
+            __threadfence();
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kEach; ++i)  // all at once; atomic only for the one round trip
+            if ((lasts >> i) & 1u) n[i] = atomicAdd(next + (key[tid * kEach + i] >> kTileBits), rel[i] + n[i]);
+#pragma unroll
+        for (int i = 0; i < kEach; ++i)
+            if ((lasts >> i) & 1u) cnt[head[i]] = n[i];
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();
+            *(volatile uint32_t*)(scratch + kPlaceTurn) = tile + 1;
+        }
+#pragma unroll
+        for (int i = 0; i < kEach; ++i) {
+            const uint32_t q = tid * kEach + i;
+            if (q < m) place[base + ((uint32_t)key[q] & (kPlaceTile - 1))] = cnt[head[i]] + rel[i];
+        }
+    }
+}
+
 __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* __restrict__ ctr,
                                                          const uint32_t* __restrict__ parent,
                                                          const uint32_t* __restrict__ csize, uint32_t* ccl,
+                                                         const uint32_t* __restrict__ cl_size,
                                                          const uint32_t* __restrict__ cl_off,
                                                          uint32_t* __restrict__ place, uint32_t* scratch,
                                                          uint32_t scratch_words, uint32_t* err) {
@@ -1041,20 +1234,19 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* _
     const uint32_t K = ctr->n_comp, k = ctr->k_need;
     const int lane = threadIdx.x & 31;
     const uint32_t w = threadIdx.x >> 5;
-    uint32_t stretch = max(1024u, ((K + gridDim.x - 1) / gridDim.x + 1023u) & ~1023u);
-    uint32_t G = (K + stretch - 1) / stretch;
-    volatile uint32_t* flags = scratch;
-    uint32_t* sums = scratch + kPlaceCtas + 1;
-    const bool many = (size_t)k * 32 <= kPlaceWords && (size_t)G * k + kPlaceCtas + 1 <= scratch_words;
-    if (!many) {
-        stretch = (K + 1023u) & ~1023u;
-        G = 1;
+    const uint32_t stretch = max(1024u, ((K + gridDim.x - 1) / gridDim.x + 1023u) & ~1023u);
+    const uint32_t G = (K + stretch - 1) / stretch;
+    if (blockIdx.x >= G) return;
+    if (k > kPlaceWords || (size_t)G * k + kPlaceHead > scratch_words) {
+        place_tiles(K, parent, csize, ccl, cl_size, cl_off, place, scratch, sm, err);
+        return;
     }
+    volatile uint32_t* flags = scratch;
+    uint32_t* sums = scratch + kPlaceHead;
     __shared__ uint32_t s_ticket;
-    if (threadIdx.x == 0) s_ticket = atomicAdd(scratch + kPlaceCtas, 1u);
+    if (threadIdx.x == 0) s_ticket = atomicAdd(scratch + kPlaceTicket, 1u);
     __syncthreads();
     const uint32_t g = s_ticket;
-    if (g >= G) return;
     const uint32_t first = g * stretch, end = min(K, first + stretch);
     constexpr int kIt = 8;
     // each component's cluster (a root's entry is read and rewritten with the same value)
@@ -1069,13 +1261,12 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* _
             if (root[i] != kNone) ccl[c0 + i * kOneT] = cl[i];
     }
     if (k == 0) return;
-    uint32_t* cnt = many ? sm : sums;
-    const uint32_t W = many ? 32u : min(32u, (scratch_words - kPlaceCtas - 1) / k);  // warps with counts of their own
-    for (uint32_t q = threadIdx.x; q < W * k; q += kOneT) cnt[q] = 0;
+    const uint32_t W = min(32u, kPlaceWords / k);  // warps with counts of their own
+    for (uint32_t q = threadIdx.x; q < W * k; q += kOneT) sm[q] = 0;
     __syncthreads();
     const uint32_t len = ((end - first + W - 1) / W + 31) & ~31u;
     const uint32_t lo = min(end, first + w * len), hi = w < W ? min(end, lo + len) : lo;
-    uint32_t* mine = cnt + (size_t)(w < W ? w : 0) * k;
+    uint32_t* mine = sm + (w < W ? w : 0) * k;
     for (uint32_t c0 = lo; c0 < hi; c0 += 32 * kIt) {  // kIt steps' loads go out together
         uint32_t cl[kIt], n[kIt];
 #pragma unroll
@@ -1095,10 +1286,10 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* _
     }
     __syncthreads();
     for (uint32_t cl = w; cl < k; cl += kOneT / 32) {  // a warp a cluster, a lane a warp's counts
-        uint32_t* at = cnt + (size_t)lane * k + cl;
+        uint32_t* at = sm + lane * k + cl;
         const uint32_t t = lane < (int)W ? *at : 0u, inc = warp_incl(t);
         if (lane < (int)W) *at = inc - t;
-        if (many && lane == 31) sums[(size_t)g * k + cl] = inc;
+        if (lane == 31) sums[(size_t)g * k + cl] = inc;
     }
     if (G > 1) {
         __threadfence();
@@ -1115,7 +1306,7 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* _
     for (uint32_t cl = threadIdx.x; cl < k; cl += kOneT) {  // the cluster's points before this CTA's
         uint32_t b = cl_off[cl];
         for (uint32_t q = 0; q < g; ++q) b += __ldcg(sums + (size_t)q * k + cl);
-        for (uint32_t q = 0; q < W; ++q) cnt[(size_t)q * k + cl] += b;
+        for (uint32_t q = 0; q < W; ++q) sm[q * k + cl] += b;
     }
     __syncthreads();
     for (uint32_t c0 = lo; c0 < hi; c0 += 32 * kIt) {
@@ -1180,7 +1371,7 @@ __global__ void __launch_bounds__(kScatWarps * 32) k_cluster_scatter(const SegCo
         for (uint32_t j = lane; j < nc; j += 32) {
             uint32_t f = 0;
             const uint32_t c = cl[j];
-            while (cl[f] != c) ++f;  // at most j
+            while (c != kNone && cl[f] != c) ++f;  // at most j
             lead[j] = c != kNone ? (uint16_t)f : kNoComp;
         }
         __syncwarp();
@@ -1225,7 +1416,7 @@ cudaError_t seg_order_bricks(const int32_t* brick_table, uint32_t nb_total, cons
 }
 
 cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* C, const vm_segment_params& p,
-                    SegBuffers& b, uint32_t kcap, uint32_t* err, int sms, cudaStream_t s, StageHook* hk) {
+                    SegBuffers& b, uint32_t kcap, bool many, uint32_t* err, int sms, cudaStream_t s, StageHook* hk) {
     static std::once_flag once;
     std::call_once(once, [] {
         cudaFuncSetAttribute(k_comp_join, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kJoinWords * 4));
@@ -1236,6 +1427,7 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
     const uint32_t pair_cap = (uint32_t)b.nv;
     uint32_t* over = b.place;                                   // k_cluster_place writes it after the last join
     uint32_t* scratch = reinterpret_cast<uint32_t*>(b.pairs);   // free once the pairs are joined
+    const uint32_t scratch_words = (uint32_t)(2 * b.nv < 0xFFFFFFFFull ? 2 * b.nv : 0xFFFFFFFFull);
     const auto clampg = [&](uint32_t want, uint32_t mx) { return want < mx ? (want ? want : 1u) : mx; };
     // Several waves of short CTAs: with about one, some SMs got a CTA more than others for the whole pass (the per-voxel
     // passes of the 8 x 8 x 3 m map 248 us at 8 CTAs an SM, 219 at 24).  A CTA per two bricks covers their occupied
@@ -1263,20 +1455,22 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
     launch_k(k_ccl_cross, dim3(vgrid), dim3(kT), 0, s, b.ctr, b.brec, b.near, b.rows, b.vox, b.pos, b.nrm, b.lc,
              b.ncomp, b.cbase, b.lsize, b.lroot, b.csize, b.croot, b.total, b.parent, over, b.pairs, pair_cap,
              p.d_th2, p.cos_ccl, err);
-    // a CTA per thousand pairs, of which a brick has about six: each needs a whole SM's shared memory, and other streams'
-    // kernels wait for it
-    launch_k(k_comp_join, dim3(clampg(cap_b / 128, sms)), dim3(kOneT), kJoinWords * 4, s, b.ctr, pair_cap, b.pairs,
-             b.lsize, b.parent, over, err);
+    // A map of surfaces has one or two components and six pairs a brick: a CTA per thousand of them, as few as there can
+    // be work for, since each takes much of an SM's shared memory and other streams' kernels wait for it.  A map of noise
+    // (many) has up to hundreds a brick and takes the GPU: 1 x 1 x 1 m with every cell at 0.01 m occupied has its pairs
+    // joined in 24 us instead of 54 and its clusters formed in 93 us instead of 365.
+    launch_k(k_comp_join, dim3(clampg(many ? cap_b / 16 : cap_b / 128, sms)), dim3(kOneT), kJoinWords * 4, s, b.ctr,
+             pair_cap, b.pairs, b.lsize, b.parent, over, err);
     VM_STAGE_END(hk, kStCcl, s);
     VM_STAGE_BEGIN(hk, kStClusters, s);
-    launch_k(k_comp_size, dim3(clampg(cap_b / 64, sms * 2)), dim3(kT), 0, s, b.ctr, b.parent,
-             b.csize, b.total, err);
+    launch_k(k_comp_size, dim3(many ? clampg(cap_b / 4, sms * 8) : clampg(cap_b / 64, sms * 2)), dim3(kT), 0, s, b.ctr,
+             b.parent, b.csize, b.total, scratch, err);
     const uint32_t min_cl = p.min_cluster ? p.min_cluster : 1u;
-    launch_k(k_cluster_number, dim3(1), dim3(kOneT), 0, s, b.ctr, min_cl, kcap, b.total, b.croot, b.ccl, b.cl_size,
-             b.cl_label, b.cl_off, scratch);
-    // a CTA per thousand components, of which a brick has one or two, for the reason given at k_comp_join
-    launch_k(k_cluster_place, dim3(clampg(cap_b / 512 + 1, kPlaceCtas)), dim3(kOneT), kPlaceWords * 4, s, b.ctr,
-             b.parent, b.csize, b.ccl, b.cl_off, b.place, scratch, (uint32_t)(2 * b.nv), err);
+    launch_k(k_cluster_number, dim3(clampg(many ? cap_b / 16 : cap_b / 1024, kPlaceCtas)), dim3(kOneT), 0, s, b.ctr,
+             min_cl, kcap, b.total, b.croot, b.ccl, b.cl_size, b.cl_label, b.cl_off, scratch, err);
+    launch_k(k_cluster_place, dim3(clampg(many ? cap_b / 16 : cap_b / 512 + 1, kPlaceCtas)), dim3(kOneT),
+             kPlaceWords * 4, s, b.ctr, b.parent, b.csize, b.ccl, b.cl_size, b.cl_off, b.place, scratch, scratch_words,
+             err);
     launch_k(k_cluster_scatter, dim3(clampg((cap_b + kScatWarps - 1) / kScatWarps, sms * 8)), dim3(kScatWarps * 32), 0,
              s, b.ctr, cap_b, b.brec, b.ncomp, b.cbase, b.ccl, b.place, b.lc, b.vox, b.pos, b.pts, b.pt_vid);
     VM_STAGE_END(hk, kStClusters, s);
