@@ -1623,8 +1623,11 @@ __global__ void __launch_bounds__(kT) k_score_warp(const float* __restrict__ pts
 // ---------------------------------------------------------------- stage b, large fits
 // The reference plane of each cluster for k_score_slab: the hypothesis with the
 // most inliers among kRefPts points spread over the cluster (any plane serves;
-// a good one decides more tiles at once).  w is infinite when no hypothesis is
-// valid.  One CTA a cluster, a thread per hypothesis.
+// a good one decides more tiles at once).  Its normal frames the tiles' boxes and
+// so has to be a unit vector: a hypothesis whose samples are closer than 1e-9 m, or
+// farther than 1e9 m, apart has none, as the square of its cross product leaves the
+// range of normal floats.  w is infinite when no hypothesis will do.  One CTA a
+// cluster, a thread per hypothesis.
 constexpr int kRefPts = 64;
 __global__ void __launch_bounds__(kT) k_score_ref(const float* __restrict__ pts, const uint32_t* __restrict__ off,
                                                   const uint32_t* __restrict__ kp, int H,
@@ -1644,7 +1647,8 @@ __global__ void __launch_bounds__(kT) k_score_ref(const float* __restrict__ pts,
         unsigned long long best = 0;  // inliers + 1 << 32 | ~h
         for (int h = threadIdx.x; h < H; h += kT) {
             const float4 pl[1] = {hyp[(size_t)c * H + h]};
-            if (!(fabsf(pl[0].w) < __int_as_float(0x7f800000))) continue;
+            const float n2 = pl[0].x * pl[0].x + pl[0].y * pl[0].y + pl[0].z * pl[0].z;
+            if (!(fabsf(pl[0].w) < __int_as_float(0x7f800000)) || !(fabsf(n2 - 1.0f) < 9.5367431640625e-07f)) continue;
             uint32_t in[1] = {1u};
             for (uint32_t q = 0; q < m; ++q) count_point<1>(pl, sp[q], eps, in);
             const unsigned long long key = ((unsigned long long)in[0] << 32) | (uint32_t)~(uint32_t)h;
@@ -1861,10 +1865,7 @@ __global__ void __launch_bounds__(kT) k_score_slab(const float* __restrict__ pts
         ay -= along * r0.y;
         az -= along * r0.z;
         const float len2 = ax * ax + ay * ay + az * az;
-        // else the axis-aligned box alone: no direction, or a normal whose square left the range of normal floats
-        // (samples closer than 1e-9 m, or beyond 1e9 m, apart) and that is not a unit vector
-        const float n2 = r0.x * r0.x + r0.y * r0.y + r0.z * r0.z;
-        const bool framed = len2 > 1e-12f && len2 < 1e12f && fabsf(n2 - 1.0f) < 9.5367431640625e-07f;  // 2^-20
+        const bool framed = len2 > 1e-12f && len2 < 1e12f;  // else the axis-aligned box alone
         const float il = framed ? rsqrtf(len2) : 0.0f;
         ax *= il;
         ay *= il;
