@@ -137,7 +137,7 @@ vm_status fit_prepare(FitContext& fc, size_t kcap, size_t npts, int H, int tile,
     fit_layout(c, fb, k2, n2, c2, h2);
     VM_CUDA(cudaMemsetAsync(fb.scan_tmp, 0, scan_tmp_words(k2 + 1) * sizeof(uint32_t), s));  // scan state
     fb.kcap = k2;
-    fb.npts_cap = fb.npts_expect = n2;
+    fb.npts_cap = n2;
     fb.items_cap = c2;
     fc.fb = fb;
     fc.gen++;
@@ -227,17 +227,20 @@ static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* 
     memset(out, 0, sizeof(*out));
     if (k == 0) return VM_OK;
     size_t npts = fc.npts;
+    bool large = fc.large();
     if (!fc.mem.p || k > fc.kcap || (size_t)k * p.n_hyp > fc.slots) {  // the scratch grows in any case: learn the point count
         uint32_t n = 0;
         VM_CUDA(cudaMemcpyAsync(&n, off + k, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         VM_CUDA(cudaStreamSynchronize(s));
         npts = n;
+        large = n > kLargeFitPoints;
     }
     StageHook* hk = fc.timer.hook();
     FitHeader h;
     for (int attempt = 0;; ++attempt) {
         VM_TRY(fit_prepare(fc, k, npts, (int)p.n_hyp, tune.tile, s));
         FitBuffers& fb = fc.fb;
+        fb.large = large;
         VM_CUDA(fit_open(off, k, (uint32_t)(fc.npts < 0xFFFFFFFFull ? fc.npts : 0xFFFFFFFFull), fb, s));
         VM_CUDA(launch_fit(pts, off, labels, fb.kdev, k, p, fb, tune, device_sms(), s, hk));
         size_t hull = (size_t)k * 48 + 4096;
@@ -262,7 +265,9 @@ static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* 
             return VM_ERR_OUT_OF_MEMORY;
         }
         npts = h.n_points;
+        large = npts > kLargeFitPoints;
     }
+    fc.saw(h.n_points);
     const size_t b_planes = (size_t)k * sizeof(vm_plane);
     const size_t b_xy = (size_t)h.n_hull * 2 * sizeof(int32_t);
     const size_t b_xyz = (size_t)h.n_hull * 3 * sizeof(float);
@@ -490,7 +495,7 @@ cudaError_t enqueue_segment(vm_map* m, const vm_segment_params& p, StageHook* hk
     SegBuffers& b = m->seg;
     FitBuffers& fb = m->fit.fb;
     // the scratch has room for every slot of the bricks; about a fifth hold a clustered voxel
-    fb.npts_expect = m->last.n_kept ? (size_t)m->last.n_kept + m->last.n_kept / 4 : m->seg_nv / 4;
+    fb.large = (m->last.n_kept ? (size_t)m->last.n_kept + m->last.n_kept / 4 : m->seg_nv / 4) > kLargeFitPoints;
     cudaError_t e;
     if ((e = enqueue_front(m, p, hk, fb.err)) != cudaSuccess) return e;
     char* d = m->out_dev;

@@ -38,8 +38,6 @@ namespace {
 constexpr int kT = 256;
 constexpr int kHullCap = 2048;   // hull candidates sorted in shared memory
 constexpr int kSurvCap = 10240;  // first-filter survivors staged in shared memory: two CTAs of k_hull fit an SM
-constexpr size_t kFusedFitPoints = size_t(4) << 20;  // fits expected to have at most this many points: per-cluster
-                                                     // tails fused, every test of stage b made
 
 // ---------------------------------------------------------------- Philox
 __device__ __forceinline__ void philox4x64_10(const unsigned long long ctr[4], const unsigned long long key[2],
@@ -2122,7 +2120,7 @@ cudaError_t launch_fit(const float* pts, const uint32_t* off, const uint32_t* la
     // Large fits also score by k_score_slab, which makes two passes more and
     // far fewer tests (small ones are bound by their launches).  Results are
     // the same.
-    uint32_t* done = fb.npts_expect <= kFusedFitPoints ? fb.done : nullptr;
+    uint32_t* done = fb.large ? nullptr : fb.done;
     const bool slab = !done && !warp && p.eps < 1e6f;
     const size_t kh = (size_t)kcap * H;
     const unsigned hgrid = (unsigned)((kh + kT - 1) / kT < (size_t)sms * 16 ? (kh + kT - 1) / kT : (size_t)sms * 16);

@@ -77,13 +77,15 @@ struct vm_fit_plan {
     uint32_t out_kcap = 0, out_hcap = 0;
     uint32_t* k_host = nullptr;  // pinned: the cluster count the graph copies to the device
     uint64_t gen = 0;            // bumps when scratch, result block or tuning change
-    // captured fit
-    cudaGraphExec_t gexec = nullptr;
-    uint64_t ggen = ~0ull;
-    const float* gx = nullptr;
-    const uint32_t* goff = nullptr;
-    const uint32_t* glab = nullptr;
-    unsigned long long glaunches = 0;
+    // captured fits: with the kernels for small batches, and for large ones
+    struct Captured {
+        cudaGraphExec_t exec = nullptr;
+        uint64_t gen = ~0ull;
+        const float* x = nullptr;
+        const uint32_t* off = nullptr;
+        const uint32_t* lab = nullptr;
+        unsigned long long launches = 0;
+    } graph[2];
     // the launch in flight
     bool pending = false;
     const float* px = nullptr;
@@ -138,6 +140,7 @@ vm_status plan_size(vm_fit_plan* f, uint32_t k, uint32_t n, uint32_t hull) {
 cudaError_t enqueue_fit(vm_fit_plan* f, const float* x, const uint32_t* off, const uint32_t* lab, StageHook* hk) {
     cudaStream_t s = f->s;
     FitBuffers& fb = f->fc.fb;
+    fb.large = f->fc.large();
     const uint32_t kcap = (uint32_t)f->fc.kcap;
     cudaError_t e;
     if ((e = cudaMemcpyAsync(fb.kdev, f->k_host, sizeof(uint32_t), cudaMemcpyHostToDevice, s)) != cudaSuccess)
@@ -157,10 +160,11 @@ cudaError_t enqueue_fit(vm_fit_plan* f, const float* x, const uint32_t* off, con
     return cudaGetLastError();
 }
 
-vm_status capture_fit(vm_fit_plan* f, const float* x, const uint32_t* off, const uint32_t* lab) {
-    if (f->gexec) {
-        cudaGraphExecDestroy(f->gexec);
-        f->gexec = nullptr;
+vm_status capture_fit(vm_fit_plan* f, vm_fit_plan::Captured& g, const float* x, const uint32_t* off,
+                      const uint32_t* lab) {
+    if (g.exec) {
+        cudaGraphExecDestroy(g.exec);
+        g.exec = nullptr;
     }
     fit_init_attributes();
     cudaGraph_t graph = nullptr;
@@ -176,17 +180,17 @@ vm_status capture_fit(vm_fit_plan* f, const float* x, const uint32_t* off, const
         return cuda_status(e, "fit capture");
     }
     if (e2 != cudaSuccess) return cuda_status(e2, "cudaStreamEndCapture");
-    e = cudaGraphInstantiate(&f->gexec, graph, 0);
+    e = cudaGraphInstantiate(&g.exec, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) {
-        f->gexec = nullptr;
+        g.exec = nullptr;
         return cuda_status(e, "cudaGraphInstantiate");
     }
-    f->glaunches = n;
-    f->ggen = f->gen;
-    f->gx = x;
-    f->goff = off;
-    f->glab = lab;
+    g.launches = n;
+    g.gen = f->gen;
+    g.x = x;
+    g.off = off;
+    g.lab = lab;
     return VM_OK;
 }
 
@@ -195,10 +199,11 @@ vm_status plan_enqueue(vm_fit_plan* f, const float* x, const uint32_t* off, cons
     StageHook* hk = f->fc.timer.hook();
     const bool graph = !(f->flags & VM_FIT_EAGER) && !hk;
     if (graph) {
-        if (!f->gexec || f->ggen != f->gen || f->gx != x || f->goff != off || f->glab != lab)
-            VM_TRY(capture_fit(f, x, off, lab));
-        VM_CUDA(cudaGraphLaunch(f->gexec, f->s));
-        count_launch((int)f->glaunches);
+        vm_fit_plan::Captured& g = f->graph[f->fc.large()];
+        if (!g.exec || g.gen != f->gen || g.x != x || g.off != off || g.lab != lab)
+            VM_TRY(capture_fit(f, g, x, off, lab));
+        VM_CUDA(cudaGraphLaunch(g.exec, f->s));
+        count_launch((int)g.launches);
     } else {
         VM_CUDA(enqueue_fit(f, x, off, lab, hk));
     }
@@ -248,9 +253,11 @@ vm_status plan_wait(vm_fit_plan* f, vm_planes* out) {
             set_error("fit scratch could not be sized for this batch");
             return VM_ERR_OUT_OF_MEMORY;
         }
+        if (scratch) f->fc.saw(h->n_points);
         VM_TRY(plan_size(f, f->pk, scratch ? h->n_points : 0, hull ? h->n_hull : 0));
         VM_TRY(plan_enqueue(f, f->px, f->poff, f->plab, f->pk));
     }
+    f->fc.saw(h->n_points);
     if (out) {
         const uint32_t K = h->k, n_hull = h->n_hull;
         const size_t b_planes = (size_t)K * sizeof(vm_plane);
@@ -341,6 +348,7 @@ vm_status vm_fit_plan_create(uint32_t k_cap, uint32_t n_cap, const vm_segment_pa
         return cuda_status(e, "cudaMallocHost");
     }
     f->k_host = static_cast<uint32_t*>(kh);
+    f->fc.expect = n_cap;
     const vm_status st = plan_size(f, k_cap, n_cap, 0);
     if (st != VM_OK) {
         vm_fit_plan_destroy(f);
@@ -353,7 +361,8 @@ vm_status vm_fit_plan_create(uint32_t k_cap, uint32_t n_cap, const vm_segment_pa
 vm_status vm_fit_plan_destroy(vm_fit_plan* f) {
     if (!f) return VM_OK;
     if (f->s) cudaStreamSynchronize(f->s);
-    if (f->gexec) cudaGraphExecDestroy(f->gexec);
+    for (auto& g : f->graph)
+        if (g.exec) cudaGraphExecDestroy(g.exec);
     fit_release(f->fc);
     if (f->out_host) cudaFreeHost(f->out_host);
     if (f->k_host) cudaFreeHost(f->k_host);
@@ -479,6 +488,12 @@ vm_status vm_fit_plan_autotune(vm_fit_plan* f, const float* xyz, const uint32_t*
     // Size for the smallest tile first so that no candidate re-allocates.
     f->tune.tile = tiles_warp[0];
     st = plan_size(f, 0, 0, 0);
+    if (st == VM_OK) st = plan_launch(f, xyz, off, labels, k);
+    if (st == VM_OK) st = plan_wait(f, nullptr);
+    if (st == VM_OK) {  // the candidates take the kernels for this batch
+        f->fc.expect = static_cast<const FitHeader*>(f->out_host)->n_points;
+        f->fc.smaller = 0;
+    }
     for (size_t i = 0; st == VM_OK && i < cand.size(); ++i) {
         st = apply_tuning(f, cand[i]);
         if (st != VM_OK) break;

@@ -87,6 +87,17 @@ struct FitContext {
     DevBuf mem;
     FitBuffers fb{};
     size_t kcap = 0, npts = 0, items = 0, slots = 0;  // slots: hypotheses of all clusters
+    // Points the next batch is expected to have, and the smaller batches since the
+    // last large one.  Batches that alternate keep the kernels for large ones: those
+    // cost a small batch 30 us, and the others cost a large batch milliseconds.
+    size_t expect = 0;
+    uint32_t smaller = 0;
+    bool large() const { return expect > kLargeFitPoints; }
+    void saw(size_t n) {
+        if (n <= kLargeFitPoints && large() && ++smaller < 8) return;
+        expect = n;
+        smaller = 0;
+    }
     // result block of vm_fit_planes: mapped pinned host memory, laid out as a plan's
     void* host = nullptr;
     char* host_dev = nullptr;

@@ -191,9 +191,11 @@ struct BatchFit {
     BatchTable* htab[kMaxSlots] = {};
     BatchStatus* hstat[kMaxSlots] = {};
     BatchStatus* dstat[kMaxSlots] = {};
-    cudaGraphExec_t gexec[kMaxSlots] = {};
-    uint64_t ggen[kMaxSlots] = {};
-    unsigned long long glaunches[kMaxSlots] = {};
+    struct Captured {
+        cudaGraphExec_t exec;
+        uint64_t gen;
+        unsigned long long launches;
+    } graph[kMaxSlots][2] = {};  // with the kernels for small batches, and for large ones
     uint64_t gen = 1;
 };
 
@@ -308,11 +310,14 @@ cudaError_t enqueue_batch(Server* S, int slot) {
     return cudaGetLastError();
 }
 
-vm_status launch_batch(Server* S, int slot) {
+// expect: points the batch is expected to have (picks the kernels).
+vm_status launch_batch(Server* S, int slot, size_t expect) {
     BatchFit& b = S->bf;
-    if (!b.gexec[slot] || b.ggen[slot] != b.gen) {
-        if (b.gexec[slot]) cudaGraphExecDestroy(b.gexec[slot]);
-        b.gexec[slot] = nullptr;
+    b.fc.fb.large = expect > kLargeFitPoints;
+    BatchFit::Captured& g = b.graph[slot][b.fc.fb.large];
+    if (!g.exec || g.gen != b.gen) {
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+        g.exec = nullptr;
         fit_init_attributes();
         cudaGraph_t graph = nullptr;
         const unsigned long long l0 = launch_total();
@@ -320,23 +325,23 @@ vm_status launch_batch(Server* S, int slot) {
         VM_CUDA(cudaStreamBeginCapture(S->fit_stream, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = enqueue_batch(S, slot);
         cudaError_t e2 = cudaStreamEndCapture(S->fit_stream, &graph);
-        b.glaunches[slot] = launch_total() - l0;
-        uncount_launch(b.glaunches[slot]);
+        g.launches = launch_total() - l0;
+        uncount_launch(g.launches);
         if (e != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
             return cuda_status(e, "batched fit capture");
         }
         if (e2 != cudaSuccess) return cuda_status(e2, "cudaStreamEndCapture");
-        e = cudaGraphInstantiate(&b.gexec[slot], graph, 0);
+        e = cudaGraphInstantiate(&g.exec, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) {
-            b.gexec[slot] = nullptr;
+            g.exec = nullptr;
             return cuda_status(e, "cudaGraphInstantiate");
         }
-        b.ggen[slot] = b.gen;
+        g.gen = b.gen;
     }
-    VM_CUDA(cudaGraphLaunch(b.gexec[slot], S->fit_stream));
-    count_launch((int)b.glaunches[slot]);
+    VM_CUDA(cudaGraphLaunch(g.exec, S->fit_stream));
+    count_launch((int)g.launches);
     return VM_OK;
 }
 
@@ -426,7 +431,7 @@ void launch_step(Server* S, Server::Step& st) {
     if (!batched || st.reqs.empty()) return;
     tab->n_maps = n_maps;
     vm_status s = bf_size(S, k_hint, n_hint);
-    if (s == VM_OK) s = launch_batch(S, st.slot);
+    if (s == VM_OK) s = launch_batch(S, st.slot, n_hint);
     if (s == VM_OK) {
         st.done = get_event(S);
         if (!st.done || cudaEventRecord(st.done, S->fit_stream) != cudaSuccess)
@@ -470,7 +475,7 @@ void complete_step(Server* S, Server::Step& st) {
         BatchStatus* bs = S->bf.hstat[st.slot];  // written before st.done was recorded
         for (int attempt = 0; attempt < 3 && (bs->err & kErrScratch); ++attempt) {  // the arena was too small
             if (bf_size(S, bs->K_need, bs->N_need) != VM_OK) break;
-            if (launch_batch(S, st.slot) != VM_OK) break;
+            if (launch_batch(S, st.slot, bs->N_need) != VM_OK) break;
             cudaStreamSynchronize(S->fit_stream);
         }
     }
@@ -693,7 +698,8 @@ void release_server(Server* S) {
     S->free_events.clear();
     BatchFit& b = S->bf;
     for (int k = 0; k < kMaxSlots; ++k) {
-        if (b.gexec[k]) cudaGraphExecDestroy(b.gexec[k]);
+        for (auto& g : b.graph[k])
+            if (g.exec) cudaGraphExecDestroy(g.exec);
         if (b.htab[k]) cudaFreeHost(b.htab[k]);
         if (b.hstat[k]) cudaFreeHost(b.hstat[k]);
     }

@@ -407,6 +407,9 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
                     SegBuffers& b, uint32_t kcap, bool many, uint32_t* err, int sms, cudaStream_t s, StageHook* hk);
 
 // ---------------------------------------------------------------- fit.cu
+// A fit expected to have more points takes the kernels for large ones: the
+// per-cluster tails in kernels of their own, and tests of stage b bounded.
+constexpr size_t kLargeFitPoints = size_t(4) << 20;
 struct FitBuffers {
     float4* hyp;            // [kcap * H]
     uint8_t* hyp_valid;     // [kcap * H]
@@ -430,7 +433,7 @@ struct FitBuffers {
     uint32_t* kdev;         // cluster count when the caller supplies it
     uint32_t* done;         // [kcap][3] per-cluster completion counters (scoring, extraction, filter)
     size_t kcap, npts_cap, items_cap;  // items_cap: 256-point partial-sum chunks
-    size_t npts_expect;     // points a fit is likely to have (picks kernels; results do not depend on it)
+    bool large;             // kernels for more than kLargeFitPoints points (results do not depend on it)
 };
 
 struct FitTuning {

@@ -94,3 +94,55 @@ def test_many_small_clusters_with_over_a_million_hull_vertices():
     want = vm.FitPlan(k, k * 24, prm).run(xyz, off)
     for key in ("planes", "hull_xy", "hull_xyz"):
         assert got[key].tobytes() == want[key].tobytes(), key
+
+
+def _same(a, b):
+    return all(a[key].tobytes() == b[key].tobytes() for key in ("planes", "hull_xy", "hull_xyz"))
+
+
+def test_direct_fits_take_the_kernels_for_the_points_they_have():
+    """A large batch (over four million points) takes more kernels than a small one; small ones after it come back to
+    their own within eight calls, and where the two alternate the large ones keep theirs.  The outputs are the same."""
+    from paper_2510_01592_gb300 import vm
+    small, large, prm = _clusters(16, 5000, 1), _clusters(40, 120000, 2), vm.segment_params(n_hyp=32, seed=3)
+
+    def call(b, res=None):
+        c = _cost(vm, lambda: (res if res is not None else []).append(vm.fit_planes(*b, prm)))
+        return c[0]
+
+    def work():
+        res = []
+        call(small)
+        few = call(small, res)
+        call(large)
+        many = call(large, res)
+        assert many > few
+        after = [call(small, res) for _ in range(10)]
+        assert after[-1] == few and _same(res[0], res[2]) and _same(res[0], res[-1])
+        call(large)  # from here on in turn
+        for _ in range(4):
+            call(small)
+            assert call(large, res) == many
+        assert _same(res[1], res[-1])
+
+    _in_thread(work)
+
+
+def test_a_plan_takes_the_kernels_for_the_points_it_has():
+    """Likewise a plan that is sized for more: and once both kinds of batch have run, none is captured again."""
+    from paper_2510_01592_gb300 import vm
+    small, large, prm = _clusters(16, 5000, 1), _clusters(40, 120000, 2), vm.segment_params(n_hyp=32, seed=3)
+    plan, own = vm.FitPlan(40, 4_800_000, prm), vm.FitPlan(16, 80000, prm)
+    want = own.run(*small)
+    few = _cost(vm, lambda: own.run(*small))[0]
+    for _ in range(10):
+        assert _same(plan.run(*small), want)
+    assert _cost(vm, lambda: plan.run(*small))[0] == few
+    first = plan.run(*large)
+    many = _cost(vm, lambda: plan.run(*large))[0]
+    assert many > few
+    captures = vm.capture_count()
+    for _ in range(10):
+        assert _same(plan.run(*large), first)
+        assert _cost(vm, lambda: plan.run(*large))[0] == many
+    assert vm.capture_count() == captures
