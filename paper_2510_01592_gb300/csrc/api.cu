@@ -494,8 +494,7 @@ cudaError_t enqueue_segment(vm_map* m, const vm_segment_params& p, StageHook* hk
     const int sms = device_sms();
     SegBuffers& b = m->seg;
     FitBuffers& fb = m->fit.fb;
-    // the scratch has room for every slot of the bricks; about a fifth hold a clustered voxel
-    fb.large = (m->last.n_kept ? (size_t)m->last.n_kept + m->last.n_kept / 4 : m->seg_nv / 4) > kLargeFitPoints;
+    fb.large = m->large;
     cudaError_t e;
     if ((e = enqueue_front(m, p, hk, fb.err)) != cudaSuccess) return e;
     char* d = m->out_dev;
@@ -580,6 +579,7 @@ vm_status capture_segment(vm_map* m, const vm_segment_params& p) {
     m->ggen = m->gen;
     m->gprm = p;
     m->gmany = m->many;
+    m->glarge = m->large;
     return VM_OK;
 }
 
@@ -601,9 +601,14 @@ vm_status launch_segment(vm_map* m, const vm_segment_params& p) {
     }
     VM_TRY(plan_capacity(m, p, true));
     m->seg_rounds = p.planes_per_cluster > 1 ? p.planes_per_cluster : 1;
+    // The points that the fit is likely to have: the last ones with headroom; before any, a quarter of the scratch, which
+    // has room for every slot of the bricks.  The kernels for large fits stay until they are a quarter below the limit, as
+    // the graph is captured anew where the choice changes.
+    const size_t expect = m->fitted ? (size_t)m->last.n_kept + m->last.n_kept / 4 : m->seg_nv / 4;
+    m->large = expect > (m->large ? kLargeFitPoints / 4 * 3 : kLargeFitPoints);
     StageHook* hk = m->fit.timer.hook();
     if (m->use_graph && !hk && (!m->gexec || m->ggen != m->gen || m->gmany != m->many ||
-                                memcmp(&m->gprm, &p, sizeof(p)) != 0)) {
+                                m->glarge != m->large || memcmp(&m->gprm, &p, sizeof(p)) != 0)) {
         if (capture_segment(m, p) != VM_OK) {  // e.g. a stream that cannot be captured: launch eagerly
             cudaGetLastError();
             m->use_graph = false;
@@ -704,8 +709,7 @@ vm_status finish_segment(vm_map* m, const vm_segment_params& p, vm_planes* out) 
 vm_status read_result(vm_map* m, vm_planes* out) {
     const SegCounters* hdr = static_cast<const SegCounters*>(m->out_host);
     m->last = *hdr;
-
-    m->segmented = true;
+    m->segmented = m->fitted = true;
     const uint32_t K = hdr->n_planes, n_hull = hdr->n_hull;
     const size_t b_planes = (size_t)K * sizeof(vm_plane);
     out->planes = static_cast<vm_plane*>(malloc(b_planes ? b_planes : 1));

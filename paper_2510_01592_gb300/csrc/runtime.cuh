@@ -189,13 +189,15 @@ struct vm_map {
     uint32_t kcap = 0;            // kept-cluster capacity of the scratch
     uint32_t brick_hint = 0, k_hint = 0, hull_hint = 0;
     bool many = false;            // the map has many components a brick
+    bool large = false;           // its fit takes the kernels for large ones
+    bool fitted = false;          // last holds the counts of a segmentation
     uint64_t gen = 0;             // bumps whenever scratch or outputs move
     // captured segmentation (one CUDA graph, replayed per call)
     bool use_graph = true;
     cudaGraphExec_t gexec = nullptr;
     uint64_t ggen = ~0ull;
     vm_segment_params gprm{};
-    bool gmany = false;
+    bool gmany = false, glarge = false;
     unsigned long long glaunches = 0;
     uint32_t gnodes = 0, gedges = 0, gprog = 0;  // the captured graph's nodes, edges and programmatic edges
     // captured front half (brick order .. cluster points), for batched serving
