@@ -230,7 +230,8 @@ typedef struct vm_fit_plan vm_fit_plan; /* opaque, library-owned */
 
 typedef struct {
     uint32_t tile;           /* points per work item, a multiple of 256 in 256..16384 (the default
-                                schedule takes a smaller one for a fit too small to fill the GPU) */
+                                schedule, 2048 / 4 / 4 / 0, takes a smaller one for a fit too small
+                                to fill the GPU) */
     uint32_t hyp_per_thread; /* hypotheses each thread holds in registers: 1, 2, 4 or 8    */
     uint32_t ctas_per_sm;    /* persistent scoring CTAs per SM, 1..16                      */
     uint32_t schedule;       /* 0: a 256-thread CTA per work item; 1: a warp per work item  */
@@ -262,7 +263,7 @@ vm_status vm_fit_plan_set_tuning(vm_fit_plan* plan, const vm_fit_tuning* tuning)
 vm_status vm_fit_plan_get_tuning(const vm_fit_plan* plan, vm_fit_tuning* tuning);
 /* Autotuner (no counterpart in the paper): times the whole fit of this batch
  * (CUDA events around graph replays, reps timed runs after one warm-up run)
- * for each candidate tuning -- CTA-per-item tiles of 1024..8192 points and
+ * for each candidate tuning -- the default, CTA-per-item tiles of 1024..8192 points and
  * warp-per-item tiles of 256..1024 points, 2..8 hypotheses per thread,
  * persistent CTAs per SM up to the occupancy limit -- and keeps the fastest.
  * *best and *best_ms (either may be NULL) receive it; *n_tried the number of
@@ -341,7 +342,7 @@ vm_status vm_set_fit_tuning(vm_map* map, const vm_fit_tuning* tuning);
 vm_status vm_get_fit_tuning(vm_map* map, vm_fit_tuning* tuning);
 /* Autotuner for a map's segmentation (no counterpart in the paper): replays
  * the segmentation of the map as it stands (segmenting does not change the
- * map) under each candidate schedule -- CTA-per-item tiles of 512..4096
+ * map) under each candidate schedule -- the default, CTA-per-item tiles of 512..4096
  * points, warp-per-item tiles of 256..1024 points, 2..8 hypotheses per
  * thread, 2..8 scoring CTAs per SM within the occupancy limit -- timing reps
  * runs of each with CUDA events after one warm-up run, and keeps the fastest.

@@ -1033,8 +1033,7 @@ vm_status vm_set_fit_tuning(vm_map* m, const vm_fit_tuning* t) {
                   "ctas_per_sm 1..16, schedule 0/1)");
         return VM_ERR_INVALID_ARG;
     }
-    m->tune = t ? FitTuning{(int)t->tile, (int)t->hyp_per_thread, (int)t->ctas_per_sm, (int)t->schedule}
-                : default_tuning();
+    m->tune = t ? tuning_of(*t) : default_tuning();
     m->gen++;  // the captured graph holds the old schedule
     return VM_OK;
 }
@@ -1059,7 +1058,7 @@ vm_status vm_autotune_segment(vm_map* m, const vm_segment_params* params, uint32
     if (reps < 1) reps = 1;
     const vm_segment_params& p = *params;
     const int H = (int)p.n_hyp;
-    std::vector<FitTuning> cand;
+    std::vector<FitTuning> cand{default_tuning()};  // which chooses its tile: no other candidate is like it
     const int tiles_cta[] = {512, 1024, 2048, 4096};
     const int tiles_warp[] = {256, 512, 1024};
     const int rs[] = {2, 4, 8};
@@ -1074,9 +1073,8 @@ vm_status vm_autotune_segment(vm_map* m, const vm_segment_params* params, uint32
                 const int occ = score_max_ctas_per_sm(base, H);
                 for (int c : ctas) {
                     if (c > occ) break;
-                    FitTuning t = base;
-                    t.ctas_per_sm = c;
-                    cand.push_back(t);
+                    const FitTuning t = tuning_of({(uint32_t)base.tile, (uint32_t)r, (uint32_t)c, (uint32_t)sched});
+                    if (!t.adapt) cand.push_back(t);
                 }
             }
     }

@@ -2015,6 +2015,14 @@ __global__ void k_set_u32(uint32_t* __restrict__ p, uint32_t v) { pdl_gate(); *p
 
 FitTuning default_tuning() { return FitTuning{2048, 4, 4, 0, 1}; }
 
+FitTuning tuning_of(const vm_fit_tuning& t) {
+    FitTuning f{(int)t.tile, (int)t.hyp_per_thread, (int)t.ctas_per_sm, (int)t.schedule, 0};
+    const FitTuning d = default_tuning();
+    f.adapt = f.tile == d.tile && f.hyp_per_thread == d.hyp_per_thread && f.ctas_per_sm == d.ctas_per_sm &&
+              f.schedule == d.schedule;
+    return f;
+}
+
 // The scoring variant launch_fit picks for t and H: hypotheses per thread
 // and whether the warp schedule applies.
 static void score_variant(const FitTuning& t, int H, int& R, bool& warp) {

@@ -426,7 +426,7 @@ vm_status vm_fit_plan_set_tuning(vm_fit_plan* f, const vm_fit_tuning* t) {
         set_error("a launch is in flight on this plan");
         return VM_ERR_INVALID_ARG;
     }
-    return apply_tuning(f, FitTuning{(int)t->tile, (int)t->hyp_per_thread, (int)t->ctas_per_sm, (int)t->schedule});
+    return apply_tuning(f, tuning_of(*t));
 }
 
 vm_status vm_fit_plan_get_tuning(const vm_fit_plan* f, vm_fit_tuning* t) {
@@ -453,7 +453,7 @@ vm_status vm_fit_plan_autotune(vm_fit_plan* f, const float* xyz, const uint32_t*
     }
     if (reps < 1) reps = 1;
     const int H = (int)f->prm.n_hyp;
-    std::vector<FitTuning> cand;
+    std::vector<FitTuning> cand{default_tuning()};  // which chooses its tile: no other candidate is like it
     const int tiles_cta[] = {1024, 2048, 4096, 8192};
     const int tiles_warp[] = {256, 512, 768, 1024};
     const int rs[] = {2, 4, 8};
@@ -467,9 +467,8 @@ vm_status vm_fit_plan_autotune(vm_fit_plan* f, const float* xyz, const uint32_t*
                 const int occ = score_max_ctas_per_sm(base, H);
                 for (int c : ctas) {
                     if (c > occ) break;
-                    FitTuning t = base;
-                    t.ctas_per_sm = c;
-                    cand.push_back(t);
+                    const FitTuning t = tuning_of({(uint32_t)base.tile, (uint32_t)r, (uint32_t)c, (uint32_t)sched});
+                    if (!t.adapt) cand.push_back(t);
                 }
             }
         }

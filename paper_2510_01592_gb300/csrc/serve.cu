@@ -751,8 +751,7 @@ vm_status vm_server_create(const vm_server_params* params, vm_server** out) {
     S->t0 = std::chrono::steady_clock::now();
     S->captures0 = capture_total();
     S->allocs0 = alloc_total();
-    S->bf.tune = t.tile ? FitTuning{(int)t.tile, (int)t.hyp_per_thread, (int)t.ctas_per_sm, (int)t.schedule}
-                        : default_tuning();
+    S->bf.tune = t.tile ? tuning_of(t) : default_tuning();
     vm_status st = VM_OK;
     size_t free_b = 0, total_b = 0;
     cudaError_t e = cudaMemGetInfo(&free_b, &total_b);

@@ -444,6 +444,9 @@ struct FitTuning {
     int adapt;              // 1: a small fit may take a smaller tile (the default schedule)
 };
 FitTuning default_tuning();
+// A caller's schedule; the default's values mean the default, which also chooses
+// its tile, so that a schedule that was read can be set again.
+FitTuning tuning_of(const vm_fit_tuning& t);
 // Resident scoring CTAs per SM for tuning t and H hypotheses (0 on error).
 int score_max_ctas_per_sm(const FitTuning& t, int H);
 size_t fit_hull_smem();
