@@ -831,6 +831,9 @@ vm_status vm_create(const vm_map_params* params, void* cuda_stream, vm_map** out
     m->scroll_tmp = c.take<uint32_t>(scroll_tmp_words(m->capacity));
     m->po_dev = c.take<float>(4);
     g.po = m->po_dev;
+    // Diagnostic: a shorter list of joined pairs.  A map has six a brick and the list room for hundreds, so that without
+    // it nothing short of a made-up map reaches the forest for the pairs beyond.
+    if (const char* v = getenv("VOXMPS_PAIR_CAP")) m->seg.pair_cap = (uint32_t)strtoul(v, nullptr, 10);
     // brick-level segmentation arrays
     Carver bd{nullptr};
     brick_layout(bd, m->seg, m->nb_total, m->capacity);

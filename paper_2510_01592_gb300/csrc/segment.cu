@@ -1424,7 +1424,7 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
     });
     const uint32_t cap_b = (uint32_t)(b.nv / kBrickVox);
     const size_t stride = b.nv;
-    const uint32_t pair_cap = (uint32_t)b.nv;
+    const uint32_t pair_cap = b.nv < b.pair_cap ? (uint32_t)b.nv : b.pair_cap;
     uint32_t* over = b.place;                                   // k_cluster_place writes it after the last join
     uint32_t* scratch = reinterpret_cast<uint32_t*>(b.pairs);   // free once the pairs are joined
     const uint32_t scratch_words = (uint32_t)(2 * b.nv < 0xFFFFFFFFull ? 2 * b.nv : 0xFFFFFFFFull);

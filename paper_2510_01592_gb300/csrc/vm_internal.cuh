@@ -388,6 +388,7 @@ struct SegBuffers {
     uint32_t* scan_tmp;     // look-back state of the segmentation's scans
     SegCounters* ctr;       // device
     size_t nv, kcap;
+    uint32_t pair_cap = kNone;  // joined pairs listed at most (and nv)
 };
 constexpr uint16_t kNoComp = 0xFFFFu;
 
