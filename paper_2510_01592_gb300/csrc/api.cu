@@ -94,7 +94,7 @@ static void fit_layout(Carver& c, FitBuffers& fb, size_t kcap, size_t npts, size
     fb.err = c.take<uint32_t>(4);
     fb.tot = c.take<uint32_t>(4);
     fb.kdev = c.take<uint32_t>(4);
-    fb.done = c.take<uint32_t>(kcap * 3);
+    fb.done = c.take<uint32_t>(kcap * 2);
 }
 
 static size_t fit_bytes(size_t kcap, size_t npts, size_t chunks, size_t slots) {
@@ -228,7 +228,7 @@ static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* 
     if (k == 0) return VM_OK;
     size_t npts = fc.npts;
     bool large = fc.large();
-    if (!fc.mem.p || k > fc.kcap || (size_t)k * p.n_hyp > fc.slots) {  // the scratch grows in any case: learn the point count
+    if (!fc.mem.p || k > fc.kcap || (size_t)k * p.n_hyp > fc.slots) {  // it grows in any case: learn the point count
         uint32_t n = 0;
         VM_CUDA(cudaMemcpyAsync(&n, off + k, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         VM_CUDA(cudaStreamSynchronize(s));
@@ -441,8 +441,8 @@ vm_status plan_capacity(vm_map* m, const vm_segment_params& p, bool with_fit) {
     const size_t nv = m->seg_nv;
     // Cluster capacity from the last count with headroom (a segmentation with
     // more clusters flags itself and is re-run with the count it needed): the
-    // fit's grids, the sort's digit passes and the fit scratch all scale with
-    // it, so it tracks the map rather than the worst case nv / min_cluster.
+    // fit's grids and scratch scale with it, so it tracks the map rather than the
+    // worst case nv / min_cluster.
     size_t kcap = (size_t)m->k_hint + m->k_hint / 4 + 64;
     if (kcap < 256) kcap = 256;
     if (kcap > nv) kcap = nv;
@@ -601,9 +601,9 @@ vm_status launch_segment(vm_map* m, const vm_segment_params& p) {
     }
     VM_TRY(plan_capacity(m, p, true));
     m->seg_rounds = p.planes_per_cluster > 1 ? p.planes_per_cluster : 1;
-    // The points that the fit is likely to have: the last ones with headroom; before any, a quarter of the scratch, which
-    // has room for every slot of the bricks.  The kernels for large fits stay until they are a quarter below the limit, as
-    // the graph is captured anew where the choice changes.
+    // The points that the fit is likely to have: the last ones with headroom; before any, a quarter of the scratch,
+    // which has room for every slot of the bricks.  The kernels for large fits stay until they are a quarter below the
+    // limit, as the graph is captured anew where the choice changes.
     const size_t expect = m->fitted ? (size_t)m->last.n_kept + m->last.n_kept / 4 : m->seg_nv / 4;
     m->large = expect > (m->large ? kLargeFitPoints / 4 * 3 : kLargeFitPoints);
     StageHook* hk = m->fit.timer.hook();
@@ -1173,7 +1173,6 @@ vm_status vm_get_stats(vm_map* m, vm_stats* out) {
     out->voxels_cleared = c.cleared;
     out->voxels_evicted = c.evicted;
     out->device_bytes = m->pool.bytes + m->stage.bytes + m->brick_mem.bytes + m->vox_mem.bytes + m->fit.mem.bytes;
-    (void)0;
     if (c.err & kErrCapacity) {
         set_error("brick pool full");
         return VM_ERR_CAPACITY;

@@ -243,11 +243,10 @@ __global__ void k_select(const float* __restrict__ pts, const uint32_t* __restri
 }
 
 // Per-cluster completion: every work item of a cluster, after its results
-// are visible device-wide, counts itself done; the CTA (or warp) that
-// completes the cluster's last item runs the cluster's next serial step
-// (stage c after scoring, the centroid after extraction, the refit after the
-// filter) in place of a kernel of its own.  done: three counters a cluster,
-// cleared before the fit.
+// are visible device-wide, counts itself done; the CTA that completes the
+// cluster's last item runs the cluster's next serial step (the centroid after
+// extraction, the refit after the filter) in place of a kernel of its own.
+// done: two counters a cluster, cleared before the fit.
 __device__ __forceinline__ bool cta_last_item(uint32_t* done, uint32_t n_items, uint32_t* flag) {
     __threadfence();
     __syncthreads();
@@ -608,7 +607,7 @@ __device__ __noinline__ void extract_tail(uint32_t c, const float* __restrict__ 
                                           uint32_t* __restrict__ done) {
     __shared__ CentroidShared sm;
     __shared__ uint32_t s_last;
-    if (cta_last_item(done + 3 * (size_t)c + 1, item_off[c + 1] - item_off[c], &s_last))
+    if (cta_last_item(done + 2 * (size_t)c, item_off[c + 1] - item_off[c], &s_last))
         centroid_cta(c, pts, off, item_off, cpt, part, cl, cen, poly, sm);
 }
 
@@ -721,7 +720,7 @@ __device__ __noinline__ void filter_tail(uint32_t c, const uint32_t* __restrict_
                                          FitCluster* __restrict__ cl, uint32_t* __restrict__ done) {
     __shared__ RefitShared sm;
     __shared__ uint32_t s_last;
-    if (cta_last_item(done + 3 * (size_t)c + 2, item_off[c + 1] - item_off[c], &s_last))
+    if (cta_last_item(done + 2 * (size_t)c + 1, item_off[c + 1] - item_off[c], &s_last))
         refit_cta(c, off, item_off, cpt, part, cen, cl, sm);
 }
 
@@ -1485,7 +1484,7 @@ __global__ void k_items(const uint32_t* __restrict__ off, const uint32_t* __rest
     for (uint32_t c = blockIdx.x * kT + threadIdx.x; c < k; c += gridDim.x * kT) {
         const uint32_t n = off[c + 1] - off[c];
         item_cnt[c] = n ? (n + T - 1) / T : 1u;
-        if (done) done[3 * (size_t)c] = done[3 * (size_t)c + 1] = done[3 * (size_t)c + 2] = 0u;
+        if (done) done[2 * (size_t)c] = done[2 * (size_t)c + 1] = 0u;
     }
 }
 
@@ -1511,7 +1510,7 @@ __global__ void __launch_bounds__(kItemsScanT) k_items_scan(const uint32_t* __re
         if (c < k) {
             const uint32_t n = off[c + 1] - off[c];
             v = n ? (n + T - 1) / T : 1u;
-            if (done) done[3 * (size_t)c] = done[3 * (size_t)c + 1] = done[3 * (size_t)c + 2] = 0u;
+            if (done) done[2 * (size_t)c] = done[2 * (size_t)c + 1] = 0u;
         }
         uint32_t inc = v;
 #pragma unroll

@@ -223,8 +223,8 @@ enum Stage {
     kStNormals,        // Eq. 3 window moments (k_moments)
     kStEigen,          // Eq. 3 eigen-solve + Eq. 4 (k_eigen)
     kStCclLocal,       // Algorithm 1 inside bricks (k_ccl_local)
-    kStCcl,            // Algorithm 1 across bricks (k_ccl_cross, k_ccl_compress)
-    kStClusters,       // sizes, numbering, compaction, sort, gather
+    kStCcl,            // Algorithm 1 across bricks (k_comp_number, k_ccl_cross, k_comp_join)
+    kStClusters,       // sizes, numbering, placement, point lists
     kStHyp,            // stage a
     kStScore,          // stage b
     kStExtract,        // stage c, inliers, centroid, filter
@@ -286,8 +286,8 @@ vm_status ensure(DevBuf& b, size_t bytes);
 // look-back wait ran out.  end: also write the sum at out[n] (n the device
 // count clamped to n_cap; out then holds n_cap + 1 words), the closing offset
 // of an offsets array.
-// Elements per tile of the single-pass scan; its look-back state is a
-// ticket, a done count, an epoch, a pad word and one 64-bit word per tile.
+// Elements per tile of the single-pass scan; its look-back state is a 64-bit
+// word that holds the ticket and the epoch, one unused, and one per tile.
 constexpr size_t kScanTileElems = 2048;
 constexpr size_t scan_tmp_words(size_t n) { return 4 + 2 * ((n + kScanTileElems - 1) / kScanTileElems) + 2; }
 cudaError_t exclusive_scan_dev(const uint32_t* in, uint32_t* out, uint32_t* total, const uint32_t* n_dev, size_t n_cap,
@@ -336,12 +336,14 @@ cudaError_t launch_scroll(const Grid& g, const Grid& g2, const int32_t shift[3],
 cudaError_t launch_integrate(const float* xyz, uint32_t n, const Pose& pose, const Grid& g, int32_t* brick_table,
                              int32_t* slot_key, unsigned long long* S, uint32_t* C, uint32_t* occ,
                              uint32_t* deferred, MapCounters* ctr, uint32_t capacity, cudaStream_t s);
+// Empties the map: the slots that were claimed, the brick table and the
+// counters.
+cudaError_t launch_reset(int32_t* brick_table, uint32_t nb_total, unsigned long long* S, uint32_t* C, uint32_t* occ,
+                         uint32_t* mark, MapCounters* ctr, uint32_t capacity, cudaStream_t s);
 // Voxel information clearing (Sec. III.B, Eq. 2): marks every occupied voxel
 // that a point's ray from the sensor passes through before the point's own
 // voxel (mark: one bit per voxel slot, capacity * 16 words, zero between
 // calls), then clears the marked voxels and the marks.
-cudaError_t launch_reset(int32_t* brick_table, uint32_t nb_total, unsigned long long* S, uint32_t* C, uint32_t* occ,
-                         uint32_t* mark, MapCounters* ctr, uint32_t capacity, cudaStream_t s);
 cudaError_t launch_clear(const float* xyz, uint32_t n, const Pose& pose, const Grid& g,
                          const int32_t* brick_table, unsigned long long* S, uint32_t* C, uint32_t* occ,
                          uint32_t* mark, MapCounters* ctr, uint32_t capacity, cudaStream_t s);
@@ -410,6 +412,11 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
 // ---------------------------------------------------------------- fit.cu
 // A fit expected to have more points takes the kernels for large ones: the
 // per-cluster tails in kernels of their own, and tests of stage b bounded.
+// Whole fits with the kernels for small / large ones, us: 16 clusters of 1 M
+// points together 114 / 128 at H = 100 and 162 / 158 at H = 256, of 4 M 264 / 217
+// and 430 / 279; 2,000 clusters of 1 M points 265 / 290 and 323 / 338, of 4 M 399 /
+// 388 and 562 / 506.  They cross between one and three million points, by the
+// hypotheses and the clusters; at the limit the large ones are ahead in each.
 constexpr size_t kLargeFitPoints = size_t(4) << 20;
 struct FitBuffers {
     float4* hyp;            // [kcap * H]
@@ -432,7 +439,7 @@ struct FitBuffers {
     uint32_t* err;          // device error word
     uint32_t* tot;          // [4] scan totals
     uint32_t* kdev;         // cluster count when the caller supplies it
-    uint32_t* done;         // [kcap][3] per-cluster completion counters (scoring, extraction, filter)
+    uint32_t* done;         // [kcap][2] per-cluster completion counters (extraction, filter)
     size_t kcap, npts_cap, items_cap;  // items_cap: 256-point partial-sum chunks
     bool large;             // kernels for more than kLargeFitPoints points (results do not depend on it)
 };
@@ -451,7 +458,6 @@ FitTuning tuning_of(const vm_fit_tuning& t);
 // Resident scoring CTAs per SM for tuning t and H hypotheses (0 on error).
 int score_max_ctas_per_sm(const FitTuning& t, int H);
 size_t fit_hull_smem();
-
 
 // Runs RANSAC, selection, extraction, refit and hull for the clusters whose
 // points are pts[off[c]..off[c+1]) (device), labels (device, or nullptr for
