@@ -601,10 +601,11 @@ vm_status launch_segment(vm_map* m, const vm_segment_params& p) {
     }
     VM_TRY(plan_capacity(m, p, true));
     m->seg_rounds = p.planes_per_cluster > 1 ? p.planes_per_cluster : 1;
-    // The points that the fit is likely to have: the last ones with headroom; before any, a quarter of the scratch,
-    // which has room for every slot of the bricks.  The kernels for large fits stay until they are a quarter below the
+    // The points that the fit is likely to have: the last ones with headroom; before any, a quarter of the bricks' slots
+    // (a fifth of them hold a voxel of a surface).  The kernels for large fits stay until they are a quarter below the
     // limit, as the graph is captured anew where the choice changes.
-    const size_t expect = m->fitted ? (size_t)m->last.n_kept + m->last.n_kept / 4 : m->seg_nv / 4;
+    const size_t expect = m->fitted ? (size_t)m->last.n_kept + m->last.n_kept / 4
+                                    : (size_t)m->brick_hint * (kBrickVox / 4);
     m->large = expect > (m->large ? kLargeFitPoints / 4 * 3 : kLargeFitPoints);
     StageHook* hk = m->fit.timer.hook();
     if (m->use_graph && !hk && (!m->gexec || m->ggen != m->gen || m->gmany != m->many ||

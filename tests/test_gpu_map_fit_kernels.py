@@ -20,7 +20,7 @@ def test_many_bricks_with_few_clustered_points():
     prm = vm.segment_params(n_hyp=32)
     floor = (np.stack(np.meshgrid(np.arange(60), np.arange(60), [20]), -1).reshape(-1, 3) + 0.5) * 0.01
     want = None
-    for spread in (0, 25000):  # scattered points: a brick each, none in a cluster
+    for spread in (0, 25000, 60000):  # scattered points: a brick each or so, none in a cluster
         m = vm.VoxelMap((800, 800, 100), (0.0, 0.0, 0.0), 0.01)
         pts = np.concatenate([floor, rng.uniform(0, 1, (spread, 3)) * [6.9, 7.9, 0.9] + [1.0, 0, 0]])
         m.integrate(pts.astype(np.float32), POSE)
