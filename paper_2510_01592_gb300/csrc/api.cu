@@ -688,8 +688,10 @@ bool take_hints(vm_map* m) {
     m->k_hint = hdr->k_need > hdr->k ? hdr->k_need : hdr->k;
     m->hull_hint = hdr->n_hull;
     m->rec_hint = hdr->n_planes;
-    // more than eight components a brick, until they are fewer than four: the graph is captured anew where it changes
-    m->many = hdr->n_comp > (uint64_t)hdr->n_sorted * (m->many ? 4 : 8);
+    // more than eight components a brick, or the clusters; until they are fewer than half and two thirds, as the graph is
+    // captured anew where it changes
+    m->many = hdr->n_comp > (uint64_t)hdr->n_sorted * (m->many ? 4 : 8) ||
+              m->k_hint > (m->many ? kSurfaceClusters / 3 * 2 : kSurfaceClusters);
     return (hdr->err & kErrScratch) || hdr->n_hull > m->out_hcap || hdr->n_planes > m->out_kcap;
 }
 

@@ -188,7 +188,7 @@ struct vm_map {
     uint32_t out_kcap = 0, out_hcap = 0;
     uint32_t kcap = 0;            // kept-cluster capacity of the scratch
     uint32_t brick_hint = 0, k_hint = 0, hull_hint = 0;
-    bool many = false;            // the map has many components a brick
+    bool many = false;            // the map has many components a brick, or clusters
     bool large = false;           // its fit takes the kernels for large ones
     bool fitted = false;          // last holds the counts of a segmentation
     uint64_t gen = 0;             // bumps whenever scratch or outputs move

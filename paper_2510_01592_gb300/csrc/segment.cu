@@ -354,6 +354,24 @@ __device__ __forceinline__ uint32_t cta_warps_excl(uint32_t v, uint32_t* ws, uin
     __syncthreads();
     return out;
 }
+// The same for two values at once (ws: 66 words).
+__device__ __forceinline__ uint2 cta_warps_excl2(uint32_t a, uint32_t b, uint32_t* ws, uint32_t* ta, uint32_t* tb) {
+    const uint32_t w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane < 2) ws[33 * lane + w] = lane ? b : a;
+    __syncthreads();
+    if (w < 2) {
+        uint32_t* p = ws + 33 * w;
+        const uint32_t t = p[lane], ti = warp_incl(t);
+        p[lane] = ti - t;
+        if (lane == 31) p[32] = ti;
+    }
+    __syncthreads();
+    const uint2 out = make_uint2(ws[w], ws[33 + w]);
+    *ta = ws[32];
+    *tb = ws[65];
+    __syncthreads();
+    return out;
+}
 // Exclusive scan over a 1024-thread CTA (ws: 33 words); *total: the sum.
 __device__ __forceinline__ uint32_t cta_excl(uint32_t v, uint32_t* ws, uint32_t* total) {
     const uint32_t inc = warp_incl(v);
@@ -935,9 +953,12 @@ __device__ __forceinline__ uint32_t uf_root(const uint32_t* P, uint32_t x, uint3
     return x;
 }
 
-// Words of the scratch that k_cluster_number and k_cluster_place share, zero when
-// they start (k_comp_size): a flag a CTA of the placement, the tickets, and whose
-// turn a tile of the placement is; then a 64-bit word a CTA of the numbering.
+// A map with many components numbers and places its clusters with kernels of their
+// own (k_cluster_number_many, k_cluster_place<true>): what they need made those for
+// surfaces, which run on every frame, a little longer.  Words of the scratch that
+// they share, zero when they start (k_comp_size, clear): a flag a CTA of the
+// placement, the tickets, and whose turn a tile of the placement is; then a 64-bit
+// word a CTA of the numbering.
 constexpr uint32_t kPlaceCtas = 128;  // CTAs of either at most
 constexpr uint32_t kPlaceTicket = kPlaceCtas, kPlaceTurn = kPlaceCtas + 1, kNumberTicket = kPlaceCtas + 2;
 constexpr uint32_t kNumberWords = kPlaceCtas + 4, kPlaceHead = kNumberWords + 2 * kPlaceCtas;
@@ -946,11 +967,11 @@ constexpr uint32_t kNumberWords = kPlaceCtas + 4, kPlaceHead = kNumberWords + 2 
 // root (lanes with equal roots add up first).
 __global__ void __launch_bounds__(kT) k_comp_size(const SegCounters* __restrict__ ctr, uint32_t* parent,
                                                   const uint32_t* __restrict__ csize, uint32_t* __restrict__ total,
-                                                  uint32_t* __restrict__ scratch, uint32_t* err) {
+                                                  uint32_t* __restrict__ clear, uint32_t* err) {
     pdl_gate();
     const uint32_t K = ctr->n_comp;
-    if (blockIdx.x == 0)
-        for (uint32_t q = threadIdx.x; q < kPlaceHead; q += kT) scratch[q] = 0;
+    if (clear && blockIdx.x == 0)
+        for (uint32_t q = threadIdx.x; q < kPlaceHead; q += kT) clear[q] = 0;
     for (uint32_t base = (blockIdx.x * kT + threadIdx.x) & ~31u; base < K; base += gridDim.x * kT) {
         const uint32_t c = base + (threadIdx.x & 31);
         uint32_t root = kNone, n = 0;
@@ -966,61 +987,112 @@ __global__ void __launch_bounds__(kT) k_comp_size(const SegCounters* __restrict_
 }
 
 // Kept components (at least min_cluster vertices) numbered in the order of
-// their roots (= label order) with their sizes, labels and offsets.  One CTA
-// takes up to kNumberRun components; more are cut into stretches, a CTA each,
-// which adds up its own, publishes the two sums and waits for the CTAs before it
-// (a ticket numbers them as they start, so each of those is running; the wait is
-// bounded).  Clusters beyond the scratch flag a re-run, and the count is clamped
-// for the kernels after this one.  next: the offsets again, which the placement
-// moves on where it goes tile by tile.  (A floor has a component or two a brick
-// and one CTA is done with its few thousand in 5 us; a 1 x 1 x 1 m map with every
-// second cell at 0.01 m occupied has hundreds a brick: 191 us in one CTA, 12 so.)
-constexpr uint32_t kNumberRun = kOneT * kRun;
+// their roots (= label order) with their sizes and labels, and the cluster
+// offsets, in one CTA.  Clusters beyond the scratch flag a re-run, and the
+// count is clamped for the kernels after this one.
 __global__ void __launch_bounds__(kOneT, 1) k_cluster_number(SegCounters* __restrict__ ctr, uint32_t min_cluster,
                                                           uint32_t kcap, const uint32_t* __restrict__ total,
                                                           const uint32_t* __restrict__ croot,
                                                           uint32_t* __restrict__ ccl, uint32_t* __restrict__ cl_size,
                                                           uint32_t* __restrict__ cl_label,
-                                                          uint32_t* __restrict__ cl_off, uint32_t* scratch,
-                                                          uint32_t* err) {
+                                                          uint32_t* __restrict__ cl_off,
+                                                          uint32_t* __restrict__ flags) {
     pdl_gate();
     __shared__ uint32_t ws[33];
+    const int lane = threadIdx.x & 31;
+    const uint32_t K = ctr->n_comp;
+    if (threadIdx.x <= kPlaceCtas) flags[threadIdx.x] = 0;  // k_cluster_place's, and its ticket
+    uint32_t k = 0;
+    for (uint32_t b0 = 0; b0 < K; b0 += kOneT * kRun) {
+        const uint32_t c0 = b0 + (threadIdx.x >> 5) * (32 * kRun) + lane;
+        uint32_t sz[kRun], kept[kRun], sum = 0;
+#pragma unroll
+        for (int i = 0; i < kRun; ++i) sz[i] = c0 + i * 32 < K ? total[c0 + i * 32] : 0u;  // 0 but at roots
+#pragma unroll
+        for (int i = 0; i < kRun; ++i) {
+            if (sz[i] < min_cluster) sz[i] = 0;
+            kept[i] = __ballot_sync(0xffffffffu, sz[i] != 0);
+            sum += __popc(kept[i]);
+        }
+        uint32_t tot;
+        uint32_t at = k + cta_warps_excl(sum, ws, &tot);
+#pragma unroll
+        for (int i = 0; i < kRun; ++i) {
+            const uint32_t c = c0 + i * 32, me = at + __popc(kept[i] & ((1u << lane) - 1u));
+            if (c < K) ccl[c] = sz[i] ? me : kNone;  // of roots; the others follow in k_cluster_place
+            if (sz[i]) {
+                cl_size[me] = sz[i];
+                cl_label[me] = croot[c];
+            }
+            at += __popc(kept[i]);
+        }
+        k += tot;
+    }
+    __syncthreads();  // cl_size, by this CTA
+    uint32_t off = 0;
+    for (uint32_t b0 = 0; b0 < k; b0 += kOneT) {
+        const uint32_t c = b0 + threadIdx.x;
+        uint32_t tot;
+        const uint32_t at = off + cta_excl(c < k ? cl_size[c] : 0u, ws, &tot);
+        if (c < k) cl_off[c] = at;
+        off += tot;
+    }
+    if (threadIdx.x == 0) {
+        cl_off[k] = off;
+        ctr->n_kept = off;
+        ctr->tot = off;
+        ctr->k_need = k;
+        ctr->k = k < kcap ? k : kcap;
+        if (k > kcap) atomicOr(&ctr->err, kErrScratch);
+    }
+}
+
+// The same for a map with many components: they are cut into stretches, a CTA each,
+// which adds up its own, publishes the two sums and waits for the CTAs before it (a
+// ticket numbers them as they start, so each of those is running; the wait is
+// bounded); then it goes over the stretch again.  next: the offsets again, which the
+// placement moves on where it goes tile by tile.  (1 x 1 x 1 m with every second cell
+// at 0.01 m occupied, hundreds of components a brick: 191 us in one CTA, 12 so.)
+constexpr uint32_t kNumberRun = kOneT * kRun;
+__global__ void __launch_bounds__(kOneT, 1) k_cluster_number_many(SegCounters* __restrict__ ctr, uint32_t min_cluster,
+                                                               uint32_t kcap, const uint32_t* __restrict__ total,
+                                                               const uint32_t* __restrict__ croot,
+                                                               uint32_t* __restrict__ ccl,
+                                                               uint32_t* __restrict__ cl_size,
+                                                               uint32_t* __restrict__ cl_label,
+                                                               uint32_t* __restrict__ cl_off, uint32_t* scratch,
+                                                               uint32_t* err) {
+    pdl_gate();
+    __shared__ uint32_t ws[66];
     __shared__ uint32_t s_ticket;
     const int lane = threadIdx.x & 31;
     const uint32_t w = threadIdx.x >> 5, K = ctr->n_comp;
     const uint32_t stretch = max(kNumberRun, ((K + gridDim.x - 1) / gridDim.x + 1023u) & ~1023u);
     const uint32_t G = max(1u, (K + stretch - 1) / stretch);
     if (blockIdx.x >= G) return;
-    uint32_t g = 0, k = 0, off = 0;  // this CTA, the clusters and the vertices before it
-    uint32_t tot, tot2;
-    if (G > 1) {
-        volatile unsigned long long* words = reinterpret_cast<volatile unsigned long long*>(scratch + kNumberWords);
-        if (threadIdx.x == 0) s_ticket = atomicAdd(scratch + kNumberTicket, 1u);
-        __syncthreads();
-        g = s_ticket;
-        uint32_t mk = 0, mv = 0;
-        const uint32_t end = min(K, (g + 1) * stretch);
+    volatile unsigned long long* words = reinterpret_cast<volatile unsigned long long*>(scratch + kNumberWords);
+    if (threadIdx.x == 0) s_ticket = atomicAdd(scratch + kNumberTicket, 1u);
+    __syncthreads();
+    const uint32_t g = s_ticket, first = g * stretch, end = min(K, first + stretch);
+    uint32_t k, off, tot, tot2, mk = 0, mv = 0;
 #pragma unroll 8
-        for (uint32_t c = g * stretch + threadIdx.x; c < end; c += kOneT) {
-            const uint32_t n = total[c];  // 0 but at roots
-            mk += n >= min_cluster;
-            mv += n >= min_cluster ? n : 0u;
-        }
-        cta_warps_excl(__reduce_add_sync(0xffffffffu, mk), ws, &tot);
-        cta_warps_excl(__reduce_add_sync(0xffffffffu, mv), ws, &tot2);
-        // one word: the sums and that they are there
-        if (threadIdx.x == 0) words[g] = 1ull << 63 | (unsigned long long)tot << 32 | tot2;
-        unsigned long long before = 0;
-        if (threadIdx.x < g) {
-            int it = 0;
-            while (!((before = words[threadIdx.x]) >> 63) && it < kLoopCap) ++it;
-            if (it == kLoopCap) atomicOr(err, kErrTimeout);
-        }
-        cta_warps_excl(__reduce_add_sync(0xffffffffu, (uint32_t)(before >> 32) & 0x7fffffffu), ws, &k);
-        cta_warps_excl(__reduce_add_sync(0xffffffffu, (uint32_t)before), ws, &off);
+    for (uint32_t c = first + threadIdx.x; c < end; c += kOneT) {
+        const uint32_t n = total[c];  // 0 but at roots
+        mk += n >= min_cluster;
+        mv += n >= min_cluster ? n : 0u;
     }
+    cta_warps_excl2(__reduce_add_sync(0xffffffffu, mk), __reduce_add_sync(0xffffffffu, mv), ws, &tot, &tot2);
+    // one word: the sums and that they are there
+    if (threadIdx.x == 0) words[g] = 1ull << 63 | (unsigned long long)tot << 32 | tot2;
+    unsigned long long before = 0;
+    if (threadIdx.x < g) {
+        int it = 0;
+        while (!((before = words[threadIdx.x]) >> 63) && it < kLoopCap) ++it;
+        if (it == kLoopCap) atomicOr(err, kErrTimeout);
+    }
+    cta_warps_excl2(__reduce_add_sync(0xffffffffu, (uint32_t)(before >> 32) & 0x7fffffffu),
+                    __reduce_add_sync(0xffffffffu, (uint32_t)before), ws, &k, &off);  // before this CTA
     uint32_t* next = scratch + kPlaceHead;
-    const uint32_t first = g * stretch, end = min(K, first + stretch);
     for (uint32_t b0 = first; b0 < end; b0 += kNumberRun) {
         const uint32_t c0 = b0 + w * (32 * kRun) + lane;
         uint32_t sz[kRun], kept[kRun], inc[kRun], nk = 0, nv = 0;
@@ -1031,11 +1103,15 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_number(SegCounters* __rest
             if (sz[i] < min_cluster) sz[i] = 0;
             kept[i] = __ballot_sync(0xffffffffu, sz[i] != 0);
             nk += __popc(kept[i]);
-            inc[i] = nv + warp_incl(sz[i]);
-            nv = __shfl_sync(0xffffffffu, inc[i], 31);
+            inc[i] = 0;
+            if (kept[i]) {  // most steps of a map of surfaces keep none
+                inc[i] = nv + warp_incl(sz[i]);
+                nv = __shfl_sync(0xffffffffu, inc[i], 31);
+            }
         }
-        uint32_t at = k + cta_warps_excl(nk, ws, &tot);
-        const uint32_t av = off + cta_warps_excl(nv, ws, &tot2);
+        const uint2 ex = cta_warps_excl2(nk, nv, ws, &tot, &tot2);
+        uint32_t at = k + ex.x;
+        const uint32_t av = off + ex.y;
 #pragma unroll
         for (int i = 0; i < kRun; ++i) {
             const uint32_t c = c0 + i * 32, me = at + __popc(kept[i] & ((1u << lane) - 1u));
@@ -1062,23 +1138,26 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_number(SegCounters* __rest
 
 // Where each in-brick component's points start in the cluster lists: its
 // cluster's offset plus the vertices of the cluster's components before it.
-// The components are cut into stretches, a CTA each, and a CTA's into at most 32,
-// a warp each: a warp adds up its components' vertices per cluster, the sums are
+// The components are cut into stretches, a CTA each, and a CTA's into 32, a
+// warp each: a warp adds up its components' vertices per cluster, the sums are
 // scanned over the CTA's warps, each CTA publishes its sums per cluster and
 // waits for the CTAs before it (a ticket numbers them as they start, so each
 // of those is running; the wait is bounded), and each warp walks its components
-// again, 32 at a time, one scan per cluster among them.  scratch: kPlaceHead words,
-// then the CTAs' sums.  The counts of 32 warps fit shared memory up to kPlaceWords /
-// 32 clusters; with more, fewer warps count.  Where one warp's do not fit, or the
-// sums the scratch, the CTAs take tiles of kPlaceTile components instead
-// (place_tiles).  With all of it in one CTA from 1,536 clusters on, 4 x 4 x 1 m of
-// noise at 0.01 m took 1.75 ms for 12 thousand clusters (0.28 with one warp a CTA
-// counting) and 36.7 ms for 616 thousand (0.46 tile by tile) with the numbering and
-// the lists.
-constexpr uint32_t kPlaceWords = 24576;  // 96 KB: another stream's kernels fit the SM beside it
-constexpr uint32_t kPlaceTile = 8192;    // its keys and counts take them all
+// again, 32 at a time, one scan per cluster among them.  scratch: a flag per CTA and
+// the ticket (zero at launch), then the CTAs' sums.  Where the warps' counts do not
+// fit shared memory or the sums the scratch, one CTA takes everything, its counts in
+// scratch.
+// kMany, for maps with many components or clusters: fewer warps count where the
+// counts of 32 do not fit, and where one warp's do not, or the sums the scratch, the
+// CTAs take tiles of kPlaceTile components (place_tiles).  4 x 4 x 1 m of noise at 0.01
+// m with 12 thousand clusters: 1.75 ms in one CTA, 0.28 with a warp a CTA counting, and
+// with 616 thousand 36.7 ms and 0.27 tile by tile, numbering and lists included.
+template <bool kMany>
+constexpr uint32_t kPlaceWords = kMany ? 24576 : 49152;  // 96 KB (other kernels fit the SM beside it), 192 KB
+constexpr uint32_t kPlaceTile = 8192;                     // its keys and counts take the 96 KB
 constexpr uint32_t kTileBits = 13;
-static_assert(kPlaceTile == 1u << kTileBits && kPlaceTile * 3 <= kPlaceWords, "a tile's keys and counts fit");
+static_assert(kPlaceTile == 1u << kTileBits && kPlaceTile * 3 <= kPlaceWords<true>, "a tile's keys and counts fit");
+static_assert(kSurfaceClusters * 32 == kPlaceWords<false>, "with more, one CTA places them all");
 
 // The placement tile by tile, however many clusters there are.  A component that is
 // its whole cluster starts at the cluster's offset.  A tile's others are sorted by
@@ -1222,6 +1301,7 @@ __device__ __noinline__ void place_tiles(uint32_t K, const uint32_t* __restrict_
     }
 }
 
+template <bool kMany>
 __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* __restrict__ ctr,
                                                          const uint32_t* __restrict__ parent,
                                                          const uint32_t* __restrict__ csize, uint32_t* ccl,
@@ -1234,19 +1314,27 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* _
     const uint32_t K = ctr->n_comp, k = ctr->k_need;
     const int lane = threadIdx.x & 31;
     const uint32_t w = threadIdx.x >> 5;
-    const uint32_t stretch = max(1024u, ((K + gridDim.x - 1) / gridDim.x + 1023u) & ~1023u);
-    const uint32_t G = (K + stretch - 1) / stretch;
-    if (blockIdx.x >= G) return;
-    if (k > kPlaceWords || (size_t)G * k + kPlaceHead > scratch_words) {
-        place_tiles(K, parent, csize, ccl, cl_size, cl_off, place, scratch, sm, err);
-        return;
-    }
+    uint32_t stretch = max(1024u, ((K + gridDim.x - 1) / gridDim.x + 1023u) & ~1023u);
+    uint32_t G = (K + stretch - 1) / stretch;
+    constexpr uint32_t kHead = kMany ? kPlaceHead : kPlaceCtas + 1;
     volatile uint32_t* flags = scratch;
-    uint32_t* sums = scratch + kPlaceHead;
+    uint32_t* sums = scratch + kHead;
+    const bool fit = (size_t)k * (kMany ? 1 : 32) <= kPlaceWords<kMany> && (size_t)G * k + kHead <= scratch_words;
+    if constexpr (kMany) {
+        if (blockIdx.x >= G) return;
+        if (!fit) {
+            place_tiles(K, parent, csize, ccl, cl_size, cl_off, place, scratch, sm, err);
+            return;
+        }
+    } else if (!fit) {
+        stretch = (K + 1023u) & ~1023u;
+        G = 1;
+    }
     __shared__ uint32_t s_ticket;
     if (threadIdx.x == 0) s_ticket = atomicAdd(scratch + kPlaceTicket, 1u);
     __syncthreads();
     const uint32_t g = s_ticket;
+    if (g >= G) return;
     const uint32_t first = g * stretch, end = min(K, first + stretch);
     constexpr int kIt = 8;
     // each component's cluster (a root's entry is read and rewritten with the same value)
@@ -1261,12 +1349,14 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* _
             if (root[i] != kNone) ccl[c0 + i * kOneT] = cl[i];
     }
     if (k == 0) return;
-    const uint32_t W = min(32u, kPlaceWords / k);  // warps with counts of their own
-    for (uint32_t q = threadIdx.x; q < W * k; q += kOneT) sm[q] = 0;
+    uint32_t* cnt = kMany || fit ? sm : sums;
+    // warps with counts of their own
+    const uint32_t W = kMany ? min(32u, kPlaceWords<kMany> / k) : (fit ? 32u : min(32u, (scratch_words - kHead) / k));
+    for (uint32_t q = threadIdx.x; q < W * k; q += kOneT) cnt[q] = 0;
     __syncthreads();
     const uint32_t len = ((end - first + W - 1) / W + 31) & ~31u;
     const uint32_t lo = min(end, first + w * len), hi = w < W ? min(end, lo + len) : lo;
-    uint32_t* mine = sm + (w < W ? w : 0) * k;
+    uint32_t* mine = cnt + (size_t)(w < W ? w : 0) * k;
     for (uint32_t c0 = lo; c0 < hi; c0 += 32 * kIt) {  // kIt steps' loads go out together
         uint32_t cl[kIt], n[kIt];
 #pragma unroll
@@ -1286,10 +1376,10 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* _
     }
     __syncthreads();
     for (uint32_t cl = w; cl < k; cl += kOneT / 32) {  // a warp a cluster, a lane a warp's counts
-        uint32_t* at = sm + lane * k + cl;
+        uint32_t* at = cnt + (size_t)lane * k + cl;
         const uint32_t t = lane < (int)W ? *at : 0u, inc = warp_incl(t);
         if (lane < (int)W) *at = inc - t;
-        if (lane == 31) sums[(size_t)g * k + cl] = inc;
+        if ((kMany || fit) && lane == 31) sums[(size_t)g * k + cl] = inc;
     }
     if (G > 1) {
         __threadfence();
@@ -1306,7 +1396,7 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* _
     for (uint32_t cl = threadIdx.x; cl < k; cl += kOneT) {  // the cluster's points before this CTA's
         uint32_t b = cl_off[cl];
         for (uint32_t q = 0; q < g; ++q) b += __ldcg(sums + (size_t)q * k + cl);
-        for (uint32_t q = 0; q < W; ++q) sm[q * k + cl] += b;
+        for (uint32_t q = 0; q < W; ++q) cnt[(size_t)q * k + cl] += b;
     }
     __syncthreads();
     for (uint32_t c0 = lo; c0 < hi; c0 += 32 * kIt) {
@@ -1420,7 +1510,10 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
     static std::once_flag once;
     std::call_once(once, [] {
         cudaFuncSetAttribute(k_comp_join, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kJoinWords * 4));
-        cudaFuncSetAttribute(k_cluster_place, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kPlaceWords * 4));
+        cudaFuncSetAttribute(k_cluster_place<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kPlaceWords<false> * 4));
+        cudaFuncSetAttribute(k_cluster_place<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kPlaceWords<true> * 4));
     });
     const uint32_t cap_b = (uint32_t)(b.nv / kBrickVox);
     const size_t stride = b.nv;
@@ -1464,13 +1557,19 @@ cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* 
     VM_STAGE_END(hk, kStCcl, s);
     VM_STAGE_BEGIN(hk, kStClusters, s);
     launch_k(k_comp_size, dim3(many ? clampg(cap_b / 4, sms * 8) : clampg(cap_b / 64, sms * 2)), dim3(kT), 0, s, b.ctr,
-             b.parent, b.csize, b.total, scratch, err);
+             b.parent, b.csize, b.total, many ? scratch : nullptr, err);
     const uint32_t min_cl = p.min_cluster ? p.min_cluster : 1u;
-    launch_k(k_cluster_number, dim3(clampg(many ? cap_b / 16 : cap_b / 1024, kPlaceCtas)), dim3(kOneT), 0, s, b.ctr,
-             min_cl, kcap, b.total, b.croot, b.ccl, b.cl_size, b.cl_label, b.cl_off, scratch, err);
-    launch_k(k_cluster_place, dim3(clampg(many ? cap_b / 16 : cap_b / 512 + 1, kPlaceCtas)), dim3(kOneT),
-             kPlaceWords * 4, s, b.ctr, b.parent, b.csize, b.ccl, b.cl_size, b.cl_off, b.place, scratch, scratch_words,
-             err);
+    if (many) {
+        launch_k(k_cluster_number_many, dim3(clampg(cap_b / 16, kPlaceCtas)), dim3(kOneT), 0, s, b.ctr, min_cl, kcap,
+                 b.total, b.croot, b.ccl, b.cl_size, b.cl_label, b.cl_off, scratch, err);
+        launch_k(k_cluster_place<true>, dim3(clampg(cap_b / 16, kPlaceCtas)), dim3(kOneT), kPlaceWords<true> * 4, s,
+                 b.ctr, b.parent, b.csize, b.ccl, b.cl_size, b.cl_off, b.place, scratch, scratch_words, err);
+    } else {
+        launch_k(k_cluster_number, dim3(1), dim3(kOneT), 0, s, b.ctr, min_cl, kcap, b.total, b.croot, b.ccl, b.cl_size,
+                 b.cl_label, b.cl_off, scratch);
+        launch_k(k_cluster_place<false>, dim3(clampg(cap_b / 512 + 1, kPlaceCtas)), dim3(kOneT), kPlaceWords<false> * 4,
+                 s, b.ctr, b.parent, b.csize, b.ccl, b.cl_size, b.cl_off, b.place, scratch, scratch_words, err);
+    }
     launch_k(k_cluster_scatter, dim3(clampg((cap_b + kScatWarps - 1) / kScatWarps, sms * 8)), dim3(kScatWarps * 32), 0,
              s, b.ctr, cap_b, b.brec, b.ncomp, b.cbase, b.ccl, b.place, b.lc, b.vox, b.pos, b.pts, b.pt_vid);
     VM_STAGE_END(hk, kStClusters, s);

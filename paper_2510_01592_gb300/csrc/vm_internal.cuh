@@ -404,8 +404,9 @@ cudaError_t seg_order_bricks(const int32_t* brick_table, uint32_t nb_total, cons
 // seg_order_bricks.  Every count is read on the device (clamped to the
 // scratch, with kErrScratch raised when it does not fit), so the launch
 // sequence is fixed and can be captured in a CUDA graph.  kcap bounds the
-// kept clusters.  many: grids for a map with many components a brick (results do
-// not depend on it).
+// kept clusters.  many: kernels and grids for a map with many components a brick, or
+// more than kSurfaceClusters clusters (results do not depend on it).
+constexpr uint32_t kSurfaceClusters = 1536;
 cudaError_t seg_run(const Grid& g, const unsigned long long* S, const uint32_t* C, const vm_segment_params& p,
                     SegBuffers& b, uint32_t kcap, bool many, uint32_t* err, int sms, cudaStream_t s, StageHook* hk);
 
