@@ -1146,7 +1146,8 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_number_many(SegCounters* _
 // again, 32 at a time, one scan per cluster among them.  scratch: a flag per CTA and
 // the ticket (zero at launch), then the CTAs' sums.  Where the warps' counts do not
 // fit shared memory or the sums the scratch, one CTA takes everything, its counts in
-// scratch.
+// scratch (and where the run is one to be repeated, the places are left at zero, from
+// where the lists stay inside their arrays).
 // kMany, for maps with many components or clusters: fewer warps count where the
 // counts of 32 do not fit, and where one warp's do not, or the sums the scratch, the
 // CTAs take tiles of kPlaceTile components (place_tiles).  4 x 4 x 1 m of noise at 0.01
@@ -1327,6 +1328,10 @@ __global__ void __launch_bounds__(kOneT, 1) k_cluster_place(const SegCounters* _
             return;
         }
     } else if (!fit) {
+        if (k > ctr->k) {  // more clusters than the scratch has room for: the host runs it all again, with kMany
+            for (uint32_t c = blockIdx.x * kOneT + threadIdx.x; c < K; c += gridDim.x * kOneT) place[c] = 0;
+            return;
+        }
         stretch = (K + 1023u) & ~1023u;
         G = 1;
     }

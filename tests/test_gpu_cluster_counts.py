@@ -64,3 +64,20 @@ def test_clusters_of_noise_cost_no_more_than_its_voxels(density, min_cluster):
         ratio = t["clusters"] / (t["finalize"] + t["moments"] + t["eigen"])
         best = ratio if best is None else min(best, ratio)
     assert best < 3.0, best
+
+
+def test_the_first_segmentation_of_noise_is_not_held_up():
+    """A map's first segmentation goes by no counts, and is repeated where the scratch has no room for the clusters: both
+    runs' clustering together take at most ten times as long as the means and normals."""
+    from paper_2510_01592_gb300 import vm
+    best = None
+    for _ in range(3):
+        m = vm.VoxelMap((200, 200, 100), (0.0, 0.0, 0.0), 0.01, stage_timing=True)
+        m.integrate(_noise((200, 200, 100), 0.05, 3), POSE)
+        m.stage_times()
+        m.segment(vm.segment_params(n_hyp=4, classify=0, min_cluster=1))
+        t = {k: v[0] for k, v in m.stage_times().items()}
+        ratio = t["clusters"] / (t["finalize"] + t["moments"] + t["eigen"])
+        best = ratio if best is None else min(best, ratio)
+        m.close()
+    assert best < 10.0, best
