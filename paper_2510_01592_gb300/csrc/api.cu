@@ -239,14 +239,14 @@ static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* 
     FitHeader h;
     for (int attempt = 0;; ++attempt) {
         VM_TRY(fit_prepare(fc, k, npts, (int)p.n_hyp, tune.tile, s));
+        size_t hull = (size_t)k * 48 + 4096;
+        if (hull > (1u << 20)) hull = 1u << 20;
+        VM_TRY(fit_out(fc, k, (uint32_t)hull));  // no work is in flight where it fails, here or below
         FitBuffers& fb = fc.fb;
         fb.large = large;
         VM_CUDA(fit_open(off, k, (uint32_t)(fc.npts < 0xFFFFFFFFull ? fc.npts : 0xFFFFFFFFull), fb, s));
         VM_CUDA(launch_fit(pts, off, labels, fb.kdev, k, p, fb, tune, device_sms(), s, hk));
-        size_t hull = (size_t)k * 48 + 4096;
-        if (hull > (1u << 20)) hull = 1u << 20;
-        do {
-            VM_TRY(fit_out(fc, k, (uint32_t)(hull < 0xFFFFFFFFull ? hull : 0xFFFFFFFFull)));
+        for (;;) {
             char* d = fc.host_dev;
             VM_STAGE_BEGIN(hk, kStPack, s);
             VM_CUDA(launch_pack(fb, off, labels, fb.kdev, k, reinterpret_cast<vm_plane*>(d + out_planes_off()),
@@ -257,8 +257,10 @@ static vm_status fit_and_pack(FitContext& fc, const float* pts, const uint32_t* 
             VM_CUDA(cudaStreamSynchronize(s));
             fc.timer.fold();
             h = *static_cast<const FitHeader*>(fc.host);
+            if (h.n_hull <= fc.out_hcap) break;
             hull = (size_t)h.n_hull + h.n_hull / 4;
-        } while (h.n_hull > fc.out_hcap);
+            VM_TRY(fit_out(fc, k, (uint32_t)(hull < 0xFFFFFFFFull ? hull : 0xFFFFFFFFull)));
+        }
         if (!(h.err & kErrScratch)) break;
         if (attempt == 3) {
             set_error("fit scratch could not be sized for this batch");
