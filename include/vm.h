@@ -133,7 +133,8 @@ vm_status vm_create(const vm_map_params* params, void* cuda_stream, vm_map** out
  * Each point is transformed, keyed to its voxel, and accumulated as exact
  * fixed-point sums (2^-20 m units) plus a count; NaN/Inf points and points
  * outside the grid are dropped and counted.  Asynchronous on the map's stream
- * unless xyz is pageable host memory.  Errors: VM_ERR_INVALID_ARG,
+ * unless xyz is pageable host memory: xyz must stay valid until the stream has
+ * passed the call (the next call that synchronises it).  Errors: VM_ERR_INVALID_ARG,
  * VM_ERR_CUDA; a full brick pool is reported by the next vm_segment /
  * vm_get_stats as VM_ERR_CAPACITY. */
 vm_status vm_integrate(vm_map* map, const float* xyz, uint32_t n, const float pose3x4[12], int xyz_on_device);

@@ -266,6 +266,7 @@ class VoxelMap:
                           float(voxel_size), int(brick_capacity), flags)
         h = C.c_void_p()
         self._stream = stream
+        self._reading = []  # frames that the map's stream may still read
         _check(L.vm_create(C.byref(p), _stream_handle(stream), C.byref(h)))
         self._h = h
 
@@ -273,6 +274,7 @@ class VoxelMap:
         if getattr(self, "_h", None):
             load().vm_destroy(self._h)
             self._h = None
+            self._reading.clear()
 
     def __del__(self):
         try:
@@ -282,7 +284,8 @@ class VoxelMap:
 
     def integrate(self, xyz, pose, clear=False):
         """xyz: float32 [n, 3] torch tensor (CUDA or CPU) or numpy array; pose: 12 floats, sensor->map.
-        clear: first clear the voxels the points' rays pass through (Eq. 2)."""
+        clear: first clear the voxels the points' rays pass through (Eq. 2).  Returns before the frame has been
+        read; the map holds on to it until then."""
         pose = _pose(pose)
         on_dev = 1 if (hasattr(xyz, "is_cuda") and xyz.is_cuda) else 0
         if hasattr(xyz, "is_contiguous"):
@@ -292,6 +295,9 @@ class VoxelMap:
             xyz = np.ascontiguousarray(xyz, np.float32)
             n = xyz.size // 3
         order_after_torch(xyz, self._stream)
+        if len(self._reading) >= 64:  # frames without a segmentation in between
+            self.stats()
+        self._reading.append(xyz)
         _check(load().vm_integrate_ex(self._h, _ptr(xyz), n, pose, on_dev, VM_INTEGRATE_CLEAR if clear else 0))
 
     def segment(self, params: vm_segment_params | None = None):
@@ -301,6 +307,7 @@ class VoxelMap:
         try:
             if st not in (VM_OK, VM_ERR_CAPACITY):
                 _check(st)
+            self._reading.clear()  # the call waits for the map's stream
             res = _planes_to_numpy(out)
             res["status"] = st
         finally:
@@ -366,6 +373,7 @@ class VoxelMap:
         st = load().vm_get_stats(self._h, C.byref(s))
         if st not in (VM_OK, VM_ERR_CAPACITY):
             _check(st)
+        self._reading.clear()  # the call waits for the map's stream
         return {f: getattr(s, f) for f, _ in vm_stats._fields_} | {"status": st}
 
     def graph_shape(self):
