@@ -255,7 +255,8 @@ vm_status vm_fit_plan_create(uint32_t k_cap, uint32_t n_cap, const vm_segment_pa
 vm_status vm_fit_plan_run(vm_fit_plan* plan, const float* xyz, const uint32_t* off, const uint32_t* labels,
                           uint32_t k, vm_planes* out);
 /* Asynchronous half of a run: enqueues the fit on the plan's stream and
- * returns; vm_fit_plan_wait synchronises and fills *out (NULL: only waits).
+ * returns (the pointers must stay valid until the wait); vm_fit_plan_wait
+ * synchronises and fills *out (NULL: only waits).
  * One launch at a time per plan. */
 vm_status vm_fit_plan_launch(vm_fit_plan* plan, const float* xyz, const uint32_t* off, const uint32_t* labels,
                              uint32_t k);

@@ -447,7 +447,8 @@ def _tuning_dict(t: vm_fit_tuning):
 
 class FitPlan:
     """A reusable batched fit (vm_fit_plan_*): buffers sized once, the whole fit
-    replayed as one CUDA graph per run.  xyz, off, labels are CUDA tensors."""
+    replayed as one CUDA graph per run.  xyz, off, labels are CUDA tensors whose
+    values are there (a stream of the plan's own does not wait for torch's)."""
 
     def __init__(self, k_cap, n_cap, params: vm_segment_params | None = None, stream=None, eager=False,
                  stage_timing=False):
@@ -457,6 +458,7 @@ class FitPlan:
         _check(load().vm_fit_plan_create(int(k_cap), int(n_cap), C.byref(self.params), _stream_handle(stream),
                                          flags, C.byref(h)))
         self._h = h
+        self._reading = None  # the inputs of a launch in flight
 
     def stage_times(self):
         """{stage: (ms, calls)} since the previous call (plans made with stage_timing=True)."""
@@ -471,6 +473,7 @@ class FitPlan:
         if getattr(self, "_h", None):
             load().vm_fit_plan_destroy(self._h)
             self._h = None
+            self._reading = None
 
     def __del__(self):
         try:
@@ -488,10 +491,13 @@ class FitPlan:
             load().vm_planes_free(C.byref(out))
 
     def launch(self, xyz, off, labels=None):
+        """Enqueues the fit; the plan holds on to its inputs until wait."""
         _check(load().vm_fit_plan_launch(self._h, _ptr(xyz), _ptr(off), _ptr(labels), int(off.numel()) - 1))
+        self._reading = xyz, off, labels
 
     def wait(self):
         _check(load().vm_fit_plan_wait(self._h, None))
+        self._reading = None
 
     @property
     def tuning(self):

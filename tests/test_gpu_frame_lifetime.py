@@ -1,4 +1,5 @@
-"""GPU: a frame may be let go of as soon as integrate has been called, although
+"""GPU: a frame may be let go of as soon as integrate has been called, and the
+inputs of a fit as soon as it has been launched, although
 the map's stream reads it later: its memory, device or pinned, is not given to
 another tensor before."""
 import numpy as np
@@ -60,3 +61,22 @@ def test_frames_without_a_segmentation_are_let_go_of():
     m.segment(vm.segment_params(min_cluster=1))
     gc.collect()
     assert not any(r() is not None for r in kept)
+
+
+def test_a_launched_fit_holds_its_inputs_until_it_is_waited_for():
+    import gc
+    import weakref
+
+    import torch
+    from paper_2510_01592_gb300 import vm
+    plan = vm.FitPlan(4, 4000, vm.segment_params(n_hyp=32))
+    xyz, off = torch.rand(4000, 3, device="cuda"), torch.arange(0, 4001, 1000, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    refs = weakref.ref(xyz), weakref.ref(off)
+    plan.launch(xyz, off)
+    del xyz, off
+    gc.collect()
+    assert all(r() is not None for r in refs)
+    plan.wait()
+    gc.collect()
+    assert not any(r() is not None for r in refs)
